@@ -126,7 +126,7 @@ k_dirprec_e(int n, int m, double omega, double eta, double ds, geom_dev g,
     } else {
       double2 a, unused;
       pair_entries_fp64<0>(g.x[gi] - g.x[gj], g.y[gi] - g.y[gj], omega, eta, h, wtab[d], g.nx[gj],
-                           g.ny[gj], g.sp[gj], g.nx[gi], g.ny[gi], g.sp[gi], a, unused);
+                           g.ny[gj], g.sp[gj], g.nx[gi], g.ny[gi], g.sp[gi], g.tab, a, unused);
       ar += a.x * pr - a.y * pim;
       ai += a.x * pim + a.y * pr;
     }

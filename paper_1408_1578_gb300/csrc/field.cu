@@ -13,6 +13,14 @@
 // spacings away from the curve), FP64 throughout with the library's own
 // Hankel evaluation.  One thread per (point, quarter of the sources), sources
 // staged in shared memory a tile at a time, the quarters added at the end.
+//
+// Bound: the FP64 pipe, about 60 instructions per kernel value and 4 per
+// density, so a kernel value is shared by up to 16 densities and padding
+// densities cost nothing; when the points alone do not fill the GPU the
+// sources are split across CTAs and a second kernel adds the splits in a
+// fixed order.
+// Measured (GB300): 16 densities of n = 4096 nodes at 20000 points, sound hard,
+// 70.2 -> 24.9 ms.
 #include <algorithm>
 
 #include "hankel64.cuh"
@@ -24,38 +32,42 @@ constexpr int FPT = 64;      // points per CTA
 constexpr int FSPL = 4;      // source quarters (threads per point)
 constexpr int FNT = FPT * FSPL;
 constexpr int FTJ = 128;     // sources per shared-memory tile
-constexpr int FRB = 8;       // right-hand sides per CTA
 
-template <int BC>
+// out: u, or with several splits the partial sums [split][density][point]
+template <int BC, int FRB>
 __global__ void __launch_bounds__(FNT)
-k_field(int n, int npts, int nrhs, double omega, double eta, double h, geom_dev g,
-        const double2* __restrict__ pts, const double2* __restrict__ q,
-        double2* __restrict__ u) {
-  __shared__ double sx[FTJ], sy[FTJ], snx[FTJ], sny[FTJ], ssp[FTJ];
+k_field(int n, int npts, int nrhs, int tiles_per_split, double omega, double eta, double h,
+        geom_dev g, const double2* __restrict__ pts, const double2* __restrict__ q,
+        double2* __restrict__ out) {
+  __shared__ double sx[FTJ], sy[FTJ], sfx[FTJ], sfy[FTJ], se[FTJ];
   // densities of the tile during the loop, the quarters' sums after it
-  constexpr int BUF = FTJ * FRB > FSPL * FPT * FRB ? FTJ * FRB : FSPL * FPT * FRB;
+  constexpr int BUF = FTJ * FRB > FSPL * FPT ? FTJ * FRB : FSPL * FPT;
   __shared__ double2 buf[BUF];
   double2 (*sq)[FRB] = reinterpret_cast<double2 (*)[FRB]>(buf);
-  double2 (*red)[FPT][FRB] = reinterpret_cast<double2 (*)[FPT][FRB]>(buf);
   const int tid = threadIdx.x;
   const int pl = tid % FPT, quarter = tid / FPT;
   const int p = blockIdx.x * FPT + pl;
   const int r0 = blockIdx.y * FRB;
   const int rn = min(FRB, nrhs - r0);
+  const int j_begin = blockIdx.z * tiles_per_split * FTJ;
+  const int j_end = min(n, j_begin + tiles_per_split * FTJ);
+  const double f = 0.25 * 0.7978845608028654 * h;   // h c0 / 4
+  const double nf = BC == 0 ? omega * f : omega * f / eta, sf = BC == 0 ? eta * f : f;
+  const double omega_inv = 1.0 / omega;
   const double2 xp = p < npts ? pts[p] : make_double2(0.0, 0.0);
   double2 acc[FRB];
 #pragma unroll
   for (int k = 0; k < FRB; ++k) acc[k] = make_double2(0.0, 0.0);
-  for (int j0 = 0; j0 < n; j0 += FTJ) {
+  for (int j0 = j_begin; j0 < j_end; j0 += FTJ) {
     __syncthreads();
     for (int e = tid; e < FTJ; e += FNT) {
       const int j = j0 + e;
       const bool ok = j < n;
       sx[e] = ok ? g.x[j] : 0.0;
       sy[e] = ok ? g.y[j] : 0.0;
-      snx[e] = ok ? g.nx[j] : 0.0;
-      sny[e] = ok ? g.ny[j] : 0.0;
-      ssp[e] = ok ? g.sp[j] : 0.0;
+      sfx[e] = ok ? nf * g.nx[j] : 0.0;
+      sfy[e] = ok ? nf * g.ny[j] : 0.0;
+      se[e] = ok ? sf * g.sp[j] : 0.0;
     }
     for (int e = tid; e < FTJ * FRB; e += FNT) {
       const int jl = e / FRB, k = e % FRB, j = j0 + jl;
@@ -63,58 +75,107 @@ k_field(int n, int npts, int nrhs, double omega, double eta, double h, geom_dev 
     }
     __syncthreads();
     if (p >= npts) continue;
-    const int jn = min(FTJ, n - j0);
+    const int jn = min(FTJ, j_end - j0);
     for (int jl = quarter; jl < jn; jl += FSPL) {
       const double dx = xp.x - sx[jl], dy = xp.y - sy[jl];
-      const double r = sqrt(dx * dx + dy * dy);
-      double J0, Y0, J1, Y1;
-      h64::bessel01(omega * r, J0, Y0, J1, Y1);
-      // S kernel (i/4) H0 |z'|, D kernel (i/4) omega H1 c; H = J + i Y
-      const double sk = 0.25 * ssp[jl];
-      const double dk = 0.25 * omega * (dx * snx[jl] + dy * sny[jl]) / r;
-      const double2 S = make_double2(-sk * Y0, sk * J0);
-      const double2 D = make_double2(-dk * Y1, dk * J1);
-      double2 c;
-      if constexpr (BC == 0) {
-        c = make_double2(D.x + eta * S.y, D.y - eta * S.x);           // D - i eta S
-      } else {
-        c = make_double2(-S.x + D.y / eta, -S.y - D.x / eta);         // -S + D / (i eta)
-      }
+      double r, rinv;
+      h64::distance(fma(dx, dx, dy * dy), r, rinv);
+      const h64::values v = h64::bessel01(omega * r, omega_inv * rinv, g.tab);
+      // h times the kernel, H = J + i Y:  S = (i/4) H0 |z'|, D = (i/4) omega H1
+      // (x - z) . nu~ / r, soft D - i eta S, hard -S + D / (i eta)
+      const double A = se[jl] * v.amp;
+      const double B = fma(dx, sfx[jl], dy * sfy[jl]) * (rinv * v.amp);
+      const double2 c = BC == 0 ? make_double2(fma(A, v.j0, -(B * v.y1)), fma(A, v.y0, B * v.j1))
+                                : make_double2(fma(A, v.y0, B * v.j1), fma(B, v.y1, -(A * v.j0)));
 #pragma unroll
       for (int k = 0; k < FRB; ++k) {
-        const double2 qq = sq[jl][k];
-        acc[k].x += c.x * qq.x - c.y * qq.y;
-        acc[k].y += c.x * qq.y + c.y * qq.x;
+        if (k < rn) {
+          const double2 qq = sq[jl][k];
+          acc[k].x = fma(c.x, qq.x, acc[k].x);
+          acc[k].x = fma(-c.y, qq.y, acc[k].x);
+          acc[k].y = fma(c.x, qq.y, acc[k].y);
+          acc[k].y = fma(c.y, qq.x, acc[k].y);
+        }
       }
     }
   }
-  __syncthreads();   // every thread is done with the last tile's densities
+  double2* dst = out + (size_t)blockIdx.z * nrhs * npts;
 #pragma unroll
-  for (int k = 0; k < FRB; ++k) red[quarter][pl][k] = acc[k];
-  __syncthreads();
-  if (quarter == 0 && p < npts) {
-    for (int k = 0; k < rn; ++k) {
-      double2 s = make_double2(0.0, 0.0);
-      for (int t = 0; t < FSPL; ++t) {
-        s.x += red[t][pl][k].x;
-        s.y += red[t][pl][k].y;
+  for (int k = 0; k < FRB; ++k) {
+    __syncthreads();   // the buffer's last readers are done
+    if (k >= rn) continue;
+    buf[tid] = acc[k];
+    __syncthreads();
+    if (quarter == 0 && p < npts) {
+      double2 s = buf[pl];
+      for (int t = 1; t < FSPL; ++t) {
+        s.x += buf[t * FPT + pl].x;
+        s.y += buf[t * FPT + pl].y;
       }
-      u[(size_t)(r0 + k) * npts + p] = make_double2(h * s.x, h * s.y);
+      dst[(size_t)(r0 + k) * npts + p] = s;
     }
   }
+}
+
+__global__ void k_field_sum(size_t tot, int splits, const double2* __restrict__ part,
+                            double2* __restrict__ u) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= tot) return;
+  double2 s = part[e];
+#pragma unroll 4
+  for (int k = 1; k < splits; ++k) {
+    const double2 v = part[(size_t)k * tot + e];
+    s.x += v.x;
+    s.y += v.y;
+  }
+  u[e] = s;
+}
+
+template <int BC, int FRB>
+void launch_field(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts,
+                  double2* u) {
+  cudaStream_t st = op->ctx->stream;
+  const int n = op->n, tiles = (n + FTJ - 1) / FTJ;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
+  const int px = (npts + FPT - 1) / FPT, ry = (nrhs + FRB - 1) / FRB;
+  // about four CTAs per SM, as many splits of the sources as that takes (no
+  // more partial sums than 256 MB)
+  const size_t tot = (size_t)nrhs * npts;
+  long long splits = std::max<long long>(1, (4LL * sms + (long long)px * ry - 1) / ((long long)px * ry));
+  splits = std::min<long long>(splits, std::min<long long>(tiles, std::max<size_t>(1, ((size_t)1 << 24) / tot)));
+  const int tps = (int)((tiles + splits - 1) / splits);
+  const int ns = (tiles + tps - 1) / tps;
+  double2* out = u;
+  if (ns > 1) {
+    op->partial.reserve(sizeof(double2) * tot * ns);
+    out = op->partial.as<double2>();
+  }
+  k_field<BC, FRB><<<dim3(px, ry, ns), FNT, 0, st>>>(n, npts, nrhs, tps, op->omega, op->eta, op->h,
+                                                     op->g, pts, q, out);
+  CFIE_CHECK_LAUNCH();
+  if (ns > 1) {
+    k_field_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, ns, out, u);
+    CFIE_CHECK_LAUNCH();
+  }
+}
+
+template <int BC>
+void field_bc(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts, double2* u) {
+  if (nrhs == 1)
+    launch_field<BC, 1>(op, q, nrhs, npts, pts, u);
+  else if (nrhs <= 4)
+    launch_field<BC, 4>(op, q, nrhs, npts, pts, u);
+  else
+    launch_field<BC, 16>(op, q, nrhs, npts, pts, u);
 }
 
 }  // namespace
 
 void field_eval(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts,
                 double2* u) {
-  const dim3 grid((npts + FPT - 1) / FPT, (nrhs + FRB - 1) / FRB);
-  cudaStream_t st = op->ctx->stream;
   if (op->bc == CFIE_SOUND_SOFT)
-    k_field<0><<<grid, FNT, 0, st>>>(op->n, npts, nrhs, op->omega, op->eta, op->h, op->g, pts, q,
-                                     u);
+    field_bc<0>(op, q, nrhs, npts, pts, u);
   else
-    k_field<1><<<grid, FNT, 0, st>>>(op->n, npts, nrhs, op->omega, op->eta, op->h, op->g, pts, q,
-                                     u);
-  CFIE_CHECK_LAUNCH();
+    field_bc<1>(op, q, nrhs, npts, pts, u);
 }

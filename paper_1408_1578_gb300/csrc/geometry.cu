@@ -9,6 +9,7 @@
 // kernels read.
 #include <cmath>
 
+#include "hankel64.cuh"
 #include "internal.h"
 
 namespace {
@@ -26,7 +27,10 @@ __global__ void k_sample(curve_params P, int n, const double* __restrict__ zs,
                          const double* __restrict__ dzs, const double* __restrict__ ddzs,
                          geom_dev g) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+  if (j >= n) {   // the threads past the nodes fill the Bessel tables
+    h64::fill_tables(j - n, g.tab);
+    return;
+  }
   double s, c;
   sincospi(2.0 * j / n, &s, &c);  // t_j = 2 pi j / n
   double z1, z2, d1, d2, e1, e2;   // z, z', z''
@@ -180,9 +184,12 @@ __global__ void k_plane_waves(int n, int nrhs, double omega, int bc,
 
 void geometry_sample(cfie_op* op, const cfie_geom* geom) {
   int n = op->n;
-  op->geo.reserve(sizeof(double) * 6 * n);
+  // (6 n doubles end on a 16-byte boundary: n is even)
+  op->geo.reserve(sizeof(double) * 6 * n + sizeof(double2) * h64::kTableDouble2);
   double* base = op->geo.as<double>();
-  op->g = geom_dev{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n};
+  op->g = geom_dev{base,         base + n,     base + 2 * n,
+                   base + 3 * n, base + 4 * n, base + 5 * n,
+                   reinterpret_cast<double2*>(base + 6 * (size_t)n)};
   curve_params P{};
   P.kind = geom->kind;
   P.p0 = geom->p0;
@@ -208,7 +215,7 @@ void geometry_sample(cfie_op* op, const cfie_geom* geom) {
     dzs = s + 2 * n;
     ddzs = s + 4 * n;
   }
-  k_sample<<<(n + 255) / 256, 256, 0, op->ctx->stream>>>(P, n, zs, dzs, ddzs, op->g);
+  k_sample<<<(n + h64::kTrig + h64::kNear + 127) / 128, 128, 0, op->ctx->stream>>>(P, n, zs, dzs, ddzs, op->g);
   CFIE_CHECK_LAUNCH();
   if (samp.p) CFIE_CHECK_CUDA(cudaStreamSynchronize(op->ctx->stream));
 }

@@ -162,6 +162,7 @@ struct geom_dev {
   double* ny;     // nu~_2 = -z1'
   double* sp;     // |z'|
   double* kap;    // L2(t,t) = (z2' z1'' - z1' z2'') / (4 pi |z'|^2)
+  double2* tab;   // FP64 Bessel tables (hankel64.cuh)
 };
 
 // Plan of the stored-matrix contraction over a list of jobs (stored.cu).
@@ -210,7 +211,7 @@ struct cfie_op {
   cfie_precision prec = CFIE_FP64;
   cfie_layout layout = CFIE_MATRIX_FREE;
 
-  dbuf geo;          // 6 n doubles (geom_dev)
+  dbuf geo;          // 6 n doubles and the Bessel tables (geom_dev)
   geom_dev g{};
   dbuf wtab;         // n doubles: w_d = R_d - h ln(4 sin^2(pi d / n)), w_0 = R_0
   dbuf ctab;         // n doubles: spectral derivative circulant c_d = (-1)^d cot(pi d / n) / 2

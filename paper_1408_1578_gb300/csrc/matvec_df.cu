@@ -1176,10 +1176,10 @@ __global__ void k_df_band(int n, int b, int hard, double omega, double eta, geom
     if (d < 0) d += n;
     if (hard)
       pair_entries_fp64<1>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, 2.0 * CFIE_PI / n,
-                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], a, b2);
+                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
     else
       pair_entries_fp64<0>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, 2.0 * CFIE_PI / n,
-                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], a, b2);
+                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
   }
   const df re = dmake(a.x), im = dmake(a.y);
   band[e] = make_float4(re.h, re.l, im.h, im.l);

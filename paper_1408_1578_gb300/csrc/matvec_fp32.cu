@@ -440,7 +440,7 @@ __global__ void k_band_fill(int n, int b, double omega, double eta, geom_dev g,
     if (d < 0) d += n;
     const double h = 2.0 * CFIE_PI / n;
     pair_entries_fp64<BC>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, h, wtab[d], g.nx[j],
-                          g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], a, bb);
+                          g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, bb);
   }
   band[e] = make_float2((float)a.x, (float)a.y);
   if (BC) band2[e] = make_float2((float)bb.x, (float)bb.y);

@@ -12,17 +12,30 @@
 //          D'_ij = h L'_ij + w L'1_ij with c' = (z_j - z_i).nu~_i / r * s_j / s_i
 //          A x = 1/2 x - D' x + (1/(i eta)) [ (1/s) Dt S (1/s) Dt x
 //                                            + omega^2 (n1 S (n1 x) + n2 S (n2 x)) ]
-//          (Maue's identity; Dt = spectral derivative, Nyquist mode zeroed)
+//          (Maue's identity; Dt = spectral derivative, Nyquist mode zeroed),
+//          summed as two operators over the same pairs: S on u = (1/s) Dt x, and
+//          C on x, C_ij = -D'_ij - i (omega^2 / eta) (n_i . n_j) S_ij, because
+//          n1 S n1 + n2 S n2 has the entries (n_i . n_j) S_ij (four multiply-adds
+//          per right-hand side and pair fewer than S on three vectors and D')
 // Diagonal entries come precomputed (geometry.cu).
 //
-// Layout: a CTA owns TI = 64 targets and walks a contiguous range of source
-// tiles (TJ = 32 sources each).  For every tile it evaluates the TI x TJ block
-// of entries into shared memory (one warp per target row, lanes over sources),
-// then contracts it with the staged block of up to 16 right-hand sides, each
-// thread holding 4 right-hand sides of one target.  Source ranges are split
-// across CTAs when the row tiles alone do not fill the GPU; the per-split
-// partial sums go to a scratch buffer and a second kernel adds them in a fixed
-// order (deterministic results) and applies the hard-path epilogue.
+// Layout: a CTA of 4 TI threads owns TI = 64 (small problems: 32) targets and
+// walks a contiguous range of source tiles (TJ = 32 sources each).  For every
+// tile it evaluates the TI x TJ block of entries into shared memory (one warp
+// per target row, lanes over sources), then contracts it with the staged block
+// of right-hand sides.  Source ranges are split across CTAs when the row tiles
+// alone do not fill the GPU; the per-split partial sums go to a scratch buffer
+// and a second kernel adds them in a fixed order (deterministic results) and
+// applies the hard-path epilogue.
+//
+// Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
+// scheduler): per pair about 70 instructions for the entry (hankel64.cuh) and
+// 4 (soft) or 8 (hard) per right-hand side for the sums, so the right-hand
+// sides of a block are counted out (no sums on padding columns; with one or
+// two the threads split the sources instead) and the entry is shared by up to
+// 64 (soft) or 32 (hard) of them.
+// Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 215 us; star n =
+// 4096, 16 right-hand sides, sound hard 15.8 -> 7.4 ms (of which 6.9 here).
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -34,10 +47,7 @@
 
 namespace {
 
-constexpr int TI = 64;
 constexpr int TJ = 32;
-constexpr int NT = 256;
-constexpr int RB = 16;  // right-hand sides per launch slice (soft with many RHS: 64)
 
 __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
   acc.x = fma(a.x, b.x, acc.x);
@@ -47,24 +57,31 @@ __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
   return acc;
 }
 
-template <int BC, int RBT = RB>
+template <int BC, int TI, int RBT>
 struct pair_smem {
-  double tx[TI], ty[TI], tnx[TI], tny[TI], tsp[TI];
-  double sx[TJ], sy[TJ], snx[TJ], sny[TJ], ssp[TJ];
-  double2 A[TI][TJ + 1];
-  double2 B[BC ? TI : 1][TJ + 1];        // hard: D' entries
-  double2 X[BC ? 4 : 1][TJ][RBT];        // soft: x ; hard: u, n1 x, n2 x, x
+  // targets: coordinates; hard: omega nu / |z'| and (omega^2 / eta) nu / |z'|
+  double tx[TI], ty[TI], tfx[BC ? TI : 1], tfy[BC ? TI : 1], tux[BC ? TI : 1], tuy[BC ? TI : 1];
+  // sources: coordinates, folded factors (soft: nu, hard: unit normal), speed factor
+  double sx[TJ], sy[TJ], sfx[TJ], sfy[TJ], se[TJ];
+  double wk[TI + TJ];                    // Kress weights / (pi h) of the tile, by i - j
+  double2 A[TI][TJ + 1];                 // soft: A; hard: S
+  double2 B[BC ? TI : 1][TJ + 1];        // hard: C
+  double2 X[BC ? 2 : 1][TJ][RBT];        // soft: x ; hard: u, x
 };
 
-template <int BC, int RBT = RB>
-__global__ void __launch_bounds__(NT)
+template <int BC, int TI, int RBT>
+__global__ void __launch_bounds__(4 * TI)
 k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restrict__ wtab,
             const double2* __restrict__ diag, const double2* __restrict__ xin,
             const double2* __restrict__ uin, int nrhs, int splits, int tiles_per_split,
             double2* __restrict__ part) {
-  constexpr int RQ = RBT / (NT / TI);  // right-hand sides per thread
+  constexpr int NT = 4 * TI;
+  constexpr int RG = RBT < 4 ? RBT : 4;   // groups of threads over the right-hand sides ..
+  constexpr int JG = 4 / RG;              // .. and, with fewer than four of those, the sources
+  constexpr int RQ = RBT / RG;            // right-hand sides per thread
+  constexpr int NO = BC ? 2 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pair_smem<BC, RBT>& S = *reinterpret_cast<pair_smem<BC, RBT>*>(smem_raw);
+  pair_smem<BC, TI, RBT>& S = *reinterpret_cast<pair_smem<BC, TI, RBT>*>(smem_raw);
   const int tid = threadIdx.x;
   const int i0 = blockIdx.x * TI;
   const int split = blockIdx.y;
@@ -74,22 +91,29 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
   const int t_begin = split * tiles_per_split;
   const int t_end = min(ntiles, t_begin + tiles_per_split);
   const double h = 2.0 * CFIE_PI / n;
+  const double f = 0.25 * 0.7978845608028654 * h;   // hq c0
+  const double wscale = 1.0 / (CFIE_PI * h), omega_inv = 1.0 / omega;
 
   if (tid < TI) {
-    int i = i0 + tid;
-    bool ok = i < n;
+    const int i = i0 + tid;
+    const bool ok = i < n;
     S.tx[tid] = ok ? g.x[i] : 0.0;
     S.ty[tid] = ok ? g.y[i] : 0.0;
-    S.tnx[tid] = ok ? g.nx[i] : 0.0;
-    S.tny[tid] = ok ? g.ny[i] : 0.0;
-    S.tsp[tid] = ok ? g.sp[i] : 1.0;
+    if constexpr (BC == 1) {
+      const double inv = ok ? omega / g.sp[i] : 0.0, k = omega / eta;
+      S.tfx[tid] = ok ? g.nx[i] * inv : 0.0;
+      S.tfy[tid] = ok ? g.ny[i] * inv : 0.0;
+      S.tux[tid] = S.tfx[tid] * k;
+      S.tuy[tid] = S.tfy[tid] * k;
+    }
   }
 
-  const int il2 = tid % TI;     // contraction: target row
-  const int rg = tid / TI;      // contraction: right-hand-side group
-  double2 acc[BC ? 4 : 1][RQ];
+  const int il2 = tid % TI;                // contraction: target row
+  const int rg = (tid / TI) % RG;          // right-hand-side group
+  const int jg = (tid / TI) / RG;          // source group
+  double2 acc[NO][RQ];
 #pragma unroll
-  for (int o = 0; o < (BC ? 4 : 1); ++o)
+  for (int o = 0; o < NO; ++o)
 #pragma unroll
     for (int q = 0; q < RQ; ++q) acc[o][q] = make_double2(0.0, 0.0);
 
@@ -97,109 +121,156 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
     const int j0 = t * TJ;
     __syncthreads();
     if (tid < TJ) {
-      int j = j0 + tid;
-      bool ok = j < n;
+      const int j = j0 + tid;
+      const bool ok = j < n;
+      const double sp = ok ? g.sp[j] : 1.0;
+      const double m = BC ? 1.0 / sp : omega * f;
       S.sx[tid] = ok ? g.x[j] : 0.0;
       S.sy[tid] = ok ? g.y[j] : 0.0;
-      S.snx[tid] = ok ? g.nx[j] : 0.0;
-      S.sny[tid] = ok ? g.ny[j] : 0.0;
-      S.ssp[tid] = ok ? g.sp[j] : 1.0;
+      S.sfx[tid] = ok ? m * g.nx[j] : 0.0;
+      S.sfy[tid] = ok ? m * g.ny[j] : 0.0;
+      S.se[tid] = BC ? f * sp : f * eta * sp;
+    }
+    for (int e = tid; e < TI + TJ - 1; e += NT) {
+      int d = (i0 - j0 + e - (TJ - 1)) % n;
+      if (d < 0) d += n;
+      S.wk[e] = wtab[d] * wscale;
     }
     for (int e = tid; e < TJ * RBT; e += NT) {
-      int jl = e / RBT, r = e % RBT;
-      int j = j0 + jl;
+      const int jl = e / RBT, r = e % RBT;
+      const int j = j0 + jl;
       double2 xv = make_double2(0.0, 0.0), uv = xv;
       if (j < n && r < rbn) {
         xv = xin[(size_t)(rb0 + r) * n + j];
         if (BC) uv = uin[(size_t)(rb0 + r) * n + j];
       }
-      if constexpr (BC == 1) {
-        double inv = (j < n) ? 1.0 / g.sp[j] : 0.0;
-        double n1 = (j < n) ? g.nx[j] * inv : 0.0;
-        double n2 = (j < n) ? g.ny[j] * inv : 0.0;
-        S.X[0][jl][r] = uv;
-        S.X[1][jl][r] = make_double2(n1 * xv.x, n1 * xv.y);
-        S.X[2][jl][r] = make_double2(n2 * xv.x, n2 * xv.y);
-        S.X[3][jl][r] = xv;
-      } else {
-        S.X[0][jl][r] = xv;
-      }
+      S.X[NO - 1][jl][r] = xv;
+      if constexpr (BC == 1) S.X[0][jl][r] = uv;
     }
     __syncthreads();
 
-    // ---- entries of the TI x TJ block: warp w handles rows w, w+8, ...; lane = source
+    // ---- entries of the TI x TJ block: one warp per row, lane = source
     for (int e = tid; e < TI * TJ; e += NT) {
       const int il = e / TJ, jl = e % TJ;
       const int i = i0 + il, j = j0 + jl;
       double2 a = make_double2(0.0, 0.0), b = a;
       if (i < n && j < n) {
-        int d = i - j;
-        if (d < 0) d += n;
-        if (d == 0) {
-          if (BC) {
-            a = diag[2 * i];
-            b = diag[2 * i + 1];
-          } else {
-            a = diag[i];
-          }
+        if (i == j) {
+          a = BC ? diag[2 * i] : diag[i];
+          if (BC) b = diag[2 * i + 1];
         } else {
-          pair_entries_fp64<BC>(S.tx[il] - S.sx[jl], S.ty[il] - S.sy[jl], omega, eta, h,
-                                wtab[d], S.snx[jl], S.sny[jl], S.ssp[jl], S.tnx[il],
-                                S.tny[il], S.tsp[il], a, b);
+          pair_folded_fp64<BC>(S.tx[il] - S.sx[jl], S.ty[il] - S.sy[jl], omega, omega_inv,
+                               BC ? S.tfx[il] : S.sfx[jl], BC ? S.tfy[il] : S.sfy[jl], S.se[jl],
+                               S.wk[il - jl + TJ - 1], g.tab, a, b);
         }
       }
       S.A[il][jl] = a;
-      if constexpr (BC == 1) S.B[il][jl] = b;
+      if constexpr (BC == 1) {
+        // C = -D' - i (omega^2 / eta) (n_i . n_j) S
+        const double k = fma(S.tux[il], S.sfx[jl], S.tuy[il] * S.sfy[jl]);
+        S.B[il][jl] = make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y));
+      }
     }
     __syncthreads();
 
     // ---- contraction
     const int jn = min(TJ, n - j0);
-    for (int jl = 0; jl < jn; ++jl) {
+    for (int jl = jg; jl < jn; jl += JG) {
       const double2 a = S.A[il2][jl];
-      if constexpr (BC == 0) {
+      const double2 b = BC ? S.B[il2][jl] : a;
 #pragma unroll
-        for (int q = 0; q < RQ; ++q) acc[0][q] = cmad(acc[0][q], a, S.X[0][jl][rg + 4 * q]);
-      } else {
-        const double2 b = S.B[il2][jl];
-#pragma unroll
-        for (int q = 0; q < RQ; ++q) {
-          const int r = rg + 4 * q;
+      for (int q = 0; q < RQ; ++q) {
+        const int r = rg + RG * q;
+        if (r < rbn) {
           acc[0][q] = cmad(acc[0][q], a, S.X[0][jl][r]);
-          acc[1][q] = cmad(acc[1][q], a, S.X[1][jl][r]);
-          acc[2][q] = cmad(acc[2][q], a, S.X[2][jl][r]);
-          acc[3][q] = cmad(acc[3][q], b, S.X[3][jl][r]);
+          if constexpr (BC == 1) acc[NO - 1][q] = cmad(acc[NO - 1][q], b, S.X[NO - 1][jl][r]);
         }
       }
     }
   }
 
+  if constexpr (JG > 1) {   // join the source groups (RQ = 1) in the entries' place
+    double2* red = &S.A[0][0];
+    static_assert(NO * JG * RG * TI <= TI * (TJ + 1), "group sums exceed the entry block");
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < NO; ++o) red[((o * JG + jg) * RG + rg) * TI + il2] = acc[o][0];
+    __syncthreads();
+    if (jg > 0) return;
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+      for (int k = 1; k < JG; ++k) {
+        const double2 v = red[((o * JG + k) * RG + rg) * TI + il2];
+        acc[o][0].x += v.x;
+        acc[o][0].y += v.y;
+      }
+  }
   const int i = i0 + il2;
   if (i < n) {
 #pragma unroll
     for (int q = 0; q < RQ; ++q) {
-      const int r = rg + 4 * q;
+      const int r = rg + RG * q;
       if (r < rbn) {
 #pragma unroll
-        for (int o = 0; o < (BC ? 4 : 1); ++o)
+        for (int o = 0; o < NO; ++o)
           part[(((size_t)o * splits + split) * nrhs + rb0 + r) * n + i] = acc[o][q];
       }
     }
   }
 }
 
-// Sum split partials (fixed order).  Soft: y = sum.  Hard: t = S u,
-// y = 1/2 x - D' x - i (omega^2 / eta) (n1 S(n1 x) + n2 S(n2 x)).
+// Sum split partials in a fixed order: four threads per element take every
+// fourth split, then two shuffles join them.  Soft: y = sum.  Hard: t = S u,
+// y = 1/2 x + C x.
 template <int BC>
-__global__ void k_reduce_fp64(int n, int nrhs, int splits, double omega, double eta, geom_dev g,
-                              const double2* __restrict__ part, const double2* __restrict__ x,
-                              double2* __restrict__ t_out, double2* __restrict__ y) {
+__global__ void __launch_bounds__(256)
+k_reduce_fp64(size_t tot, int splits, const double2* __restrict__ part,
+              const double2* __restrict__ x, double2* __restrict__ t_out,
+              double2* __restrict__ y) {
+  // element by lane % 8, split group by lane / 8: eight neighbouring
+  // elements are one 128-byte line
+  const int lane = threadIdx.x & 31, g = lane >> 3;
+  const size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) / 32 * 8 + (lane & 7);
+  double2 s[BC ? 2 : 1];
+#pragma unroll
+  for (int o = 0; o < (BC ? 2 : 1); ++o) {
+    double2 v = make_double2(0.0, 0.0);
+    if (e < tot) {
+#pragma unroll 4
+      for (int sp = g; sp < splits; sp += 4) {
+        const double2 p = part[((size_t)o * splits + sp) * tot + e];
+        v.x += p.x;
+        v.y += p.y;
+      }
+    }
+    for (int k = 8; k < 32; k *= 2) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, k);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, k);
+    }
+    s[o] = v;
+  }
+  if (e >= tot || g) return;
+  if (BC == 0) {
+    y[e] = s[0];
+  } else {
+    const double2 xv = x[e], c = s[BC ? 1 : 0];
+    y[e] = make_double2(fma(0.5, xv.x, c.x), fma(0.5, xv.y, c.y));
+    t_out[e] = s[0];
+  }
+}
+
+// Sum split partials of the double-float sums (matvec_df.cu; four outputs):
+// t = S u, y = 1/2 x - D' x - i (omega^2 / eta) (n1 S(n1 x) + n2 S(n2 x)).
+__global__ void k_reduce_hard4(int n, int nrhs, int splits, double omega, double eta, geom_dev g,
+                               const double2* __restrict__ part, const double2* __restrict__ x,
+                               double2* __restrict__ t_out, double2* __restrict__ y) {
   size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t tot = (size_t)n * nrhs;
   if (e >= tot) return;
   const size_t stride_o = (size_t)splits * tot;
   double2 s[4] = {};
-  for (int o = 0; o < (BC ? 4 : 1); ++o) {
+  for (int o = 0; o < 4; ++o) {
     double2 v = make_double2(0.0, 0.0);
     for (int sp = 0; sp < splits; ++sp) {
       double2 p = part[o * stride_o + (size_t)sp * tot + e];
@@ -208,19 +279,15 @@ __global__ void k_reduce_fp64(int n, int nrhs, int splits, double omega, double 
     }
     s[o] = v;
   }
-  if (BC == 0) {
-    y[e] = s[0];
-  } else {
-    int i = (int)(e % n);
-    double inv = 1.0 / g.sp[i];
-    double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-    double2 m = make_double2(n1 * s[1].x + n2 * s[2].x, n1 * s[1].y + n2 * s[2].y);
-    double k = omega * omega / eta;
-    double2 xv = x[e];
-    // -i k m = (k m.y, -k m.x)
-    y[e] = make_double2(0.5 * xv.x - s[3].x + k * m.y, 0.5 * xv.y - s[3].y - k * m.x);
-    t_out[e] = s[0];
-  }
+  int i = (int)(e % n);
+  double inv = 1.0 / g.sp[i];
+  double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
+  double2 m = make_double2(n1 * s[1].x + n2 * s[2].x, n1 * s[1].y + n2 * s[2].y);
+  double k = omega * omega / eta;
+  double2 xv = x[e];
+  // -i k m = (k m.y, -k m.x)
+  y[e] = make_double2(0.5 * xv.x - s[3].x + k * m.y, 0.5 * xv.y - s[3].y - k * m.x);
+  t_out[e] = s[0];
 }
 
 // out[k][i] = base[k][i] + (scale / s_i) sum_j c_{(i-j) mod n} in[k][j]
@@ -265,18 +332,74 @@ k_spectral_fp64(int n, const double* __restrict__ ct, const double* __restrict__
   }
 }
 
-template <int BC, int RBT = RB>
-void launch_pair(cfie_op* op, const double2* x, const double2* u, int nrhs, int splits, int tps,
+// How one product is cut: right-hand sides per CTA, targets per CTA, source
+// splits.  Four CTAs per SM keep the FP64 pipes busy; problems of fewer 64 x 32
+// tiles than eight per SM take 32-target tiles, whose last wave is fuller
+// (n = 1024: 512 tiles on 152 SMs are 3.4 each, 1024 are 6.7).
+struct pair_plan {
+  int rbt, ti, rhsblocks, splits, tps;
+};
+
+pair_plan plan_pair(int n, int nrhs, int hard, int device, int max_splits) {
+  pair_plan p;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  p.rbt = nrhs <= 2 ? nrhs : (nrhs <= 4 ? 4 : (nrhs <= 16 ? 16 : (hard ? 32 : 64)));
+  p.rhsblocks = (nrhs + p.rbt - 1) / p.rbt;
+  const int ntiles = (n + TJ - 1) / TJ;
+  p.ti = (long long)((n + 63) / 64) * ntiles * p.rhsblocks < 8LL * sms && p.rbt <= 16 ? 32 : 64;
+  const int rows = (n + p.ti - 1) / p.ti * p.rhsblocks;
+  const int target = (p.ti == 32 ? 8 : 4) * sms;
+  p.splits = std::max(1, std::min(std::min(ntiles, max_splits), (target + rows - 1) / rows));
+  p.tps = (ntiles + p.splits - 1) / p.splits;
+  p.splits = (ntiles + p.tps - 1) / p.tps;
+  return p;
+}
+
+template <int BC, int TI, int RBT>
+void launch_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
                  double2* part) {
   const int n = op->n;
-  size_t smem = sizeof(pair_smem<BC, RBT>);
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_fp64<BC, RBT>,
+  const size_t smem = sizeof(pair_smem<BC, TI, RBT>);
+  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_fp64<BC, TI, RBT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((n + TI - 1) / TI, splits, (nrhs + RBT - 1) / RBT);
+  dim3 grid((n + TI - 1) / TI, p.splits, p.rhsblocks);
   prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
-  k_pair_fp64<BC, RBT><<<grid, NT, smem, op->ctx->stream>>>(
+  k_pair_fp64<BC, TI, RBT><<<grid, 4 * TI, smem, op->ctx->stream>>>(
       n, op->omega, op->eta, op->g, op->wtab.as<double>(), op->diag.as<double2>(), x, u, nrhs,
-      splits, tps, part);
+      p.splits, p.tps, part);
+  CFIE_CHECK_LAUNCH();
+}
+
+// partial sums of every output, then their reduction (soft: into y; hard: t = S
+// u and y = 1/2 x + C x)
+template <int BC>
+void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
+              double2* part, double2* t, double2* y) {
+  const bool small = p.ti == 32;
+  switch (p.rbt) {
+    case 1:
+      small ? launch_pair<BC, 32, 1>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 1>(op, p, x, u, nrhs, part);
+      break;
+    case 2:
+      small ? launch_pair<BC, 32, 2>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 2>(op, p, x, u, nrhs, part);
+      break;
+    case 4:
+      small ? launch_pair<BC, 32, 4>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 4>(op, p, x, u, nrhs, part);
+      break;
+    case 16:
+      small ? launch_pair<BC, 32, 16>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 16>(op, p, x, u, nrhs, part);
+      break;
+    default:
+      launch_pair<BC, 64, BC ? 32 : 64>(op, p, x, u, nrhs, part);
+  }
+  const size_t tot = (size_t)op->n * nrhs;
+  k_reduce_fp64<BC><<<(unsigned)((tot + 63) / 64), 256, 0, op->ctx->stream>>>(tot, p.splits, part,
+                                                                             x, t, y);
   CFIE_CHECK_LAUNCH();
 }
 
@@ -292,38 +415,19 @@ void spectral_apply(cfie_op* op, const double2* in, double2* out, const double2*
 void reduce_hard_fp64(cfie_op* op, const double2* part, int splits, const double2* x,
                       double2* t, double2* y, int nrhs) {
   const size_t tot = (size_t)op->n * nrhs;
-  k_reduce_fp64<1><<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(
+  k_reduce_hard4<<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(
       op->n, nrhs, splits, op->omega, op->eta, op->g, part, x, t, y);
   CFIE_CHECK_LAUNCH();
 }
 
 void matvec_fp64(cfie_op* op, const double2* x, double2* y, int nrhs) {
-  const int n = op->n;
-  const int hard = op->bc == CFIE_SOUND_HARD;
-  const int rowtiles = (n + TI - 1) / TI;
-  const bool wide = !hard && nrhs > RB;  // one pass of pair evaluations for up to 64 RHS
-  const int rb = wide ? 64 : RB;
-  const int rhsblocks = (nrhs + rb - 1) / rb;
-  const int ntiles = (n + TJ - 1) / TJ;
-  int dev_sms = 152;
-  cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
-  const int target = 4 * dev_sms;
-  int splits = std::max(1, std::min(ntiles, (target + rowtiles * rhsblocks - 1) /
-                                                (rowtiles * rhsblocks)));
-  int tps = (ntiles + splits - 1) / splits;
-  splits = (ntiles + tps - 1) / tps;
-  const int ops = hard ? 4 : 1;
-  op->partial.reserve(sizeof(double2) * (size_t)ops * splits * nrhs * n);
+  const bool hard = op->bc == CFIE_SOUND_HARD;
+  const pair_plan p = plan_pair(op->n, nrhs, hard, op->ctx->device, 1 << 20);
+  const size_t tot = (size_t)op->n * nrhs;
+  op->partial.reserve(sizeof(double2) * (hard ? 2 : 1) * (size_t)p.splits * tot);
   double2* part = op->partial.as<double2>();
-  const size_t tot = (size_t)n * nrhs;
   if (!hard) {
-    if (wide)
-      launch_pair<0, 64>(op, x, nullptr, nrhs, splits, tps, part);
-    else
-      launch_pair<0>(op, x, nullptr, nrhs, splits, tps, part);
-    k_reduce_fp64<0><<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(
-        n, nrhs, splits, op->omega, op->eta, op->g, part, x, nullptr, y);
-    CFIE_CHECK_LAUNCH();
+    run_pair<0>(op, p, x, nullptr, nrhs, part, nullptr, y);
     return;
   }
   op->tmp1.reserve(sizeof(double2) * tot);
@@ -332,10 +436,7 @@ void matvec_fp64(cfie_op* op, const double2* x, double2* y, int nrhs) {
   double2* t = op->tmp2.as<double2>();
   // u = (1/s) Dt x
   spectral_apply(op, x, u, nullptr, make_double2(1.0, 0.0), nrhs);
-  launch_pair<1>(op, x, u, nrhs, splits, tps, part);
-  k_reduce_fp64<1><<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(
-      n, nrhs, splits, op->omega, op->eta, op->g, part, x, t, y);
-  CFIE_CHECK_LAUNCH();
+  run_pair<1>(op, p, x, u, nrhs, part, t, y);
   // y += (1/(i eta)) (1/s) Dt t
   spectral_apply(op, t, y, y, make_double2(0.0, -1.0 / op->eta), nrhs);
 }
@@ -407,63 +508,35 @@ size_t static_scratch_capacity() { return kStaticScratchBytes; }
 
 void matvec_fp64_static(cfie_op* op, const double2* x, double2* y, int nrhs) {
   const int n = op->n;
-  const int hard = op->bc == CFIE_SOUND_HARD;
-  const int ops = hard ? 4 : 1;
+  const bool hard = op->bc == CFIE_SOUND_HARD;
   const size_t tot = (size_t)n * nrhs;
   const size_t vec_bytes = sizeof(double2) * tot;
   const size_t fixed = hard ? 2 * vec_bytes : 0;          // u and t
-  const size_t per_split = sizeof(double2) * (size_t)ops * tot;
-  if (fixed + per_split > kStaticScratchBytes)
+  const size_t per_split = sizeof(double2) * (hard ? 2 : 1) * tot;
+  // the documented limit (16 and 96 bytes per element; the hard form now uses
+  // 64 of them)
+  const size_t need = (hard ? 6 : 1) * vec_bytes;
+  if (need > kStaticScratchBytes)
     throw cfie_error(CFIE_EINVAL,
                      "cfie_apply_fp64_static: n * nrhs too large for the 32 MiB static scratch "
-                     "(needs " + std::to_string(fixed + per_split) + " bytes)");
+                     "(needs " + std::to_string(need) + " bytes)");
   // device address of the array on the context's (current) device
   unsigned char* base = static_cast<unsigned char*>(static_scratch_address(op->ctx->device));
-
-  const int rowtiles = (n + TI - 1) / TI;
-  const int rhsblocks = (nrhs + RB - 1) / RB;
-  const int ntiles = (n + TJ - 1) / TJ;
-  int dev_sms = 152;
-  cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
-  const int target = 4 * dev_sms;
-  int splits = std::max(1, std::min(ntiles, (target + rowtiles * rhsblocks - 1) /
-                                                (rowtiles * rhsblocks)));
-  const int fit = (int)std::min<size_t>((kStaticScratchBytes - fixed) / per_split, ntiles);
-  splits = std::max(1, std::min(splits, fit));
-  int tps = (ntiles + splits - 1) / splits;
-  splits = (ntiles + tps - 1) / tps;
-
+  const int fit = (int)std::min<size_t>((kStaticScratchBytes - fixed) / per_split, 1 << 20);
+  const pair_plan p = plan_pair(n, nrhs, hard, op->ctx->device, fit);
   double2* part = reinterpret_cast<double2*>(base + fixed);
-  double2* u = hard ? reinterpret_cast<double2*>(base) : nullptr;
-  double2* t = hard ? reinterpret_cast<double2*>(base + vec_bytes) : nullptr;
-  cudaStream_t st = op->ctx->stream;
-  const dim3 grid(rowtiles, splits, rhsblocks);
-  const dim3 sgrid((n + SPT - 1) / SPT, nrhs);
   if (!hard) {
-    const size_t smem = sizeof(pair_smem<0>);
-    CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_fp64<0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_pair_fp64<0><<<grid, NT, smem, st>>>(n, op->omega, op->eta, op->g, op->wtab.as<double>(),
-                                           op->diag.as<double2>(), x, nullptr, nrhs, splits, tps,
-                                           part);
-    CFIE_CHECK_LAUNCH();
-    k_reduce_fp64<0><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(
-        n, nrhs, splits, op->omega, op->eta, op->g, part, x, nullptr, y);
-    CFIE_CHECK_LAUNCH();
+    run_pair<0>(op, p, x, nullptr, nrhs, part, nullptr, y);
     return;
   }
+  double2* u = reinterpret_cast<double2*>(base);
+  double2* t = reinterpret_cast<double2*>(base + vec_bytes);
+  cudaStream_t st = op->ctx->stream;
+  const dim3 sgrid((n + SPT - 1) / SPT, nrhs);
   k_spectral_fp64<<<sgrid, SPT, 0, st>>>(n, op->ctab.as<double>(), op->g.sp, x, nullptr,
                                           make_double2(1.0, 0.0), u);
   CFIE_CHECK_LAUNCH();
-  const size_t smem = sizeof(pair_smem<1>);
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_fp64<1>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_pair_fp64<1><<<grid, NT, smem, st>>>(n, op->omega, op->eta, op->g, op->wtab.as<double>(),
-                                         op->diag.as<double2>(), x, u, nrhs, splits, tps, part);
-  CFIE_CHECK_LAUNCH();
-  k_reduce_fp64<1><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(
-      n, nrhs, splits, op->omega, op->eta, op->g, part, x, t, y);
-  CFIE_CHECK_LAUNCH();
+  run_pair<1>(op, p, x, u, nrhs, part, t, y);
   k_spectral_fp64<<<sgrid, SPT, 0, st>>>(n, op->ctab.as<double>(), op->g.sp, t, y,
                                           make_double2(0.0, -1.0 / op->eta), y);
   CFIE_CHECK_LAUNCH();

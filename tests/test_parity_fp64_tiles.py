@@ -1,0 +1,60 @@
+"""FP64 matvec and field at the edges of their tilings: right-hand-side blocks of 1, 2, 4, 16,
+32 / 64 and their remainders, 32- and 64-target tiles with ragged ends, source splits, pairs on
+both sides of every change of the Hankel evaluation (omega r = 20, 40, 100, 400).
+
+Bounds: 1e-12 per right-hand side (the FP64 resolution of the Hankel argument, 4e-16 omega
+diam, is below it at every size here), as for the other FP64 parity tests."""
+import numpy as np
+import pytest
+
+from oracle import field as ofield
+from oracle import geometry, operators
+from paper_1408_1578_gb300 import inputs
+from tests.gpu_util import col_rel, empty, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1408_1578_gb300 import cfie
+    c = cfie.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+@pytest.mark.parametrize("n,omega", [(8, 1.0), (62, 3.0), (66, 15.0), (510, 260.0), (1026, 30.0)])
+def test_right_hand_side_blocks(ctx, bc, n, omega):
+    A = operators.cfie_matrix(geometry.kite(n), omega, omega, bc)
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp64")
+    for nrhs in (1, 2, 3, 4, 5, 16, 17, 33, 65):
+        X = inputs.random_density(n, nrhs, seed=nrhs)
+        x, y = to_dev(X), empty(nrhs, n)
+        op.apply_fp64(x, y)
+        want = (A @ X.T).T
+        assert np.max(col_rel(to_host(y), want)) < TOL, (nrhs, "regular")
+        y.zero_()
+        op.ctx.check(ctx.lib.cfie_apply_fp64_static(op.h, x.data_ptr(), y.data_ptr(), nrhs),
+                     "cfie_apply_fp64_static")
+        assert np.max(col_rel(to_host(y), want)) < TOL, (nrhs, "static")
+    op.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+@pytest.mark.parametrize("npts,nrhs", [(1, 1), (63, 3), (65, 5), (130, 17)])
+def test_field_splits(ctx, bc, npts, nrhs):
+    n, omega = 258, 20.0
+    c = geometry.kite(n)
+    q = inputs.random_density(n, nrhs, seed=5)
+    rng = np.random.default_rng(npts)
+    pts = rng.uniform(2.0, 30.0, npts) * np.exp(2j * np.pi * rng.uniform(size=npts))
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp64")
+    u = empty(nrhs, npts)
+    op.field_eval(to_dev(q), to_dev(pts), u)
+    xy = np.stack([pts.real, pts.imag], 1)
+    want = np.stack([ofield.scattered_field(c, omega, omega, bc, q[k], xy) for k in range(nrhs)])
+    assert np.max(np.abs(to_host(u) - want)) < TOL * np.max(np.abs(want))
+    op.close()
