@@ -195,12 +195,13 @@ struct rtc_plan {
   alignas(64) unsigned char tmB[128];
 };
 
-// Bluestein / radix-2 FFT tables of an operator's spectral derivative
-// (spectral_fft.cu): power-of-two length N >= 2 n - 1, twiddles, chirp, FFT of
-// the wrapped chirp (FP64 and FP32), work buffers.
+// FFT tables of an operator's spectral derivative (spectral_fft.cu): length N
+// (n itself when that is a power of two, else a power of two >= 2 n - 1 for
+// Bluestein's algorithm), twiddles, chirp, spectrum of the wrapped chirp (FP64
+// and FP32), output factors, work buffers.
 struct fft_plan {
-  int N = 0, L = 0;
-  dbuf tw, tw32, chirp, chirp32, bf, bf32, work, work32;
+  int N = 0, L = 0, direct = 0;
+  dbuf tw, tw32, tc, tc32, chirp, chirp32, bf, bf32, osc, work, work32;
 };
 
 struct cfie_op {

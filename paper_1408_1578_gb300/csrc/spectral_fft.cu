@@ -6,15 +6,32 @@
 //
 // then divided by |z'| (d/ds).  This is the same operator as the circulant
 // c_d = (-1)^d cot(pi d / n) / 2, at O(n log n) instead of O(n^2) per column.
-// A DFT of any length n goes through Bluestein's chirp-z identity
+// A power-of-two n is transformed directly (N = n).  A DFT of any other length
+// n goes through Bluestein's chirp-z identity
 //
 //     X_m = conj(b_m) sum_j (x_j conj(b_j)) b_(m-j),   b_k = exp(i pi k^2 / n),
 //
-// a linear convolution computed with power-of-two FFTs of length N >= 2n - 1
-// (Stockham radix-2 passes, out of place, twiddles exp(-2 pi i q / N)); the
-// inverse DFT is conj(DFT(conj(D))) / n.  The FFT of the wrapped chirp is
-// precomputed per operator.  FP64 for the true residuals, FP32 for the inner
-// matvecs (same code, element type a template parameter).
+// a linear convolution computed with power-of-two FFTs of length N >= 2n - 1;
+// the inverse DFT is conj(DFT(conj(D))) / n.  FP64 for the true residuals, FP32
+// for the inner matvecs (same code, element type a template parameter).
+//
+// A length N = N1 N2 transform is done in two kernels (Bailey's four-step
+// form, time index j = j1 N2 + j2, frequency k1 + N1 k2): N2 transforms of
+// length N1 down the columns j2, times the twiddles exp(-2 pi i j2 k1 / N),
+// then N1 transforms of length N2 along the rows k1.  The spectrum is left in
+// that order: what it is multiplied by is stored in the same order, and the
+// way back runs the steps in reverse.  So one derivative is three kernels
+// (columns; rows, times i m', rows back; columns back), with Bluestein five
+// (the middle one ends the first convolution and starts the second on the same
+// columns).  Inside a kernel the transforms are Stockham passes of radix 8, 4
+// and 2 in shared memory.
+//
+// Bound: launches and latency (a whole derivative moves a few MB).  Before,
+// one radix-2 pass per launch (61 launches at N = 16384), or one CTA per
+// column with everything in shared memory (52 passes behind barriers, 16 CTAs
+// at 16 columns).  Measured (GB300), the two derivatives of one product: n =
+// 4096, 16 columns, FP32 268 -> 45 us, FP64 500 -> 80 us; n = 32768, 1 column,
+// FP32 500 -> 30 us; n = 6002 (N = 16384), 33 columns, FP32 470 -> 110 us.
 #include <algorithm>
 
 #include "internal.h"
@@ -31,6 +48,7 @@ template <> struct cx<float2> {
   static __device__ __forceinline__ float2 make(double a, double b) {
     return make_float2((float)a, (float)b);
   }
+  static __device__ __forceinline__ float2 make(float a, float b) { return make_float2(a, b); }
 };
 
 template <typename T>
@@ -41,286 +59,365 @@ template <typename T>
 __device__ __forceinline__ T cmulc(T a, T b) {   // a * conj(b)
   return cx<T>::make(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
+template <typename T>
+__device__ __forceinline__ T cadd(T a, T b) { return cx<T>::make(a.x + b.x, a.y + b.y); }
+template <typename T>
+__device__ __forceinline__ T csub(T a, T b) { return cx<T>::make(a.x - b.x, a.y - b.y); }
 
-// twiddles exp(-2 pi i q / N), q < N / 2 (FP64 and FP32 copies)
-__global__ void k_twiddles(int N, double2* __restrict__ tw, float2* __restrict__ tw32) {
+// twiddles exp(-2 pi i q / N), q < N, and exp(-2 pi i q / N2), q < N2 (FP64 and
+// FP32 copies)
+__global__ void k_twiddles(int N, int N2, double2* __restrict__ tw, float2* __restrict__ tw32,
+                           double2* __restrict__ tc, float2* __restrict__ tc32) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= N / 2) return;
+  if (q >= N) return;
   double s, c;
   sincospi(-2.0 * q / N, &s, &c);
   tw[q] = make_double2(c, s);
   tw32[q] = make_float2((float)c, (float)s);
+  if (q % (N / N2) == 0) {
+    tc[q / (N / N2)] = make_double2(c, s);
+    tc32[q / (N / N2)] = make_float2((float)c, (float)s);
+  }
 }
 
-// chirp b_k = exp(i pi (k^2 mod 2n) / n), k < n (the square reduced exactly in
-// integers before the sine and cosine)
-__global__ void k_chirp(int n, double2* __restrict__ b, float2* __restrict__ b32) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const long long q = ((long long)k * k) % (2LL * n);
-  double s, c;
-  sincospi((double)q / n, &s, &c);
-  b[k] = make_double2(c, s);
-  b32[k] = make_float2((float)c, (float)s);
-}
-
-// its wrapped copy B[k] = b_k (k < n), B[N - k] = b_k (0 < k < n), zero elsewhere
-__global__ void k_chirp_wrap(int n, int N, const double2* __restrict__ b, double2* __restrict__ B) {
+// Bluestein's chirp b_k = exp(i pi (k^2 mod 2n) / n), k < n (the square reduced
+// exactly in integers before the sine and cosine), its wrapped copy B[k] = b_k
+// (k < n), B[N - k] = b_k (0 < k < n), zero elsewhere, and the output factors
+// 1 / (n N |z'|) (direct transform: 1 / (N |z'|))
+__global__ void k_chirp(int n, int N, int direct, const double* __restrict__ sp,
+                        double2* __restrict__ b, float2* __restrict__ b32,
+                        double2* __restrict__ B, double* __restrict__ osc) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
+  if (k < n) osc[k] = 1.0 / ((direct ? 1.0 : (double)n) * (double)N * sp[k]);
+  if (direct) return;
+  const long long m = k < n ? k : (k > N - n ? N - k : -1);
   double2 v = make_double2(0.0, 0.0);
-  if (k < n) v = b[k];
-  else if (k > N - n) v = b[N - k];
+  if (m >= 0) {
+    const long long q = (m * m) % (2LL * n);
+    double s, c;
+    sincospi((double)q / n, &s, &c);
+    v = make_double2(c, s);
+  }
   B[k] = v;
-}
-
-// one Stockham radix-2 pass over `cols` columns of length N (half-size m)
-template <typename T>
-__global__ void k_fft_pass(int N, int m, int cols, const T* __restrict__ in, T* __restrict__ out,
-                           const T* __restrict__ tw, int inverse) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (i >= N / 2 || c >= cols) return;
-  const int j = i / m, k = i - j * m;
-  T w = tw[(size_t)k * (N / (2 * m))];
-  if (inverse) w.y = -w.y;
-  const T* a = in + (size_t)c * N;
-  T* o = out + (size_t)c * N;
-  const T u = a[j * m + k], v = cmul(w, a[j * m + k + N / 2]);
-  o[2 * j * m + k] = cx<T>::make(u.x + v.x, u.y + v.y);
-  o[2 * j * m + k + m] = cx<T>::make(u.x - v.x, u.y - v.y);
-}
-
-// a[c][j] = x[c][j] conj(b_j) for j < n, 0 up to N
-template <typename T, typename X>
-__global__ void k_bs_pre(int n, int N, int cols, const X* __restrict__ x, const T* __restrict__ b,
-                         T* __restrict__ a) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (j >= N) return;
-  T v = cx<T>::make(0.0, 0.0);
-  if (j < n) {
-    const X xv = x[(size_t)c * n + j];
-    v = cmulc(cx<T>::make(xv.x, xv.y), b[j]);
+  if (k < n) {
+    b[k] = v;
+    b32[k] = make_float2((float)v.x, (float)v.y);
   }
-  a[(size_t)c * N + j] = v;
 }
 
-// a *= Bf (pointwise, every column)
-template <typename T>
-__global__ void k_bs_mul(int N, int cols, T* __restrict__ a, const T* __restrict__ bf) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (k >= N) return;
-  a[(size_t)c * N + k] = cmul(a[(size_t)c * N + k], bf[k]);
+// discrete Fourier transforms of 2, 4 and 8 values in registers (sign -1, or +1
+// when INV)
+template <typename T, bool INV>
+__device__ __forceinline__ T mul_i(T a) {   // a * (-i), INV: a * i
+  return INV ? cx<T>::make(-a.y, a.x) : cx<T>::make(a.y, -a.x);
 }
-
-// X_m = conj(b_m) conv_m / N; D_m = i m' X_m; a2_m = conj(D_m) conj(b_m), 0 up to N
-template <typename T>
-__global__ void k_bs_mid(int n, int N, int cols, const T* __restrict__ conv,
-                         const T* __restrict__ b, T* __restrict__ a2) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (m >= N) return;
-  using S = typename cx<T>::S;
-  T v = cx<T>::make(0.0, 0.0);
-  if (m < n) {
-    const T X = cmulc(conv[(size_t)c * N + m], b[m]);
-    const S mm = (S)(2 * m < n ? m : (2 * m == n ? 0 : m - n)) / (S)N;
-    const T D = cx<T>::make(-mm * X.y, mm * X.x);      // i m' X / N
-    v = cmulc(cx<T>::make(D.x, -D.y), b[m]);          // conj(D) conj(b)
-  }
-  a2[(size_t)c * N + m] = v;
-}
-
-// out_j = base_j + (scale / |z'_j|) (1 / n) conj(conj(b_j) conv2_j / N)
-template <typename T, typename O>
-__global__ void k_bs_out(int n, int N, int cols, const T* __restrict__ conv2,
-                         const T* __restrict__ b, const double* __restrict__ sp, double2 scale,
-                         const O* __restrict__ base, O* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (j >= n) return;
-  const T w = cmulc(conv2[(size_t)c * N + j], b[j]);
-  const double f = 1.0 / ((double)n * (double)N * sp[j]);
-  const double dx = (double)w.x * f, dy = -(double)w.y * f;     // conj
-  double ox = scale.x * dx - scale.y * dy, oy = scale.x * dy + scale.y * dx;
-  if (base) {
-    const O bv = base[(size_t)c * n + j];
-    ox += (double)bv.x;
-    oy += (double)bv.y;
-  }
-  O r;
-  r.x = ox;
-  r.y = oy;
-  out[(size_t)c * n + j] = r;
-}
-
-// The whole derivative of one column in one CTA when both length-N work
-// buffers fit in shared memory: chirp premultiply, FFT, times Bf, inverse FFT,
-// derivative, FFT, times Bf, inverse FFT, output, with barriers between passes.
-template <typename T>
-__device__ __forceinline__ void smem_fft(int N, int L, T* a, T* b, const T* __restrict__ tw,
-                                         int inverse, T*& res) {
-  int m = 1;
-  for (int p = 0; p < L; ++p, m *= 2) {
-    for (int i = threadIdx.x; i < N / 2; i += blockDim.x) {
-      const int j = i / m, k = i - j * m;
-      T w = tw[(size_t)k * (N / (2 * m))];
-      if (inverse) w.y = -w.y;
-      const T u = a[j * m + k], v = cmul(w, a[j * m + k + N / 2]);
-      b[2 * j * m + k] = cx<T>::make(u.x + v.x, u.y + v.y);
-      b[2 * j * m + k + m] = cx<T>::make(u.x - v.x, u.y - v.y);
+template <typename T, bool INV, int R>
+__device__ __forceinline__ void dft(T* v) {
+  if constexpr (R == 2) {
+    const T a = v[0], b = v[1];
+    v[0] = cadd(a, b);
+    v[1] = csub(a, b);
+  } else if constexpr (R == 4) {
+    const T a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+    const T c = cadd(v[1], v[3]), d = mul_i<T, INV>(csub(v[1], v[3]));
+    v[0] = cadd(a, c);
+    v[1] = cadd(b, d);
+    v[2] = csub(a, c);
+    v[3] = csub(b, d);
+  } else {
+    using S = typename cx<T>::S;
+    T e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+    dft<T, INV, 4>(e);
+    dft<T, INV, 4>(o);
+    const S h = (S)0.70710678118654752440;
+    const T w1 = cx<T>::make(h, INV ? h : -h), w3 = cx<T>::make(-h, INV ? h : -h);
+    o[1] = cmul(o[1], w1);
+    o[2] = mul_i<T, INV>(o[2]);
+    o[3] = cmul(o[3], w3);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = cadd(e[k], o[k]);
+      v[k + 4] = csub(e[k], o[k]);
     }
-    __syncthreads();
+  }
+}
+
+// One Stockham pass of radix R over 2^lc transforms of length M in shared
+// memory (element e of transform c at e es + c): m = product of the radices so
+// far, butterfly (j, k), k < m, reads elements i + q M / R (i = j m + k), times
+// exp(-2 pi i q k / (R m)), and writes elements R j m + k + p m.  tc: the N2
+// twiddles, N2 = M ts.
+template <typename T, bool INV, int R>
+__device__ __forceinline__ void fft_pass(const T* __restrict__ a, T* __restrict__ o, int M, int lc,
+                                         int es, int lm, const T* __restrict__ tc, int ts) {
+  const int m = 1 << lm, nb = (M / R) << lc;
+  const int tstep = (M / R >> lm) * ts;
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    const int c = b & ((1 << lc) - 1), i = b >> lc;
+    const int k = i & (m - 1), j = i >> lm;
+    T v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) v[q] = a[(i + q * (M / R)) * es + c];
+    if (lm) {
+#pragma unroll
+      for (int q = 1; q < R; ++q) {
+        const T w = __ldg(tc + q * k * tstep);
+        v[q] = INV ? cmulc(v[q], w) : cmul(v[q], w);
+      }
+    }
+    dft<T, INV, R>(v);
+#pragma unroll
+    for (int p = 0; p < R; ++p) o[(R * j * m + k + p * m) * es + c] = v[p];
+  }
+  __syncthreads();
+}
+
+// 2^lc transforms of length M = 2^lM from buffer a, b the other buffer; returns
+// the one that holds the result (natural order).  The caller synchronises
+// before the call.
+template <typename T, bool INV>
+__device__ T* fft_smem(T* a, T* b, int lM, int lc, int es, const T* __restrict__ tc, int ts) {
+  const int M = 1 << lM;
+  for (int lm = 0; lm < lM;) {
+    const int rem = lM - lm;
+    if (rem >= 5 || rem == 3) {
+      fft_pass<T, INV, 8>(a, b, M, lc, es, lm, tc, ts);
+      lm += 3;
+    } else if (rem >= 2) {
+      fft_pass<T, INV, 4>(a, b, M, lc, es, lm, tc, ts);
+      lm += 2;
+    } else {
+      fft_pass<T, INV, 2>(a, b, M, lc, es, lm, tc, ts);
+      lm += 1;
+    }
     T* t = a;
     a = b;
     b = t;
-  }
-  res = a;
-}
-
-template <typename T, typename X, typename O>
-__global__ void __launch_bounds__(512)
-k_spectral_smem(int n, int N, int L, const X* __restrict__ in, const T* __restrict__ ch,
-                const T* __restrict__ bf, const T* __restrict__ tw, const double* __restrict__ sp,
-                double2 scale, const O* __restrict__ base, O* __restrict__ out) {
-  using S = typename cx<T>::S;
-  extern __shared__ __align__(16) unsigned char raw[];
-  T* a = reinterpret_cast<T*>(raw);
-  T* b = a + N;
-  const int c = blockIdx.x;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    T v = cx<T>::make(0.0, 0.0);
-    if (j < n) {
-      const X xv = in[(size_t)c * n + j];
-      v = cmulc(cx<T>::make(xv.x, xv.y), ch[j]);
-    }
-    a[j] = v;
-  }
-  __syncthreads();
-  T* r;
-  smem_fft(N, L, a, b, tw, 0, r);
-  for (int k = threadIdx.x; k < N; k += blockDim.x) r[k] = cmul(r[k], bf[k]);
-  __syncthreads();
-  T* o = r == a ? b : a;
-  smem_fft(N, L, r, o, tw, 1, r);
-  o = r == a ? b : a;
-  for (int m = threadIdx.x; m < N; m += blockDim.x) {
-    T v = cx<T>::make(0.0, 0.0);
-    if (m < n) {
-      const T Xm = cmulc(r[m], ch[m]);
-      const S mm = (S)(2 * m < n ? m : (2 * m == n ? 0 : m - n)) / (S)N;
-      const T D = cx<T>::make(-mm * Xm.y, mm * Xm.x);
-      v = cmulc(cx<T>::make(D.x, -D.y), ch[m]);
-    }
-    o[m] = v;
-  }
-  __syncthreads();
-  smem_fft(N, L, o, r, tw, 0, r);
-  for (int k = threadIdx.x; k < N; k += blockDim.x) r[k] = cmul(r[k], bf[k]);
-  __syncthreads();
-  o = r == a ? b : a;
-  smem_fft(N, L, r, o, tw, 1, r);
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    const T w = cmulc(r[j], ch[j]);
-    const double f = 1.0 / ((double)n * (double)N * sp[j]);
-    const double dx = (double)w.x * f, dy = -(double)w.y * f;
-    double ox = scale.x * dx - scale.y * dy, oy = scale.x * dy + scale.y * dx;
-    if (base) {
-      const O bv = base[(size_t)c * n + j];
-      ox += (double)bv.x;
-      oy += (double)bv.y;
-    }
-    O q;
-    q.x = ox;
-    q.y = oy;
-    out[(size_t)c * n + j] = q;
-  }
-}
-
-unsigned nb(size_t len, int t = 256) { return (unsigned)((len + t - 1) / t); }
-
-// FFT of `cols` columns of length N between the two work buffers; returns the
-// buffer holding the result
-template <typename T>
-T* fft(cudaStream_t st, int N, int L, int cols, T* a, T* b, const T* tw, int inverse) {
-  int m = 1;
-  for (int p = 0; p < L; ++p, m *= 2) {
-    k_fft_pass<T><<<dim3(nb(N / 2), cols), 256, 0, st>>>(N, m, cols, a, b, tw, inverse);
-    CFIE_CHECK_LAUNCH();
-    std::swap(a, b);
   }
   return a;
 }
 
 template <typename T>
-const T* tw_of(const fft_plan& F);
-template <> const double2* tw_of<double2>(const fft_plan& F) { return F.tw.as<double2>(); }
-template <> const float2* tw_of<float2>(const fft_plan& F) { return F.tw32.as<float2>(); }
-template <typename T>
-const T* chirp_of(const fft_plan& F);
-template <> const double2* chirp_of<double2>(const fft_plan& F) { return F.chirp.as<double2>(); }
-template <> const float2* chirp_of<float2>(const fft_plan& F) { return F.chirp32.as<float2>(); }
-template <typename T>
-const T* bf_of(const fft_plan& F);
-template <> const double2* bf_of<double2>(const fft_plan& F) { return F.bf.as<double2>(); }
-template <> const float2* bf_of<float2>(const fft_plan& F) { return F.bf32.as<float2>(); }
+struct fft_args {
+  int n, N, l1, l2, lc, direct;   // N = 2^(l1 + l2); 2^lc transforms per CTA
+  const T* tw;                    // exp(-2 pi i q / N), q < N
+  const T* tc;                    // exp(-2 pi i q / 2^l2)
+  const T* ch;                    // chirp
+  const T* bf;                    // spectrum of the wrapped chirp, [k1][k2]
+  T* work;                        // [column][N]
+};
+
+// Transforms down the columns j2 = 2^lc blockIdx.x .. of density column
+// blockIdx.y.  COL_IN: from x (times the chirp) to the rows; COL_RAW: the same
+// from the work buffer; COL_OUT: from the rows to the output; COL_MID: from the
+// rows to the time domain (the end of Bluestein's first convolution), times
+// i m', and on to the rows of the second.
+enum { COL_IN = 1, COL_OUT = 2, COL_MID = 3, COL_RAW = 4 };
+
+template <typename T, int MODE, typename X, typename O>
+__global__ void __launch_bounds__(256)
+k_fft_cols(fft_args<T> F, const X* __restrict__ x, const double* __restrict__ osc, double2 scale,
+           const O* base, O* out) {
+  using S = typename cx<T>::S;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int N1 = 1 << F.l1, N2 = 1 << F.l2, C = 1 << F.lc, es = C + 1;
+  const int col = blockIdx.y, c0 = blockIdx.x << F.lc, n = F.n;
+  T* a = reinterpret_cast<T*>(raw);
+  T* b = a + (size_t)N1 * es;
+  T* w = F.work + (size_t)col * F.N;
+  const int tot = N1 << F.lc, ts = N2 >> F.l1;
+  if constexpr (MODE == COL_IN || MODE == COL_RAW) {
+    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+      const int c = e & (C - 1), j1 = e >> F.lc, j = j1 * N2 + c0 + c;
+      T v = cx<T>::make((S)0, (S)0);
+      if (MODE == COL_RAW) {
+        v = w[j];
+      } else if (j < n) {
+        const X xv = x[(size_t)col * n + j];
+        v = cx<T>::make((S)xv.x, (S)xv.y);
+        if (!F.direct) v = cmulc(v, F.ch[j]);
+      }
+      a[j1 * es + c] = v;
+    }
+    __syncthreads();
+  } else {
+    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+      const int c = e & (C - 1), k1 = e >> F.lc, j2 = c0 + c;
+      a[k1 * es + c] = cmulc(w[k1 * N2 + j2], __ldg(F.tw + k1 * j2));
+    }
+    __syncthreads();
+    T* r = fft_smem<T, true>(a, b, F.l1, F.lc, es, F.tc, ts);
+    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+      const int c = e & (C - 1), j1 = e >> F.lc, j = j1 * N2 + c0 + c;
+      T v = r[j1 * es + c];
+      if constexpr (MODE == COL_OUT) {
+        // out_j = base_j + scale osc_j conj(conj(b_j) conv_j) (direct: scale osc_j v_j)
+        if (j >= n) continue;
+        if (!F.direct) {
+          v = cmulc(v, F.ch[j]);
+          v.y = -v.y;
+        }
+        const double f = osc[j];
+        const double dx = (double)v.x * f, dy = (double)v.y * f;
+        double ox = scale.x * dx - scale.y * dy, oy = scale.x * dy + scale.y * dx;
+        if (base) {
+          const O bv = base[(size_t)col * n + j];
+          ox += (double)bv.x;
+          oy += (double)bv.y;
+        }
+        O q;
+        q.x = ox;
+        q.y = oy;
+        out[(size_t)col * n + j] = q;
+      } else {
+        // X_m = conj(b_m) conv_m; D_m = i m' X_m / N; next input conj(D_m) conj(b_m)
+        T d = cx<T>::make((S)0, (S)0);
+        if (j < n) {
+          const T ch = F.ch[j];
+          const T Xm = cmulc(v, ch);
+          const S mm = (S)(2 * j < n ? j : (2 * j == n ? 0 : j - n)) / (S)F.N;
+          d = cmulc(cx<T>::make(-mm * Xm.y, -mm * Xm.x), ch);
+        }
+        r[j1 * es + c] = d;
+      }
+    }
+    __syncthreads();
+    if (r != a) {
+      b = a;
+      a = r;
+    }
+  }
+  if constexpr (MODE != COL_OUT) {
+    T* r = fft_smem<T, false>(a, b, F.l1, F.lc, es, F.tc, ts);
+    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+      const int c = e & (C - 1), k1 = e >> F.lc, j2 = c0 + c;
+      w[k1 * N2 + j2] = cmul(r[k1 * es + c], __ldg(F.tw + k1 * j2));
+    }
+  }
+}
+
+// rows k1 = 2^lc blockIdx.x ..: forward transform along the row, times the
+// chirp's spectrum (direct: i m'), back transform; FWD_ONLY: forward alone
+template <typename T, bool FWD_ONLY>
+__global__ void __launch_bounds__(256) k_fft_rows(fft_args<T> F) {
+  using S = typename cx<T>::S;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int N1 = 1 << F.l1, N2 = 1 << F.l2, C = 1 << F.lc, es = C + 1;
+  const int r0 = blockIdx.x << F.lc, n = F.n;
+  T* a = reinterpret_cast<T*>(raw);
+  T* b = a + (size_t)N2 * es;
+  T* w = F.work + (size_t)blockIdx.y * F.N + (size_t)r0 * N2;
+  const int tot = N2 << F.lc;
+  for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+    const int c = e >> F.l2, j = e & (N2 - 1);
+    a[j * es + c] = w[e];
+  }
+  __syncthreads();
+  T* r = fft_smem<T, false>(a, b, F.l2, F.lc, es, F.tc, 1);
+  if constexpr (!FWD_ONLY) {
+    for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+      const int c = e >> F.l2, k2 = e & (N2 - 1);
+      T v = r[k2 * es + c];
+      if (F.direct) {
+        const int m = r0 + c + N1 * k2;
+        const S mm = (S)(2 * m < n ? m : (2 * m == n ? 0 : m - n));
+        v = cx<T>::make(-mm * v.y, mm * v.x);
+      } else {
+        v = cmul(v, F.bf[(size_t)(r0 + c) * N2 + k2]);
+      }
+      r[k2 * es + c] = v;
+    }
+    __syncthreads();
+    r = fft_smem<T, true>(r, r == a ? b : a, F.l2, F.lc, es, F.tc, 1);
+  }
+  for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+    const int c = e >> F.l2, j = e & (N2 - 1);
+    w[e] = r[j * es + c];
+  }
+}
+
+unsigned nb(size_t len, int t = 256) { return (unsigned)((len + t - 1) / t); }
 
 __global__ void k_to_f32(size_t len, const double2* __restrict__ a, float2* __restrict__ b) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < len) b[e] = make_float2((float)a[e].x, (float)a[e].y);
 }
 
+template <typename T>
+fft_args<T> args_of(const fft_plan& F, int n, T* work) {
+  fft_args<T> A{};
+  A.n = n;
+  A.N = F.N;
+  A.l1 = F.L / 2;
+  A.l2 = F.L - F.L / 2;
+  A.direct = F.direct;
+  if constexpr (sizeof(T) == 16) {
+    A.tw = F.tw.as<double2>();
+    A.tc = F.tc.as<double2>();
+    A.ch = F.chirp.as<double2>();
+    A.bf = F.bf.as<double2>();
+  } else {
+    A.tw = F.tw32.as<float2>();
+    A.tc = F.tc32.as<float2>();
+    A.ch = F.chirp32.as<float2>();
+    A.bf = F.bf32.as<float2>();
+  }
+  A.work = work;
+  return A;
+}
+
+// Transforms per CTA (2^lc of length 2^lM, out of 2^lOther): about 2048
+// elements, at least 64 contiguous bytes per row of the columns, fewer when
+// the launch would leave SMs idle.  Shared memory: two buffers, at most
+// 2 (2^11 elements x 2) or 2 (2^10 x (4 + 1)) of 16 bytes, 164 KB.
+template <typename T>
+int per_cta(int lM, int lOther, int cols, int lmin) {
+  int lc = std::max(lmin, 11 - lM);
+  lc = std::min(lc, lOther);
+  while (lc > std::min(lmin, lOther) && ((long long)cols << (lOther - lc)) < 152) --lc;
+  return lc;
+}
+template <typename T>
+size_t smem_of(int lM, int lc) {
+  return 2 * sizeof(T) * (((size_t)1 << lM) * (((size_t)1 << lc) + 1));
+}
+constexpr size_t kSmemMax = (size_t)200 * 1024;
+
+// the attribute is the bound of every launch of the kernel, not this one's
+// size: it is per kernel and process-wide, and operators of other sizes launch
+// the same kernel from other host threads (server slots)
+#define FFT_LAUNCH(kernel, grid, smem, st, ...)                                               \
+  do {                                                                                        \
+    CFIE_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                         (int)kSmemMax));                                     \
+    kernel<<<grid, 256, smem, st>>>(__VA_ARGS__);                                             \
+    CFIE_CHECK_LAUNCH();                                                                      \
+  } while (0)
+
 // out = base + scale (1/|z'|) d/dt in, columns of length n, element type T for
 // the transforms
 template <typename T, typename X, typename O>
 void spectral_fft(cfie_op* op, const X* in, O* out, const O* base, double2 scale, int cols) {
   fft_plan& F = op->fft;
-  const int n = op->n, N = F.N, L = F.L;
   cudaStream_t st = op->ctx->stream;
-  const size_t smem = 2 * sizeof(T) * (size_t)N;
-  constexpr size_t kSmemMax = (size_t)128 * 1024;
-  if (smem <= kSmemMax) {
-    // one CTA per column, everything in shared memory.  The attribute is the
-    // bound of this branch, not this launch's size: it is per kernel and
-    // process-wide, and operators of other sizes launch the same kernel from
-    // other host threads (server slots)
-    prof_scope ps(op->ctx, CFIE_K_SPECTRAL);
-    CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_spectral_smem<T, X, O>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemMax));
-    k_spectral_smem<T, X, O><<<cols, 512, smem, st>>>(n, N, L, in, chirp_of<T>(F), bf_of<T>(F),
-                                                     tw_of<T>(F), op->g.sp, scale, base, out);
-    CFIE_CHECK_LAUNCH();
-    return;
-  }
-  dbuf& w = sizeof(T) == 16 ? F.work : F.work32;
-  w.reserve(sizeof(T) * 2 * (size_t)N * cols);
-  T* a = w.as<T>();
-  T* b = a + (size_t)N * cols;
-  const T* tw = tw_of<T>(F);
-  const T* ch = chirp_of<T>(F);
-  const T* bf = bf_of<T>(F);
-  const dim3 gN(nb(N), cols), gn(nb(n), cols);
+  dbuf& wb = sizeof(T) == 16 ? F.work : F.work32;
+  wb.reserve(sizeof(T) * (size_t)F.N * cols);
+  fft_args<T> C = args_of<T>(F, op->n, wb.as<T>()), R = C;
+  constexpr int lmin = sizeof(T) == 16 ? 2 : 3;
+  C.lc = per_cta<T>(C.l1, C.l2, cols, lmin);
+  R.lc = per_cta<T>(R.l2, R.l1, cols, 0);
+  const dim3 gc(1u << (C.l2 - C.lc), cols), gr(1u << (R.l1 - R.lc), cols);
+  const size_t sc = smem_of<T>(C.l1, C.lc), sr = smem_of<T>(R.l2, R.lc);
+  const double* osc = F.osc.as<double>();
   prof_scope ps(op->ctx, CFIE_K_SPECTRAL);
-  k_bs_pre<T, X><<<gN, 256, 0, st>>>(n, N, cols, in, ch, a);
-  CFIE_CHECK_LAUNCH();
-  T* r = fft<T>(st, N, L, cols, a, b, tw, 0);
-  k_bs_mul<T><<<gN, 256, 0, st>>>(N, cols, r, bf);
-  CFIE_CHECK_LAUNCH();
-  T* o = r == a ? b : a;
-  r = fft<T>(st, N, L, cols, r, o, tw, 1);
-  o = r == a ? b : a;
-  k_bs_mid<T><<<gN, 256, 0, st>>>(n, N, cols, r, ch, o);
-  CFIE_CHECK_LAUNCH();
-  r = fft<T>(st, N, L, cols, o, r, tw, 0);
-  k_bs_mul<T><<<gN, 256, 0, st>>>(N, cols, r, bf);
-  CFIE_CHECK_LAUNCH();
-  o = r == a ? b : a;
-  r = fft<T>(st, N, L, cols, r, o, tw, 1);
-  k_bs_out<T, O><<<gn, 256, 0, st>>>(n, N, cols, r, ch, op->g.sp, scale, base, out);
-  CFIE_CHECK_LAUNCH();
+  FFT_LAUNCH((k_fft_cols<T, COL_IN, X, O>), gc, sc, st, C, in, osc, scale, base, out);
+  FFT_LAUNCH((k_fft_rows<T, false>), gr, sr, st, R);
+  if (!F.direct) {
+    FFT_LAUNCH((k_fft_cols<T, COL_MID, X, O>), gc, sc, st, C, in, osc, scale, base, out);
+    FFT_LAUNCH((k_fft_rows<T, false>), gr, sr, st, R);
+  }
+  FFT_LAUNCH((k_fft_cols<T, COL_OUT, X, O>), gc, sc, st, C, in, osc, scale, base, out);
 }
 
 }  // namespace
@@ -328,32 +425,43 @@ void spectral_fft(cfie_op* op, const X* in, O* out, const O* base, double2 scale
 void fft_prepare(cfie_op* op) {
   fft_plan& F = op->fft;
   const int n = op->n;
+  F.direct = (n & (n - 1)) == 0;
   int N = 1, L = 0;
-  while (N < 2 * n - 1) {
+  while (N < (F.direct ? n : 2 * n - 1)) {
     N *= 2;
     ++L;
   }
   F.N = N;
   F.L = L;
+  const int N2 = 1 << (L - L / 2);
   cudaStream_t st = op->ctx->stream;
-  F.tw.reserve(sizeof(double2) * (N / 2));
-  F.tw32.reserve(sizeof(float2) * (N / 2));
-  F.chirp.reserve(sizeof(double2) * n);
-  F.chirp32.reserve(sizeof(float2) * n);
-  F.bf.reserve(sizeof(double2) * N);
-  F.bf32.reserve(sizeof(float2) * N);
-  k_twiddles<<<nb(N / 2), 256, 0, st>>>(N, F.tw.as<double2>(), F.tw32.as<float2>());
+  F.tw.reserve(sizeof(double2) * N);
+  F.tw32.reserve(sizeof(float2) * N);
+  F.tc.reserve(sizeof(double2) * N2);
+  F.tc32.reserve(sizeof(float2) * N2);
+  F.osc.reserve(sizeof(double) * n);
+  k_twiddles<<<nb(N), 256, 0, st>>>(N, N2, F.tw.as<double2>(), F.tw32.as<float2>(),
+                                    F.tc.as<double2>(), F.tc32.as<float2>());
   CFIE_CHECK_LAUNCH();
-  k_chirp<<<nb(n), 256, 0, st>>>(n, F.chirp.as<double2>(), F.chirp32.as<float2>());
+  if (!F.direct) {
+    F.chirp.reserve(sizeof(double2) * n);
+    F.chirp32.reserve(sizeof(float2) * n);
+    F.bf.reserve(sizeof(double2) * N);
+    F.bf32.reserve(sizeof(float2) * N);
+  }
+  // the wrapped chirp, then its spectrum (FP64, in place) and the FP32 copy
+  k_chirp<<<nb(N), 256, 0, st>>>(n, N, F.direct, op->g.sp, F.chirp.as<double2>(),
+                                 F.chirp32.as<float2>(), F.bf.as<double2>(), F.osc.as<double>());
   CFIE_CHECK_LAUNCH();
-  // Bf = FFT of the wrapped chirp (FP64), then its FP32 copy
-  dbuf tmp;
-  tmp.reserve(sizeof(double2) * 2 * (size_t)N);
-  double2* a = tmp.as<double2>();
-  k_chirp_wrap<<<nb(N), 256, 0, st>>>(n, N, F.chirp.as<double2>(), a);
-  CFIE_CHECK_LAUNCH();
-  double2* r = fft<double2>(st, N, L, 1, a, a + N, F.tw.as<double2>(), 0);
-  CFIE_CHECK_CUDA(cudaMemcpyAsync(F.bf.p, r, sizeof(double2) * N, cudaMemcpyDeviceToDevice, st));
+  if (F.direct) return;
+  fft_args<double2> C = args_of<double2>(F, n, F.bf.as<double2>()), R = C;
+  C.lc = per_cta<double2>(C.l1, C.l2, 1, 2);
+  R.lc = per_cta<double2>(R.l2, R.l1, 1, 0);
+  FFT_LAUNCH((k_fft_cols<double2, COL_RAW, double2, double2>), dim3(1u << (C.l2 - C.lc), 1),
+             smem_of<double2>(C.l1, C.lc), st, C, nullptr, nullptr, make_double2(0.0, 0.0), nullptr,
+             nullptr);
+  FFT_LAUNCH((k_fft_rows<double2, true>), dim3(1u << (R.l1 - R.lc), 1),
+             smem_of<double2>(R.l2, R.lc), st, R);
   k_to_f32<<<nb(N), 256, 0, st>>>(N, F.bf.as<double2>(), F.bf32.as<float2>());
   CFIE_CHECK_LAUNCH();
 }

@@ -43,6 +43,22 @@ def test_right_hand_side_blocks(ctx, bc, n, omega):
     op.close()
 
 
+@pytest.mark.parametrize("n,nrhs", [(16, 3), (128, 2), (256, 5), (2048, 4), (4098, 2), (32768, 1)])
+def test_spectral_derivative_lengths(ctx, n, nrhs):
+    """The FFT derivative (direct for powers of two, Bluestein otherwise, both splits of each
+    length) against the circulant one of the allocation-free matvec, inside the sound-hard
+    product.  The derivative's modes reach n / 2, so the product carries ~2^-53 n / omega."""
+    omega = n / 16.0
+    op = ctx.kite().discretise(n, omega, bc="hard", precision="fp64")
+    x = to_dev(inputs.random_density(n, nrhs, seed=n))
+    y, z = empty(nrhs, n), empty(nrhs, n)
+    op.apply_fp64(x, y)
+    op.ctx.check(ctx.lib.cfie_apply_fp64_static(op.h, x.data_ptr(), z.data_ptr(), nrhs),
+                 "cfie_apply_fp64_static")
+    assert np.max(col_rel(to_host(y), to_host(z))) < TOL
+    op.close()
+
+
 @pytest.mark.parametrize("bc", ["soft", "hard"])
 @pytest.mark.parametrize("npts,nrhs", [(1, 1), (63, 3), (65, 5), (130, 17)])
 def test_field_splits(ctx, bc, npts, nrhs):
