@@ -107,8 +107,23 @@ namespace {
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int>, int> g_tuned;
 
+// Sizes at which a product is launches and latency in either variant (tens of
+// microseconds; timed on a GB300, both within a third of each other) take the
+// CUDA-core sums without timing: they are the more accurate, 1e-6 against 2e-6
+// (sound soft) and 6e-6 (sound hard) relative.  Sound soft, one right-hand
+// side: 27 against 37 us at n = 1024, 51 against 50 at 2050; sound hard:
+// 85 against 104 us at n = 512, 64 right-hand sides, 114 against 110 at n =
+// 2048, 8 (CUDA cores against tensor cores).
+bool prefers_fp32_sums(const cfie_op* op, int nrhs) {
+  const int n = op->n;
+  if (nrhs == 1 && n <= 2304) return true;
+  return op->bc == CFIE_SOUND_HARD &&
+         (n <= 1152 || (n <= 1600 && nrhs < 32) || (n <= 2304 && nrhs < 16));
+}
+
 int tuned_variant(cfie_op* op, const double2* x, double2* y, int nrhs) {
   if (op->variant) return op->variant;
+  if (prefers_fp32_sums(op, nrhs)) return 1;
   // decisions are shared by operators of similar shape (n up to the next power
   // of two, right-hand sides in octaves), so that a server seeing a new n and
   // nrhs with every request does not time both variants every time

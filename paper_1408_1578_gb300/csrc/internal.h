@@ -228,7 +228,7 @@ struct cfie_op {
   dbuf band;         // near-field band entries (complex64), n x (2 b + 1) per operator
   int band_b = -1;
   dbuf xin32, xin32b; // FP32 staging of the input (and hard-path helpers)
-  dbuf tcv, tcs;      // sound-hard tensor-core path: S inputs, S and D' outputs
+  dbuf tcv, tcs;      // sound-hard tensor-core residual: S inputs, S and D' outputs
   fft_plan fft;       // sound hard: FFT spectral derivative
 
   // FP64-accurate residual matvec in double-float arithmetic (sound-soft)
@@ -241,7 +241,7 @@ struct cfie_op {
   // FP32 matvec variant: 0 = autotuned, 1 = FP32-pipe contraction, 2 = tensor cores
   int variant = 0, tuned_nrhs = -1, tuned_choice = 1;
   int basis32 = 1;   // inner Krylov basis in FP32 for the refined precisions
-  tc_plan tc[2];   // 32- and 64-right-hand-side plans
+  tc_plan tc[3];   // plans: up to 32, up to 64 right-hand sides; S and C together, up to 32
 
   // stored path (CFIE_STORED): bf16 hi/lo planes of A and the contraction plan
   dbuf stored;
@@ -327,6 +327,7 @@ void fft_prepare(cfie_op* op);
 void spectral_fft64(cfie_op* op, const double2* in, double2* out, const double2* base,
                     double2 scale, int nrhs);
 void spectral_fft32_apply(cfie_op* op, const float2* in, float2* out, int nrhs);
+void spectral_fft32_apply(cfie_op* op, const double2* in, float2* out, int nrhs);
 void spectral_fft32_accumulate(cfie_op* op, const float2* in, double2* y, double2 scale,
                                int nrhs);
 // sound-hard combination of the four FP64-layout partial sums (S u, S n1 x,
@@ -338,10 +339,10 @@ size_t static_scratch_capacity();
 // matvec_fp32.cu
 void fp32_prepare(cfie_op* op);
 void fp32_band(cfie_op* op);   // after df_prepare
-// FP32 helpers shared with the tensor-core kernels: x32 = x, u32 = (1/|z'|) d/dt x32,
+// FP32 helpers shared with the tensor-core kernels: u32 = (1/|z'|) d/dt x,
 // y += (1/(i eta)) (1/|z'|) d/dt t32
-void k_to32_fp32(cfie_op* op, const double2* x, float2* x32, size_t tot);
 void spectral32_apply(cfie_op* op, const float2* x32, float2* u32, int nrhs);
+void spectral32_apply(cfie_op* op, const double2* x, float2* u32, int nrhs);
 void spectral32_accumulate(cfie_op* op, const float2* t32, double2* y, int nrhs);
 void matvec_fp32(cfie_op* op, const double2* x, double2* y, int nrhs);
 // stored.cu

@@ -52,6 +52,7 @@ struct pair_params : omega32 {
   const float2* band2;   // hard: D'
   const float2* xin;     // [k][j] complex64 (hard: x)
   const float2* uin;     // hard: (1/s) Dt x
+  float k2;              // hard: omega^2 / eta
   float2* part;          // [o][split][k][i]
 };
 
@@ -66,16 +67,16 @@ __device__ __forceinline__ float2 cmul_add(float2 acc, float2 a, float2 x) {
 template <int BC, int R>
 struct smem32 {
   float txh[TI], txl[TI], tyh[TI], tyl[TI], tnx[TI], tny[TI], tsp[TI];
-  float2 A[TJ][TI + 1];
-  float2 B[BC ? TJ : 1][TI + 1];
-  float2 X[BC ? 4 : 1][TJ][R];
+  float2 A[TJ][TI + 1];              // soft A; hard S
+  float2 B[BC ? TJ : 1][TI + 1];     // hard C
+  float2 X[BC ? 2 : 1][TJ][R];       // soft x; hard u, x
 };
 
 template <int BC, int R>
 __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
   extern __shared__ __align__(16) unsigned char raw[];
   smem32<BC, R>& S = *reinterpret_cast<smem32<BC, R>*>(raw);
-  constexpr int RQ = R / 8;
+  constexpr int RQ = R / 8, NO = BC ? 2 : 1;
   const int n = P.n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int i0 = blockIdx.x * TI;
@@ -99,9 +100,9 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
     S.tsp[q] = ok ? P.g.sp[i] : 1.f;
   }
 
-  float2 acc[BC ? 4 : 1][4][RQ];
+  float2 acc[NO][4][RQ];
 #pragma unroll
-  for (int o = 0; o < (BC ? 4 : 1); ++o)
+  for (int o = 0; o < NO; ++o)
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
@@ -121,23 +122,15 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
         xv = P.xin[(size_t)(rb0 + r) * n + jj];
         if (BC) uv = P.uin[(size_t)(rb0 + r) * n + jj];
       }
-      if constexpr (BC == 1) {
-        const float inv = jj < n ? 1.0f / P.g.sp[jj] : 0.f;
-        const float n1 = jj < n ? P.g.nx[jj] * inv : 0.f;
-        const float n2 = jj < n ? P.g.ny[jj] * inv : 0.f;
-        S.X[0][jl][r] = uv;
-        S.X[1][jl][r] = make_float2(n1 * xv.x, n1 * xv.y);
-        S.X[2][jl][r] = make_float2(n2 * xv.x, n2 * xv.y);
-        S.X[3][jl][r] = xv;
-      } else {
-        S.X[0][jl][r] = xv;
-      }
+      S.X[NO - 1][jl][r] = xv;
+      if constexpr (BC == 1) S.X[0][jl][r] = uv;
     }
     // this lane's source
     const float sxh = jok ? P.g.xh[j] : 0.f, sxl = jok ? P.g.xl[j] : 0.f;
     const float syh = jok ? P.g.yh[j] : 0.f, syl = jok ? P.g.yl[j] : 0.f;
     const float snx = jok ? P.g.nx[j] : 0.f, sny = jok ? P.g.ny[j] : 0.f;
     const float ssp = jok ? P.g.sp[j] : 1.f;
+    const float sux = snx / ssp, suy = sny / ssp;   // unit normal (hard)
     __syncthreads();  // target geometry (first tile) and X are in place
 
     // ---- entries: warp handles rows warp + 8 q, lane = source
@@ -160,7 +153,11 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
         }
       }
       S.A[lane][il] = a;
-      if constexpr (BC == 1) S.B[lane][il] = b;
+      if constexpr (BC == 1) {
+        // C = -D' - i (omega^2 / eta) (n_i . n_j) S
+        const float kn = P.k2 / S.tsp[il] * fmaf(S.tnx[il], sux, S.tny[il] * suy);
+        S.B[lane][il] = make_float2(fmaf(kn, a.y, -b.x), -fmaf(kn, a.x, b.y));
+      }
     }
     __syncthreads();
 
@@ -184,14 +181,11 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
 #pragma unroll
         for (int q = 0; q < RQ; ++q) {
           const int r = warp * RQ + q;
-          const float2 x0 = S.X[0][jl][r], x1 = S.X[1][jl][r], x2 = S.X[2][jl][r],
-                       x3 = S.X[3][jl][r];
+          const float2 x0 = S.X[0][jl][r], x1 = S.X[NO - 1][jl][r];
 #pragma unroll
           for (int p = 0; p < 4; ++p) {
             acc[0][p][q] = cmul_add(acc[0][p][q], av[p], x0);
-            acc[1][p][q] = cmul_add(acc[1][p][q], av[p], x1);
-            acc[2][p][q] = cmul_add(acc[2][p][q], av[p], x2);
-            acc[3 * BC][p][q] = cmul_add(acc[3 * BC][p][q], bv[p], x3);
+            acc[NO - 1][p][q] = cmul_add(acc[NO - 1][p][q], bv[p], x1);
           }
         }
       }
@@ -207,42 +201,43 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
       const int r = warp * RQ + q;
       if (r >= rbn) continue;
 #pragma unroll
-      for (int o = 0; o < (BC ? 4 : 1); ++o)
+      for (int o = 0; o < NO; ++o)
         P.part[(((size_t)o * P.splits + split) * P.nrhs + rb0 + r) * n + i] = acc[o][p][q];
     }
   }
 }
 
-// y = sum of split partials in FP64; hard: t = S u (complex64 for the
-// derivative) and y = 1/2 x - D' x - i (omega^2/eta)(n1 S n1 x + n2 S n2 x)
+// y = sum of split partials, as FP32 pairs (TwoSum, errors gathered: 48 bits,
+// without the FP64 pipe); hard: t = S u (complex64 for the derivative) and
+// y = 1/2 x + C x
 template <int BC>
-__global__ void k_reduce32(int n, int nrhs, int splits, double omega, double eta, geom_dev g,
-                           const float2* __restrict__ part, const double2* __restrict__ x,
-                           float2* __restrict__ t_out, double2* __restrict__ y) {
+__global__ void k_reduce32(size_t tot, int splits, const float2* __restrict__ part,
+                           const double2* __restrict__ x, float2* __restrict__ t_out,
+                           double2* __restrict__ y) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t tot = (size_t)n * nrhs;
   if (e >= tot) return;
-  const size_t so = (size_t)splits * tot;
-  double2 s[4] = {};
-  for (int o = 0; o < (BC ? 4 : 1); ++o) {
-    double2 v = make_double2(0.0, 0.0);
+  auto two_sum = [](float& s, float& err, float p) {
+    const float t = s + p, v = t - s;
+    err += (s - (t - v)) + (p - v);
+    s = t;
+  };
+  double2 s[BC ? 2 : 1];
+#pragma unroll
+  for (int o = 0; o < (BC ? 2 : 1); ++o) {
+    float2 v = make_float2(0.f, 0.f), err = v;
+#pragma unroll 4
     for (int sp = 0; sp < splits; ++sp) {
-      const float2 p = part[o * so + (size_t)sp * tot + e];
-      v.x += p.x;
-      v.y += p.y;
+      const float2 p = part[((size_t)o * splits + sp) * tot + e];
+      two_sum(v.x, err.x, p.x);
+      two_sum(v.y, err.y, p.y);
     }
-    s[o] = v;
+    s[o] = make_double2((double)v.x + (double)err.x, (double)v.y + (double)err.y);
   }
   if (BC == 0) {
     y[e] = s[0];
   } else {
-    const int i = (int)(e % n);
-    const double inv = 1.0 / g.sp[i];
-    const double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-    const double2 m = make_double2(n1 * s[1].x + n2 * s[2].x, n1 * s[1].y + n2 * s[2].y);
-    const double k = omega * omega / eta;
-    const double2 xv = x[e];
-    y[e] = make_double2(0.5 * xv.x - s[3].x + k * m.y, 0.5 * xv.y - s[3].y - k * m.x);
+    const double2 xv = x[e], c = s[BC ? 1 : 0];
+    y[e] = make_double2(fma(0.5, xv.x, c.x), fma(0.5, xv.y, c.y));
     t_out[e] = make_float2((float)s[0].x, (float)s[0].y);
   }
 }
@@ -321,7 +316,7 @@ __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w
                         const double* __restrict__ ct, const unsigned* __restrict__ bound,
                         double omega, double eta, double h, float* __restrict__ w32,
                         float* __restrict__ c32, float4* __restrict__ pk,
-                        float2* __restrict__ wkt) {
+                        float2* __restrict__ wkt, int hard, float* __restrict__ sp4) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < 8) wkt[2 * n + i] = make_float2(0.f, 0.f);
   if (i >= n) return;
@@ -355,6 +350,17 @@ __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w
   pk[n + i] = make_float4((float)(omega * f * nx), (float)(omega * f * ny),
                           (float)(f * eta * sp), (float)(f * sp));
   pk[2 * n + i] = make_float4((float)(omega * nx / sp), (float)(omega * ny / sp), 0.f, 0.f);
+  // source data by pairs: value v of node i at 4 (i / 2 * 2 + v / 2) + 2 (v % 2) + i % 2
+  float* sq = sp4 + (size_t)(i / 2) * 8 + (i & 1);
+  sq[0] = -xh;
+  sq[2] = -xl;
+  sq[4] = -yh;
+  sq[6] = -yl;
+  sq += (size_t)4 * n;
+  sq[0] = (float)(hard ? omega / eta * nx / sp : omega * f * nx);
+  sq[2] = (float)(hard ? omega / eta * ny / sp : omega * f * ny);
+  sq[4] = (float)(hard ? f * sp : f * eta * sp);
+  sq[6] = 0.f;
 }
 
 // Largest cyclic index distance |i - j| of a pair with omega r < X0 (with a
@@ -475,7 +481,7 @@ int launch32(cfie_op* op, pair_params P, int rowtiles, int slices) {
   int tps = (ntiles + best_s - 1) / best_s;
   P.splits = (ntiles + tps - 1) / tps;
   P.tiles_per_split = tps;
-  const int ops = BC ? 4 : 1;
+  const int ops = BC ? 2 : 1;
   op->partial.reserve(sizeof(float2) * (size_t)ops * P.splits * P.nrhs * P.n);
   P.part = op->partial.as<float2>();
   dim3 grid(rowtiles, P.splits, slices);
@@ -528,7 +534,8 @@ void fp32_prepare(cfie_op* op) {
   k_geo32<<<nblk(n), 256, 0, st>>>(n, op->g, o, op->wtab.as<double>(), op->ctab.as<double>(),
                                     bound, op->omega, op->eta, op->h, w32, c32,
                                     reinterpret_cast<float4*>(base + geo32_pack_offset(n)),
-                                    reinterpret_cast<float2*>(base + geo32_wk_offset(n)));
+                                    reinterpret_cast<float2*>(base + geo32_wk_offset(n)),
+                                    op->bc == CFIE_SOUND_HARD, base + geo32_pair_offset(n));
   CFIE_CHECK_LAUNCH();
 }
 
@@ -557,13 +564,12 @@ void fp32_band(cfie_op* op) {
   CFIE_CHECK_CUDA(cudaStreamSynchronize(st));
 }
 
-void k_to32_fp32(cfie_op* op, const double2* x, float2* x32, size_t tot) {
-  k_to32<<<nblk(tot), 256, 0, op->ctx->stream>>>(tot, x, x32);
-  CFIE_CHECK_LAUNCH();
-}
-
 void spectral32_apply(cfie_op* op, const float2* x32, float2* u32, int nrhs) {
   spectral_fft32_apply(op, x32, u32, nrhs);
+}
+
+void spectral32_apply(cfie_op* op, const double2* x, float2* u32, int nrhs) {
+  spectral_fft32_apply(op, x, u32, nrhs);
 }
 
 void spectral32_accumulate(cfie_op* op, const float2* t32, double2* y, int nrhs) {
@@ -602,8 +608,7 @@ void matvec_fp32(cfie_op* op, const double2* x, double2* y, int nrhs) {
       splits = launch32<0, 16>(op, P, rowtiles, 1);
     else
       splits = launch32<0, 8>(op, P, rowtiles, 1);
-    k_reduce32<0><<<nblk(tot), 256, 0, st>>>(n, nrhs, splits, op->omega, op->eta, op->g,
-                                             op->partial.as<float2>(), x, nullptr, y);
+    k_reduce32<0><<<nblk(tot), 256, 0, st>>>(tot, splits, op->partial.as<float2>(), x, nullptr, y);
     CFIE_CHECK_LAUNCH();
     return;
   }
@@ -611,13 +616,15 @@ void matvec_fp32(cfie_op* op, const double2* x, double2* y, int nrhs) {
   float2* t32 = x32 + 2 * tot;
   spectral32_apply(op, x32, u32, nrhs);
   P.uin = u32;
+  P.k2 = (float)(op->omega * op->omega / op->eta);
   int splits;
-  if (nrhs > 8)
-    splits = launch32<1, 16>(op, P, rowtiles, (nrhs + 15) / 16);
+  if (nrhs > 16)
+    splits = launch32<1, 32>(op, P, rowtiles, (nrhs + 31) / 32);
+  else if (nrhs > 8)
+    splits = launch32<1, 16>(op, P, rowtiles, 1);
   else
     splits = launch32<1, 8>(op, P, rowtiles, 1);
-  k_reduce32<1><<<nblk(tot), 256, 0, st>>>(n, nrhs, splits, op->omega, op->eta, op->g,
-                                           op->partial.as<float2>(), x, t32, y);
+  k_reduce32<1><<<nblk(tot), 256, 0, st>>>(tot, splits, op->partial.as<float2>(), x, t32, y);
   CFIE_CHECK_LAUNCH();
   // y += (1/(i eta)) (1/s) Dt t
   spectral32_accumulate(op, t32, y, nrhs);

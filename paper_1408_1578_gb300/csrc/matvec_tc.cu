@@ -1,24 +1,38 @@
 // Matrix-free FP32 matvec with the source summation on the tensor cores.
 //
-// Same entries as the FP32 fused kernel (sound-soft operator of eq. 1: FP32
-// pair evaluation with two-float phase and Hankel asymptotics, FP64-evaluated
-// near band), but instead of the register-blocked FP32 contraction the entries
-// of each 128 x 32 tile are written, split as bf16 hi + lo, straight into
-// shared memory in the tensor cores' 64-byte-swizzled K-major layout, and one
-// thread issues tcgen05.mma against the right-hand-side block (bf16 hi / lo
-// planes brought in by TMA):
+// Same entries as the FP32 fused kernel (FP32 pair evaluation with two-float
+// phase and Hankel asymptotics, FP64-evaluated near band), but instead of the
+// register-blocked FP32 contraction the entries of each 128 x 32 tile are
+// written, split as bf16 hi + lo, straight into shared memory in the tensor
+// cores' 64-byte-swizzled K-major layout, and one thread issues tcgen05.mma
+// against the right-hand-side block (bf16 hi / lo planes brought in by TMA):
 //
 //     [Yr | Yi] += Ar [Xr | Xi] + Ai [-Xi | Xr],  each product hi*hi + hi*lo + lo*hi,
 //
-// FP32 accumulation in tensor memory.  Work is split stream-K: the
-// (128-row tile, 32-source tile) pairs form one list and each CTA (one per SM)
-// takes a contiguous range, cut into segments that end at row-tile boundaries.
-// Warp roles (22 warps): 0-15 evaluate pair entries into the stage ring, 16
-// issues the TMA loads of the right-hand sides, of each tile's source geometry
-// and of its Kress window, 17 issues the MMAs (double-buffered accumulators),
-// 18-21 drain finished accumulators into per-segment partial sums, which a
-// second kernel adds in a fixed order.  All mbarrier waits are bounded (error
-// flag, drain, TMEM freed on every path).
+// FP32 accumulation in tensor memory.  The sound-hard operator (eq. 2 with
+// Maue's identity) is two operators over the same pairs, S on u = d/ds x and
+// C = -D' - i (omega^2 / eta) (n_i . n_j) S on x (n1 S n1 + n2 S n2 has the
+// entries (n_i . n_j) S_ij); up to 32 right-hand sides one pass evaluates both
+// from one phase, above that each has a pass of its own (both sets of operand
+// planes of 64 right-hand sides do not fit two stages of shared memory).
+// Work is split stream-K: the (128-row tile, 32-source tile) pairs form one
+// list and each CTA (one per SM) takes a contiguous range, cut into segments
+// that end at row-tile boundaries.  Warp roles (22 warps): 0-15 evaluate pair
+// entries into the stage ring, 16 issues the TMA loads of the right-hand sides,
+// of each tile's source geometry and of its Kress window, 17 issues the MMAs
+// (double-buffered accumulators), 18-21 drain finished accumulators into
+// per-segment partial sums, which a second kernel adds in a fixed order.  All
+// mbarrier waits are bounded (error flag, drain, TMEM freed on every path).
+//
+// Bound: the producers' FP32 arithmetic (FMA pipe 75 % busy, ncu).  A lane keeps
+// one target and evaluates the entries of eight adjacent sources in packed FP32
+// pairs (pair32.cuh), which issue half as often as scalar instructions, four
+// independent chains at a time; the sources are warp-uniform loads from a ring
+// filled three tiles ahead.  Measured (GB300), kernel alone: kite n = 32768, 64
+// right-hand sides 2.95 -> 2.53 ms (packed pairs in the former layout, a row
+// per half warp: 2.97, bound by shared-memory cycles and by waits for the
+// source loads); ellipse n = 32768, 1 right-hand side, sound hard, 4.90 (S and
+// D' in two passes) -> 2.98 ms; two pairs at a time instead of four: 2.60 ms.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -36,7 +50,6 @@ namespace {
 
 constexpr int TBM = 128;     // targets per tile (UMMA M)
 constexpr int TBK = 32;      // sources per tile (32 bf16 = one 64-byte swizzle row)
-constexpr int TSTAGES = 3;
 // Source tiles accumulated in one tensor-memory accumulator before the epilogue
 // warps add it into their running sums.  The tensor core's FP32 accumulation
 // does not round to nearest: its error grows with the number of MMAs summed
@@ -45,54 +58,127 @@ constexpr int TSTAGES = 3;
 // to nearest) and the FP64 segment reduction add only unbiased rounding.
 constexpr int CK = 8;
 constexpr int WKW = TBM + TBK + 2;   // Kress window of a tile (+ alignment slack)
+// Source data (geometry, Kress window) are fetched this many tiles ahead, into
+// a ring of their own: with the operand stages' ring the producers stood idle
+// for the latency of these loads whenever a stage came free
+constexpr int LOOK = 3;
 constexpr int NPROD = 16;    // producer warps
 constexpr int WTMA = NPROD, WMMA = NPROD + 1;   // then the epilogue warps
-constexpr int TNT = (NPROD + 6) * 32;
-constexpr int QI = 2;        // rows whose entries a producer lane evaluates together
+constexpr int NEPI = 4;      // epilogue warps
+// six warpgroups of 128 threads: four of producers, then the other roles and
+// two warps that only make the last warpgroup whole
+constexpr int TNT = (NPROD + 8) * 32;
+// Registers per thread: the launch has TNT x 80; the producers take 96 (their
+// constants are packed pairs), the others give up what that costs (512 x 96 +
+// 256 x 48 = 768 x 80)
+constexpr int RLAUNCH = 80, RPRODUCER = 96, ROTHER = 48;
+static_assert(NPROD * 32 * RPRODUCER + (TNT - NPROD * 32) * ROTHER <= TNT * RLAUNCH,
+              "register shares exceed the launch's total");
 
 struct tc_params {
   int n, b, ktiles;
   const float2* wext;    // Kress table / (pi h) at i - j + n, paired with the next source's
   const float4* pk;      // packed coordinates, source factors, target factors (n each)
-  const float2* band;    // near entries of the evaluated kind (soft A, or S, or D')
+  const float4* spk;     // source coordinates by pairs, source factors by pairs (n each)
+  const float2* band;    // near entries: soft A, or S, then D'
 };
 
-// bf16 hi / lo split of two entries of one row (adjacent sources k, k + 1)
-// into the four A planes: one packed 32-bit word per plane at byte offset o
-__device__ __forceinline__ void store_split2(unsigned char* a0, unsigned char* a1,
-                                             unsigned char* a2, unsigned char* a3, uint32_t o,
-                                             float2 e0, float2 e1) {
-  const __nv_bfloat162 hr = __floats2bfloat162_rn(e0.x, e1.x);
-  const __nv_bfloat162 hi = __floats2bfloat162_rn(e0.y, e1.y);
-  const __nv_bfloat162 lr =
-      __floats2bfloat162_rn(e0.x - __low2float(hr), e1.x - __high2float(hr));
-  const __nv_bfloat162 li =
-      __floats2bfloat162_rn(e0.y - __low2float(hi), e1.y - __high2float(hi));
-  *reinterpret_cast<__nv_bfloat162*>(a0 + o) = hr;
-  *reinterpret_cast<__nv_bfloat162*>(a1 + o) = hi;
-  *reinterpret_cast<__nv_bfloat162*>(a2 + o) = lr;
-  *reinterpret_cast<__nv_bfloat162*>(a3 + o) = li;
+// bf16 hi / lo split of eight entries of one row (adjacent sources): the packed
+// words of the four planes (hi re, hi im, lo re, lo im) of each operator
+template <int NO>
+struct split_words {
+  uint32_t v[NO][4][4];
+  __device__ __forceinline__ static void split(float2 e, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(e.x, e.y);
+    hi = *reinterpret_cast<const uint32_t*>(&b);
+    const float2 h = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+    const float2 d = add2(e, neg2(h));
+    const __nv_bfloat162 c = __floats2bfloat162_rn(d.x, d.y);
+    lo = *reinterpret_cast<const uint32_t*>(&c);
+  }
+  __device__ __forceinline__ void put(int p, const entry_pair& e) {
+    split(e.re, v[0][0][p], v[0][2][p]);
+    split(e.im, v[0][1][p], v[0][3][p]);
+    if constexpr (NO == 2) {
+      split(e.re2, v[1][0][p], v[1][2][p]);
+      split(e.im2, v[1][1][p], v[1][3][p]);
+    }
+  }
+  // planes `plane` bytes apart, operators four planes apart
+  __device__ __forceinline__ void store(unsigned char* a, uint32_t plane) const {
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<uint4*>(a + (4 * o + c) * plane) =
+            make_uint4(v[o][c][0], v[o][c][1], v[o][c][2], v[o][c][3]);
+  }
+};
+
+// Two entries of a tile that the near band or the end of the curve touches:
+// band entries replace the far ones, rows and sources past n are zero
+template <int OP>
+__device__ __forceinline__ entry_pair near_pair(const tc_params& P, float4 t0, float4 t1, float4 tn,
+                                                const float4* sc, const float4* sf, int i, int j) {
+  entry_pair e;
+  e.re = e.im = e.re2 = e.im2 = f2(0.f);
+  const int n = P.n;
+  if (i >= n || j >= n) return e;                    // n is even: j + 1 < n as well
+  const float4 g0 = sf[0];
+  e = finish32_pair<OP>(phase32_pair(t0, t1, sc[0], sc[1]), tn, g0, lo2(sf[1]), P.wext[i - j + n]);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    int d = i - j - u;
+    if (d < 0) d += n;
+    const int dd = d <= P.b ? d : (d >= n - P.b ? d - n : INT_MAX);
+    if (dd == INT_MAX) continue;
+    const size_t bw = 2 * (size_t)P.b + 1, at = (size_t)i * bw + dd + P.b;
+    const float2 bv = P.band[at];                    // soft A, or S
+    float2 s = bv, c = f2(0.f);
+    if constexpr (OP != OP_SOFT) s = make_float2(bv.y, -bv.x);   // S' = -i S
+    if constexpr (OP == OP_C || OP == OP_SC) {
+      // C = -D' + (omega^2 / eta) (n_i . n_j) S'
+      const float2 dp = P.band[(size_t)n * bw + at];
+      const float kn = tn.x * (u ? g0.y : g0.x) + tn.z * (u ? g0.w : g0.z);
+      c = make_float2(fmaf(kn, s.x, -dp.x), fmaf(kn, s.y, -dp.y));
+    }
+    const float2 first = OP == OP_C ? c : s;
+    if (u) {
+      e.re.y = first.x, e.im.y = first.y;
+      e.re2.y = c.x, e.im2.y = c.y;
+    } else {
+      e.re.x = first.x, e.im.x = first.y;
+      e.re2.x = c.x, e.im2.x = c.y;
+    }
+  }
+  return e;
 }
 
-template <int NP>
+// operators evaluated by a pass, and the stages that fit
+template <int OP>
+__host__ __device__ constexpr int tc_ops() { return OP == OP_SC ? 2 : 1; }
+template <int NP, int OP>
+__host__ __device__ constexpr int tc_stages() { return OP == OP_SC ? 2 : 3; }
+
+template <int NP, int OP>
 struct tc_smem {
-  __nv_bfloat16 A[TSTAGES][4][TBM * TBK];   // hi_re, hi_im, lo_re, lo_im
-  __nv_bfloat16 B[TSTAGES][4][NP * TBK];    // B1 hi, B1 lo, B2 hi, B2 lo
-  float4 tgt[TBM];                          // targets (x hi, x lo, y hi, y lo)
-  float4 tgn[TBM];                          // target factors (D' only)
-  float4 src[TSTAGES][2][TBK];              // sources: coordinates, factors
-  float2 wk[TSTAGES][WKW];                  // Kress weight pairs / (pi h) of a plain tile
-  uint64_t full[TSTAGES], empty[TSTAGES], sfull[TSTAGES], tfull[2], tempty[2];
+  static constexpr int NO = tc_ops<OP>(), ST = tc_stages<NP, OP>(), SD = ST + LOOK;
+  __nv_bfloat16 A[ST][NO][4][TBM * TBK];    // per operator: hi_re, hi_im, lo_re, lo_im
+  __nv_bfloat16 B[ST][NO][4][NP * TBK];     // per operator: B1 hi, B1 lo, B2 hi, B2 lo
+  float4 src[SD][2][TBK];                   // sources by pairs: coordinates, factors
+  float2 wk[SD][WKW];                       // Kress weight pairs / (pi h) of a plain tile
+  uint64_t full[ST], empty[ST], sfull[SD], tfull[2], tempty[2];
   uint64_t mdone;                           // completion of every MMA issued (abort path)
   uint32_t tmem_base;
   int abort;
-  int issued[TSTAGES], sissued[TSTAGES];
-  int wofs[TSTAGES];                        // plain tile: window entry of (row 0, source 0); else -1
+  int issued[ST], sissued[SD];
+  int wofs[SD];                             // plain tile: window entry of (row 0, source 0); else -1
 };
 
-template <int NP>
+template <int NP, int OP>
 constexpr size_t tc_smem_bytes() {
-  return sizeof(tc_smem<NP>) + 1024;
+  static_assert(sizeof(tc_smem<NP, OP>) + 1024 <= 227 * 1024, "stages exceed shared memory");
+  return sizeof(tc_smem<NP, OP>) + 1024;
 }
 
 // byte offset of element (row r, k) in a 64-byte-swizzled K-major tile
@@ -100,18 +186,22 @@ __device__ __forceinline__ uint32_t sw64(int r, int k) {
   return (uint32_t)(r * 64 + ((((k >> 3) ^ (r >> 1)) & 3) << 4) + (k & 7) * 2);
 }
 
-template <int NP, int KIND>
+template <int NP, int OP>
 __global__ void __launch_bounds__(TNT, 1)
 k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __restrict__ segs,
            const int* __restrict__ cbeg, float2* __restrict__ partial, int* __restrict__ err) {
-  constexpr int NR = NP / 2;
-  // two accumulator buffers, then the epilogue's running sums (NP columns each)
-  constexpr uint32_t TMEM_COLS = 3 * NP <= 256 ? 256 : 512;
-  constexpr uint32_t RUN = 2 * NP;
-  constexpr uint32_t B_BYTES = 4u * NP * TBK * 2u;
+  constexpr int NR = NP / 2, NO = tc_ops<OP>(), TSTAGES = tc_stages<NP, OP>();
+  constexpr int SD = TSTAGES + LOOK;
+  constexpr bool HAS_TQ = OP == OP_C || OP == OP_SC;
+  // per operator two accumulator buffers, then the epilogue's running sums
+  // (NP columns each)
+  constexpr uint32_t TMEM_COLS = 3 * NO * NP <= 256 ? 256 : 512;
+  static_assert(3 * NO * NP <= 512, "accumulators exceed the tensor memory");
+  constexpr uint32_t RUN = 2 * NO * NP;
+  constexpr uint32_t B_BYTES = 4u * NO * NP * TBK * 2u;
+  constexpr uint32_t APLANE = TBM * TBK * 2u;    // bytes of one A plane
   extern __shared__ unsigned char raw[];
-  tc_smem<NP>& S = *reinterpret_cast<tc_smem<NP>*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
-                                                    ~uintptr_t(1023));
+  tc_smem<NP, OP>& S = smem_aligned<tc_smem<NP, OP>>(raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sb = cbeg[blockIdx.x], se = cbeg[blockIdx.x + 1];
   const int n = P.n;
@@ -120,13 +210,15 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
     for (int s = 0; s < TSTAGES; ++s) {
       mbar_init(&S.full[s], NPROD + 1);        // one arrival per producer warp + the TMA thread
       mbar_init(&S.empty[s], 1);
-      mbar_init(&S.sfull[s], 1);
       S.issued[s] = -1;
+    }
+    for (int s = 0; s < SD; ++s) {
+      mbar_init(&S.sfull[s], 1);
       S.sissued[s] = -1;
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&S.tfull[b], 1);
-      mbar_init(&S.tempty[b], 4);
+      mbar_init(&S.tempty[b], NEPI);
     }
     mbar_init(&S.mdone, 1);
     S.abort = 0;
@@ -142,116 +234,75 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
   const uint32_t tmem = S.tmem_base;
 
   if (warp < NPROD) {
-    // ---- pair-entry producers.  Warp w owns rows w + NPROD q (q < TBM / NPROD);
-    // each step of its loop covers two of them: lanes 0-15 the first, lanes
-    // 16-31 the second, lane l the two adjacent sources 2 (l % 16), +1, so
-    // that the bf16 pairs go to shared memory as packed 32-bit words.
-    const int half = lane >> 4, jp = 2 * (lane & 15);
-    // byte offset of the lane's two sources in its first row of a step; the
-    // rows of step q lie 2 NPROD q rows further on, a multiple of the 8-row
-    // period of the 64-byte swizzle, hence 2 NPROD q 64 bytes further
-    static_assert((2 * NPROD) % 8 == 0, "row step must keep the swizzle phase");
-    const uint32_t sbase = sw64(warp + NPROD * half, jp);
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RPRODUCER));
+    // ---- pair-entry producers.  Lane l of warp w owns row 32 (w % 4) + l of
+    // the tile and the eight sources 8 (w / 4) .. + 7: the target stays in
+    // registers for the whole segment, the sources are warp-uniform shared
+    // loads, and the bf16 entries of a plane are one 16-byte chunk of the
+    // swizzled tile, which 8 consecutive rows store without a bank conflict.
+    // (A row per half warp, sources across its lanes, spent 65 % of the
+    // shared-memory cycles on the strided source loads, the targets and
+    // two-way conflicted stores.)
+    const int row = 32 * (warp & 3) + lane, js = 8 * (warp >> 2);
+    const uint32_t off = sw64(row, js);
     int it = 0;
     for (int s = sb; s < se; ++s) {
       const int4 sg = segs[s];
       const int m0 = sg.y * TBM;
-      // stage the target geometry of this warp's own rows: no other warp
-      // reads them, so a warp-level barrier is enough
-      __syncwarp();
-      if (lane < TBM / NPROD) {
-        const int r = warp + NPROD * lane;
-        const int i = m0 + r;
-        const bool ok = i < n;
-        S.tgt[r] = ok ? P.pk[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (KIND == KIND_DP) S.tgn[r] = ok ? P.pk[2 * n + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int i = m0 + row;
+      float4 t0, t1, tn;
+      {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 g = i < n ? P.pk[i] : z;
+        t0 = make_float4(g.x, g.x, g.y, g.y);
+        t1 = make_float4(g.z, g.z, g.w, g.w);
+        const float4 q = HAS_TQ && i < n ? P.pk[2 * n + i] : z;
+        tn = make_float4(q.x, q.x, q.y, q.y);
       }
-      __syncwarp();
       for (int k = sg.z; k < sg.w; ++k, ++it) {
         const int st = it % TSTAGES;
-        const int j0 = k * TBK;
-        const int j = j0 + jp;                       // first of the lane's two sources
+        const int j = k * TBK + js;                  // first of the lane's eight sources
         // exits are warp-uniform: the warp arrives on the stage barrier as one
         if (__any_sync(0xffffffffu, *(volatile int*)&S.abort)) break;
-        // this tile's source geometry and Kress window, brought in by the TMA
-        // warp once the MMAs of the stage's previous tile were done (so the A
-        // planes of the stage are free as well)
-        if (!__all_sync(0xffffffffu, mbar_wait(&S.sfull[st], (it / TSTAGES) & 1))) {
+        // this tile's source geometry and Kress window (from the TMA warp),
+        // and the stage's A planes (the MMAs of its previous tile are done)
+        const int sl = it % SD;
+        bool ok = mbar_wait_sleep<40>(&S.sfull[sl], (it / SD) & 1);
+        if (ok && it >= TSTAGES) ok = mbar_wait_sleep<40>(&S.empty[st], ((it / TSTAGES) - 1) & 1);
+        if (!__all_sync(0xffffffffu, ok)) {
           if (lane == 0) {
             atomicExch(err, 15);
             S.abort = 1;
           }
           break;
         }
-        const float4 sc[2] = {S.src[st][0][jp], S.src[st][0][jp + 1]};
-        const float4 sn[2] = {S.src[st][1][jp], S.src[st][1][jp + 1]};
-        unsigned char* a0 = reinterpret_cast<unsigned char*>(S.A[st][0]);
-        unsigned char* a1 = reinterpret_cast<unsigned char*>(S.A[st][1]);
-        unsigned char* a2 = reinterpret_cast<unsigned char*>(S.A[st][2]);
-        unsigned char* a3 = reinterpret_cast<unsigned char*>(S.A[st][3]);
+        unsigned char* a = reinterpret_cast<unsigned char*>(S.A[st][0][0]) + off;
+        const float4* sc = S.src[sl][0] + js;
+        const float4* sf = S.src[sl][1] + js;
         // Plain tiles (all but ~1%, flagged by the TMA warp) skip the per-pair
         // range and band tests and take the Kress weights from the staged
         // window of the unwrapped table (entry i - j + n)
-        const int wofs = S.wofs[st];
-        constexpr int QS = TBM / NPROD / 2;          // loop steps (two rows each)
+        const int wofs = S.wofs[sl];
+        const float2* wq = S.wk[sl] + wofs + row - js;
+        split_words<NO> w;
+        entry_pair e[4];
         if (wofs >= 0) {
-          const float2* wq = S.wk[st] + wofs + warp + NPROD * half - jp;
-          float2 wv[QS];
+          // the phases (special-function ops) of the four pairs of sources
+          // first, then the series and assembly, so that the chains interleave
+          pair_phase2 f[4];
 #pragma unroll
-          for (int q = 0; q < QS; ++q) wv[q] = wq[2 * NPROD * q];
-          // QI rows at a time: the phases (special-function ops) of their
-          // 2 QI entries first, then the series and assembly, so that the
-          // independent chains interleave
+          for (int u = 0; u < 4; ++u) f[u] = phase32_pair(t0, t1, sc[2 * u], sc[2 * u + 1]);
 #pragma unroll
-          for (int q0 = 0; q0 < QS; q0 += QI) {
-            pair_phase f[QI][2];
-            float4 tn[QI];
-#pragma unroll
-            for (int r = 0; r < QI; ++r) {
-              const int il = warp + NPROD * (2 * (q0 + r) + half);
-              const float4 tg = S.tgt[il];
-              tn[r] = KIND == KIND_DP ? S.tgn[il] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-              for (int u = 0; u < 2; ++u)
-                f[r][u] = pair_phase32_tc(tg.x, tg.y, tg.z, tg.w, sc[u].x, sc[u].y, sc[u].z,
-                                          sc[u].w);
-            }
-#pragma unroll
-            for (int r = 0; r < QI; ++r) {
-              const int q = q0 + r;
-              float2 e[2];
-#pragma unroll
-              for (int u = 0; u < 2; ++u)
-                e[u] = entry_finish32<KIND>(f[r][u], tn[r], sn[u], u ? wv[q].y : wv[q].x);
-              store_split2(a0, a1, a2, a3, sbase + (uint32_t)(2 * NPROD * 64 * q), e[0], e[1]);
-            }
-          }
+          for (int u = 0; u < 4; ++u)
+            e[u] = finish32_pair<OP>(f[u], tn, sf[2 * u], lo2(sf[2 * u + 1]), wq[-2 * u]);
         } else {
-#pragma unroll 1
-          for (int q = 0; q < QS; ++q) {
-            const int il = warp + NPROD * (2 * q + half);
-            const int i = m0 + il;
-            const float4 tg = S.tgt[il];
-            const float4 tn = KIND == KIND_DP ? S.tgn[il] : make_float4(0.f, 0.f, 0.f, 0.f);
-            float2 e[2];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const int jj = j + u;
-              float2 a = make_float2(0.f, 0.f);
-              if (i < n && jj < n) {
-                int d = i - jj;
-                if (d < 0) d += n;
-                const int dd = d <= P.b ? d : (d >= n - P.b ? d - n : INT_MAX);
-                if (dd != INT_MAX)
-                  a = P.band[(size_t)i * (2 * P.b + 1) + dd + P.b];
-                else
-                  a = entry_folded32<KIND>(tg, tn, sc[u], sn[u], P.wext[i - jj + n].x);
-              }
-              e[u] = a;
-            }
-            store_split2(a0, a1, a2, a3, sbase + (uint32_t)(2 * NPROD * 64 * q), e[0], e[1]);
-          }
+          for (int u = 0; u < 4; ++u)
+            e[u] = near_pair<OP>(P, t0, t1, tn, sc + 2 * u, sf + 2 * u, i, j + 2 * u);
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w.put(u, e[u]);
+        w.store(a, APLANE);
         // generic-proxy writes become visible to the tensor core's async proxy;
         // the warp's writes are ordered before its one arrival by __syncwarp
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -260,16 +311,44 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
       }
       if (__any_sync(0xffffffffu, *(volatile int*)&S.abort)) break;
     }
-  } else if (warp == WTMA) {
-    if (lane == 0) {
-      // ---- TMA producer of the right-hand-side planes
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ROTHER));
+    if (warp == WTMA && lane == 0) {
+      // ---- TMA producer of the right-hand-side planes and the source data
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+      // Source data of the next tile of the list (segment ls, source tile lk,
+      // running number lt).  A tile is plain when it holds full rows and
+      // sources and no pair of the near band: d = i - j spans [dlo, dhi] there,
+      // and the band is |d - t n| <= b for t = -1, 0, 1; a plain tile also gets
+      // the window of the Kress table (entries dlo + n ... dhi + n) from the
+      // 16-byte boundary below it.  Window bytes: WKW float2 = 1296, a multiple
+      // of 16.
+      int ls = sb, lt = 0, lk = sb < se ? segs[sb].z : 0;
+      auto load_sources = [&] {
+        if (ls >= se) return;
+        const int4 sg = segs[ls];
+        const int sl = lt % SD, m0 = sg.y * TBM, j0 = lk * TBK;
+        const int dlo = m0 - j0 - (TBK - 1), dhi = m0 + TBM - 1 - j0;
+        bool near = false;
+#pragma unroll
+        for (int t = -1; t <= 1; ++t) near |= (dhi >= t * n - P.b) && (dlo <= t * n + P.b);
+        const bool plain = !near && m0 + TBM <= n && j0 + TBK <= n;
+        S.wofs[sl] = plain ? m0 - j0 + n - ((dlo + n) & ~1) : -1;
+        mbar_arrive_expect_tx(&S.sfull[sl], 2u * TBK * 16u + (plain ? WKW * 8u : 0u));
+        S.sissued[sl] = (lt / SD) & 1;
+        bulk_load(S.src[sl][0], P.spk + j0, TBK * 16u, &S.sfull[sl]);
+        bulk_load(S.src[sl][1], P.spk + n + j0, TBK * 16u, &S.sfull[sl]);
+        if (plain) bulk_load(S.wk[sl], P.wext + ((dlo + n) & ~1), WKW * 8u, &S.sfull[sl]);
+        ++lt;
+        if (++lk == sg.w && ++ls < se) lk = segs[ls].z;
+      };
+      for (int q = 0; q < LOOK; ++q) load_sources();
       int it = 0;
       for (int s = sb; s < se && !*(volatile int*)&S.abort; ++s) {
         const int4 sg = segs[s];
         for (int k = sg.z; k < sg.w; ++k, ++it) {
           const int st = it % TSTAGES;
-          if (it >= TSTAGES && !mbar_wait(&S.empty[st], ((it / TSTAGES) - 1) & 1)) {
+          if (it >= TSTAGES && !mbar_wait_sleep<40>(&S.empty[st], ((it / TSTAGES) - 1) & 1)) {
             atomicExch(err, 12);
             S.abort = 1;
             break;
@@ -277,30 +356,15 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
           mbar_arrive_expect_tx(&S.full[st], B_BYTES);
           S.issued[st] = (it / TSTAGES) & 1;
 #pragma unroll
-          for (int p = 0; p < 4; ++p) tma_load_2d(S.B[st][p], &tmB, &S.full[st], k * TBK, p * NP);
-          // Source coordinates and factors of the tile.  A tile is plain when
-          // it holds full rows and sources and no pair of the near band: d =
-          // i - j spans [dlo, dhi] there, and the band is |d - t n| <= b for
-          // t = -1, 0, 1; a plain tile also gets the window of the Kress table
-          // (entries dlo + n ... dhi + n) from the 16-byte boundary below it.
-          // Window bytes: WKW float2 = 1296, a multiple of 16.
-          const int m0 = sg.y * TBM, j0 = k * TBK;
-          const int dlo = m0 - j0 - (TBK - 1), dhi = m0 + TBM - 1 - j0;
-          bool near = false;
-#pragma unroll
-          for (int t = -1; t <= 1; ++t) near |= (dhi >= t * n - P.b) && (dlo <= t * n + P.b);
-          const bool plain = !near && m0 + TBM <= n && j0 + TBK <= n;
-          S.wofs[st] = plain ? m0 - j0 + n - ((dlo + n) & ~1) : -1;
-          mbar_arrive_expect_tx(&S.sfull[st], 2u * TBK * 16u + (plain ? WKW * 8u : 0u));
-          S.sissued[st] = (it / TSTAGES) & 1;
-          bulk_load(S.src[st][0], P.pk + j0, TBK * 16u, &S.sfull[st]);
-          bulk_load(S.src[st][1], P.pk + n + j0, TBK * 16u, &S.sfull[st]);
-          if (plain) bulk_load(S.wk[st], P.wext + ((dlo + n) & ~1), WKW * 8u, &S.sfull[st]);
+          for (int p = 0; p < 4 * NO; ++p)
+            tma_load_2d(S.B[st][p / 4][p % 4], &tmB, &S.full[st], k * TBK, p * NP);
+          // the slot of tile it + LOOK held tile it - TSTAGES, whose MMAs, and
+          // so whose producers, are done
+          load_sources();
         }
       }
     }
-  } else if (warp == WMMA) {
-    if (lane == 0) {
+    if (warp == WMMA && lane == 0) {
       // ---- MMA issuer: one accumulator buffer per chunk of CK source tiles
       constexpr uint32_t idesc = make_idesc(TBM, NP);
       int it = 0, cc = 0;
@@ -309,35 +373,38 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
         for (int c0 = sg.z; c0 < sg.w; c0 += CK, ++cc) {
           const int c1 = min(sg.w, c0 + CK);
           const int tb = cc & 1, use = cc >> 1;
-          if (use >= 1 && !mbar_wait(&S.tempty[tb], (use - 1) & 1)) {
+          if (use >= 1 && !mbar_wait_sleep<40>(&S.tempty[tb], (use - 1) & 1)) {
             atomicExch(err, 14);
             S.abort = 1;
           }
           if (*(volatile int*)&S.abort) break;
           tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)(tb * NP);
           for (int k = c0; k < c1; ++k, ++it) {
             const int st = it % TSTAGES;
-            if (!mbar_wait(&S.full[st], (it / TSTAGES) & 1)) {
+            if (!mbar_wait_sleep<40>(&S.full[st], (it / TSTAGES) & 1)) {
               atomicExch(err, 13);
               S.abort = 1;
               break;
             }
             tc_fence_after();
-            const uint32_t a0 = smem_u32(S.A[st][0]), a1 = smem_u32(S.A[st][1]);
-            const uint32_t a2 = smem_u32(S.A[st][2]), a3 = smem_u32(S.A[st][3]);
-            const uint32_t b0 = smem_u32(S.B[st][0]), b1 = smem_u32(S.B[st][1]);
-            const uint32_t b2 = smem_u32(S.B[st][2]), b3 = smem_u32(S.B[st][3]);
 #pragma unroll
-            for (int kk = 0; kk < TBK / 16; ++kk) {
-              const uint32_t off = kk * 32;
-              const uint32_t acc0 = (k > c0 || kk > 0) ? 1u : 0u;
-              umma_bf16(d, smem_desc_sw64(a0 + off), smem_desc_sw64(b0 + off), idesc, acc0);
-              umma_bf16(d, smem_desc_sw64(a0 + off), smem_desc_sw64(b1 + off), idesc, 1u);
-              umma_bf16(d, smem_desc_sw64(a2 + off), smem_desc_sw64(b0 + off), idesc, 1u);
-              umma_bf16(d, smem_desc_sw64(a1 + off), smem_desc_sw64(b2 + off), idesc, 1u);
-              umma_bf16(d, smem_desc_sw64(a1 + off), smem_desc_sw64(b3 + off), idesc, 1u);
-              umma_bf16(d, smem_desc_sw64(a3 + off), smem_desc_sw64(b2 + off), idesc, 1u);
+            for (int o = 0; o < NO; ++o) {
+              const uint32_t d = tmem + (uint32_t)((2 * o + tb) * NP);
+              const uint32_t a0 = smem_u32(S.A[st][o][0]), a1 = smem_u32(S.A[st][o][1]);
+              const uint32_t a2 = smem_u32(S.A[st][o][2]), a3 = smem_u32(S.A[st][o][3]);
+              const uint32_t b0 = smem_u32(S.B[st][o][0]), b1 = smem_u32(S.B[st][o][1]);
+              const uint32_t b2 = smem_u32(S.B[st][o][2]), b3 = smem_u32(S.B[st][o][3]);
+#pragma unroll
+              for (int kk = 0; kk < TBK / 16; ++kk) {
+                const uint32_t off = kk * 32;
+                const uint32_t acc0 = (k > c0 || kk > 0) ? 1u : 0u;
+                umma_bf16(d, smem_desc_sw64(a0 + off), smem_desc_sw64(b0 + off), idesc, acc0);
+                umma_bf16(d, smem_desc_sw64(a0 + off), smem_desc_sw64(b1 + off), idesc, 1u);
+                umma_bf16(d, smem_desc_sw64(a2 + off), smem_desc_sw64(b0 + off), idesc, 1u);
+                umma_bf16(d, smem_desc_sw64(a1 + off), smem_desc_sw64(b2 + off), idesc, 1u);
+                umma_bf16(d, smem_desc_sw64(a1 + off), smem_desc_sw64(b3 + off), idesc, 1u);
+                umma_bf16(d, smem_desc_sw64(a3 + off), smem_desc_sw64(b2 + off), idesc, 1u);
+              }
             }
             umma_commit(&S.empty[st]);
           }
@@ -345,7 +412,7 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
         }
       }
     }
-  } else {
+    if (warp > WMMA && warp <= WMMA + NEPI) {
     // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, one row per
     // thread, and keeps the segment's running sums in the same lanes of the
     // last NP tensor-memory columns (FP32 adds, rounded to nearest)
@@ -358,7 +425,7 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
       const int4 sg = segs[s];
       for (int c0 = sg.z; c0 < sg.w; c0 += CK, ++cc) {
         const int tb = cc & 1, use = cc >> 1;
-        if (*(volatile int*)&S.abort || !mbar_wait(&S.tfull[tb], use & 1)) {
+        if (*(volatile int*)&S.abort || !mbar_wait_sleep<400>(&S.tfull[tb], use & 1)) {
           if (lane == 0) {
             atomicExch(err, 15);
             S.abort = 1;
@@ -368,34 +435,43 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
         }
         __syncwarp();
         tc_fence_after();
-        const uint32_t base = lanes + (uint32_t)(tb * NP);
         const bool first = c0 == sg.z;
-#pragma unroll 2
-        for (int cb = 0; cb < NP; cb += 16) {
-          float v[16];
-          tmem_ld16(base + (uint32_t)cb, v);
-          if (!first) {
-            float r[16];
-            tmem_ld16(lanes + RUN + (uint32_t)cb, r);
+#pragma unroll 1
+        for (int o = 0; o < NO; ++o) {
+          const uint32_t base = lanes + (uint32_t)((2 * o + tb) * NP);
+          const uint32_t run = lanes + RUN + (uint32_t)(o * NP);
+#pragma unroll 1
+          for (int cb = 0; cb < NP; cb += 16) {
+            float v[16];
+            tmem_ld16(base + (uint32_t)cb, v);
+            if (!first) {
+              float r[16];
+              tmem_ld16(run + (uint32_t)cb, r);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) v[k] += r[k];
+              for (int k = 0; k < 16; ++k) v[k] += r[k];
+            }
+            tmem_st16(run + (uint32_t)cb, v);
           }
-          tmem_st16(lanes + RUN + (uint32_t)cb, v);
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.tempty[tb]);
       }
       if (stop) break;
-      float2* dst = partial + (size_t)s * TBM * NR + row;
 #pragma unroll 1
-      for (int cb = 0; cb < NR; cb += 16) {
-        float re[16], im[16];
-        tmem_ld16(lanes + RUN + (uint32_t)cb, re);
-        tmem_ld16(lanes + RUN + (uint32_t)(NR + cb), im);
+      for (int o = 0; o < NO; ++o) {
+        float2* dst = partial + ((size_t)s * NO + o) * TBM * NR + row;
+        const uint32_t run = lanes + RUN + (uint32_t)(o * NP);
+#pragma unroll 1
+        for (int cb = 0; cb < NR; cb += 16) {
+          float re[16], im[16];
+          tmem_ld16(run + (uint32_t)cb, re);
+          tmem_ld16(run + (uint32_t)(NR + cb), im);
 #pragma unroll
-        for (int k = 0; k < 16; ++k) dst[(size_t)(cb + k) * TBM] = make_float2(re[k], im[k]);
+          for (int k = 0; k < 16; ++k) dst[(size_t)(cb + k) * TBM] = make_float2(re[k], im[k]);
+        }
       }
+    }
     }
   }
   __syncthreads();
@@ -403,8 +479,8 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
   // issued, then free TMEM
   if (*(volatile int*)&S.abort) {
     if (threadIdx.x == 0)
-      for (int s = 0; s < TSTAGES; ++s) {
-        if (S.issued[s] >= 0) mbar_wait(&S.full[s], (uint32_t)S.issued[s]);
+      for (int s = 0; s < SD; ++s) {
+        if (s < TSTAGES && S.issued[s] >= 0) mbar_wait(&S.full[s], (uint32_t)S.issued[s]);
         if (S.sissued[s] >= 0) mbar_wait(&S.sfull[s], (uint32_t)S.sissued[s]);
       }
     if (warp == WMMA && lane == 0) {
@@ -419,33 +495,50 @@ k_fused_tc(tc_params P, const __grid_constant__ CUtensorMap tmB, const int4* __r
   }
 }
 
-// y[r][i] = sum of the (one to a few) segment partials of row tile i / 128, in
-// a fixed order; FP32 adds (the partials are FP32 sums of bf16 products: FP64
-// adds would buy nothing here and run at 1/64 of the FP32 rate)
+// Sums of the (one to a few) segment partials of row tile i / 128, in a fixed
+// order; FP32 adds (the partials are FP32 sums of bf16 products: FP64 adds
+// would buy nothing here and run at 1/64 of the FP32 rate).  Soft: y = A x.
+// OP_S: t = S u = i S' u.  OP_C: y = x / 2 + C x.  OP_SC: both.
+template <int OP>
 __global__ void k_reduce_tc(int n, int nr, int NR, const int2* __restrict__ mt_seg,
-                            const float2* __restrict__ partial, double2* __restrict__ y) {
+                            const float2* __restrict__ partial, const double2* __restrict__ x,
+                            float2* __restrict__ t, double2* __restrict__ y) {
+  constexpr int NO = tc_ops<OP>();
   const int m = blockIdx.x, r = blockIdx.y, row = threadIdx.x;
   const int i = m * TBM + row;
   if (i >= n || r >= nr) return;
   const int2 sr = mt_seg[m];
-  float sx = 0.f, sy = 0.f;
+  float2 v[NO];
+#pragma unroll
+  for (int o = 0; o < NO; ++o) v[o] = make_float2(0.f, 0.f);
   for (int s = sr.x; s < sr.x + sr.y; ++s) {
-    const float2 p = partial[((size_t)s * NR + r) * TBM + row];
-    sx += p.x;
-    sy += p.y;
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      const float2 p = partial[(((size_t)s * NO + o) * NR + r) * TBM + row];
+      v[o].x += p.x;
+      v[o].y += p.y;
+    }
   }
-  y[(size_t)r * n + i] = make_double2(sx, sy);
+  const size_t e = (size_t)r * n + i;
+  if constexpr (OP == OP_SOFT) y[e] = make_double2(v[0].x, v[0].y);
+  if constexpr (OP == OP_S || OP == OP_SC) t[e] = make_float2(-v[0].y, v[0].x);
+  if constexpr (OP == OP_C || OP == OP_SC) {
+    const double2 xv = x[e];
+    y[e] = make_double2(fma(0.5, xv.x, (double)v[NO - 1].x), fma(0.5, xv.y, (double)v[NO - 1].y));
+  }
 }
 
-unsigned nb(size_t len, int t = 256) { return (unsigned)((len + t - 1) / t); }
-
-template <int NP, int KIND>
-void run_fused(cfie_op* op, const double2* x, double2* y, int r0, int nr) {
-  constexpr int NR = NP / 2;
-  tc_plan& T = op->tc[NP == 64 ? 0 : 1];
+// One pass for the right-hand sides r0 .. r0 + nr - 1: soft x -> y; S: u -> t;
+// C: x -> y; SC: u, x -> t, y
+template <int NP, int OP>
+void run_fused(cfie_op* op, const double2* x, const float2* u, float2* t, double2* y, int r0,
+               int nr) {
+  constexpr int NR = NP / 2, NO = tc_ops<OP>();
+  tc_plan& T = op->tc[OP == OP_SC ? 2 : (NP == 64 ? 0 : 1)];
   const int n = op->n;
   cudaStream_t st = op->ctx->stream;
   const int pitch = (n + 63) / 64 * 64;
+  const size_t planes = 4 * (size_t)NP * pitch;
   if (!T.built) {
     const int mtiles = (n + TBM - 1) / TBM, ktiles = (n + TBK - 1) / TBK;
     int sms = 152;
@@ -468,17 +561,21 @@ void run_fused(cfie_op* op, const double2* x, double2* y, int r0, int nr) {
                                     cudaMemcpyHostToDevice, st));
     CFIE_CHECK_CUDA(cudaMemcpyAsync(tb + T.o_mts, mt_seg.data(), sizeof(int2) * mt_seg.size(),
                                     cudaMemcpyHostToDevice, st));
-    T.bt.reserve(sizeof(__nv_bfloat16) * 4 * (size_t)NP * pitch);
-    T.partial.reserve(sizeof(float2) * (size_t)T.nsegs * TBM * NR);
+    T.bt.reserve(sizeof(__nv_bfloat16) * NO * planes);
+    T.partial.reserve(sizeof(float2) * (size_t)T.nsegs * NO * TBM * NR);
     T.err.reserve(sizeof(int));
     CFIE_CHECK_CUDA(cudaMemsetAsync(T.err.p, 0, sizeof(int), st));
-    const CUtensorMap mb = tc_make_map(T.bt.p, 4 * (uint64_t)NP, (uint64_t)pitch, pitch, NP,
+    const CUtensorMap mb = tc_make_map(T.bt.p, 4 * NO * (uint64_t)NP, (uint64_t)pitch, pitch, NP,
                                        TBK, CU_TENSOR_MAP_SWIZZLE_64B);
     std::memcpy(T.tmB, &mb, sizeof(mb));
     CFIE_CHECK_CUDA(cudaStreamSynchronize(st));
     T.built = true;
   }
-  prep_b_planes(op->ctx, n, pitch, NP, nr, x + (size_t)r0 * n, T.bt.as<__nv_bfloat16>());
+  __nv_bfloat16* bt = T.bt.as<__nv_bfloat16>();
+  const size_t at = (size_t)r0 * n;
+  if constexpr (OP == OP_S || OP == OP_SC) prep_b_planes(op->ctx, n, pitch, NP, nr, u + at, bt);
+  if constexpr (OP != OP_S)
+    prep_b_planes(op->ctx, n, pitch, NP, nr, x + at, bt + (NO - 1) * planes);
   tc_params P{};
   P.n = n;
   P.b = op->band_b;
@@ -486,100 +583,57 @@ void run_fused(cfie_op* op, const double2* x, double2* y, int r0, int nr) {
   float* base = op->geo32.as<float>();
   P.wext = reinterpret_cast<const float2*>(base + geo32_wk_offset(n));
   P.pk = reinterpret_cast<const float4*>(base + geo32_pack_offset(n));
-  // the FP32 band holds the soft entries, or S then D' for the hard operator
-  P.band = op->band.as<float2>() +
-           (KIND == KIND_DP ? (size_t)n * (2 * (size_t)op->band_b + 1) : (size_t)0);
-  const size_t smem = tc_smem_bytes<NP>();
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_fused_tc<NP, KIND>,
+  P.spk = reinterpret_cast<const float4*>(base + geo32_pair_offset(n));
+  P.band = op->band.as<float2>();
+  const size_t smem = tc_smem_bytes<NP, OP>();
+  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_fused_tc<NP, OP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   char* tb = T.tables.as<char>();
   {
     prof_scope ps(op->ctx, CFIE_K_MATVEC_FP32);
-    k_fused_tc<NP, KIND><<<T.grid, TNT, smem, st>>>(P, *reinterpret_cast<const CUtensorMap*>(T.tmB),
-                                             reinterpret_cast<const int4*>(tb),
-                                             reinterpret_cast<const int*>(tb + T.o_cbeg),
-                                             T.partial.as<float2>(), T.err.as<int>());
+    k_fused_tc<NP, OP><<<T.grid, TNT, smem, st>>>(P, *reinterpret_cast<const CUtensorMap*>(T.tmB),
+                                                  reinterpret_cast<const int4*>(tb),
+                                                  reinterpret_cast<const int*>(tb + T.o_cbeg),
+                                                  T.partial.as<float2>(), T.err.as<int>());
     CFIE_CHECK_LAUNCH();
   }
-  k_reduce_tc<<<dim3(T.mtiles, nr), TBM, 0, st>>>(n, nr, NR,
-                                                 reinterpret_cast<const int2*>(tb + T.o_mts),
-                                                 T.partial.as<float2>(), y + (size_t)r0 * n);
+  k_reduce_tc<OP><<<dim3(T.mtiles, nr), TBM, 0, st>>>(
+      n, nr, NR, reinterpret_cast<const int2*>(tb + T.o_mts), T.partial.as<float2>(),
+      x ? x + at : nullptr, t ? t + at : nullptr, y ? y + at : nullptr);
   CFIE_CHECK_LAUNCH();
 }
 
-template <int KIND>
-void run_blocks(cfie_op* op, const double2* x, double2* y, int nrhs) {
+template <int OP>
+void run_blocks(cfie_op* op, const double2* x, const float2* u, float2* t, double2* y, int nrhs) {
   for (int r0 = 0; r0 < nrhs; r0 += 64) {
     const int nr = std::min(64, nrhs - r0);
     if (nr > 32)
-      run_fused<128, KIND>(op, x, y, r0, nr);
+      run_fused<128, OP>(op, x, u, t, y, r0, nr);
     else
-      run_fused<64, KIND>(op, x, y, r0, nr);
+      run_fused<64, OP>(op, x, u, t, y, r0, nr);
   }
-}
-
-// hard operator inputs of the S sums: [u, n1 x, n2 x] (u = (1/|z'|) d/dt x)
-__global__ void k_hard_inputs(int n, size_t tot, const double2* __restrict__ x,
-                              const float2* __restrict__ u32, geom_dev g,
-                              double2* __restrict__ v) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= tot) return;
-  const int i = (int)(e % n);
-  const double inv = 1.0 / g.sp[i];
-  const double2 xv = x[e];
-  const float2 uv = u32[e];
-  v[e] = make_double2(uv.x, uv.y);
-  v[tot + e] = make_double2(g.nx[i] * inv * xv.x, g.nx[i] * inv * xv.y);
-  v[2 * tot + e] = make_double2(g.ny[i] * inv * xv.x, g.ny[i] * inv * xv.y);
-}
-
-// y = x/2 - D' x - i (omega^2 / eta) (n1 S(n1 x) + n2 S(n2 x)), t = S u (FP32)
-__global__ void k_hard_combine(int n, size_t tot, double omega, double eta, geom_dev g,
-                               const double2* __restrict__ x, const double2* __restrict__ ys,
-                               const double2* __restrict__ yd, float2* __restrict__ t32,
-                               double2* __restrict__ y) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= tot) return;
-  const int i = (int)(e % n);
-  const double inv = 1.0 / g.sp[i];
-  const double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-  const double2 s1 = ys[tot + e], s2 = ys[2 * tot + e];
-  const double2 m = make_double2(n1 * s1.x + n2 * s2.x, n1 * s1.y + n2 * s2.y);
-  const double k = omega * omega / eta;
-  const double2 xv = x[e], d = yd[e];
-  y[e] = make_double2(0.5 * xv.x - d.x + k * m.y, 0.5 * xv.y - d.y - k * m.x);
-  t32[e] = make_float2((float)ys[e].x, (float)ys[e].y);
 }
 
 }  // namespace
 
 void matvec_fp32_tc(cfie_op* op, const double2* x, double2* y, int nrhs) {
   if (op->bc == CFIE_SOUND_SOFT) {
-    run_blocks<KIND_SOFT>(op, x, y, nrhs);
+    run_blocks<OP_SOFT>(op, x, nullptr, nullptr, y, nrhs);
     return;
   }
-  // sound hard (eq. 2 with Maue's identity): S applied to [u, n1 x, n2 x] and
-  // D' to x, each with the tensor-core sums, then the spectral derivative
-  const int n = op->n;
-  const size_t tot = (size_t)n * nrhs;
-  cudaStream_t st = op->ctx->stream;
+  // sound hard: S on u = (1/|z'|) d/dt x and C on x, then the spectral
+  // derivative of S u
+  const size_t tot = (size_t)op->n * nrhs;
   op->xin32.reserve(sizeof(float2) * tot * 3);
-  float2* x32 = op->xin32.as<float2>();
-  float2* u32 = x32 + tot;
-  float2* t32 = x32 + 2 * tot;
-  op->tcv.reserve(sizeof(double2) * tot * 4);
-  double2* v = op->tcv.as<double2>();        // [u, n1 x, n2 x], then S of them
-  op->tcs.reserve(sizeof(double2) * tot * 4);
-  double2* ys = op->tcs.as<double2>();       // S [u, n1 x, n2 x], then D' x
-  k_to32_fp32(op, x, x32, tot);
-  spectral32_apply(op, x32, u32, nrhs);
-  k_hard_inputs<<<nb(tot), 256, 0, st>>>(n, tot, x, u32, op->g, v);
-  CFIE_CHECK_LAUNCH();
-  run_blocks<KIND_S>(op, v, ys, 3 * nrhs);
-  run_blocks<KIND_DP>(op, x, ys + 3 * tot, nrhs);
-  k_hard_combine<<<nb(tot), 256, 0, st>>>(n, tot, op->omega, op->eta, op->g, x, ys, ys + 3 * tot,
-                                          t32, y);
-  CFIE_CHECK_LAUNCH();
+  float2* u32 = op->xin32.as<float2>();
+  float2* t32 = u32 + tot;
+  spectral32_apply(op, x, u32, nrhs);
+  if (nrhs <= 32) {
+    run_fused<64, OP_SC>(op, x, u32, t32, y, 0, nrhs);
+  } else {
+    run_blocks<OP_S>(op, nullptr, u32, t32, nullptr, nrhs);
+    run_blocks<OP_C>(op, x, nullptr, nullptr, y, nrhs);
+  }
   spectral32_accumulate(op, t32, y, nrhs);
 }
 

@@ -15,6 +15,11 @@
 //   2 n + 8 float2: the Kress table twice over divided by pi h, entry
 //   k = i - j + n holding the weights of sources j and j + 1,
 //   (w_{k mod n}, w_{(k - 1) mod n}) / (pi h), then zeros
+//   n float4 source coordinates by pairs j, j + 1 (n is even), negated:
+//   (-xh_j, -xh_j+1, -xl_j, -xl_j+1), (-yh_j, ..)
+//   n float4 source factors by pairs, (a_j, a_j+1, b_j, b_j+1), (c_j, c_j+1, 0, 0):
+//   soft a, b = omega hq c0 nu, c = hq c0 eta |z'|; hard a, b = (omega / eta)
+//   nu / |z'|, c = hq c0 |z'|
 // with hq = h / 4 and c0 = sqrt(2 / pi) (nu = unnormalised normal, |z'| = speed).
 struct geo32 {
   float *xh, *xl, *yh, *yl, *nx, *ny, *sp;
@@ -22,8 +27,11 @@ struct geo32 {
 
 inline size_t geo32_pack_offset(int n) { return ((size_t)9 * n + 3) & ~size_t(3); }
 inline size_t geo32_wk_offset(int n) { return geo32_pack_offset(n) + (size_t)12 * n; }
-// (+ 128 floats of slack: the fused kernel copies whole 32-source tiles)
-inline size_t geo32_floats(int n) { return geo32_wk_offset(n) + (size_t)4 * n + 16 + 128; }
+inline size_t geo32_pair_offset(int n) {
+  return (geo32_wk_offset(n) + (size_t)4 * n + 16 + 3) & ~size_t(3);
+}
+// (+ 256 floats of slack: the fused kernel copies whole 32-source tiles)
+inline size_t geo32_floats(int n) { return geo32_pair_offset(n) + (size_t)8 * n + 256; }
 
 inline geo32 geo32_at(float* base, int n) {
   return geo32{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n,
@@ -240,4 +248,119 @@ __device__ __forceinline__ float2 entry_folded32(float4 tg, float4 tq, float4 sc
                                                  float wk) {
   return entry_finish32<KIND>(pair_phase32_tc(tg.x, tg.y, tg.z, tg.w, sc.x, sc.y, sc.z, sc.w), tq,
                               sq, wk);
+}
+
+// ---------------------------------------------------------------------------
+// Two entries of one target at once (the adjacent sources j, j + 1), in packed
+// FP32 pairs: add, mul and fma on float2 issue once for two lanes of
+// arithmetic (measured: the same 121 lane-ops per clock and SM as scalar FMAs
+// at half the issue slots), and the producers of the fused kernel are bound by
+// issue slots.  Signs sit in the per-node data and in the constants
+// where they can.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+
+// as pair_phase, for the two sources
+struct pair_phase2 {
+  float2 dx, dy, xinv, ra, s, c;
+};
+
+// pair_phase32_tc for both sources: t0, t1 the target's (xh, xh, xl, xl), (yh,
+// ..), s0, s1 the sources' negated coordinates by pairs.  k is rounded by adding
+// and subtracting 1.5 2^23 (k < 2^14), -pi/4 joins the lo part of x.
+__device__ __forceinline__ pair_phase2 phase32_pair(float4 t0, float4 t1, float4 s0, float4 s1) {
+  pair_phase2 f;
+  const float2 dxh = add2(lo2(t0), lo2(s0)), dxl = add2(hi2(t0), hi2(s0));   // dxh, dyh exact
+  const float2 dyh = add2(lo2(t1), lo2(s1)), dyl = add2(hi2(t1), hi2(s1));
+  const float2 H = fma2(dxh, dxh, mul2(dyh, dyh));                           // exact
+  f.dx = add2(dxh, dxl);
+  f.dy = add2(dyh, dyl);
+  const float2 C = fma2(dxl, add2(dxh, f.dx), mul2(dyl, add2(dyh, f.dy)));
+  const float2 x2 = add2(H, C);
+  f.xinv = make_float2(rsqrt_sfu(x2.x), rsqrt_sfu(x2.y));
+  const float2 xh = mul2(x2, f.xinv);
+  f.ra = make_float2(rsqrt_sfu(xh.x), rsqrt_sfu(xh.y));
+  const float2 e = add2(fma2(neg2(xh), xh, H), C);                // x^2 - xh^2
+  const float2 xl = fma2(e, mul2(f.xinv, f2(0.5f)), f2(-kPi4H));             // x lo - pi/4
+  const float2 kr = add2(fma2(xh, f2(kInv2Pi), f2(-0.125f)), f2(12582912.0f));
+  const float2 k = add2(kr, f2(-12582912.0f));
+  const float2 chi = add2(fma2(k, f2(-kC2), fma2(k, f2(-kC1), xh)), xl);     // first fma exact
+  sincos_sfu(chi.x, &f.s.x, &f.c.x);
+  sincos_sfu(chi.y, &f.s.y, &f.c.y);
+  return f;
+}
+
+// j0, w0 = y0 + wk j0, j1, w1 = y1 + wk j1 of both sources (hankel_asym32_tc)
+struct hankel_pair {
+  float2 j0, w0, j1, w1;
+};
+__device__ __forceinline__ hankel_pair hankel32_pair(const pair_phase2& f, float2 wk) {
+  const float2 ti = f.xinv, t2 = mul2(ti, ti);
+  const float2 ns = neg2(f.s);
+  const float2 P0 = fma2(t2, f2(-0.0703125f), f2(1.0f));
+  const float2 Q0 = mul2(ti, fma2(t2, f2(0.0732421875f), f2(-0.125f)));
+  const float2 P1n = fma2(t2, f2(-0.1171875f), f2(-1.0f));
+  const float2 Q1 = mul2(ti, fma2(t2, f2(-0.1025390625f), f2(0.375f)));
+  hankel_pair h;
+  h.j0 = fma2(P0, f.c, mul2(Q0, ns));
+  h.w0 = fma2(wk, h.j0, fma2(P0, f.s, mul2(Q0, f.c)));
+  h.j1 = fma2(P1n, ns, mul2(Q1, f.c));
+  h.w1 = fma2(wk, h.j1, fma2(P1n, f.c, mul2(Q1, f.s)));
+  return h;
+}
+
+// Operators of the fused kernel: the sound-soft one (eq. 1); of the sound-hard
+// one (eq. 2, Maue's identity summed over the pairs) S' = -i S, applied to u =
+// d/ds x, and C = -D' - i (omega^2 / eta) (n_i . n_j) S, applied to x; or both
+// from one phase.  With A = c ra, B (soft) = (a, b).(dx, dy) ra / x, D =
+// (tq).(dx, dy) A / x, kn = tq.(a, b) = (omega^2 / eta) n_i . n_j:
+//   soft: re = A j0 - B w1,           im = A w0 + B j1
+//   S':   re = A j0,                  im = A w0
+//   C:    re = kn A j0 - D w1,        im = kn A w0 + D j1
+enum { OP_SOFT = 0, OP_S = 1, OP_C = 2, OP_SC = 3 };
+
+struct entry_pair {
+  float2 re, im;     // soft, S' or C
+  float2 re2, im2;   // OP_SC: C (the first is S')
+};
+
+// tq = (tx, tx, ty, ty) target factors omega nu / |z'| (hard), s2, s3 the source
+// factors by pairs
+template <int OP>
+__device__ __forceinline__ entry_pair finish32_pair(const pair_phase2& f, float4 tq, float4 s2,
+                                                    float2 sc, float2 wk) {
+  const hankel_pair h = hankel32_pair(f, wk);
+  const float2 A = mul2(sc, f.ra);
+  entry_pair e;
+  if constexpr (OP == OP_SOFT) {
+    const float2 B = mul2(fma2(f.dx, lo2(s2), mul2(f.dy, hi2(s2))), mul2(f.xinv, f.ra));
+    e.re = fma2(A, h.j0, mul2(neg2(B), h.w1));
+    e.im = fma2(A, h.w0, mul2(B, h.j1));
+  } else {
+    const float2 sr = mul2(A, h.j0), si = mul2(A, h.w0);
+    if constexpr (OP == OP_S || OP == OP_SC) {
+      e.re = sr;
+      e.im = si;
+    }
+    if constexpr (OP == OP_C || OP == OP_SC) {
+      const float2 D = mul2(fma2(f.dx, lo2(tq), mul2(f.dy, hi2(tq))), mul2(f.xinv, A));
+      const float2 kn = fma2(lo2(tq), lo2(s2), mul2(hi2(tq), hi2(s2)));
+      const float2 cr = fma2(kn, sr, mul2(neg2(D), h.w1));
+      const float2 ci = fma2(kn, si, mul2(D, h.j1));
+      if constexpr (OP == OP_C) {
+        e.re = cr;
+        e.im = ci;
+      } else {
+        e.re2 = cr;
+        e.im2 = ci;
+      }
+    }
+  }
+  return e;
 }

@@ -475,6 +475,10 @@ void spectral_fft32_apply(cfie_op* op, const float2* in, float2* out, int nrhs) 
   spectral_fft<float2, float2, float2>(op, in, out, nullptr, make_double2(1.0, 0.0), nrhs);
 }
 
+void spectral_fft32_apply(cfie_op* op, const double2* in, float2* out, int nrhs) {
+  spectral_fft<float2, double2, float2>(op, in, out, nullptr, make_double2(1.0, 0.0), nrhs);
+}
+
 void spectral_fft32_accumulate(cfie_op* op, const float2* in, double2* y, double2 scale,
                                int nrhs) {
   spectral_fft<float2, float2, double2>(op, in, y, y, scale, nrhs);

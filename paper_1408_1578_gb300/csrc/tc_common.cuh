@@ -44,7 +44,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 // taking issue slots from the warps that do the work
 constexpr uint32_t kSuspendNs = 1000000;
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity, uint32_t ns) {
   uint32_t ok;
   asm volatile(
       "{\n"
@@ -53,7 +53,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       "selp.u32 %0, 1, 0, p;\n"
       "}\n"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
       : "memory");
   return ok != 0;
 }
@@ -61,10 +61,32 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // bounded wait on the phase of parity `parity`; false on timeout
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
+  while (!mbar_try_wait(bar, parity, kSuspendNs)) {
     if (clock64() - t0 > kTimeoutCycles) return false;
   }
   return true;
+}
+
+// The same with about NS nanoseconds of sleep between the tries: for roles
+// that wait a long time next to busy warps (the drain, TMA and MMA warps of
+// the fused kernel issued a third of all its instructions in mbar_wait's loop)
+template <int NS>
+__device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity, 0)) return true;
+  const long long t0 = clock64();
+  do {
+    __nanosleep(NS);
+    if (mbar_try_wait(bar, parity, 0)) return true;
+  } while (clock64() - t0 <= kTimeoutCycles);
+  return false;
+}
+
+// start of a kernel's dynamic shared memory, rounded up to 1024 bytes (the
+// swizzled tiles' alignment) by pointer arithmetic: a detour over an integer
+// would lose the address space and turn every access into a generic one
+template <typename T>
+__device__ __forceinline__ T& smem_aligned(unsigned char* raw) {
+  return *reinterpret_cast<T*>(raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u));
 }
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar,
@@ -322,11 +344,12 @@ inline void streamk_segments(int mtiles, int ktiles, int grid_max, std::vector<i
   cbeg[grid] = (int)segs.size();
 }
 
-// B operand planes [4][NP][pitch] for nr right-hand sides (complex128, [r][j]):
+// B operand planes [4][NP][pitch] for nr right-hand sides (complex128 or complex64, [r][j]):
 // B1 = [Xr | Xi], B2 = [-Xi | Xr] (rows = output columns), hi / lo bf16 split
 // (of the FP32-rounded value, in FP32).  One thread per right-hand side r and
 // source pair j, j + 1: x read once, packed bf16 pairs stored.
-__global__ void k_prep_b_planes(int n, int pitch, int NP, int nr, const double2* __restrict__ x,
+template <typename X>
+__global__ void k_prep_b_planes(int n, int pitch, int NP, int nr, const X* __restrict__ x,
                                 __nv_bfloat16* __restrict__ bt) {
   const int r = blockIdx.y;                       // < NP / 2
   const int j = 2 * (blockIdx.x * 256 + threadIdx.x);
@@ -337,7 +360,7 @@ __global__ void k_prep_b_planes(int n, int pitch, int NP, int nr, const double2*
 #pragma unroll
     for (int u = 0; u < 2; ++u)
       if (j + u < n) {
-        const double2 v = x[(size_t)r * n + j + u];
+        const X v = x[(size_t)r * n + j + u];
         re[u] = (float)v.x;
         im[u] = (float)v.y;
       }
@@ -363,9 +386,10 @@ __global__ void k_prep_b_planes(int n, int pitch, int NP, int nr, const double2*
   b[3 * p2 + e1] = lr;
 }
 
-inline void prep_b_planes(cfie_ctx* ctx, int n, int pitch, int NP, int nr, const double2* x,
-                          __nv_bfloat16* bt) {
-  k_prep_b_planes<<<dim3((unsigned)((pitch / 2 + 255) / 256), NP / 2), 256, 0, ctx->stream>>>(
+template <typename X>
+void prep_b_planes(cfie_ctx* ctx, int n, int pitch, int NP, int nr, const X* x,
+                   __nv_bfloat16* bt) {
+  k_prep_b_planes<X><<<dim3((unsigned)((pitch / 2 + 255) / 256), NP / 2), 256, 0, ctx->stream>>>(
       n, pitch, NP, nr, x, bt);
   CFIE_CHECK_LAUNCH();
 }
