@@ -321,3 +321,12 @@ __device__ __forceinline__ void pair_entries_fp64(double dx, double dy, double o
     pair_folded_fp64<1>(dx, dy, omega, 1.0 / omega, omega * nxi / si, omega * nyi / si, f * sj, wk,
                         tab, a, b);
 }
+
+// C_ij = -D'_ij - i (omega^2 / eta) (n_i . n_j) S_ij, the operator that the
+// sound-hard sums apply to x (n the unit normals; i == j: the diagonal entries)
+__device__ __forceinline__ double2 hard_combined(const geom_dev& g, double omega, double eta, int i,
+                                                 int j, double2 S, double2 Dp) {
+  const double k = omega * omega / eta / (g.sp[i] * g.sp[j]) *
+                   fma(g.nx[i], g.nx[j], g.ny[i] * g.ny[j]);
+  return make_double2(fma(k, S.y, -Dp.x), -fma(k, S.x, Dp.y));
+}

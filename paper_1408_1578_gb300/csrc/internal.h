@@ -228,7 +228,6 @@ struct cfie_op {
   dbuf band;         // near-field band entries (complex64), n x (2 b + 1) per operator
   int band_b = -1;
   dbuf xin32, xin32b; // FP32 staging of the input (and hard-path helpers)
-  dbuf tcv, tcs;      // sound-hard tensor-core residual: S inputs, S and D' outputs
   fft_plan fft;       // sound hard: FFT spectral derivative
 
   // FP64-accurate residual matvec in double-float arithmetic (sound-soft)
@@ -330,10 +329,10 @@ void spectral_fft32_apply(cfie_op* op, const float2* in, float2* out, int nrhs);
 void spectral_fft32_apply(cfie_op* op, const double2* in, float2* out, int nrhs);
 void spectral_fft32_accumulate(cfie_op* op, const float2* in, double2* y, double2 scale,
                                int nrhs);
-// sound-hard combination of the four FP64-layout partial sums (S u, S n1 x,
-// S n2 x, D' x): t = S u, y = x / 2 - D' x - i (omega^2 / eta) (n1 S n1 x + n2 S n2 x)
-void reduce_hard_fp64(cfie_op* op, const double2* part, int splits, const double2* x,
-                      double2* t, double2* y, int nrhs);
+// split partial sums (part[output][split][k][i]) added in a fixed order: soft
+// y = sum; hard t = S u, y = x / 2 + C x
+void reduce_fp64(cfie_op* op, const double2* part, int splits, const double2* x, double2* t,
+                 double2* y, int nrhs);
 void matvec_fp64_static(cfie_op* op, const double2* x, double2* y, int nrhs);
 size_t static_scratch_capacity();
 // matvec_fp32.cu

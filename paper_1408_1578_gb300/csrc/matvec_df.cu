@@ -1,31 +1,19 @@
 // FP64-accurate matvec on the FP32 pipe (compensated arithmetic), used for the
 // true residuals of the refined solves: the sound-soft operator of eq. 1, and
-// the sound-hard operator of eq. 2 with N by Maue's identity (the S and D'
-// sums here, the spectral derivatives by the FP64 circulant kernel).
+// the sound-hard operator of eq. 2 with N by Maue's identity, as two operators
+// over the same pairs (S on u = d/ds x and C = -D' - i (omega^2 / eta)
+// (n_i . n_j) S on x; the spectral derivatives by FP64 FFT).
 //
 // GB300 runs FP64 at a small fraction of its FP32 rate, and the two residual
 // matvecs of a refined solve cost more than all its inner FP32 matvecs when
 // computed in FP64.  These kernels evaluate the same Nystrom entries as the
-// FP64 kernel (Kress log-split rule) in double-float arithmetic: every
-// quantity is an unevaluated sum hi + lo of two FP32 numbers (~48 significant
-// bits), products and sums use error-free transformations (TwoProd with fmaf,
-// TwoSum), reciprocals and square roots start from the special-function
-// unit's approximations and take one double-float correction; coordinates are
-// stored times omega (the node distance is the Hankel argument) and the
-// per-node factors of each entry are folded into per-node vectors; and
-//  * Hankel's asymptotic expansion (A&S 9.2.5, 9.2.9, 9.2.10) carries its
-//    leading terms in double-float and the small corrections in FP32: for
-//    omega r >= 40 four terms of P and Q, for 20 <= omega r < 40 (pairs next to
-//    the band) seven and their first corrections in double-float; the dropped
-//    terms are below 1e-13;
-//  * the phase omega r - pi/4 is reduced modulo 2 pi with a three-part
-//    constant, then sin / cos come from a 64-entry double-float table of
-//    sin(j pi/32), cos(j pi/32) and Taylor series of the remainder |d| <= pi/64;
-//  * pairs with omega r < 20 come from a band of entries evaluated in FP64.
-// Source sums use Dot2 (Ogita, Rump & Oishi) inside each 32-source tile and
-// double-float additions across tiles; the densities are converted to
-// double-float once per matvec.  Relative accuracy a few 1e-12 (the FP32
-// corrections of P and Q at omega r ~ 40 bound it; tests ask 1e-11).
+// FP64 kernel (Kress log-split rule) in double-float arithmetic (pairdf.cuh:
+// unevaluated sums hi + lo of two FP32 numbers, ~48 significant bits, two
+// sources at a time in packed FP32 pairs).  Pairs with omega r < 20 come from a
+// band of entries evaluated in FP64.  Source sums use Dot2 (Ogita, Rump &
+// Oishi) inside each 32-source tile and double-float additions across tiles, or
+// the tensor cores on exact slices (below); the densities are converted to
+// double-float once per matvec.  Relative accuracy a few 1e-12 (tests ask 1e-11).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -40,7 +28,7 @@
 
 #include "hankel64.cuh"
 #include "internal.h"
-#include "pair32.cuh"
+#include "pairdf.cuh"
 #include "tc_common.cuh"
 
 namespace {
@@ -48,370 +36,52 @@ namespace {
 constexpr int DTI = 64;
 constexpr int DTJ = 32;
 constexpr int DNT = 256;
-constexpr float kXD = 20.0f;   // asymptotic expansion in this kernel for omega r >= 20
-constexpr float kXS = 40.0f;   // short series (leading terms in FP32) for omega r >= 40
 
-struct df {
-  float h, l;
-};
-
-__device__ __forceinline__ df quick(float a, float b) {
-  const float s = a + b;
-  return {s, b - (s - a)};
-}
-__device__ __forceinline__ df dadd(df a, df b) {
-  const float s = a.h + b.h;
-  const float v = s - a.h;
-  const float e = (a.h - (s - v)) + (b.h - v) + a.l + b.l;
-  return quick(s, e);
-}
-__device__ __forceinline__ df dneg(df a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ df dsub(df a, df b) { return dadd(a, dneg(b)); }
-__device__ __forceinline__ df dmul(df a, df b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  return quick(p, e);
-}
-__device__ __forceinline__ df dmulf(df a, float b) {
-  const float p = a.h * b;
-  float e = fmaf(a.h, b, -p);
-  e = fmaf(a.l, b, e);
-  return quick(p, e);
-}
-__host__ __device__ __forceinline__ df dmake(double v) {
-  const float h = (float)v;
-  return {h, (float)(v - (double)h)};
-}
-// 1 / a from the special-function unit's approximation q (~1 ulp): with
-// e = 1 - a q, 1 / a = q (1 + e + e^2 + ...), kept to second order
-__device__ __forceinline__ df drcp(df a) {
-  float q;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(a.h));
-  const float e = fmaf(-a.h, q, 1.0f) - a.l * q;
-  return quick(q, q * fmaf(e, e, e));
-}
-// sqrt(a), a > 0: r = a rs with rs ~ 1/sqrt(a.h) (one Newton step on the
-// special-function unit's value), then one Newton correction in double-float
-__device__ __forceinline__ df dsqrt(df a) {
-  float rs;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(a.h));
-  rs = rs * fmaf(-0.5f * a.h * rs, rs, 1.5f);
-  const float r = a.h * rs;
-  const float e = fmaf(-r, r, a.h) + a.l;           // a - r^2
-  return quick(r, e * (0.5f * rs));
-}
-
-// sin(j pi / 32), cos(j pi / 32) for j = -32 .. 32 as hi / lo pairs
-__constant__ float4 kSinCos[65] = {
-    {0.0f, 0.0f, -1.0f, 0.0f}, {-0.0980171412229538f, 8.933931927579408e-10f, -0.9951847195625305f, -7.109666189109021e-09f},
-    {-0.19509032368659973f, 1.670471427850373e-09f, -0.9807852506637573f, -2.9739473106360492e-08f}, {-0.290284663438797f, -1.3815665056426951e-08f, -0.9569403529167175f, 1.7184508038781132e-08f},
-    {-0.3826834261417389f, -6.2233507236442165e-09f, -0.9238795042037964f, -2.830748968563057e-08f}, {-0.4713967442512512f, 7.425253745196869e-09f, -0.8819212913513184f, 2.7002963420841297e-08f},
-    {-0.5555702447891235f, 1.1769521357507529e-08f, -0.8314695954322815f, -1.687026340846387e-08f}, {-0.6343932747840881f, -9.37955757507325e-09f, -0.7730104327201843f, -2.0642552556182636e-08f},
-    {-0.7071067690849304f, -1.2101617485882343e-08f, -0.7071067690849304f, -1.2101617485882343e-08f}, {-0.7730104327201843f, -2.0642552556182636e-08f, -0.6343932747840881f, -9.37955757507325e-09f},
-    {-0.8314695954322815f, -1.687026340846387e-08f, -0.5555702447891235f, 1.1769521357507529e-08f}, {-0.8819212913513184f, 2.7002963420841297e-08f, -0.4713967442512512f, 7.425253745196869e-09f},
-    {-0.9238795042037964f, -2.830748968563057e-08f, -0.3826834261417389f, -6.2233507236442165e-09f}, {-0.9569403529167175f, 1.7184508038781132e-08f, -0.290284663438797f, -1.3815665056426951e-08f},
-    {-0.9807852506637573f, -2.9739473106360492e-08f, -0.19509032368659973f, 1.670471427850373e-09f}, {-0.9951847195625305f, -7.109666189109021e-09f, -0.0980171412229538f, 8.933931927579408e-10f},
-    {-1.0f, 0.0f, 0.0f, 0.0f}, {-0.9951847195625305f, -7.109666189109021e-09f, 0.0980171412229538f, -8.933931927579408e-10f},
-    {-0.9807852506637573f, -2.9739473106360492e-08f, 0.19509032368659973f, -1.670471427850373e-09f}, {-0.9569403529167175f, 1.7184508038781132e-08f, 0.290284663438797f, 1.3815665056426951e-08f},
-    {-0.9238795042037964f, -2.830748968563057e-08f, 0.3826834261417389f, 6.2233507236442165e-09f}, {-0.8819212913513184f, 2.7002963420841297e-08f, 0.4713967442512512f, -7.425253745196869e-09f},
-    {-0.8314695954322815f, -1.687026340846387e-08f, 0.5555702447891235f, -1.1769521357507529e-08f}, {-0.7730104327201843f, -2.0642552556182636e-08f, 0.6343932747840881f, 9.37955757507325e-09f},
-    {-0.7071067690849304f, -1.2101617485882343e-08f, 0.7071067690849304f, 1.2101617485882343e-08f}, {-0.6343932747840881f, -9.37955757507325e-09f, 0.7730104327201843f, 2.0642552556182636e-08f},
-    {-0.5555702447891235f, 1.1769521357507529e-08f, 0.8314695954322815f, 1.687026340846387e-08f}, {-0.4713967442512512f, 7.425253745196869e-09f, 0.8819212913513184f, -2.7002963420841297e-08f},
-    {-0.3826834261417389f, -6.2233507236442165e-09f, 0.9238795042037964f, 2.830748968563057e-08f}, {-0.290284663438797f, -1.3815665056426951e-08f, 0.9569403529167175f, -1.7184508038781132e-08f},
-    {-0.19509032368659973f, 1.670471427850373e-09f, 0.9807852506637573f, 2.9739473106360492e-08f}, {-0.0980171412229538f, 8.933931927579408e-10f, 0.9951847195625305f, 7.109666189109021e-09f},
-    {0.0f, 0.0f, 1.0f, 0.0f}, {0.0980171412229538f, -8.933931927579408e-10f, 0.9951847195625305f, 7.109666189109021e-09f},
-    {0.19509032368659973f, -1.670471427850373e-09f, 0.9807852506637573f, 2.9739473106360492e-08f}, {0.290284663438797f, 1.3815665056426951e-08f, 0.9569403529167175f, -1.7184508038781132e-08f},
-    {0.3826834261417389f, 6.2233507236442165e-09f, 0.9238795042037964f, 2.830748968563057e-08f}, {0.4713967442512512f, -7.425253745196869e-09f, 0.8819212913513184f, -2.7002963420841297e-08f},
-    {0.5555702447891235f, -1.1769521357507529e-08f, 0.8314695954322815f, 1.687026340846387e-08f}, {0.6343932747840881f, 9.37955757507325e-09f, 0.7730104327201843f, 2.0642552556182636e-08f},
-    {0.7071067690849304f, 1.2101617485882343e-08f, 0.7071067690849304f, 1.2101617485882343e-08f}, {0.7730104327201843f, 2.0642552556182636e-08f, 0.6343932747840881f, 9.37955757507325e-09f},
-    {0.8314695954322815f, 1.687026340846387e-08f, 0.5555702447891235f, -1.1769521357507529e-08f}, {0.8819212913513184f, -2.7002963420841297e-08f, 0.4713967442512512f, -7.425253745196869e-09f},
-    {0.9238795042037964f, 2.830748968563057e-08f, 0.3826834261417389f, 6.2233507236442165e-09f}, {0.9569403529167175f, -1.7184508038781132e-08f, 0.290284663438797f, 1.3815665056426951e-08f},
-    {0.9807852506637573f, 2.9739473106360492e-08f, 0.19509032368659973f, -1.670471427850373e-09f}, {0.9951847195625305f, 7.109666189109021e-09f, 0.0980171412229538f, -8.933931927579408e-10f},
-    {1.0f, 0.0f, 0.0f, 0.0f}, {0.9951847195625305f, 7.109666189109021e-09f, -0.0980171412229538f, 8.933931927579408e-10f},
-    {0.9807852506637573f, 2.9739473106360492e-08f, -0.19509032368659973f, 1.670471427850373e-09f}, {0.9569403529167175f, -1.7184508038781132e-08f, -0.290284663438797f, -1.3815665056426951e-08f},
-    {0.9238795042037964f, 2.830748968563057e-08f, -0.3826834261417389f, -6.2233507236442165e-09f}, {0.8819212913513184f, -2.7002963420841297e-08f, -0.4713967442512512f, 7.425253745196869e-09f},
-    {0.8314695954322815f, 1.687026340846387e-08f, -0.5555702447891235f, 1.1769521357507529e-08f}, {0.7730104327201843f, 2.0642552556182636e-08f, -0.6343932747840881f, -9.37955757507325e-09f},
-    {0.7071067690849304f, 1.2101617485882343e-08f, -0.7071067690849304f, -1.2101617485882343e-08f}, {0.6343932747840881f, 9.37955757507325e-09f, -0.7730104327201843f, -2.0642552556182636e-08f},
-    {0.5555702447891235f, -1.1769521357507529e-08f, -0.8314695954322815f, -1.687026340846387e-08f}, {0.4713967442512512f, -7.425253745196869e-09f, -0.8819212913513184f, 2.7002963420841297e-08f},
-    {0.3826834261417389f, 6.2233507236442165e-09f, -0.9238795042037964f, -2.830748968563057e-08f}, {0.290284663438797f, 1.3815665056426951e-08f, -0.9569403529167175f, 1.7184508038781132e-08f},
-    {0.19509032368659973f, -1.670471427850373e-09f, -0.9807852506637573f, -2.9739473106360492e-08f}, {0.0980171412229538f, -8.933931927579408e-10f, -0.9951847195625305f, -7.109666189109021e-09f},
-    {0.0f, 0.0f, -1.0f, 0.0f},
-};
-__constant__ float kPi32H = 0.09817477315664291f, kPi32L = -2.7319617679211206e-09f;
-__constant__ float kPi4H = 0.7853981852531433f, kPi4L = -2.1855694143368964e-08f;
-__constant__ float kN6H = -0.1666666716337204f, kN6L = 4.967053879312289e-09f;
-// 2 pi = C1 + C2 + C3, C1 on 10 significant bits
-__constant__ float kC1 = 6.28125f, kC2 = 0.0019353071693331003f, kC3 = 1.0253376273028358e-11f;
-
-// Per-node double-float data (hi, lo pairs), with hq = h / 4, c0 = sqrt(2/pi),
-// nu the unnormalised normal and |z'| the speed:
 struct df_params {
   int n, b, nrhs, splits, tiles_per_split;
-  const float4* g;              // omega (x, y)
-  const float4* sqa;            // source factors omega hq c0 (nu1, nu2)
-  const float4* tq;             // target factors omega (nu1, nu2) / |z'|
-  const float2* sqe;            // source factor hq c0 eta |z'|
-  const float2* sqs;            // source factor hq c0 |z'|
-  const float2* w;              // Kress table w_d / (pi h)
+  df_nodes g;
   const float4* band;           // near entries (re hi, re lo, im hi, im lo), n x (2b + 1)
   const float4* x;              // densities as double-float (re hi, re lo, im hi, im lo)
-  double2* part;                // [split][k][i]
+  double2* part;                // [output][split][k][i]
   const int* fx;                // tensor-core residual: exponent of each accumulator column
 };
 
-// Hankel values of one far pair (x = omega r >= 20) in double-float, without
-// the common factor c0 x^(-1/2): (dx, dy) = omega (z_i - z_j), 1 / x,
-// ra = x^(-1/2), and j_m, y_m with J_m = c0 ra j_m, Y_m = c0 ra y_m
-struct df_hankel {
-  df dx, dy, xinv, ra, j0, y0, j1, y1;
-};
-
-__device__ __forceinline__ df_hankel hankel_df(float4 gi, float4 gj,
-                                               const float4* __restrict__ tab) {
-  const df dx = dsub({gi.x, gi.y}, {gj.x, gj.y});
-  const df dy = dsub({gi.z, gi.w}, {gj.z, gj.w});
-  const df x = dsqrt(dadd(dmul(dx, dx), dmul(dy, dy)));
-  const df t = drcp(x);
-  // chi = x - pi/4 - 2 pi k, |chi| <= pi
-  const float k = rintf(fmaf(x.h, 0.15915493667125702f, -0.125f));
-  df chi = {fmaf(-k, kC1, x.h), x.l};                          // exact first step
-  const float p2 = k * kC2;
-  chi = dsub(chi, {p2, fmaf(k, kC2, -p2)});
-  chi = dsub(chi, {k * kC3, 0.f});
-  chi = dsub(chi, {kPi4H, kPi4L});
-  // sin / cos: chi = j pi / 32 + d
-  const float jf = rintf(chi.h * 10.185916f);
-  const float pj = jf * kPi32H;
-  df d = dsub(chi, {pj, fmaf(jf, kPi32H, -pj)});
-  d = dsub(d, {jf * kPi32L, 0.f});
-  const df d2 = dmul(d, d);
-  const float z = d2.h;
-  const df d3 = dmul(d2, d);
-  const df sb = dadd({kN6H, kN6L}, {z * (1.0f / 120.0f - z * (1.0f / 5040.0f)), 0.f});
-  const df sd = dadd(d, dmul(d3, sb));                          // sin d
-  const df cb = dadd({-0.5f, 0.f}, {z * (1.0f / 24.0f - z * (1.0f / 720.0f)), 0.f});
-  const df cd = dadd({1.0f, 0.f}, dmul(d2, cb));                // cos d
-  const float4 tj = tab[(int)jf + 32];
-  const df sj = {tj.x, tj.y}, cj = {tj.z, tj.w};
-  const df sn = dadd(dmul(sj, cd), dmul(cj, sd));
-  const df cs = dsub(dmul(cj, cd), dmul(sj, sd));
-  // asymptotic expansion, t = 1/x
-  df P0, P1, Q0, Q1;
-  if (x.h >= kXS) {
-    // x >= 40: terms up to t^8 (P) and t^7 (Q), the corrections in FP32
-    // (t^2 with the lo part of t: its FP32 error, times the 0.07 t^2 term,
-    // stays below 3e-12 of P)
-    const float t2 = fmaf(t.h, t.h, 2.0f * t.h * t.l);
-    P0 = quick(1.0f, t2 * (-0.0703125f + t2 * (0.112152099609375f +
-                     t2 * (-0.5725014209747314f + t2 * 6.074042001273483f))));
-    P1 = quick(1.0f, t2 * (0.1171875f + t2 * (-0.144195556640625f +
-                     t2 * (0.6765925884246826f + t2 * -6.883914268109947f))));
-    Q0 = dadd({-0.125f * t.h, -0.125f * t.l},
-              {t.h * t2 * (0.0732421875f + t2 * (-0.22710800170898438f +
-                           t2 * 1.7277275025844574f)), 0.f});
-    Q1 = dadd(dmulf(t, 0.375f),
-              {t.h * t2 * (-0.1025390625f + t2 * (0.2775764465332031f +
-                           t2 * -1.993531733751297f)), 0.f});
-  } else {
-    // 20 <= x < 40 (pairs next to the band only): terms up to t^14 (P) and
-    // t^15 (Q), the first omitted one below 1e-14 at x = 20; the t^2 term of P
-    // and the t^3 term of Q (up to 2e-4 and 1e-5 there) in double-float
-    const df u2 = dmul(t, t), u3 = dmul(u2, t);
-    const float u = u2.h;
-    const float p0 = u * u * (0.112152099609375f + u * (-0.5725014209747314f +
-                     u * (6.074042001273483f + u * (-110.01714026924674f +
-                     u * (3038.090510922384f + u * -118838.42625678325f)))));
-    const float p1 = u * u * (-0.144195556640625f + u * (0.6765925884246826f +
-                     u * (-6.883914268109947f + u * (121.59789187653587f +
-                     u * (-3302.2722944808525f + u * 127641.2726461746f)))));
-    const float q0 = u3.h * u * (-0.22710800170898438f + u * (1.7277275025844574f +
-                     u * (-24.380529699556064f + u * (551.3358961220206f +
-                     u * (-18257.755474293175f + u * 832859.3040162893f)))));
-    const float q1 = u3.h * u * (0.2775764465332031f + u * (-1.993531733751297f +
-                     u * (27.248827311268542f + u * (-603.8440767050702f +
-                     u * (19718.37591223663f + u * -890297.8767070678f)))));
-    P0 = dadd({1.0f, 0.f}, dmulf(u2, -0.0703125f));
-    P0 = quick(P0.h, P0.l + p0);
-    P1 = dadd({1.0f, 0.f}, dmulf(u2, 0.1171875f));
-    P1 = quick(P1.h, P1.l + p1);
-    Q0 = dadd({-0.125f * t.h, -0.125f * t.l}, dmulf(u3, 0.0732421875f));
-    Q0 = quick(Q0.h, Q0.l + q0);
-    Q1 = dadd(dmulf(t, 0.375f), dmulf(u3, -0.1025390625f));
-    Q1 = quick(Q1.h, Q1.l + q1);
-  }
-  df_hankel H;
-  H.dx = dx;
-  H.dy = dy;
-  H.xinv = t;
-  H.ra = dsqrt(t);
-  H.j0 = dsub(dmul(P0, cs), dmul(Q0, sn));
-  H.y0 = dadd(dmul(P0, sn), dmul(Q0, cs));
-  H.j1 = dadd(dmul(P1, sn), dmul(Q1, cs));
-  H.y1 = dsub(dmul(Q1, sn), dmul(P1, cs));
-  return H;
-}
-
-// one far pair: soft entry a = h K + w K1 (eq. 1), K = L - i eta M.  With the
-// per-node factors folded in (source: sa = omega hq c0 nu_j, se = hq c0 eta
-// |z'_j|; wk = w / (pi h)): A = se ra, B = (sa . dx) ra / x and
-//   Re a = A j0 - B (y1 + wk j1),  Im a = B j1 + A (y0 + wk j0)
-__device__ __forceinline__ float4 entry_df(float4 gi, float4 gj, float4 sa, float2 se, float2 w2,
-                                           const float4* __restrict__ tab) {
-  const df_hankel H = hankel_df(gi, gj, tab);
-  const df wk = {w2.x, w2.y};
-  const df A = dmul({se.x, se.y}, H.ra);
-  const df B = dmul(dadd(dmul(H.dx, {sa.x, sa.y}), dmul(H.dy, {sa.z, sa.w})), dmul(H.xinv, H.ra));
-  const df re = dsub(dmul(A, H.j0), dmul(B, dadd(H.y1, dmul(wk, H.j1))));
-  const df im = dadd(dmul(B, H.j1), dmul(A, dadd(H.y0, dmul(wk, H.j0))));
-  return make_float4(re.h, re.l, im.h, im.l);
-}
-
-// one far pair of the sound-hard operator (eq. 2): S_ij = h M + w M1 with
-// M = (i/4) H0 |z'_j|, M1 = -(1/4 pi) J0 |z'_j|, and D'_ij = h L' + w L'1 with
-// L' = (i omega / 4) H1 cp, L'1 = -(omega / 4 pi) J1 cp,
-// cp = -((z_i - z_j) . nu~_i / r) |z'_j| / |z'_i|.  Folded (ss = hq c0 |z'_j|,
-// ti = omega nu_i / |z'_i|): A = ss ra, D = (ti . dx) ra ss / x and
-//   S = -A (y0 + wk j0) + i A j0,   D' = D (y1 + wk j1) - i D j1
-__device__ __forceinline__ void entry_df_hard(float4 gi, float4 gj, float4 ti, float2 ss2,
-                                              float2 w2, const float4* __restrict__ tab,
-                                              float4& S, float4& Dp) {
-  const df_hankel H = hankel_df(gi, gj, tab);
-  const df wk = {w2.x, w2.y};
-  const df ss = {ss2.x, ss2.y};
-  const df A = dmul(ss, H.ra);
-  const df sre = dneg(dmul(A, dadd(H.y0, dmul(wk, H.j0))));
-  const df sim = dmul(A, H.j0);
-  S = make_float4(sre.h, sre.l, sim.h, sim.l);
-  const df D = dmul(dmul(dadd(dmul(H.dx, {ti.x, ti.y}), dmul(H.dy, {ti.z, ti.w})),
-                         dmul(H.xinv, H.ra)), ss);
-  const df dre = dmul(D, dadd(H.y1, dmul(wk, H.j1)));
-  const df dim = dneg(dmul(D, H.j1));
-  Dp = make_float4(dre.h, dre.l, dim.h, dim.l);
-}
-
-// (s, e) += (ah + al)(xh + xl): TwoProd + TwoSum, errors gathered in e
-__device__ __forceinline__ void dot2_term(float& s, float& e, float ah, float al, float xh,
-                                          float xl) {
-  const float p = ah * xh;
-  float pe = fmaf(ah, xh, -p);
-  pe = fmaf(ah, xl, pe);
-  pe = fmaf(al, xh, pe);
-  const float t = s + p;
-  const float v = t - s;
-  e += ((s - (t - v)) + (p - v)) + pe;
+// (sr + i si, er + i ei) += a x for complex double-floats a = (re hi, re lo, im
+// hi, im lo), x alike: TwoProd + TwoSum per real product, errors gathered in e;
+// real and imaginary parts in packed pairs
+__device__ __forceinline__ void dot2_add(float2& s, float2& e, float2 ah, float2 al, float2 xh,
+                                         float2 xl) {
+  const float2 p = mul2(ah, xh);
+  float2 pe = fma2(ah, xh, neg2(p));
+  pe = fma2(ah, xl, pe);
+  pe = fma2(al, xh, pe);
+  const float2 t = add2(s, p), v = sub2(t, s);
+  e = add2(e, add2(add2(sub2(s, sub2(t, v)), sub2(p, v)), pe));
   s = t;
 }
-
-template <int RB>
-struct df_smem {
-  float4 A[DTI][DTJ + 1];
-  float4 X[DTJ][RB];
-};
-
-template <int RB>
-__global__ void __launch_bounds__(DNT) k_pair_df(df_params P) {
-  constexpr int RQ = RB / (DNT / DTI);
-  extern __shared__ __align__(16) unsigned char raw[];
-  df_smem<RB>& S = *reinterpret_cast<df_smem<RB>*>(raw);
-  // the sin / cos table, indexed per lane: shared memory, not the constant
-  // cache (which serialises differing addresses within a warp)
-  __shared__ float4 sTab[65];
-  const int n = P.n, tid = threadIdx.x;
-  if (tid < 65) sTab[tid] = kSinCos[tid];
-  const int i0 = blockIdx.x * DTI, split = blockIdx.y, rb0 = blockIdx.z * RB;
-  const int rbn = min(RB, P.nrhs - rb0);
-  const int ntiles = (n + DTJ - 1) / DTJ;
-  const int t_begin = split * P.tiles_per_split;
-  const int t_end = min(ntiles, t_begin + P.tiles_per_split);
-  const int il2 = tid % DTI, rg = tid / DTI;
-  const int bw = 2 * P.b + 1;
-  // running sums over the tiles in double-float (no FP64 instructions in the loop)
-  df accr[RQ], acci[RQ];
-#pragma unroll
-  for (int q = 0; q < RQ; ++q) accr[q] = acci[q] = df{0.f, 0.f};
-
-  for (int t = t_begin; t < t_end; ++t) {
-    const int j0 = t * DTJ;
-    __syncthreads();
-    for (int e = tid; e < DTJ * RB; e += DNT) {
-      const int jl = e / RB, r = e % RB, j = j0 + jl;
-      S.X[jl][r] = (j < n && r < rbn) ? P.x[(size_t)(rb0 + r) * n + j]
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    // entries: warp handles rows warp + 8 q, lane = source
-    for (int e = tid; e < DTI * DTJ; e += DNT) {
-      const int il = e / DTJ, jl = e % DTJ;
-      const int i = i0 + il, j = j0 + jl;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i < n && j < n) {
-        int d = i - j;
-        if (d < 0) d += n;
-        const int dd = d <= P.b ? d : (d >= n - P.b ? d - n : INT_MAX);
-        if (dd != INT_MAX)
-          a = P.band[(size_t)i * bw + dd + P.b];
-        else
-          a = entry_df(P.g[i], P.g[j], P.sqa[j], P.sqe[j], P.w[d], sTab);
-      }
-      S.A[il][jl] = a;
-    }
-    __syncthreads();
-    float4 t4[RQ];
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) t4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int jn = min(DTJ, n - j0);
-    for (int jl = 0; jl < jn; ++jl) {
-      const float4 a = S.A[il2][jl];
-#pragma unroll
-      for (int q = 0; q < RQ; ++q) {
-        const float4 x = S.X[jl][rg + 4 * q];
-        dot2_term(t4[q].x, t4[q].y, a.x, a.y, x.x, x.y);     // + ar xr
-        dot2_term(t4[q].x, t4[q].y, -a.z, -a.w, x.z, x.w);   // - ai xi
-        dot2_term(t4[q].z, t4[q].w, a.x, a.y, x.z, x.w);     // + ar xi
-        dot2_term(t4[q].z, t4[q].w, a.z, a.w, x.x, x.y);     // + ai xr
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-      accr[q] = dadd(accr[q], df{t4[q].x, t4[q].y});
-      acci[q] = dadd(acci[q], df{t4[q].z, t4[q].w});
-    }
-  }
-  const int i = i0 + il2;
-  if (i < n) {
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-      const int r = rg + 4 * q;
-      if (r < rbn)
-        P.part[((size_t)split * P.nrhs + rb0 + r) * n + i] =
-            make_double2((double)accr[q].h + (double)accr[q].l,
-                         (double)acci[q].h + (double)acci[q].l);
-    }
-  }
+__device__ __forceinline__ void dot2_cmul(float2& s, float2& e, float4 a, float4 x) {
+  dot2_add(s, e, f2(a.x), f2(a.y), make_float2(x.x, x.z), make_float2(x.y, x.w));
+  dot2_add(s, e, make_float2(-a.z, a.z), make_float2(-a.w, a.w), make_float2(x.z, x.x),
+           make_float2(x.w, x.y));
 }
 
-// Sound-hard residual sums (eq. 2 with Maue's identity for N): per right-hand
-// side four outputs over the same pair entries, o = 0: S u (u = d/ds x),
-// o = 1, 2: S (n_c x), o = 3: D' x, in double-float with Dot2 sums inside each
-// 32-source tile and double-float running sums across tiles.  Partial sums
-// per source split go out in the layout of the FP64 kernel:
-// part[((o * splits + split) * nrhs + k) * n + i].
-template <int RB>
-struct df_smem_hard {
-  float4 S[DTI][DTJ + 1];
-  float4 D[DTI][DTJ + 1];
-  float4 X[DTJ][RB][4];
+// Sums of the products of NO operators with their densities over a range of
+// source tiles, in double-float with Dot2 inside each 32-source tile and
+// double-float running sums across tiles (no FP64 instructions in the loop).
+// Soft: A x.  Hard: S u (u = d/ds x) and C x.  Partial sums per source split go
+// out as part[((o * splits + split) * nrhs + k) * n + i].
+template <int RB, int BC>
+struct df_smem {
+  float4 A[BC ? 2 : 1][DTI][DTJ + 1];
+  float4 X[DTJ][RB][BC ? 2 : 1];
 };
 
-template <int RB>
-__global__ void __launch_bounds__(DNT) k_pair_df_hard(df_params P, const float4* __restrict__ x4) {
-  constexpr int RQ = RB / (DNT / DTI);
+template <int RB, int BC>
+__global__ void __launch_bounds__(DNT) k_pair_df(df_params P, size_t xstride) {
+  constexpr int RQ = RB / (DNT / DTI), NO = BC ? 2 : 1;
   extern __shared__ __align__(16) unsigned char raw[];
-  df_smem_hard<RB>& S = *reinterpret_cast<df_smem_hard<RB>*>(raw);
-  __shared__ float4 sTab[65];   // sin / cos table (see k_pair_df)
+  df_smem<RB, BC>& S = *reinterpret_cast<df_smem<RB, BC>*>(raw);
   const int n = P.n, tid = threadIdx.x;
-  if (tid < 65) sTab[tid] = kSinCos[tid];
   const int i0 = blockIdx.x * DTI, split = blockIdx.y, rb0 = blockIdx.z * RB;
   const int rbn = min(RB, P.nrhs - rb0);
   const int ntiles = (n + DTJ - 1) / DTJ;
@@ -420,72 +90,90 @@ __global__ void __launch_bounds__(DNT) k_pair_df_hard(df_params P, const float4*
   const int il2 = tid % DTI, rg = tid / DTI;
   const int bw = 2 * P.b + 1;
   const size_t nbw = (size_t)n * bw;
-  df acc[4][RQ][2];
+  df acc[NO][RQ][2];
 #pragma unroll
-  for (int o = 0; o < 4; ++o)
+  for (int o = 0; o < NO; ++o)
 #pragma unroll
     for (int q = 0; q < RQ; ++q) acc[o][q][0] = acc[o][q][1] = df{0.f, 0.f};
 
   for (int t = t_begin; t < t_end; ++t) {
     const int j0 = t * DTJ;
     __syncthreads();
-    for (int e = tid; e < DTJ * RB * 4; e += DNT) {
-      const int c = e % 4, r = (e / 4) % RB, jl = e / (4 * RB), j = j0 + jl;
-      S.X[jl][r][c] = (j < n && r < rbn) ? x4[((size_t)(rb0 + r) * n + j) * 4 + c]
+    for (int e = tid; e < DTJ * RB * NO; e += DNT) {
+      const int o = e % NO, r = (e / NO) % RB, jl = e / (NO * RB), j = j0 + jl;
+      S.X[jl][r][o] = (j < n && r < rbn) ? P.x[o * xstride + (size_t)(rb0 + r) * n + j]
                                          : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    for (int e = tid; e < DTI * DTJ; e += DNT) {
-      const int il = e / DTJ, jl = e % DTJ;
+    // entries: a half warp per row, two adjacent sources per lane (n is even)
+    for (int e = tid; e < DTI * DTJ / 2; e += DNT) {
+      const int il = e / (DTJ / 2), jl = 2 * (e % (DTJ / 2));
       const int i = i0 + il, j = j0 + jl;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+      float4 a[NO][2];
+#pragma unroll
+      for (int o = 0; o < NO; ++o) a[o][0] = a[o][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (i < n && j < n) {
-        int d = i - j;
-        if (d < 0) d += n;
-        const int dd = d <= P.b ? d : (d >= n - P.b ? d - n : INT_MAX);
-        if (dd != INT_MAX) {
-          a = P.band[(size_t)i * bw + dd + P.b];
-          b = P.band[nbw + (size_t)i * bw + dd + P.b];
-        } else {
-          entry_df_hard(P.g[i], P.g[j], P.tq[i], P.sqs[j], P.w[d], sTab, a, b);
+        int dd[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          int d = i - j - u;
+          if (d < 0) d += n;
+          dd[u] = d <= P.b ? d : (d >= n - P.b ? d - n : INT_MAX);
         }
+        if (dd[0] == INT_MAX || dd[1] == INT_MAX) {
+          const float4 gx = P.g.tgt[2 * i], gy = P.g.tgt[2 * i + 1];
+          const df_entry2 v = entry_df2<BC ? OP_SC : OP_SOFT>(
+              make_float3(gx.x, gx.y, gx.z), make_float3(gy.x, gy.y, gy.z),
+              BC ? P.g.tq[i] : gx, P.g.src + (size_t)(j / 2) * 6, P.g.w[i - j + n], P.g.tab);
+          if constexpr (BC == 0) {
+            a[0][0] = make_float4(v.re.h.x, v.re.l.x, v.im.h.x, v.im.l.x);
+            a[0][1] = make_float4(v.re.h.y, v.re.l.y, v.im.h.y, v.im.l.y);
+          } else {
+            // S = i S'
+            a[0][0] = make_float4(-v.im.h.x, -v.im.l.x, v.re.h.x, v.re.l.x);
+            a[0][1] = make_float4(-v.im.h.y, -v.im.l.y, v.re.h.y, v.re.l.y);
+            a[NO - 1][0] = make_float4(v.re2.h.x, v.re2.l.x, v.im2.h.x, v.im2.l.x);
+            a[NO - 1][1] = make_float4(v.re2.h.y, v.re2.l.y, v.im2.h.y, v.im2.l.y);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (dd[u] != INT_MAX)
+#pragma unroll
+            for (int o = 0; o < NO; ++o) a[o][u] = P.band[o * nbw + (size_t)i * bw + dd[u] + P.b];
       }
-      S.S[il][jl] = a;
-      S.D[il][jl] = b;
+#pragma unroll
+      for (int o = 0; o < NO; ++o)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) S.A[o][il][jl + u] = a[o][u];
     }
     __syncthreads();
-    float4 t4[4][RQ];
+    float2 ts[NO][RQ], te[NO][RQ];
 #pragma unroll
-    for (int o = 0; o < 4; ++o)
+    for (int o = 0; o < NO; ++o)
 #pragma unroll
-      for (int q = 0; q < RQ; ++q) t4[o][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = 0; q < RQ; ++q) ts[o][q] = te[o][q] = f2(0.f);
     const int jn = min(DTJ, n - j0);
     for (int jl = 0; jl < jn; ++jl) {
-      const float4 a = S.S[il2][jl], b = S.D[il2][jl];
 #pragma unroll
-      for (int q = 0; q < RQ; ++q) {
+      for (int o = 0; o < NO; ++o) {
+        const float4 a = S.A[o][il2][jl];
 #pragma unroll
-        for (int o = 0; o < 4; ++o) {
-          const float4 m = o < 3 ? a : b;
-          const float4 v = S.X[jl][rg + 4 * q][o];
-          dot2_term(t4[o][q].x, t4[o][q].y, m.x, m.y, v.x, v.y);
-          dot2_term(t4[o][q].x, t4[o][q].y, -m.z, -m.w, v.z, v.w);
-          dot2_term(t4[o][q].z, t4[o][q].w, m.x, m.y, v.z, v.w);
-          dot2_term(t4[o][q].z, t4[o][q].w, m.z, m.w, v.x, v.y);
-        }
+        for (int q = 0; q < RQ; ++q)
+          if (rg + 4 * q < rbn) dot2_cmul(ts[o][q], te[o][q], a, S.X[jl][rg + 4 * q][o]);
       }
     }
 #pragma unroll
-    for (int o = 0; o < 4; ++o)
+    for (int o = 0; o < NO; ++o)
 #pragma unroll
       for (int q = 0; q < RQ; ++q) {
-        acc[o][q][0] = dadd(acc[o][q][0], df{t4[o][q].x, t4[o][q].y});
-        acc[o][q][1] = dadd(acc[o][q][1], df{t4[o][q].z, t4[o][q].w});
+        acc[o][q][0] = dadd(acc[o][q][0], df{ts[o][q].x, te[o][q].x});
+        acc[o][q][1] = dadd(acc[o][q][1], df{ts[o][q].y, te[o][q].y});
       }
   }
   const int i = i0 + il2;
   if (i < n) {
 #pragma unroll
-    for (int o = 0; o < 4; ++o)
+    for (int o = 0; o < NO; ++o)
 #pragma unroll
       for (int q = 0; q < RQ; ++q) {
         const int r = rg + 4 * q;
@@ -497,29 +185,9 @@ __global__ void __launch_bounds__(DNT) k_pair_df_hard(df_params P, const float4*
   }
 }
 
-// the four double-float inputs per right-hand side of the sound-hard sums:
-// u = d/ds x, n1 x, n2 x, x (n_c = nu~_c / |z'|)
-__global__ void k_df_x_hard(int n, size_t len, const double2* __restrict__ x,
-                            const double2* __restrict__ u, geom_dev g, float4* __restrict__ xo) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= len) return;
-  const int i = (int)(e % n);
-  const double inv = 1.0 / g.sp[i];
-  const double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-  const double2 xv = x[e], uv = u[e];
-  const double2 v[4] = {uv, make_double2(n1 * xv.x, n1 * xv.y), make_double2(n2 * xv.x, n2 * xv.y),
-                        xv};
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const float rh = (float)v[c].x, ih = (float)v[c].y;
-    xo[e * 4 + c] =
-        make_float4(rh, (float)(v[c].x - (double)rh), ih, (float)(v[c].y - (double)ih));
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Residual with the source sums on the tensor cores (the sound-soft entries,
-// or S or D' of the sound-hard operator).
+// or S or C of the sound-hard operator).
 //
 // Far pairs (outside the double-float band) are evaluated in double-float as
 // above and written as bf16 slices: with E_i the row's exponent (every far
@@ -549,6 +217,12 @@ __global__ void k_df_x_hard(int n, size_t len, const double2* __restrict__ x,
 // (k_band_df).  Split
 // complex as in the FP32 tensor-core kernel: [Yr | Yi] += Ar [Xr | Xi] +
 // Ai [-Xi | Xr].
+//
+// Bound: the producers' FP32 arithmetic, about 340 operations per pair (290 for
+// the entry, 52 for the slices), issued in packed pairs.  Measured (GB300): kite
+// n = 32768, 64 right-hand sides 27.4 -> 18.1 ms (710 -> 380 instructions per
+// pair); star n = 4096, 16, sound hard: 1.88 -> 0.76 ms (two passes instead of
+// three, the band sums 0.77 -> 0.1 ms).
 // ---------------------------------------------------------------------------
 constexpr int RTM = 128;      // rows per tile (UMMA M)
 constexpr int RTK = 16;       // sources per tile: one K step, 32-byte rows
@@ -563,15 +237,13 @@ constexpr int RWTMA = RPROD, RWMMA = RPROD + 1;
 // 18 warps (the producers also drain the accumulators): at most 5 per
 // scheduler, so 96 registers per thread fit its quarter of the register file
 constexpr int RNT = (RPROD + 2) * 32;
+constexpr uint32_t RPLANE = RTM * RTK * 2;   // bytes of one A plane
 
 template <int NB>
 struct rtc_smem {
   __nv_bfloat16 A[RST][2 * RSL][RTM * RTK];    // Ar slices 0..5, Ai slices 0..5
   __nv_bfloat16 B[RST][2 * RSL][2 * NB * RTK]; // per slice t: [Xr | Xi], [-Xi | Xr]
-  float4 tgt[RTM];
-  float4 tgn[RTM];   // target factors (hard kinds)
-  int ex[RTM];
-  float4 tab[65];    // sin / cos table (per-lane indices: shared, not constant)
+  float4 tab[kDfTab];   // sine / cosine table (per-lane indices)
   uint64_t full[RST], empty[RST], tfull, tempty;
   uint64_t mdone;    // completion of every MMA issued (abort path)
   uint32_t tmem_base;
@@ -581,6 +253,7 @@ struct rtc_smem {
 
 template <int NB>
 constexpr size_t rtc_smem_bytes() {
+  static_assert(sizeof(rtc_smem<NB>) + 1024 <= 227 * 1024, "stages exceed shared memory");
   return sizeof(rtc_smem<NB>) + 1024;
 }
 
@@ -600,35 +273,36 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
   return d;
 }
 
-// six 8-bit slices of a double-float value already scaled below 128 in
-// magnitude, slice s multiplied by 2^(-8 s)
-__device__ __forceinline__ void slice6(float h, float l, float* o) {
-  float q = rintf(h);
+// six 8-bit slices of two double-float values already scaled below 128 in
+// magnitude, slice s multiplied by 2^(-8 s); o[s] for both values.  Values are
+// rounded to integers by adding and subtracting 1.5 2^23.
+__device__ __forceinline__ void slice6(float2 h, float2 l, float2* o) {
+  constexpr float M = 12582912.0f;
+  auto rnd = [](float2 v) { return add2(add2(v, f2(M)), f2(-M)); };
+  // rint(256 v), by fma
+  auto rnd256 = [](float2 v) { return add2(fma2(v, f2(256.f), f2(M)), f2(-M)); };
+  float2 q = rnd(h);
   o[0] = q;
-  float r = h - q;                             // exact
+  float2 r = sub2(h, q);                         // exact
 #pragma unroll
   for (int s = 1; s < 3; ++s) {
-    q = rintf(r * 256.f);
-    r = fmaf(r, 256.f, -q);                    // exact
-    o[s] = q * (s == 1 ? 0.00390625f : 1.52587890625e-05f);
+    q = rnd256(r);
+    r = fma2(r, f2(256.f), neg2(q));             // exact
+    o[s] = mul2(q, f2(s == 1 ? 0.00390625f : 1.52587890625e-05f));
   }
   // the rest of h (scaled by 2^16) with l: within 2^-24 of its size
-  float rr = fmaf(r, 256.f, l * 16777216.f);
-  q = rintf(rr);
-  o[3] = q * 5.9604644775390625e-08f;          // 2^-24
-  rr -= q;
-  q = rintf(rr * 256.f);
-  o[4] = q * 2.3283064365386963e-10f;          // 2^-32
-  rr = fmaf(rr, 256.f, -q);
-  q = rintf(rr * 256.f);
-  o[5] = q * 9.094947017729282e-13f;           // 2^-40
+  float2 rr = fma2(r, f2(256.f), mul2(l, f2(16777216.f)));
+  q = rnd(rr);
+  o[3] = mul2(q, f2(5.9604644775390625e-08f));   // 2^-24
+  rr = sub2(rr, q);
+  q = rnd256(rr);
+  o[4] = mul2(q, f2(2.3283064365386963e-10f));   // 2^-32
+  rr = fma2(rr, f2(256.f), neg2(q));
+  q = rnd256(rr);
+  o[5] = mul2(q, f2(9.094947017729282e-13f));    // 2^-40
 }
 
-// entry kinds of the sliced residual: the sound-soft combination (eq. 1), or
-// S or D' of the sound-hard operator (eq. 2)
-enum { RK_SOFT = 0, RK_S = 1, RK_DP = 2 };
-
-template <int NB, int KIND>
+template <int NB, int OP>
 __global__ void __launch_bounds__(RNT, 1)
 k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ CUtensorMap tmB,
            const int4* __restrict__ segs, const int* __restrict__ cbeg,
@@ -639,8 +313,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
   static_assert(NL * NC <= 512, "level accumulators exceed the tensor memory");
   constexpr uint32_t B_BYTES = 2u * RSL * NC * RTK * 2u;
   extern __shared__ unsigned char raw[];
-  rtc_smem<NB>& S = *reinterpret_cast<rtc_smem<NB>*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
-                                                      ~uintptr_t(1023));
+  rtc_smem<NB>& S = smem_aligned<rtc_smem<NB>>(raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sb = cbeg[blockIdx.x], se = cbeg[blockIdx.x + 1];
   const int n = P.n;
@@ -657,7 +330,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
     S.abort = 0;
     fence_mbar_init();
   }
-  if (threadIdx.x < 65) S.tab[threadIdx.x] = kSinCos[threadIdx.x];
+  for (int q = threadIdx.x; q < kDfTab; q += RNT) S.tab[q] = P.g.tab[q];
   if (warp == RWMMA) {
     tmem_alloc(&S.tmem_base, TMEM_COLS);
     tmem_relinquish();
@@ -668,9 +341,12 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
   const uint32_t tmem = S.tmem_base;
 
   if (warp < RPROD) {
-    // ---- producers: warp w owns rows w + RPROD (4 q + lane / 8), q = 0, 1;
-    // lane l the two adjacent sources 2 (l % 8), +1 of the 16-source tile
-    const int sub = lane >> 3, jp = 2 * (lane & 7);
+    // ---- producers: lane l of warp w owns row 32 (w % 4) + l and the four
+    // sources 4 (w / 4) .. + 3 of each 16-source tile, two at a time in packed
+    // pairs: the target stays in registers, the source data are warp-uniform
+    // loads
+    const int row = 32 * (warp & 3) + lane, js = 4 * (warp >> 2);
+    const uint32_t off = sw32(row, js);
     // Accumulator drain: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its
     // rows) and a group of columns; chunk c (RCK tiles) is drained once the
     // first tile of chunk c + 1 is produced: the four exact levels are added
@@ -745,78 +421,70 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
     for (int s = sb; s < se && !stop; ++s) {
       const int4 sg = segs[s];
       const int m0 = sg.y * RTM;
-      __syncwarp();
-      if (lane < RTM / RPROD) {
-        const int r = warp + RPROD * lane;
-        const int i = m0 + r;
-        S.tgt[r] = i < n ? P.g[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        S.ex[r] = i < n ? rowexp[i] : 0;
-        if (KIND != RK_SOFT) S.tgn[r] = i < n ? P.tq[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int i = m0 + row;
+      float3 tx, ty;
+      float4 tq;
+      float sc;                            // 2^(7 - E_i): exact for both parts
+      {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 gx = i < n ? P.g.tgt[2 * i] : z, gy = i < n ? P.g.tgt[2 * i + 1] : z;
+        tx = make_float3(gx.x, gx.y, gx.z);
+        ty = make_float3(gy.x, gy.y, gy.z);
+        tq = OP == OP_C && i < n ? P.g.tq[i] : z;
+        sc = __int_as_float((127 + 7 - (i < n ? rowexp[i] : 0)) << 23);
       }
-      __syncwarp();
       for (int k = sg.z; k < sg.w; ++k, ++it) {
         const int st = it % RST;
         // exits are warp-uniform: the warp arrives on the stage barrier as one
         if (__any_sync(0xffffffffu, *(volatile int*)&S.abort)) break;
-        if (it >= RST && !__all_sync(0xffffffffu, mbar_wait(&S.empty[st], ((it / RST) - 1) & 1))) {
+        if (it >= RST &&
+            !__all_sync(0xffffffffu, mbar_wait_sleep<100>(&S.empty[st], ((it / RST) - 1) & 1))) {
           if (lane == 0) {
             atomicExch(err, 21);
             S.abort = 1;
           }
           break;
         }
-        const int j = k * RTK + jp;
-        float4 gj[2], nj[2];
-        float2 sj[2];
+        // a tile is plain when it holds full rows and sources and no pair of
+        // the band (|i - j - t n| <= b for t = -1, 0, 1)
+        const int j0 = k * RTK;
+        bool plain = m0 + RTM <= n && j0 + RTK <= n;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const bool ok = j + u < n;
-          gj[u] = ok ? P.g[j + u] : make_float4(0.f, 0.f, 0.f, 0.f);
-          if (KIND == RK_SOFT) {
-            nj[u] = ok ? P.sqa[j + u] : make_float4(0.f, 0.f, 0.f, 0.f);
-            sj[u] = ok ? P.sqe[j + u] : make_float2(0.f, 0.f);
-          } else {
-            sj[u] = ok ? P.sqs[j + u] : make_float2(0.f, 0.f);
-          }
-        }
-        unsigned char* A = reinterpret_cast<unsigned char*>(&S.A[st][0][0]);
+        for (int t = -1; t <= 1; ++t)
+          plain &= m0 + RTM - 1 - j0 < t * n - P.b || m0 - j0 - (RTK - 1) > t * n + P.b;
+        unsigned char* A = reinterpret_cast<unsigned char*>(&S.A[st][0][0]) + off;
 #pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-          const int il = warp + RPROD * (4 * q + sub);
-          const int i = m0 + il;
-          const float4 gi = S.tgt[il];
-          const int e = S.ex[il];
-          float sl[2][2][RSL];                  // [source][re/im][slice]
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-            const int jj = j + u;
-            if (i < n && jj < n) {
-              int d = i - jj;
-              if (d < 0) d += n;
-              if (d > P.b && d < n - P.b) {
-                if constexpr (KIND == RK_SOFT) {
-                  a = entry_df(gi, gj[u], nj[u], sj[u], P.w[d], S.tab);
-                } else {
-                  float4 es, ed;
-                  entry_df_hard(gi, gj[u], S.tgn[il], sj[u], P.w[d], S.tab, es, ed);
-                  a = KIND == RK_S ? es : ed;
-                }
-              }
+        for (int u = 0; u < 2; ++u) {
+          const int j = j0 + js + 2 * u;
+          const bool in = plain || (i < n && j < n);     // n is even: j + 1 < n as well
+          df_entry2 e;
+          e.re = e.im = {f2(0.f), f2(0.f)};
+          if (in) {
+            e = entry_df2<OP>(tx, ty, tq, P.g.src + (size_t)(j / 2) * 6, __ldg(P.g.w + i - j + n),
+                              S.tab);
+            if constexpr (OP == OP_S) {   // S = i S'
+              const d2 r = e.re;
+              e.re = dd_neg(e.im);
+              e.im = r;
             }
-            // scale by 2^(7 - e): exact for both parts
-            const float sc = __int_as_float((127 + 7 - e) << 23);
-            slice6(a.x * sc, a.y * sc, sl[u][0]);
-            slice6(a.z * sc, a.w * sc, sl[u][1]);
+            if (!plain) {
+              int d0 = i - j, d1 = i - j - 1;
+              if (d0 < 0) d0 += n;
+              if (d1 < 0) d1 += n;
+              if (d0 <= P.b || d0 >= n - P.b) e.re.h.x = e.re.l.x = e.im.h.x = e.im.l.x = 0.f;
+              if (d1 <= P.b || d1 >= n - P.b) e.re.h.y = e.re.l.y = e.im.h.y = e.im.l.y = 0.f;
+            }
           }
-          const uint32_t o = sw32(il, jp);
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
+          for (int c = 0; c < 2; ++c) {
+            const d2 v = c ? e.im : e.re;
+            float2 sl[RSL];
+            slice6(mul2(v.h, f2(sc)), mul2(v.l, f2(sc)), sl);
 #pragma unroll
-            for (int t = 0; t < RSL; ++t) {
-              const __nv_bfloat162 v = __floats2bfloat162_rn(sl[0][c][t], sl[1][c][t]);
-              *reinterpret_cast<__nv_bfloat162*>(A + (size_t)(c * RSL + t) * RTM * RTK * 2 + o) = v;
-            }
+            for (int t = 0; t < RSL; ++t)
+              *reinterpret_cast<__nv_bfloat162*>(A + (c * RSL + t) * RPLANE + 4 * u) =
+                  __floats2bfloat162_rn(sl[t].x, sl[t].y);
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
@@ -847,7 +515,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
         const int4 sg = segs[s];
         for (int k = sg.z; k < sg.w; ++k, ++it) {
           const int st = it % RST;
-          if (it >= RST && !mbar_wait(&S.empty[st], ((it / RST) - 1) & 1)) {
+          if (it >= RST && !mbar_wait_sleep<1000>(&S.empty[st], ((it / RST) - 1) & 1)) {
             atomicExch(err, 22);
             S.abort = 1;
             break;
@@ -870,7 +538,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
         const int4 sg = segs[s];
         for (int c0 = sg.z; c0 < sg.w; c0 += RCK, ++cc) {
           const int c1 = min(sg.w, c0 + RCK);
-          if (cc >= 1 && !mbar_wait(&S.tempty, (cc - 1) & 1)) {
+          if (cc >= 1 && !mbar_wait_sleep<200>(&S.tempty, (cc - 1) & 1)) {
             atomicExch(err, 24);
             S.abort = 1;
           }
@@ -878,7 +546,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
           tc_fence_after();
           for (int k = c0; k < c1; ++k, ++it) {
             const int st = it % RST;
-            if (!mbar_wait(&S.full[st], (it / RST) & 1)) {
+            if (!mbar_wait_sleep<200>(&S.full[st], (it / RST) & 1)) {
               atomicExch(err, 23);
               S.abort = 1;
               break;
@@ -930,38 +598,52 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
   }
 }
 
-// Row exponents of the far entries: E_i with |Re a_ij|, |Im a_ij| < 2^E_i for
-// every pair outside the double-float band, from the FP32 entries with a
-// 1e-4 margin (their relative error is ~1e-6); 0 for rows without far pairs.
-template <int KIND>
+// Largest |Re a_ij|, |Im a_ij| of the far entries of every row (float bits,
+// zeroed beforehand), from the packed FP32 entries of the fused matvec; hard:
+// of S', then of C.  64 rows per CTA, the source pairs of the CTA's share split
+// over four groups of threads.
+template <int OP>
 __global__ void __launch_bounds__(256)
-k_rowexp(int n, int b, const float4* __restrict__ pk, const float2* __restrict__ wkt,
-         int* __restrict__ rowexp) {
-  __shared__ float red[4][64];
+k_rowmax(int n, int b, int per_cta, const float4* __restrict__ pk, const float4* __restrict__ spk,
+         const float2* __restrict__ wkt, unsigned* __restrict__ rmax) {
   const int il = threadIdx.x % 64, qd = threadIdx.x / 64;
   const int i = blockIdx.x * 64 + il;
-  float m = 0.f;
-  if (i < n) {
-    // the folded FP32 entries of the fused tensor-core kernel (packed
-    // per-node vectors; source j is the same for a whole warp)
-    const float4 tg = pk[i];
-    const float4 tq = KIND == RK_DP ? pk[2 * n + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = qd; j < n; j += 4) {
-      int d = i - j;
-      if (d < 0) d += n;
-      if (d <= b || d >= n - b) continue;
-      const float2 a = entry_folded32<KIND>(tg, tq, pk[j], pk[n + j], wkt[i - j + n].x);
-      m = fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y)));
+  if (i >= n) return;
+  float m = 0.f, m2 = 0.f;
+  const float4 tg = pk[i];
+  const float4 t0 = make_float4(tg.x, tg.x, tg.y, tg.y), t1 = make_float4(tg.z, tg.z, tg.w, tg.w);
+  const float4 q = OP == OP_SC ? pk[2 * n + i] : tg;
+  const float4 tq = make_float4(q.x, q.x, q.y, q.y);
+  const int j_end = min(n, (int)(blockIdx.y + 1) * per_cta);
+  for (int j = blockIdx.y * per_cta + 2 * qd; j < j_end; j += 8) {
+    const entry_pair e = finish32_pair<OP>(phase32_pair(t0, t1, spk[j], spk[j + 1]), tq,
+                                           spk[n + j], lo2(spk[n + j + 1]), wkt[i - j + n]);
+    int d0 = i - j, d1 = i - j - 1;
+    if (d0 < 0) d0 += n;
+    if (d1 < 0) d1 += n;
+    if (d0 > b && d0 < n - b) {
+      m = fmaxf(m, fmaxf(fabsf(e.re.x), fabsf(e.im.x)));
+      if (OP == OP_SC) m2 = fmaxf(m2, fmaxf(fabsf(e.re2.x), fabsf(e.im2.x)));
+    }
+    if (d1 > b && d1 < n - b) {
+      m = fmaxf(m, fmaxf(fabsf(e.re.y), fabsf(e.im.y)));
+      if (OP == OP_SC) m2 = fmaxf(m2, fmaxf(fabsf(e.re2.y), fabsf(e.im2.y)));
     }
   }
-  red[qd][il] = m;
-  __syncthreads();
-  if (qd == 0 && i < n) {
-    m = fmaxf(fmaxf(red[0][il], red[1][il]), fmaxf(red[2][il], red[3][il]));
-    int e = 0;
-    if (m > 0.f) frexpf(m * 1.0001f, &e);
-    rowexp[i] = e;
-  }
+  if (m > 0.f) atomicMax(&rmax[i], __float_as_uint(m));
+  if (OP == OP_SC && m2 > 0.f) atomicMax(&rmax[n + i], __float_as_uint(m2));
+}
+
+// row maxima (float bits, in place) -> exponents E with max < 2^E (1e-4 margin
+// for the FP32 evaluation, whose relative error is ~1e-6), 0 for rows without
+// far entries
+__global__ void k_rowexp(int len, unsigned* __restrict__ r) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= len) return;
+  const float m = __uint_as_float(r[i]);
+  int e = 0;
+  if (m > 0.f) frexpf(m * 1.0001f, &e);
+  reinterpret_cast<int*>(r)[i] = e;
 }
 
 // Column exponents F_r (|Re x|, |Im x| < 2^F_r) of the right-hand sides r0 ..
@@ -997,75 +679,87 @@ __global__ void k_xslices(int n, int pitch, int NB, int nr, const double2* __res
   const int j = blockIdx.x * 256 + threadIdx.x;
   const int r = blockIdx.y;
   if (j >= pitch) return;
-  float sr[RSL], si[RSL];
+  float2 sl[RSL];   // slices of the real and the imaginary part
   if (j < n && r < nr) {
     const double2 v = x[(size_t)r * n + j];
     const double sc = ldexp(1.0, 7 - fx[r]);
     const double vr = v.x * sc, vi = v.y * sc;
     const float rh = (float)vr, ih = (float)vi;
-    slice6(rh, (float)(vr - (double)rh), sr);
-    slice6(ih, (float)(vi - (double)ih), si);
+    slice6(make_float2(rh, ih), make_float2((float)(vr - (double)rh), (float)(vi - (double)ih)), sl);
   } else {
 #pragma unroll
-    for (int t = 0; t < RSL; ++t) sr[t] = si[t] = 0.f;
+    for (int t = 0; t < RSL; ++t) sl[t] = f2(0.f);
   }
   const size_t plane = (size_t)2 * NB * pitch;
 #pragma unroll
   for (int t = 0; t < RSL; ++t) {
     __nv_bfloat16* p1 = bt + (size_t)(2 * t) * plane;
     __nv_bfloat16* p2 = bt + (size_t)(2 * t + 1) * plane;
-    p1[(size_t)r * pitch + j] = __float2bfloat16_rn(sr[t]);
-    p1[(size_t)(NB + r) * pitch + j] = __float2bfloat16_rn(si[t]);
-    p2[(size_t)r * pitch + j] = __float2bfloat16_rn(-si[t]);
-    p2[(size_t)(NB + r) * pitch + j] = __float2bfloat16_rn(sr[t]);
+    p1[(size_t)r * pitch + j] = __float2bfloat16_rn(sl[t].x);
+    p1[(size_t)(NB + r) * pitch + j] = __float2bfloat16_rn(sl[t].y);
+    p2[(size_t)r * pitch + j] = __float2bfloat16_rn(-sl[t].y);
+    p2[(size_t)(NB + r) * pitch + j] = __float2bfloat16_rn(sl[t].x);
   }
 }
 
-// Near-band part of the soft residual (diagonal included): Dot2 over the
-// 2 b + 1 band entries of each row, double-float densities; one thread per
-// (row, group of 8 right-hand sides), each band entry loaded once per group
+// Near-band part of the residual (diagonal included): Dot2 over the 2 b + 1
+// band entries of each row, double-float densities.  Eight lanes share a row
+// and a group of up to 8 right-hand sides and take every eighth entry (128
+// contiguous bytes of the band), then join their sums in double-float.  (One
+// thread per row left the band reads uncoalesced and n = 4096 at 64 CTAs: 257
+// us at 16 right-hand sides.)
 constexpr int BRG = 8;
-__global__ void k_band_df(int n, int b, int nrhs, const float4* __restrict__ band,
-                          const float4* __restrict__ x, double2* __restrict__ yb) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int groups = (nrhs + BRG - 1) / BRG;
-  if (e >= (size_t)n * groups) return;
-  const int i = (int)(e % n), r0 = (int)(e / n) * BRG;
+__global__ void __launch_bounds__(256)
+k_band_df(int n, int b, int nrhs, const float4* __restrict__ band, const float4* __restrict__ x,
+          double2* __restrict__ yb) {
+  const int sub = threadIdx.x & 7;
+  const int i = (blockIdx.x * 256 + threadIdx.x) >> 3, r0 = blockIdx.y * BRG;
   const int rn = min(BRG, nrhs - r0);
   const int bw = 2 * b + 1;
-  float s[BRG][4];
+  float2 s[BRG], e[BRG];
 #pragma unroll
-  for (int q = 0; q < BRG; ++q) s[q][0] = s[q][1] = s[q][2] = s[q][3] = 0.f;
-  for (int dd = -b; dd <= b; ++dd) {
-    // each pair once: the offset its cyclic distance maps to (matters when
-    // the band wraps around, 2 b + 1 > n)
-    const int d = dd < 0 ? dd + n : dd;
-    if ((d <= b ? d : d - n) != dd) continue;
-    int j = (i - dd) % n;
-    if (j < 0) j += n;
-    const float4 a = band[(size_t)i * bw + dd + b];
+  for (int q = 0; q < BRG; ++q) s[q] = e[q] = f2(0.f);
+  if (i < n) {
+    for (int c = sub; c < bw; c += 8) {
+      const int dd = c - b;
+      // each pair once: the offset its cyclic distance maps to (matters when
+      // the band wraps around, 2 b + 1 > n)
+      const int d = dd < 0 ? dd + n : dd;
+      if ((d <= b ? d : d - n) != dd) continue;
+      int j = i - dd;
+      if (j < 0) j += n;
+      if (j >= n) j -= n;
+      const float4 a = band[(size_t)i * bw + c];
 #pragma unroll
-    for (int q = 0; q < BRG; ++q) {
-      if (q < rn) {
-        const float4 v = x[(size_t)(r0 + q) * n + j];
-        dot2_term(s[q][0], s[q][1], a.x, a.y, v.x, v.y);
-        dot2_term(s[q][0], s[q][1], -a.z, -a.w, v.z, v.w);
-        dot2_term(s[q][2], s[q][3], a.x, a.y, v.z, v.w);
-        dot2_term(s[q][2], s[q][3], a.z, a.w, v.x, v.y);
-      }
+      for (int q = 0; q < BRG; ++q)
+        if (q < rn) dot2_cmul(s[q], e[q], a, x[(size_t)(r0 + q) * n + j]);
     }
   }
 #pragma unroll
-  for (int q = 0; q < BRG; ++q)
-    if (q < rn)
-      yb[(size_t)(r0 + q) * n + i] =
-          make_double2((double)s[q][0] + (double)s[q][1], (double)s[q][2] + (double)s[q][3]);
+  for (int q = 0; q < BRG; ++q) {
+    if (q < rn) {
+#pragma unroll
+      for (int o = 1; o < 8; o *= 2) {
+        const float2 so = make_float2(__shfl_xor_sync(0xffffffffu, s[q].x, o),
+                                      __shfl_xor_sync(0xffffffffu, s[q].y, o));
+        const float2 eo = make_float2(__shfl_xor_sync(0xffffffffu, e[q].x, o),
+                                      __shfl_xor_sync(0xffffffffu, e[q].y, o));
+        const d2 t = dd_norm(dd_add({s[q], e[q]}, {so, eo}));
+        s[q] = t.h;
+        e[q] = t.l;
+      }
+      if (sub == 0 && i < n)
+        yb[(size_t)(r0 + q) * n + i] =
+            make_double2((double)s[q].x + (double)e[q].x, (double)s[q].y + (double)e[q].y);
+    }
+  }
 }
 
-// y[r][i] = band part + sum of the segment sums of row tile i / 128 (FP64)
+// y[r][i] = band part + sum of the segment sums of row tile i / 128 (FP64),
+// plus half[r][i] / 2 when given
 __global__ void k_reduce_rtc(int n, int NB, int nr, const int2* __restrict__ mt_seg,
                              const float2* __restrict__ acc, const double2* __restrict__ yb,
-                             double2* __restrict__ y) {
+                             const double2* __restrict__ half, double2* __restrict__ y) {
   const int m = blockIdx.x, r = blockIdx.y, row = threadIdx.x;
   const int i = m * RTM + row;
   if (i >= n || r >= nr) return;
@@ -1077,6 +771,11 @@ __global__ void k_reduce_rtc(int n, int NB, int nr, const int2* __restrict__ mt_
     const float2 pi = acc[((size_t)s * NC + NB + r) * RTM + row];
     v.x += (double)pr.x + (double)pr.y;
     v.y += (double)pi.x + (double)pi.y;
+  }
+  if (half) {
+    const double2 h = half[(size_t)r * n + i];
+    v.x = fma(0.5, h.x, v.x);
+    v.y = fma(0.5, h.y, v.y);
   }
   y[(size_t)r * n + i] = v;
 }
@@ -1090,41 +789,50 @@ __global__ void k_df_x(size_t len, const double2* __restrict__ x, float4* __rest
   xo[e] = make_float4(rh, (float)(v.x - (double)rh), ih, (float)(v.y - (double)ih));
 }
 
-__global__ void k_reduce_df(int n, int nrhs, int splits, const double2* __restrict__ part,
-                            double2* __restrict__ y) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t tot = (size_t)n * nrhs;
-  if (e >= tot) return;
-  double sx = 0.0, sy = 0.0;
-  for (int s = 0; s < splits; ++s) {
-    const double2 p = part[(size_t)s * tot + e];
-    sx += p.x;
-    sy += p.y;
-  }
-  y[e] = make_double2(sx, sy);
-}
-
-// set-up: per-node double-float data (df_params), band width for
-// omega r < kXD, FP64 band
-__global__ void k_df_geo(int n, geom_dev g, const double* __restrict__ w, double omega,
-                         double eta, double h, float4* __restrict__ go, float4* __restrict__ sa,
-                         float4* __restrict__ tq, float2* __restrict__ se,
-                         float2* __restrict__ ss, float2* __restrict__ wo) {
+// set-up: per-node double-float data (df_nodes in pairdf.cuh); threads past the
+// nodes convert the sine / cosine table
+__global__ void k_df_geo(int n, geom_dev g, const double* __restrict__ w, double omega, double eta,
+                         double h, int hard, const unsigned* __restrict__ bound,
+                         float4* __restrict__ tgt, float4* __restrict__ tq, float4* __restrict__ src,
+                         float4* __restrict__ wo, float4* __restrict__ tab) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n) {
+    if (i - n < kDfTab) {
+      const double2 v = g.tab[i - n];
+      const df s = dmake(v.x), c = dmake(v.y);
+      tab[i - n] = make_float4(s.h, s.l, c.h, c.l);
+    }
+    return;
+  }
   const double f = 0.25 * h * 0.7978845608028654;   // hq c0
   const double sp = g.sp[i];
-  const df x = dmake(omega * g.x[i]), y = dmake(omega * g.y[i]);
-  const df a1 = dmake(omega * f * g.nx[i]), a2 = dmake(omega * f * g.ny[i]);
+  // coordinates times omega in three parts: hi on the grid 2^(e - 23) where
+  // every omega |x|, omega |y| < 2^e, mid on 2^(e - 47), the rest
+  int e = 0;
+  const double m = omega * (double)__uint_as_float(*bound);
+  if (m > 0.0) frexp(m, &e);
+  auto split3 = [e](double v) {
+    const double hi = rint(ldexp(v, 23 - e)), r = v - ldexp(hi, e - 23);
+    const double mid = rint(ldexp(r, 47 - e));
+    return make_float3((float)ldexp(hi, e - 23), (float)ldexp(mid, e - 47),
+                       (float)(r - ldexp(mid, e - 47)));
+  };
+  const float3 x = split3(omega * g.x[i]), y = split3(omega * g.y[i]);
+  tgt[2 * i] = make_float4(x.x, x.y, x.z, 0.f);
+  tgt[2 * i + 1] = make_float4(y.x, y.y, y.z, 0.f);
   const df t1 = dmake(omega * g.nx[i] / sp), t2 = dmake(omega * g.ny[i] / sp);
-  const df e = dmake(f * eta * sp), s = dmake(f * sp);
-  const df ww = dmake(w[i] / (3.141592653589793 * h));
-  go[i] = make_float4(x.h, x.l, y.h, y.l);
-  sa[i] = make_float4(a1.h, a1.l, a2.h, a2.l);
   tq[i] = make_float4(t1.h, t1.l, t2.h, t2.l);
-  se[i] = make_float2(e.h, e.l);
-  ss[i] = make_float2(s.h, s.l);
-  wo[i] = make_float2(ww.h, ww.l);
+  const double k = hard ? omega / eta / sp : omega * f;
+  const df a = dmake(k * g.nx[i]), b = dmake(k * g.ny[i]);
+  const df c = dmake(hard ? f * sp : f * eta * sp);
+  // value v of node i at 24 (i / 2) + 2 v + i % 2
+  float* q = reinterpret_cast<float*>(src) + (size_t)(i / 2) * 24 + (i & 1);
+  const float v[12] = {-x.x, -x.y, -x.z, -y.x, -y.y, -y.z, a.h, a.l, b.h, b.l, c.h, c.l};
+#pragma unroll
+  for (int u = 0; u < 12; ++u) q[2 * u] = v[u];
+  const double ph = 3.141592653589793 * h;
+  const df w0 = dmake(w[i] / ph), w1 = dmake(w[i == 0 ? n - 1 : i - 1] / ph);
+  wo[i] = wo[n + i] = make_float4(w0.h, w1.h, w0.l, w1.l);
 }
 
 __global__ void __launch_bounds__(256)
@@ -1184,14 +892,15 @@ __global__ void k_df_band(int n, int b, int hard, double omega, double eta, geom
   const df re = dmake(a.x), im = dmake(a.y);
   band[e] = make_float4(re.h, re.l, im.h, im.l);
   if (hard) {
-    const df br = dmake(b2.x), bi = dmake(b2.y);
+    const double2 c = hard_combined(g, omega, eta, i, j, a, b2);
+    const df br = dmake(c.x), bi = dmake(c.y);
     band[(size_t)n * bw + e] = make_float4(br.h, br.l, bi.h, bi.l);
   }
 }
 
 unsigned nbk(size_t len, int t = 256) { return (unsigned)((len + t - 1) / t); }
 
-template <int RB>
+template <int RB, int BC>
 int launch_df(cfie_op* op, df_params P, int nrhs) {
   const int n = op->n;
   const int rowtiles = (n + DTI - 1) / DTI, slices = (nrhs + RB - 1) / RB;
@@ -1203,45 +912,22 @@ int launch_df(cfie_op* op, df_params P, int nrhs) {
   splits = (ntiles + tps - 1) / tps;
   P.splits = splits;
   P.tiles_per_split = tps;
-  op->df_part.reserve(sizeof(double2) * (size_t)splits * nrhs * n);
+  op->df_part.reserve(sizeof(double2) * (BC ? 2 : 1) * (size_t)splits * nrhs * n);
   P.part = op->df_part.as<double2>();
-  const size_t smem = sizeof(df_smem<RB>);
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_df<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-  {
-    prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
-    k_pair_df<RB><<<dim3(rowtiles, splits, slices), DNT, smem, op->ctx->stream>>>(P);
-    CFIE_CHECK_LAUNCH();
-  }
-  return splits;
-}
-
-template <int RB>
-int launch_df_hard(cfie_op* op, df_params P, const float4* x4, int nrhs) {
-  const int n = op->n;
-  const int rowtiles = (n + DTI - 1) / DTI, slices = (nrhs + RB - 1) / RB;
-  const int ntiles = (n + DTJ - 1) / DTJ;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
-  int splits = std::max(1, std::min(ntiles, (4 * sms + rowtiles * slices - 1) / (rowtiles * slices)));
-  const int tps = (ntiles + splits - 1) / splits;
-  splits = (ntiles + tps - 1) / tps;
-  P.splits = splits;
-  P.tiles_per_split = tps;
-  op->df_part.reserve(sizeof(double2) * 4 * (size_t)splits * nrhs * n);
-  P.part = op->df_part.as<double2>();
-  const size_t smem = sizeof(df_smem_hard<RB>);
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_df_hard<RB>,
+  const size_t smem = sizeof(df_smem<RB, BC>);
+  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_df<RB, BC>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   {
     prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
-    k_pair_df_hard<RB><<<dim3(rowtiles, splits, slices), DNT, smem, op->ctx->stream>>>(P, x4);
+    k_pair_df<RB, BC><<<dim3(rowtiles, splits, slices), DNT, smem, op->ctx->stream>>>(
+        P, BC ? (size_t)n * nrhs : 0);
     CFIE_CHECK_LAUNCH();
   }
   return splits;
 }
 
-template <int NB, int KIND>
+// one pass for the right-hand sides r0 .. r0 + nr - 1: y = A x, S x or x / 2 + C x
+template <int NB, int OP>
 void run_rtc(cfie_op* op, df_params P, const double2* x, double2* y, int r0, int nr) {
   constexpr int NC = 2 * NB;
   rtc_plan& T = op->rtc[NB == 16 ? 0 : (NB == 32 ? 1 : 2)];
@@ -1288,72 +974,42 @@ void run_rtc(cfie_op* op, df_params P, const double2* x, double2* y, int r0, int
   k_xslices<<<dim3((unsigned)((T.pitch + 255) / 256), NB), 256, 0, st>>>(
       n, T.pitch, NB, nr, xr, T.fx.as<int>(), T.bt.as<__nv_bfloat16>());
   CFIE_CHECK_LAUNCH();
-  const size_t tot = (size_t)n * ((nr + BRG - 1) / BRG);
-  k_band_df<<<nbk(tot), 256, 0, st>>>(n, P.b, nr, P.band, P.x + (size_t)r0 * n,
-                                      T.yb.as<double2>());
+  k_band_df<<<dim3(nbk((size_t)n * 8), (nr + BRG - 1) / BRG), 256, 0, st>>>(
+      n, P.b, nr, P.band, P.x + (size_t)r0 * n, T.yb.as<double2>());
   CFIE_CHECK_LAUNCH();
   P.fx = T.fx.as<int>();
   const size_t smem = rtc_smem_bytes<NB>();
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_resid_tc<NB, KIND>,
+  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_resid_tc<NB, OP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   char* tb = T.tables.as<char>();
   {
     prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
-    k_resid_tc<NB, KIND><<<T.grid, RNT, smem, st>>>(P, op->df_rowexp.as<int>() + (KIND == RK_DP ? n : 0),
-                                              *reinterpret_cast<const CUtensorMap*>(T.tmB),
-                                              reinterpret_cast<const int4*>(tb),
-                                              reinterpret_cast<const int*>(tb + T.o_cbeg),
-                                              T.acc.as<float2>(), T.err.as<int>());
+    k_resid_tc<NB, OP><<<T.grid, RNT, smem, st>>>(
+        P, op->df_rowexp.as<int>() + (OP == OP_C ? n : 0),
+        *reinterpret_cast<const CUtensorMap*>(T.tmB), reinterpret_cast<const int4*>(tb),
+        reinterpret_cast<const int*>(tb + T.o_cbeg), T.acc.as<float2>(), T.err.as<int>());
     CFIE_CHECK_LAUNCH();
   }
   k_reduce_rtc<<<dim3(T.mtiles, nr), RTM, 0, st>>>(n, NB, nr,
                                                   reinterpret_cast<const int2*>(tb + T.o_mts),
                                                   T.acc.as<float2>(), T.yb.as<double2>(),
-                                                  y + (size_t)r0 * n);
+                                                  OP == OP_C ? xr : nullptr, y + (size_t)r0 * n);
   CFIE_CHECK_LAUNCH();
 }
 
-template <int KIND>
+template <int OP>
 void run_rtc_block(cfie_op* op, const df_params& P, const double2* x, double2* y, int r0,
                    int nr) {
-  if (nr > 32)
-    run_rtc<64, KIND>(op, P, x, y, r0, nr);
-  else if (nr > 16)
-    run_rtc<32, KIND>(op, P, x, y, r0, nr);
+  if constexpr (OP == OP_SOFT) {
+    if (nr > 32) {
+      run_rtc<64, OP>(op, P, x, y, r0, nr);
+      return;
+    }
+  }
+  if (nr > 16)
+    run_rtc<32, OP>(op, P, x, y, r0, nr);
   else
-    run_rtc<16, KIND>(op, P, x, y, r0, nr);
-}
-
-// sound-hard inputs of the S sums, [u, n1 x, n2 x]
-__global__ void k_hard_inputs64(int n, size_t tot, const double2* __restrict__ x,
-                                const double2* __restrict__ u, geom_dev g,
-                                double2* __restrict__ v) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= tot) return;
-  const int i = (int)(e % n);
-  const double inv = 1.0 / g.sp[i];
-  const double2 xv = x[e];
-  v[e] = u[e];
-  v[tot + e] = make_double2(g.nx[i] * inv * xv.x, g.nx[i] * inv * xv.y);
-  v[2 * tot + e] = make_double2(g.ny[i] * inv * xv.x, g.ny[i] * inv * xv.y);
-}
-
-// y = x/2 - D' x - i (omega^2 / eta) (n1 S(n1 x) + n2 S(n2 x)), t = S u
-__global__ void k_hard_combine64(int n, size_t tot, double omega, double eta, geom_dev g,
-                                 const double2* __restrict__ x, const double2* __restrict__ ys,
-                                 const double2* __restrict__ yd, double2* __restrict__ t,
-                                 double2* __restrict__ y) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= tot) return;
-  const int i = (int)(e % n);
-  const double inv = 1.0 / g.sp[i];
-  const double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-  const double2 s1 = ys[tot + e], s2 = ys[2 * tot + e];
-  const double2 m = make_double2(n1 * s1.x + n2 * s2.x, n1 * s1.y + n2 * s2.y);
-  const double k = omega * omega / eta;
-  const double2 xv = x[e], d = yd[e];
-  y[e] = make_double2(0.5 * xv.x - d.x + k * m.y, 0.5 * xv.y - d.y - k * m.x);
-  t[e] = ys[e];
+    run_rtc<16, OP>(op, P, x, y, r0, nr);
 }
 
 std::mutex g_df_mu;
@@ -1415,15 +1071,15 @@ void df_prepare(cfie_op* op) {
     return;
   }
   op->df_b = b;
-  op->df_geo.reserve((sizeof(float4) * 3 + sizeof(float2) * 3) * (size_t)n);
+  op->df_geo.reserve(sizeof(float4) * ((size_t)8 * n + kDfTab));
   const int hard = op->bc == CFIE_SOUND_HARD ? 1 : 0;
   op->df_band.reserve(sizeof(float4) * (size_t)n * bw * (hard ? 2 : 1));
-  char* base = op->df_geo.as<char>();
-  const size_t f4 = sizeof(float4) * n, f2 = sizeof(float2) * n;
-  k_df_geo<<<nbk(n), 256, 0, st>>>(n, op->g, op->wtab.as<double>(), op->omega, op->eta, op->h,
-                                    (float4*)base, (float4*)(base + f4), (float4*)(base + 2 * f4),
-                                    (float2*)(base + 3 * f4), (float2*)(base + 3 * f4 + f2),
-                                    (float2*)(base + 3 * f4 + 2 * f2));
+  float4* g4 = op->df_geo.as<float4>();
+  const unsigned* bound =
+      reinterpret_cast<const unsigned*>(op->geo32.as<float>() + geo32_bound_offset(n));
+  k_df_geo<<<nbk((size_t)n + kDfTab), 256, 0, st>>>(
+      n, op->g, op->wtab.as<double>(), op->omega, op->eta, op->h, hard, bound, g4, g4 + 2 * (size_t)n,
+      g4 + 3 * (size_t)n, g4 + 6 * (size_t)n, g4 + 8 * (size_t)n);
   CFIE_CHECK_LAUNCH();
   k_df_band<<<nbk((size_t)n * bw), 256, 0, st>>>(n, b, hard, op->omega, op->eta, op->g,
                                                   op->wtab.as<double>(), op->diag.as<double2>(),
@@ -1434,14 +1090,20 @@ void df_prepare(cfie_op* op) {
     float* base = op->geo32.as<float>();
     const float4* pk = reinterpret_cast<const float4*>(base + geo32_pack_offset(n));
     const float2* wkt = reinterpret_cast<const float2*>(base + geo32_wk_offset(n));
-    const unsigned g = (unsigned)((n + 63) / 64);
-    if (hard) {
-      k_rowexp<RK_S><<<g, 256, 0, st>>>(n, b, pk, wkt, op->df_rowexp.as<int>());
-      CFIE_CHECK_LAUNCH();
-      k_rowexp<RK_DP><<<g, 256, 0, st>>>(n, b, pk, wkt, op->df_rowexp.as<int>() + n);
-    } else {
-      k_rowexp<RK_SOFT><<<g, 256, 0, st>>>(n, b, pk, wkt, op->df_rowexp.as<int>());
-    }
+    const float4* spk = reinterpret_cast<const float4*>(base + geo32_pair_offset(n));
+    unsigned* rmax = reinterpret_cast<unsigned*>(op->df_rowexp.as<int>());
+    const int len = n * (hard ? 2 : 1);
+    CFIE_CHECK_CUDA(cudaMemsetAsync(rmax, 0, sizeof(unsigned) * len, st));
+    // sources split so that the grid covers the SMs a few times
+    const int rows = (n + 63) / 64;
+    const int per = std::max(64, ((n + 1216 / rows) / (1216 / rows + 1) + 7) / 8 * 8);
+    const dim3 g(rows, (n + per - 1) / per);
+    if (hard)
+      k_rowmax<OP_SC><<<g, 256, 0, st>>>(n, b, per, pk, spk, wkt, rmax);
+    else
+      k_rowmax<OP_SOFT><<<g, 256, 0, st>>>(n, b, per, pk, spk, wkt, rmax);
+    CFIE_CHECK_LAUNCH();
+    k_rowexp<<<nbk(len), 256, 0, st>>>(len, rmax);
     CFIE_CHECK_LAUNCH();
   }
   CFIE_CHECK_CUDA(cudaStreamSynchronize(st));
@@ -1472,98 +1134,64 @@ void matvec_df(cfie_op* op, const double2* x, double2* y, int nrhs) {
   P.n = n;
   P.b = op->df_b;
   P.nrhs = nrhs;
-  char* base = op->df_geo.as<char>();
-  const size_t f4 = sizeof(float4) * n, f2 = sizeof(float2) * n;
-  P.g = (const float4*)base;
-  P.sqa = (const float4*)(base + f4);
-  P.tq = (const float4*)(base + 2 * f4);
-  P.sqe = (const float2*)(base + 3 * f4);
-  P.sqs = (const float2*)(base + 3 * f4 + f2);
-  P.w = (const float2*)(base + 3 * f4 + 2 * f2);
+  const float4* g4 = op->df_geo.as<float4>();
+  P.g = df_nodes{g4, g4 + 2 * (size_t)n, g4 + 3 * (size_t)n, g4 + 6 * (size_t)n,
+                 g4 + 8 * (size_t)n};
   P.band = op->df_band.as<float4>();
   const size_t tot = (size_t)n * nrhs;
-  if (op->bc == CFIE_SOUND_HARD && (op->res_variant == 2 || (op->res_variant == 0 && nrhs >= 8))) {
-    // S on [u, n1 x, n2 x] and D' on x with the sliced tensor-core sums
-    op->stats.residual_variant = 2;
-    cudaStream_t st = op->ctx->stream;
+  cudaStream_t st = op->ctx->stream;
+  const bool hard = op->bc == CFIE_SOUND_HARD;
+  const bool tc = op->res_variant == 2 || (op->res_variant == 0 && nrhs >= 8);
+  double2 *u = nullptr, *t = nullptr;
+  op->df_x.reserve(sizeof(float4) * tot * (hard ? 2 : 1));
+  float4* xv = op->df_x.as<float4>();
+  P.x = xv;
+  if (hard) {   // S on u = d/ds x, then C on x
     op->tmp1.reserve(sizeof(double2) * tot);
     op->tmp2.reserve(sizeof(double2) * tot);
-    double2* u = op->tmp1.as<double2>();
-    double2* t = op->tmp2.as<double2>();
+    u = op->tmp1.as<double2>();
+    t = op->tmp2.as<double2>();
     spectral_apply(op, x, u, nullptr, make_double2(1.0, 0.0), nrhs);
-    op->tcv.reserve(sizeof(double2) * tot * 4);
-    double2* v = op->tcv.as<double2>();
-    op->tcs.reserve(sizeof(double2) * tot * 4);
-    double2* ys = op->tcs.as<double2>();
-    k_hard_inputs64<<<nbk(tot), 256, 0, st>>>(n, tot, x, u, op->g, v);
+    k_df_x<<<nbk(tot), 256, 0, st>>>(tot, u, xv);
     CFIE_CHECK_LAUNCH();
-    op->df_x.reserve(sizeof(float4) * tot * 4);
-    float4* xv = op->df_x.as<float4>();
-    k_df_x<<<nbk(3 * tot), 256, 0, st>>>(3 * tot, v, xv);
-    CFIE_CHECK_LAUNCH();
-    k_df_x<<<nbk(tot), 256, 0, st>>>(tot, x, xv + 3 * tot);
-    CFIE_CHECK_LAUNCH();
-    const size_t nbw = (size_t)n * (2 * (size_t)P.b + 1);
-    df_params PS = P, PD = P;
-    PS.x = xv;
-    PD.x = xv + 3 * tot;
-    PD.band = P.band + nbw;
+  }
+  k_df_x<<<nbk(tot), 256, 0, st>>>(tot, x, hard ? xv + tot : xv);
+  CFIE_CHECK_LAUNCH();
+  if (tc) {
+    op->stats.residual_variant = 2;
+    if (!hard) {
+      for (int r0 = 0; r0 < nrhs; r0 += 64)
+        run_rtc_block<OP_SOFT>(op, P, x, y, r0, std::min(64, nrhs - r0));
+      return;
+    }
+    df_params PC = P;
+    PC.x = xv + tot;
+    PC.band = P.band + (size_t)n * (2 * (size_t)P.b + 1);
     // passes of at most 32 right-hand sides, whose tensor memory holds an
     // exact accumulator for every level up to L = 5: the hypersingular part
     // magnifies the rounding of the shared L >= 5 accumulator of 64-wide
     // passes to ~1e-11 relative (sound soft: ~1e-12)
-    for (int r0 = 0; r0 < 3 * nrhs; r0 += 32)
-      run_rtc_block<RK_S>(op, PS, v, ys, r0, std::min(32, 3 * nrhs - r0));
-    for (int r0 = 0; r0 < nrhs; r0 += 32)
-      run_rtc_block<RK_DP>(op, PD, x, ys + 3 * tot, r0, std::min(32, nrhs - r0));
-    k_hard_combine64<<<nbk(tot), 256, 0, st>>>(n, tot, op->omega, op->eta, op->g, x, ys,
-                                               ys + 3 * tot, t, y);
-    CFIE_CHECK_LAUNCH();
-    spectral_apply(op, t, y, y, make_double2(0.0, -1.0 / op->eta), nrhs);
-    return;
-  }
-  if (op->bc == CFIE_SOUND_HARD) {
-    // y = x/2 - D' x + (1/(i eta)) [d/ds S d/ds x + omega^2 sum_c n_c S (n_c x)]
-    op->tmp1.reserve(sizeof(double2) * tot);
-    op->tmp2.reserve(sizeof(double2) * tot);
-    double2* u = op->tmp1.as<double2>();
-    double2* t = op->tmp2.as<double2>();
-    spectral_apply(op, x, u, nullptr, make_double2(1.0, 0.0), nrhs);
-    op->df_x.reserve(sizeof(float4) * 4 * tot);
-    k_df_x_hard<<<nbk(tot), 256, 0, op->ctx->stream>>>(n, tot, x, u, op->g,
-                                                        op->df_x.as<float4>());
-    CFIE_CHECK_LAUNCH();
-    const float4* x4 = op->df_x.as<float4>();
-    const int splits = nrhs > 4 ? launch_df_hard<16>(op, P, x4, nrhs)
-                                : launch_df_hard<4>(op, P, x4, nrhs);
-    reduce_hard_fp64(op, op->df_part.as<double2>(), splits, x, t, y, nrhs);
-    spectral_apply(op, t, y, y, make_double2(0.0, -1.0 / op->eta), nrhs);
-    return;
-  }
-  op->df_x.reserve(sizeof(float4) * tot);
-  k_df_x<<<nbk(tot), 256, 0, op->ctx->stream>>>(tot, x, op->df_x.as<float4>());
-  CFIE_CHECK_LAUNCH();
-  P.x = op->df_x.as<float4>();
-  if (op->res_variant == 2 || (op->res_variant == 0 && nrhs >= 8)) {
-    op->stats.residual_variant = 2;
-    for (int r0 = 0; r0 < nrhs; r0 += 64) {
-      const int nr = std::min(64, nrhs - r0);
-      run_rtc_block<RK_SOFT>(op, P, x, y, r0, nr);
+    for (int r0 = 0; r0 < nrhs; r0 += 32) {
+      run_rtc_block<OP_S>(op, P, u, t, r0, std::min(32, nrhs - r0));
+      run_rtc_block<OP_C>(op, PC, x, y, r0, std::min(32, nrhs - r0));
     }
-    return;
-  }
-  int splits;
-  if (nrhs > 32) {
-    // 64 right-hand sides per CTA (one pass of entries, one CTA per SM) or 32
-    // (entries evaluated twice, two CTAs per SM): timed once per (n, nrhs)
-    const int rb = df_tile_choice(op, n, nrhs, [&](int c) {
-      return c == 64 ? launch_df<64>(op, P, nrhs) : launch_df<32>(op, P, nrhs);
-    });
-    splits = rb == 64 ? launch_df<64>(op, P, nrhs) : launch_df<32>(op, P, nrhs);
   } else {
-    splits = nrhs > 16 ? launch_df<32>(op, P, nrhs) : launch_df<16>(op, P, nrhs);
+    int splits;
+    if (hard) {
+      splits = nrhs > 4 ? launch_df<16, 1>(op, P, nrhs) : launch_df<4, 1>(op, P, nrhs);
+    } else if (nrhs > 32) {
+      // 64 right-hand sides per CTA (one pass of entries, one CTA per SM) or 32
+      // (entries evaluated twice, two CTAs per SM): timed once per (n, nrhs)
+      const int rb = df_tile_choice(op, n, nrhs, [&](int c) {
+        return c == 64 ? launch_df<64, 0>(op, P, nrhs) : launch_df<32, 0>(op, P, nrhs);
+      });
+      splits = rb == 64 ? launch_df<64, 0>(op, P, nrhs) : launch_df<32, 0>(op, P, nrhs);
+    } else if (nrhs > 4) {
+      splits = nrhs > 16 ? launch_df<32, 0>(op, P, nrhs) : launch_df<16, 0>(op, P, nrhs);
+    } else {
+      splits = launch_df<4, 0>(op, P, nrhs);
+    }
+    reduce_fp64(op, op->df_part.as<double2>(), splits, x, t, y, nrhs);
   }
-  k_reduce_df<<<nbk(tot), 256, 0, op->ctx->stream>>>(n, nrhs, splits, op->df_part.as<double2>(),
-                                                      y);
-  CFIE_CHECK_LAUNCH();
+  if (hard) spectral_apply(op, t, y, y, make_double2(0.0, -1.0 / op->eta), nrhs);
 }

@@ -49,7 +49,7 @@ struct pair_params : omega32 {
   geo32 g;
   const float* w32;
   const float2* band;    // soft: A ; hard: S
-  const float2* band2;   // hard: D'
+  const float2* band2;   // hard: C
   const float2* xin;     // [k][j] complex64 (hard: x)
   const float2* uin;     // hard: (1/s) Dt x
   float k2;              // hard: omega^2 / eta
@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
       const int il = warp + 8 * q;
       const int i = i0 + il;
       float2 a = make_float2(0.f, 0.f), b = a;
+      bool near = false;
       if (i < n && jok) {
         int d = i - j;
         if (d < 0) d += n;
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
         if (dd != INT_MAX) {
           a = P.band[(size_t)i * bw + dd + P.b];
           if (BC) b = P.band2[(size_t)i * bw + dd + P.b];
+          near = true;
         } else {
           pair_entries_fp32<BC>(P, S.txh[il], S.txl[il], S.tyh[il], S.tyl[il], S.tnx[il],
                                 S.tny[il], S.tsp[il], sxh, sxl, syh, syl, snx, sny, ssp,
@@ -154,9 +156,9 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
       }
       S.A[lane][il] = a;
       if constexpr (BC == 1) {
-        // C = -D' - i (omega^2 / eta) (n_i . n_j) S
+        // C = -D' - i (omega^2 / eta) (n_i . n_j) S (the band holds it)
         const float kn = P.k2 / S.tsp[il] * fmaf(S.tnx[il], sux, S.tny[il] * suy);
-        S.B[lane][il] = make_float2(fmaf(kn, a.y, -b.x), -fmaf(kn, a.x, b.y));
+        S.B[lane][il] = near ? b : make_float2(fmaf(kn, a.y, -b.x), -fmaf(kn, a.x, b.y));
       }
     }
     __syncthreads();
@@ -407,7 +409,7 @@ k_band_scan(int n, double omega, geom_dev g, int* __restrict__ bmax, float* __re
 
 // FP32 band entries (offsets |dd| <= b) from the double-float band of width
 // bd >= b: the high parts (the FP32 rounding of the FP64 entries); `ops`
-// bands of each kind (sound hard: S, then D')
+// bands of each kind (sound hard: S, then C)
 __global__ void k_band_from_df(int n, int b, int bd, int ops, const float4* __restrict__ dfb,
                                float2* __restrict__ band) {
   const int bw = 2 * b + 1, bwd = 2 * bd + 1;
@@ -449,7 +451,10 @@ __global__ void k_band_fill(int n, int b, double omega, double eta, geom_dev g,
                           g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, bb);
   }
   band[e] = make_float2((float)a.x, (float)a.y);
-  if (BC) band2[e] = make_float2((float)bb.x, (float)bb.y);
+  if (BC) {
+    const double2 c = hard_combined(g, omega, eta, i, j, a, bb);
+    band2[e] = make_float2((float)c.x, (float)c.y);
+  }
 }
 
 unsigned nblk(size_t len, int t = 256) { return (unsigned)((len + t - 1) / t); }
@@ -527,7 +532,7 @@ void fp32_prepare(cfie_op* op) {
   geo32 o{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n, base + 6 * n};
   float* w32 = base + 7 * n;
   float* c32 = base + 8 * n;
-  unsigned* bound = reinterpret_cast<unsigned*>(scan.as<int>() + 2);
+  unsigned* bound = reinterpret_cast<unsigned*>(base + geo32_bound_offset(n));
   CFIE_CHECK_CUDA(cudaMemsetAsync(bound, 0, sizeof(unsigned), st));
   k_coord_bound<<<nblk(n), 256, 0, st>>>(n, op->g, bound);
   CFIE_CHECK_LAUNCH();

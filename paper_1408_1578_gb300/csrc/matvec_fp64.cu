@@ -260,36 +260,6 @@ k_reduce_fp64(size_t tot, int splits, const double2* __restrict__ part,
   }
 }
 
-// Sum split partials of the double-float sums (matvec_df.cu; four outputs):
-// t = S u, y = 1/2 x - D' x - i (omega^2 / eta) (n1 S(n1 x) + n2 S(n2 x)).
-__global__ void k_reduce_hard4(int n, int nrhs, int splits, double omega, double eta, geom_dev g,
-                               const double2* __restrict__ part, const double2* __restrict__ x,
-                               double2* __restrict__ t_out, double2* __restrict__ y) {
-  size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t tot = (size_t)n * nrhs;
-  if (e >= tot) return;
-  const size_t stride_o = (size_t)splits * tot;
-  double2 s[4] = {};
-  for (int o = 0; o < 4; ++o) {
-    double2 v = make_double2(0.0, 0.0);
-    for (int sp = 0; sp < splits; ++sp) {
-      double2 p = part[o * stride_o + (size_t)sp * tot + e];
-      v.x += p.x;
-      v.y += p.y;
-    }
-    s[o] = v;
-  }
-  int i = (int)(e % n);
-  double inv = 1.0 / g.sp[i];
-  double n1 = g.nx[i] * inv, n2 = g.ny[i] * inv;
-  double2 m = make_double2(n1 * s[1].x + n2 * s[2].x, n1 * s[1].y + n2 * s[2].y);
-  double k = omega * omega / eta;
-  double2 xv = x[e];
-  // -i k m = (k m.y, -k m.x)
-  y[e] = make_double2(0.5 * xv.x - s[3].x + k * m.y, 0.5 * xv.y - s[3].y - k * m.x);
-  t_out[e] = s[0];
-}
-
 // out[k][i] = base[k][i] + (scale / s_i) sum_j c_{(i-j) mod n} in[k][j]
 // (spectral derivative as a circulant; c_d = (-1)^d cot(pi d / n) / 2)
 constexpr int SPT = 256;
@@ -397,10 +367,7 @@ void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* 
     default:
       launch_pair<BC, 64, BC ? 32 : 64>(op, p, x, u, nrhs, part);
   }
-  const size_t tot = (size_t)op->n * nrhs;
-  k_reduce_fp64<BC><<<(unsigned)((tot + 63) / 64), 256, 0, op->ctx->stream>>>(tot, p.splits, part,
-                                                                             x, t, y);
-  CFIE_CHECK_LAUNCH();
+  reduce_fp64(op, part, p.splits, x, t, y, nrhs);
 }
 
 }  // namespace
@@ -412,11 +379,14 @@ void spectral_apply(cfie_op* op, const double2* in, double2* out, const double2*
   spectral_fft64(op, in, out, base, scale, nrhs);
 }
 
-void reduce_hard_fp64(cfie_op* op, const double2* part, int splits, const double2* x,
-                      double2* t, double2* y, int nrhs) {
+void reduce_fp64(cfie_op* op, const double2* part, int splits, const double2* x, double2* t,
+                 double2* y, int nrhs) {
   const size_t tot = (size_t)op->n * nrhs;
-  k_reduce_hard4<<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(
-      op->n, nrhs, splits, op->omega, op->eta, op->g, part, x, t, y);
+  const unsigned blocks = (unsigned)((tot + 63) / 64);
+  if (op->bc == CFIE_SOUND_HARD)
+    k_reduce_fp64<1><<<blocks, 256, 0, op->ctx->stream>>>(tot, splits, part, x, t, y);
+  else
+    k_reduce_fp64<0><<<blocks, 256, 0, op->ctx->stream>>>(tot, splits, part, x, t, y);
   CFIE_CHECK_LAUNCH();
 }
 

@@ -80,7 +80,7 @@ struct tc_params {
   const float2* wext;    // Kress table / (pi h) at i - j + n, paired with the next source's
   const float4* pk;      // packed coordinates, source factors, target factors (n each)
   const float4* spk;     // source coordinates by pairs, source factors by pairs (n each)
-  const float2* band;    // near entries: soft A, or S, then D'
+  const float2* band;    // near entries: soft A, or S, then C
 };
 
 // bf16 hi / lo split of eight entries of one row (adjacent sources): the packed
@@ -136,12 +136,7 @@ __device__ __forceinline__ entry_pair near_pair(const tc_params& P, float4 t0, f
     const float2 bv = P.band[at];                    // soft A, or S
     float2 s = bv, c = f2(0.f);
     if constexpr (OP != OP_SOFT) s = make_float2(bv.y, -bv.x);   // S' = -i S
-    if constexpr (OP == OP_C || OP == OP_SC) {
-      // C = -D' + (omega^2 / eta) (n_i . n_j) S'
-      const float2 dp = P.band[(size_t)n * bw + at];
-      const float kn = tn.x * (u ? g0.y : g0.x) + tn.z * (u ? g0.w : g0.z);
-      c = make_float2(fmaf(kn, s.x, -dp.x), fmaf(kn, s.y, -dp.y));
-    }
+    if constexpr (OP == OP_C || OP == OP_SC) c = P.band[(size_t)n * bw + at];
     const float2 first = OP == OP_C ? c : s;
     if (u) {
       e.re.y = first.x, e.im.y = first.y;

@@ -33,6 +33,9 @@ inline size_t geo32_pair_offset(int n) {
 // (+ 256 floats of slack: the fused kernel copies whole 32-source tiles)
 inline size_t geo32_floats(int n) { return geo32_pair_offset(n) + (size_t)8 * n + 256; }
 
+// the last float: bit pattern of the largest |x|, |y| over the nodes
+inline size_t geo32_bound_offset(int n) { return geo32_floats(n) - 1; }
+
 inline geo32 geo32_at(float* base, int n) {
   return geo32{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n,
                base + 6 * n};
