@@ -220,9 +220,11 @@ __global__ void __launch_bounds__(DNT) k_pair_df(df_params P, size_t xstride) {
 //
 // Bound: the producers' FP32 arithmetic, about 340 operations per pair (290 for
 // the entry, 52 for the slices), issued in packed pairs.  Measured (GB300): kite
-// n = 32768, 64 right-hand sides 27.4 -> 18.1 ms (710 -> 380 instructions per
+// n = 32768, 64 right-hand sides 27.4 -> 16.8 ms (710 -> 340 instructions per
 // pair); star n = 4096, 16, sound hard: 1.88 -> 0.76 ms (two passes instead of
-// three, the band sums 0.77 -> 0.1 ms).
+// three, the band sums 0.77 -> 0.1 ms).  The drain (one pass over the accumulators
+// per 128 sources, 40 operations per element) in packed pairs of columns: 18.1 ->
+// 16.8 ms.
 // ---------------------------------------------------------------------------
 constexpr int RTM = 128;      // rows per tile (UMMA M)
 constexpr int RTK = 16;       // sources per tile: one K step, 32-byte rows
@@ -370,43 +372,38 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
         const uint32_t base = tmem + ((uint32_t)(32 * qd) << 16);
 #pragma unroll 1
         for (int cb = cg0; cb < cg0 + CPG; cb += 8) {
-          // eight columns at a time: the small levels (L >= 4) first, as one
-          // double-float (L = 4 exact, plus the rest), then L = 2, 3 exactly;
-          // the two are joined in double-float, so nothing of the exact level
-          // sums is rounded away at FP32 precision
-          float t[8], te[8], v0[8], v1[8];
-          tmem_ld8(base + (uint32_t)(3 * NC + cb), t);
+          // eight columns at a time, two per packed pair: the small levels (L >=
+          // 4) as one double-float (L = 4 exact, plus the rest), then L = 2, 3
+          // exactly; the two are joined in double-float, so nothing of the
+          // exact level sums is rounded away at FP32 precision
+          float v0[8], v1[8], v2[8], v3[8];
+          tmem_ld8(base + (uint32_t)(3 * NC + cb), v3);
           if constexpr (NL == 5) {
             tmem_ld8(base + (uint32_t)(4 * NC + cb), v0);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) t[r] += v0[r];
+            for (int r = 0; r < 8; ++r) v3[r] += v0[r];
           }
-          tmem_ld8(base + (uint32_t)(2 * NC + cb), v0);
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const float s2 = v0[r] + t[r];
-            const float b2 = s2 - v0[r];
-            te[r] = (v0[r] - (s2 - b2)) + (t[r] - b2);
-            t[r] = s2;
-          }
+          tmem_ld8(base + (uint32_t)(2 * NC + cb), v2);
           tmem_ld8(base + (uint32_t)(0 * NC + cb), v0);
           tmem_ld8(base + (uint32_t)(1 * NC + cb), v1);
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
+          for (int r = 0; r < 8; r += 2) {
             const int col = cb + r;
-            const float sh = v0[r] + v1[r];
-            const float bv = sh - v0[r];
-            const float sl = (v0[r] - (sh - bv)) + (v1[r] - bv);
-            const float fs = __int_as_float((127 + P.fx[col]) << 23);  // 2^F_col
-            df val = dadd(quick(sh, sl), df{t[r], te[r]});
-            val.h *= rs * fs;
-            val.l *= rs * fs;
+            const float2 fs = make_float2(__int_as_float((127 + P.fx[col]) << 23),     // 2^F_col
+                                          __int_as_float((127 + P.fx[col + 1]) << 23));
+            const d2 lo = two_sum(make_float2(v2[r], v2[r + 1]), make_float2(v3[r], v3[r + 1]));
+            const d2 hi = two_sum(make_float2(v0[r], v0[r + 1]), make_float2(v1[r], v1[r + 1]));
+            d2 val = dd_norm(dd_add(dd_norm(hi), lo));
+            const float2 sc2 = mul2(f2(rs), fs);
+            val.h = mul2(val.h, sc2);
+            val.l = mul2(val.l, sc2);
             float2* pp = dst + (size_t)col * RTM;
             if (!first) {
-              const float2 o = *pp;
-              val = dadd(val, df{o.x, o.y});
+              const float2 o0 = pp[0], o1 = pp[RTM];
+              val = dd_norm(dd_add(val, {make_float2(o0.x, o1.x), make_float2(o0.y, o1.y)}));
             }
-            *pp = make_float2(val.h, val.l);
+            pp[0] = make_float2(val.h.x, val.l.x);
+            pp[RTM] = make_float2(val.h.y, val.l.y);
           }
         }
       }
@@ -453,7 +450,7 @@ k_resid_tc(df_params P, const int* __restrict__ rowexp, const __grid_constant__ 
         for (int t = -1; t <= 1; ++t)
           plain &= m0 + RTM - 1 - j0 < t * n - P.b || m0 - j0 - (RTK - 1) > t * n + P.b;
         unsigned char* A = reinterpret_cast<unsigned char*>(&S.A[st][0][0]) + off;
-#pragma unroll 1
+#pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int j = j0 + js + 2 * u;
           const bool in = plain || (i < n && j < n);     // n is even: j + 1 < n as well
