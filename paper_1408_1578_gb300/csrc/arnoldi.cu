@@ -18,20 +18,31 @@
 // n x nrhs layout of the C ABI; for a batch of operators the blocks of all
 // operators are concatenated.  Basis vector j of every problem is the slice
 // V[j * L .. (j + 1) * L), so the matvec reads it directly.  The chunked kernels
-// run over a work list of (problem, 2048-element chunk) items and stream V once
-// per pass (HBM-bound); per-problem quantities (H, Givens data, norms) are
-// reduced from per-chunk partial sums in a fixed order.
+// run over a work list of (problem, chunk) items and stream V once per pass;
+// per-problem quantities (H, Givens data, norms) are reduced from per-chunk
+// partial sums in a fixed order by the problem's last CTA to finish.
+//
+// Bound: HBM (or L2, when the basis fits) for large sets, latency for small
+// ones.  The chunk length (128 to 2048 elements) is chosen so that the set has
+// about two CTAs per SM, the inner products of a small set are also split over
+// the basis vectors, loads of four basis vectors are in flight at once, the four
+// pairs of sums are reduced across a warp together (9 shuffles instead of 40;
+// on GB300 the FP64 additions of a plain reduction cost more than the products),
+// and an Arnoldi step is 5 launches instead of 9.  Measured (GB300): unrestarted
+// FP64 solve of n = 1024, 30 steps, 15.2 -> 9.1 ms (490 -> 290 us a step, 227 of
+// them the matvec); kite n = 8192, 64 directions, 88 steps, 34.2 -> 30.4 ms.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
+#include "hankel64.cuh"
 #include "internal.h"
 
 namespace {
 
-constexpr int AT = 256;          // threads per CTA
-constexpr int AE = 8;            // elements per thread
-constexpr int CH = AT * AE;      // elements per chunk
+constexpr int AT = 256;          // threads per CTA at most
+constexpr int AB = 4;            // basis vectors in flight
 constexpr int MAXJ = 512;        // largest restart length
 
 template <typename S>
@@ -64,165 +75,170 @@ __device__ __forceinline__ chunk_ref chunk_of(const pset_dev& ps, int item) {
   const int2 it = ps.items[item];
   chunk_ref r;
   r.p = it.x;
-  r.base = ps.off[it.x] + (size_t)it.y * CH;
-  r.cnt = min(CH, ps.len[it.x] - it.y * CH);
+  r.base = ps.off[it.x] + (size_t)it.y * ps.ch;
+  r.cnt = min(ps.ch, ps.len[it.x] - it.y * ps.ch);
   r.slot = ps.chb[it.x] + it.y;
   return r;
 }
 
-// partial[slot][jj] = sum over the chunk of conj(V[jj]) w, jj = 0..J
-// (products and the in-chunk sums in the basis precision, chunk partials FP64)
-template <typename T>
-__global__ void __launch_bounds__(AT)
-k_dots(int J, const T* __restrict__ V, size_t L, const T* __restrict__ w,
-       const int* __restrict__ act, pset_dev ps, double2* __restrict__ partial) {
-  using S = typename basis_t<T>::S;
-  extern __shared__ double2 red[];  // [J+1][AT/32]
-  const chunk_ref c = chunk_of(ps, blockIdx.x);
-  if (!act[c.p]) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T wr[AE];
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    wr[e] = q < c.cnt ? w[c.base + q] : basis_t<T>::make(0.0, 0.0);
-  }
-  for (int jj = 0; jj <= J; ++jj) {
-    const T* v = V + (size_t)jj * L + c.base;
-    S re = 0, im = 0;
-#pragma unroll
-    for (int e = 0; e < AE; ++e) {
-      const int q = e * AT + threadIdx.x;
-      if (q < c.cnt) {
-        const T a = v[q];
-        re = fma(a.x, wr[e].x, fma(a.y, wr[e].y, re));
-        im = fma(a.x, wr[e].y, fma(-a.y, wr[e].x, im));
-      }
-    }
-    re = warp_sum(re);
-    im = warp_sum(im);
-    if (lane == 0) red[jj * (AT / 32) + warp] = make_double2((double)re, (double)im);
-  }
-  __syncthreads();
-  for (int jj = threadIdx.x; jj <= J; jj += AT) {
-    double2 s = make_double2(0.0, 0.0);
-    for (int q = 0; q < AT / 32; ++q) {
-      s.x += red[jj * (AT / 32) + q].x;
-      s.y += red[jj * (AT / 32) + q].y;
-    }
-    partial[(size_t)c.slot * (J + 1) + jj] = s;
-  }
+// two adjacent elements (segments and chunks have even lengths and offsets)
+template <typename T> struct two { T a, b; };
+__device__ __forceinline__ two<float2> load2(const float2* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ two<double2> load2(const double2* p) { return {p[0], p[1]}; }
+__device__ __forceinline__ void store2(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void store2(double2* p, double2 a, double2 b) {
+  p[0] = a;
+  p[1] = b;
 }
 
-// h[p][jj] = sum over the problem's chunks; H[p][jj][col] = (first) or += h
-__global__ void k_dots_reduce(int J, int m, int col, int first, const int* __restrict__ act,
-                              pset_dev ps, const double2* __restrict__ partial,
-                              double2* __restrict__ hbuf, double2* __restrict__ H) {
-  const int p = blockIdx.x;
-  if (!act[p]) return;
-  const int nch = ps.nch[p], chb = ps.chb[p];
+// Whether this CTA is the last of the problem's `total` to get here; all its
+// earlier writes, and those of the others, are then visible to it.  The counter
+// is left at zero.
+__device__ __forceinline__ bool last_cta(int* counter, int total) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1) == total - 1;
+    if (last) *counter = 0;
+  }
+  __syncthreads();
+  __threadfence();
+  return last != 0;
+}
+
+// h[p][jj] = V[jj]^H w, jj = 0..J: CTA (item, y) the vectors y JB .. of one chunk
+// (products and the in-chunk sums in the basis precision, chunk partials FP64);
+// the problem's last CTA adds the chunks and H[p][jj][col] = (first) or += h
+template <typename T, int PT>
+__global__ void __launch_bounds__(AT)
+k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t L,
+       const T* __restrict__ w, const int* __restrict__ act, pset_dev ps,
+       double2* __restrict__ partial, int* __restrict__ counter, double2* __restrict__ hbuf,
+       double2* __restrict__ H) {
+  using S = typename basis_t<T>::S;
+  extern __shared__ double2 red[];  // [JB][warps]
+  const chunk_ref c = chunk_of(ps, blockIdx.x);
+  if (!act[c.p]) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int j0 = blockIdx.y * JB, j1 = min(J + 1, j0 + JB);
+  two<T> wr[PT];
+#pragma unroll
+  for (int e = 0; e < PT; ++e) {
+    const int q = 2 * (e * blockDim.x + threadIdx.x);
+    wr[e].a = wr[e].b = basis_t<T>::make(0.0, 0.0);
+    if (q < c.cnt) wr[e] = load2(w + c.base + q);
+  }
+  for (int jj = j0; jj < j1; jj += AB) {
+    two<T> v[AB][PT];
+#pragma unroll
+    for (int b = 0; b < AB; ++b)
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const int q = 2 * (e * blockDim.x + threadIdx.x);
+        v[b][e].a = v[b][e].b = basis_t<T>::make(0.0, 0.0);
+        if (q < c.cnt && jj + b < j1) v[b][e] = load2(V + (size_t)(jj + b) * L + c.base + q);
+      }
+    S s[2 * AB];
+#pragma unroll
+    for (int b = 0; b < AB; ++b) {
+      S re = 0, im = 0;
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const two<T> a = v[b][e];
+        re = fma(a.a.x, wr[e].a.x, fma(a.a.y, wr[e].a.y, re));
+        im = fma(a.a.x, wr[e].a.y, fma(-a.a.y, wr[e].a.x, im));
+        re = fma(a.b.x, wr[e].b.x, fma(a.b.y, wr[e].b.y, re));
+        im = fma(a.b.x, wr[e].b.y, fma(-a.b.y, wr[e].b.x, im));
+      }
+      s[2 * b] = re;
+      s[2 * b + 1] = im;
+    }
+    // the 2 AB = 8 sums across the warp: halve the values and double the lanes
+    // per value three times, then two plain steps; value `idx` ends in the four
+    // lanes of its group
+#pragma unroll
+    for (int n = AB, o = 16; n >= 1; n /= 2, o /= 2) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        const S mine = up ? s[k + n] : s[k];
+        const S other = up ? s[k] : s[k + n];
+        s[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    }
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+    const int idx = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+    if ((lane & 3) == 0 && jj + (idx >> 1) < j1) {
+      double* d = reinterpret_cast<double*>(red + (size_t)(jj - j0 + (idx >> 1)) * warps + warp);
+      d[idx & 1] = (double)s[0];
+    }
+  }
+  __syncthreads();
+  for (int jj = j0 + threadIdx.x; jj < j1; jj += blockDim.x) {
+    double2 t = make_double2(0.0, 0.0);
+    for (int q = 0; q < warps; ++q) {
+      t.x += red[(size_t)(jj - j0) * warps + q].x;
+      t.y += red[(size_t)(jj - j0) * warps + q].y;
+    }
+    partial[(size_t)c.slot * (J + 1) + jj] = t;
+  }
+  const int nch = ps.nch[c.p], chb = ps.chb[c.p];
+  if (!last_cta(counter + c.p, nch * gridDim.y)) return;
   for (int jj = threadIdx.x; jj <= J; jj += blockDim.x) {
-    double2 s = make_double2(0.0, 0.0);
-    for (int c = 0; c < nch; ++c) {
-      const double2 v = partial[(size_t)(chb + c) * (J + 1) + jj];
-      s.x += v.x;
-      s.y += v.y;
+    double2 t = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int k = 0; k < nch; ++k) {
+      const double2 v = __ldcg(partial + (size_t)(chb + k) * (J + 1) + jj);
+      t.x += v.x;
+      t.y += v.y;
     }
-    hbuf[(size_t)p * (J + 1) + jj] = s;
-    double2* hk = H + ((size_t)p * (m + 1) + jj) * m + col;
+    hbuf[(size_t)c.p * (J + 1) + jj] = t;
+    double2* hk = H + ((size_t)c.p * (m + 1) + jj) * m + col;
     if (first) {
-      *hk = s;
+      *hk = t;
     } else {
-      hk->x += s.x;
-      hk->y += s.y;
+      hk->x += t.x;
+      hk->y += t.y;
     }
   }
 }
 
-// w -= sum_jj V[jj] h[p][jj] on one chunk; optional |w|^2 partial per chunk
-template <typename T>
-__global__ void __launch_bounds__(AT)
-k_update(int J, const T* __restrict__ V, size_t L, const double2* __restrict__ hbuf,
-         const int* __restrict__ act, pset_dev ps, T* __restrict__ w,
-         double* __restrict__ nrm_partial) {
-  using S = typename basis_t<T>::S;
-  extern __shared__ double2 hs_raw[];
-  T* hs = reinterpret_cast<T*>(hs_raw);
-  const chunk_ref c = chunk_of(ps, blockIdx.x);
-  if (!act[c.p]) return;
-  for (int jj = threadIdx.x; jj <= J; jj += AT) {
-    const double2 h = hbuf[(size_t)c.p * (J + 1) + jj];
-    hs[jj] = basis_t<T>::make(h.x, h.y);
-  }
-  __syncthreads();
-  T acc[AE];
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    acc[e] = q < c.cnt ? w[c.base + q] : basis_t<T>::make(0.0, 0.0);
-  }
-  for (int jj = 0; jj <= J; ++jj) {
-    const T* v = V + (size_t)jj * L + c.base;
-    const T hh = hs[jj];
-#pragma unroll
-    for (int e = 0; e < AE; ++e) {
-      const int q = e * AT + threadIdx.x;
-      if (q < c.cnt) {
-        const T a = v[q];
-        acc[e].x -= a.x * hh.x - a.y * hh.y;
-        acc[e].y -= a.x * hh.y + a.y * hh.x;
-      }
-    }
-  }
-  S ss = 0;
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    if (q < c.cnt) {
-      w[c.base + q] = acc[e];
-      ss += acc[e].x * acc[e].x + acc[e].y * acc[e].y;
-    }
-  }
-  if (nrm_partial) {
-    __shared__ double red[AT / 32];
-    const double sd = warp_sum((double)ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sd;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int q = 0; q < AT / 32; ++q) t += red[q];
-      nrm_partial[c.slot] = t;
-    }
-  }
-}
+// Givens data of one cycle, per problem
+struct givens_dev {
+  double2* H;      // [m + 1][m]
+  double* cs;      // [m]
+  double2* sn;     // [m]
+  double2* gv;     // [m + 1]
+  double* hnorm;   // ||w||
+  double* res;     // residual estimate
+};
 
-// One warp per problem: ||w||, Givens rotations, residual estimate.  The
-// warp stages column j of H and the previous rotations in shared memory;
-// lane 0 applies the rotations in order (each depends on the last).
-__global__ void k_givens(int m, int j, const int* __restrict__ act, pset_dev ps,
-                         const double* __restrict__ nrm_partial, double2* __restrict__ H,
-                         double* __restrict__ cs, double2* __restrict__ sn,
-                         double2* __restrict__ gv, double* __restrict__ hnorm,
-                         double* __restrict__ res) {
-  const int p = blockIdx.x, lane = threadIdx.x;
-  if (!act[p]) return;
-  extern __shared__ double2 gsh[];
-  double2* col = gsh;                                  // m + 1
-  double2* ssn = gsh + (m + 1);                        // m
-  double* scs = reinterpret_cast<double*>(ssn + m);    // m
-  double2* Hk = H + (size_t)p * (m + 1) * m;
-  double s2 = 0.0;
-  for (int c = lane; c < ps.nch[p]; c += 32) s2 += nrm_partial[ps.chb[p] + c];
-  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+// One warp: Givens rotations on column j of H, residual estimate.  The warp
+// stages the column and the previous rotations in shared memory (m + 1, m, m
+// entries); lane 0 applies the rotations in order (each depends on the last).
+// s2 = ||w||^2.
+__device__ void givens_step(int p, int m, int j, double s2, const givens_dev& G, double2* col) {
+  const int lane = threadIdx.x & 31;
+  double2* ssn = col + (m + 1);
+  double* scs = reinterpret_cast<double*>(ssn + m);
+  double2* Hk = G.H + (size_t)p * (m + 1) * m;
   const double hn = sqrt(s2);
   for (int q = lane; q <= j; q += 32) col[q] = Hk[(size_t)q * m + j];
   for (int q = lane; q < j; q += 32) {
-    scs[q] = cs[(size_t)p * m + q];
-    ssn[q] = sn[(size_t)p * m + q];
+    scs[q] = G.cs[(size_t)p * m + q];
+    ssn[q] = G.sn[(size_t)p * m + q];
   }
   __syncwarp();
   if (lane == 0) {
-    hnorm[p] = hn;
+    G.hnorm[p] = hn;
+    const double2 gj = G.gv[(size_t)p * (m + 1) + j];
     double2 a = col[0];
     for (int q = 0; q < j; ++q) {   // previous rotations [c s; -conj(s) c] on column j
       const double2 b = col[q + 1];
@@ -234,30 +250,118 @@ __global__ void k_givens(int m, int j, const int* __restrict__ act, pset_dev ps,
     const double bn = hn;  // b = ||w|| is real
     double c;
     double2 s;
-    const double aa = hypot(a.x, a.y);
-    if (bn == 0.0) {
-      c = 1.0;
-      s = make_double2(0.0, 0.0);
-    } else if (aa == 0.0) {
-      c = 0.0;
-      s = make_double2(1.0, 0.0);
+    const double a2 = a.x * a.x + a.y * a.y, t2 = a2 + bn * bn;
+    if (bn > 0.0 && a2 > 1e-280 && t2 < 1e280) {
+      // |a|, sqrt(|a|^2 + b^2) and their reciprocals from one Newton step each
+      const double ra = h64::rsqrt_newton(a2), rt = h64::rsqrt_newton(t2);
+      c = a2 * ra * rt;
+      const double f = ra * rt * bn;       // (a/|a|) conj(b) / t
+      s = make_double2(a.x * f, a.y * f);
     } else {
-      const double t = hypot(aa, bn);
-      c = aa / t;
-      s = make_double2(a.x / aa * bn / t, a.y / aa * bn / t);  // (a/|a|) conj(b) / t
+      const double aa = hypot(a.x, a.y);
+      if (bn == 0.0) {
+        c = 1.0;
+        s = make_double2(0.0, 0.0);
+      } else if (aa == 0.0) {
+        c = 0.0;
+        s = make_double2(1.0, 0.0);
+      } else {
+        const double t = hypot(aa, bn);
+        c = aa / t;
+        s = make_double2(a.x / aa * bn / t, a.y / aa * bn / t);
+      }
     }
-    cs[(size_t)p * m + j] = c;
-    sn[(size_t)p * m + j] = s;
+    G.cs[(size_t)p * m + j] = c;
+    G.sn[(size_t)p * m + j] = s;
     col[j] = make_double2(c * a.x + s.x * bn, c * a.y + s.y * bn);
     col[j + 1] = make_double2(0.0, 0.0);
-    const double2 gj = gv[(size_t)p * (m + 1) + j];
     const double2 g1 = make_double2(-(s.x * gj.x + s.y * gj.y), -(s.x * gj.y - s.y * gj.x));
-    gv[(size_t)p * (m + 1) + j + 1] = g1;
-    gv[(size_t)p * (m + 1) + j] = make_double2(c * gj.x, c * gj.y);
-    res[p] = hypot(g1.x, g1.y);
+    G.gv[(size_t)p * (m + 1) + j + 1] = g1;
+    G.gv[(size_t)p * (m + 1) + j] = make_double2(c * gj.x, c * gj.y);
+    const double g2 = g1.x * g1.x + g1.y * g1.y;
+    G.res[p] = g2 > 1e-280 && g2 < 1e280 ? sqrt(g2) : hypot(g1.x, g1.y);
   }
   __syncwarp();
   for (int q = lane; q <= j + 1; q += 32) Hk[(size_t)q * m + j] = col[q];
+}
+
+// w -= sum_jj V[jj] h[p][jj] on one chunk; with GIVENS (the second pass) also
+// |w|^2, and the problem's last CTA adds the chunks and does the Givens step
+template <typename T, int PT, bool GIVENS>
+__global__ void __launch_bounds__(AT)
+k_update(int J, int m, const T* __restrict__ V, size_t L, const double2* __restrict__ hbuf,
+         const int* __restrict__ act, pset_dev ps, T* __restrict__ w,
+         double* __restrict__ nrm_partial, int* __restrict__ counter, givens_dev G) {
+  using S = typename basis_t<T>::S;
+  extern __shared__ double2 hs_raw[];   // h in the basis precision; then the Givens step's data
+  T* hs = reinterpret_cast<T*>(hs_raw);
+  const chunk_ref c = chunk_of(ps, blockIdx.x);
+  if (!act[c.p]) return;
+  for (int jj = threadIdx.x; jj <= J; jj += blockDim.x) {
+    const double2 h = hbuf[(size_t)c.p * (J + 1) + jj];
+    hs[jj] = basis_t<T>::make(h.x, h.y);
+  }
+  two<T> acc[PT];
+#pragma unroll
+  for (int e = 0; e < PT; ++e) {
+    const int q = 2 * (e * blockDim.x + threadIdx.x);
+    acc[e].a = acc[e].b = basis_t<T>::make(0.0, 0.0);
+    if (q < c.cnt) acc[e] = load2(w + c.base + q);
+  }
+  __syncthreads();
+  for (int jj = 0; jj <= J; jj += AB) {
+    two<T> v[AB][PT];
+#pragma unroll
+    for (int b = 0; b < AB; ++b)
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const int q = 2 * (e * blockDim.x + threadIdx.x);
+        v[b][e].a = v[b][e].b = basis_t<T>::make(0.0, 0.0);
+        if (q < c.cnt && jj + b <= J) v[b][e] = load2(V + (size_t)(jj + b) * L + c.base + q);
+      }
+#pragma unroll
+    for (int b = 0; b < AB; ++b) {
+      if (jj + b > J) break;
+      const T hh = hs[jj + b];
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const two<T> a = v[b][e];
+        acc[e].a.x = fma(-a.a.x, hh.x, fma(a.a.y, hh.y, acc[e].a.x));
+        acc[e].a.y = fma(-a.a.x, hh.y, fma(-a.a.y, hh.x, acc[e].a.y));
+        acc[e].b.x = fma(-a.b.x, hh.x, fma(a.b.y, hh.y, acc[e].b.x));
+        acc[e].b.y = fma(-a.b.x, hh.y, fma(-a.b.y, hh.x, acc[e].b.y));
+      }
+    }
+  }
+  S ss = 0;
+#pragma unroll
+  for (int e = 0; e < PT; ++e) {
+    const int q = 2 * (e * blockDim.x + threadIdx.x);
+    if (q < c.cnt) {
+      store2(w + c.base + q, acc[e].a, acc[e].b);
+      ss = fma(acc[e].a.x, acc[e].a.x, fma(acc[e].a.y, acc[e].a.y, ss));
+      ss = fma(acc[e].b.x, acc[e].b.x, fma(acc[e].b.y, acc[e].b.y, ss));
+    }
+  }
+  if constexpr (GIVENS) {
+    __shared__ double red[AT / 32];
+    const double sd = warp_sum((double)ss);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sd;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q];
+      nrm_partial[c.slot] = t;
+    }
+    const int nch = ps.nch[c.p], chb = ps.chb[c.p];
+    if (!last_cta(counter + c.p, nch)) return;
+    if (threadIdx.x < 32) {
+      double s2 = 0.0;
+      for (int k = threadIdx.x; k < nch; k += 32) s2 += __ldcg(nrm_partial + chb + k);
+      for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      givens_step(c.p, m, J, s2, G, hs_raw);
+    }
+  }
 }
 
 // vout = w / ||w|| per problem (0 on breakdown); vin (optional) = the same
@@ -272,10 +376,9 @@ k_scale(const int* __restrict__ act, pset_dev ps, const double* __restrict__ hn,
   const double inv = h > 0.0 ? 1.0 / h : 0.0;
   // the multiply in the basis precision (FP64 runs at 1/64 of the FP32 rate)
   const typename basis_t<T>::S s = (typename basis_t<T>::S)inv;
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    if (q < c.cnt) {
+#pragma unroll 4
+  for (int q = threadIdx.x; q < c.cnt; q += blockDim.x) {
+    {
       const T v = w[c.base + q];
       const T o = basis_t<T>::make(v.x * s, v.y * s);
       vout[c.base + q] = o;
@@ -292,10 +395,9 @@ k_start(const int* __restrict__ act, pset_dev ps, const double* __restrict__ bet
   const chunk_ref c = chunk_of(ps, blockIdx.x);
   const double b = beta[c.p];
   const double inv = (act[c.p] && b > 0.0) ? 1.0 / b : 0.0;
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    if (q < c.cnt) {
+#pragma unroll 4
+  for (int q = threadIdx.x; q < c.cnt; q += blockDim.x) {
+    {
       const double2 v = r[c.base + q];
       const T o = basis_t<T>::make(v.x * inv, v.y * inv);
       v0[c.base + q] = o;
@@ -310,10 +412,9 @@ k_to32(const int* __restrict__ act, pset_dev ps, const double2* __restrict__ w,
        float2* __restrict__ w32) {
   const chunk_ref c = chunk_of(ps, blockIdx.x);
   if (!act[c.p]) return;
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    if (q < c.cnt) {
+#pragma unroll 4
+  for (int q = threadIdx.x; q < c.cnt; q += blockDim.x) {
+    {
       const double2 v = w[c.base + q];
       w32[c.base + q] = make_float2((float)v.x, (float)v.y);
     }
@@ -330,32 +431,43 @@ __global__ void k_g_init(int P, int m, const int* __restrict__ act, const double
   gv[e] = make_double2(q == 0 && act[p] ? beta[p] : 0.0, 0.0);
 }
 
-// per problem: y = R^{-1} g on the leading kd x kd triangle
-__global__ void k_lsq(int P, int m, const int* __restrict__ kd, const double2* __restrict__ H,
-                      const double2* __restrict__ gv, double2* __restrict__ y) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
+// one warp per problem: y = R^{-1} g on the leading kd x kd triangle, column by
+// column from the last (each solved unknown is taken out of the rows above it,
+// one row per lane; the reciprocals of the diagonal come first)
+__global__ void __launch_bounds__(32)
+k_lsq(int m, const int* __restrict__ kd, const double2* __restrict__ H,
+      const double2* __restrict__ gv, double2* __restrict__ y) {
+  extern __shared__ double2 lsh[];   // s [m], 1 / diagonal [m]
+  const int p = blockIdx.x, lane = threadIdx.x;
   const int K = kd[p];
   const double2* Hk = H + (size_t)p * (m + 1) * m;
   double2* yk = y + (size_t)p * m;
-  for (int i = K - 1; i >= 0; --i) {
-    double2 s = gv[(size_t)p * (m + 1) + i];
-    for (int q = i + 1; q < K; ++q) {
-      const double2 h = Hk[(size_t)i * m + q], yq = yk[q];
-      s.x -= h.x * yq.x - h.y * yq.y;
-      s.y -= h.x * yq.y + h.y * yq.x;
-    }
+  double2* s = lsh;
+  double2* inv = lsh + m;
+  for (int i = lane; i < K; i += 32) {
+    s[i] = gv[(size_t)p * (m + 1) + i];
     const double2 d = Hk[(size_t)i * m + i];
     const double den = d.x * d.x + d.y * d.y;
-    yk[i] = den > 0.0 ? make_double2((s.x * d.x + s.y * d.y) / den, (s.y * d.x - s.x * d.y) / den)
-                      : make_double2(0.0, 0.0);
+    inv[i] = den > 0.0 ? make_double2(d.x / den, -d.y / den) : make_double2(0.0, 0.0);
+  }
+  __syncwarp();
+  for (int i = K - 1; i >= 0; --i) {
+    const double2 a = s[i], d = inv[i];
+    const double2 yi = make_double2(a.x * d.x - a.y * d.y, a.x * d.y + a.y * d.x);
+    if (lane == 0) yk[i] = yi;
+    for (int q = lane; q < i; q += 32) {
+      const double2 h = Hk[(size_t)q * m + i];
+      s[q].x -= h.x * yi.x - h.y * yi.y;
+      s[q].y -= h.x * yi.y + h.y * yi.x;
+    }
+    __syncwarp();
   }
 }
 
 // x += sum_{jj < kd[p]} V[jj] y[p][jj]: the sum in the basis precision (an
 // FP32 basis is orthonormal to FP32 accuracy, so |sum| ~ |y| and FP32 loses
 // nothing the inner solve's tolerance would notice), added to x in FP64
-template <typename T>
+template <typename T, int PT>
 __global__ void __launch_bounds__(AT)
 k_xupdate(int m, const int* __restrict__ kd, pset_dev ps, const T* __restrict__ V, size_t L,
           const double2* __restrict__ y, double2* __restrict__ x) {
@@ -363,29 +475,42 @@ k_xupdate(int m, const int* __restrict__ kd, pset_dev ps, const T* __restrict__ 
   const chunk_ref c = chunk_of(ps, blockIdx.x);
   const int K = kd[c.p];
   if (K == 0) return;
-  S ar[AE], ai[AE];
+  two<T> acc[PT];
 #pragma unroll
-  for (int e = 0; e < AE; ++e) ar[e] = ai[e] = 0;
-  for (int jj = 0; jj < K; ++jj) {
-    const double2 yd = y[(size_t)c.p * m + jj];
-    const S yr = (S)yd.x, yi = (S)yd.y;
-    const T* v = V + (size_t)jj * L + c.base;
+  for (int e = 0; e < PT; ++e) acc[e].a = acc[e].b = basis_t<T>::make(0.0, 0.0);
+  for (int jj = 0; jj < K; jj += AB) {
+    two<T> v[AB][PT];
 #pragma unroll
-    for (int e = 0; e < AE; ++e) {
-      const int q = e * AT + threadIdx.x;
-      if (q < c.cnt) {
-        const T a = v[q];
-        ar[e] = fma(a.x, yr, fma(-a.y, yi, ar[e]));
-        ai[e] = fma(a.x, yi, fma(a.y, yr, ai[e]));
+    for (int b = 0; b < AB; ++b)
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const int q = 2 * (e * blockDim.x + threadIdx.x);
+        v[b][e].a = v[b][e].b = basis_t<T>::make(0.0, 0.0);
+        if (q < c.cnt && jj + b < K) v[b][e] = load2(V + (size_t)(jj + b) * L + c.base + q);
+      }
+#pragma unroll
+    for (int b = 0; b < AB; ++b) {
+      if (jj + b >= K) break;
+      const double2 yd = y[(size_t)c.p * m + jj + b];
+      const S yr = (S)yd.x, yi = (S)yd.y;
+#pragma unroll
+      for (int e = 0; e < PT; ++e) {
+        const two<T> a = v[b][e];
+        acc[e].a.x = fma(a.a.x, yr, fma(-a.a.y, yi, acc[e].a.x));
+        acc[e].a.y = fma(a.a.x, yi, fma(a.a.y, yr, acc[e].a.y));
+        acc[e].b.x = fma(a.b.x, yr, fma(-a.b.y, yi, acc[e].b.x));
+        acc[e].b.y = fma(a.b.x, yi, fma(a.b.y, yr, acc[e].b.y));
       }
     }
   }
 #pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
+  for (int e = 0; e < PT; ++e) {
+    const int q = 2 * (e * blockDim.x + threadIdx.x);
     if (q < c.cnt) {
-      const double2 xo = x[c.base + q];
-      x[c.base + q] = make_double2(xo.x + (double)ar[e], xo.y + (double)ai[e]);
+      const two<double2> xo = load2(x + c.base + q);
+      store2(x + c.base + q,
+             make_double2(xo.a.x + (double)acc[e].a.x, xo.a.y + (double)acc[e].a.y),
+             make_double2(xo.b.x + (double)acc[e].b.x, xo.b.y + (double)acc[e].b.y));
     }
   }
 }
@@ -396,10 +521,9 @@ k_residual(pset_dev ps, const double2* __restrict__ f, const double2* __restrict
            double2* __restrict__ r, double* __restrict__ rr, double* __restrict__ ff) {
   const chunk_ref c = chunk_of(ps, blockIdx.x);
   double sr = 0.0, sf = 0.0;
-#pragma unroll
-  for (int e = 0; e < AE; ++e) {
-    const int q = e * AT + threadIdx.x;
-    if (q < c.cnt) {
+#pragma unroll 4
+  for (int q = threadIdx.x; q < c.cnt; q += blockDim.x) {
+    {
       const size_t idx = c.base + q;
       const double2 fv = f[idx];
       double2 v = fv;
@@ -423,7 +547,7 @@ k_residual(pset_dev ps, const double2* __restrict__ f, const double2* __restrict
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;
-    for (int q = 0; q < AT / 32; ++q) {
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
       a += red[0][q];
       b += red[1][q];
     }
@@ -477,10 +601,10 @@ struct ws {
   double2* vin = nullptr;            // FP64 copy of the newest FP32 basis vector
   double2 *V, *H, *gv, *sn, *w, *hbuf, *y, *part;
   double *cs, *hn, *res, *nrmp, *rr, *ff, *norms;
-  int *act, *kd;
+  int *act, *kd, *cnt;
 };
 
-ws workspace(krylov_ws& K, const pset& ps, int m, bool f32) {
+ws workspace(cudaStream_t st, krylov_ws& K, const pset& ps, int m, bool f32) {
   const int P = ps.P, Q = ps.Q;
   const size_t L = ps.L;
   if (f32) {
@@ -512,6 +636,7 @@ ws workspace(krylov_ws& K, const pset& ps, int m, bool f32) {
   const size_t o_norms = take(sizeof(double) * 2 * P);
   const size_t o_act = take(sizeof(int) * P);
   const size_t o_kd = take(sizeof(int) * P);
+  const size_t o_cnt = take(sizeof(int) * P);
   K.small.reserve(sm);
   char* b = K.small.as<char>();
   ws W;
@@ -536,6 +661,8 @@ ws workspace(krylov_ws& K, const pset& ps, int m, bool f32) {
   W.norms = (double*)(b + o_norms);
   W.act = (int*)(b + o_act);
   W.kd = (int*)(b + o_kd);
+  W.cnt = (int*)(b + o_cnt);
+  CFIE_CHECK_CUDA(cudaMemsetAsync(W.cnt, 0, sizeof(int) * P, st));
   if (K.host_cap < 2 * P + 8) {
     if (K.host) cudaFreeHost(K.host);
     K.host = nullptr;
@@ -550,7 +677,7 @@ void residual_norms(cudaStream_t st, krylov_ws& K, const pset& ps, const ws& W,
                     const double2* f, const double2* ax, double2* r, std::vector<double>& rn,
                     std::vector<double>& fn) {
   const int P = ps.P;
-  k_residual<<<ps.Q, AT, 0, st>>>(ps.dev, f, ax, r, W.rr, W.ff);
+  k_residual<<<ps.Q, ps.tb, 0, st>>>(ps.dev, f, ax, r, W.rr, W.ff);
   CFIE_CHECK_LAUNCH();
   k_sum_chunks<<<blocks_for(P, 64), 64, 0, st>>>(P, ps.dev, W.rr, W.ff, W.norms);
   CFIE_CHECK_LAUNCH();
@@ -559,6 +686,56 @@ void residual_norms(cudaStream_t st, krylov_ws& K, const pset& ps, const ws& W,
   CFIE_CHECK_CUDA(cudaStreamSynchronize(st));
   rn.assign(K.host, K.host + P);
   fn.assign(K.host + P, K.host + 2 * P);
+}
+
+// pairs of elements per thread of the chunked kernels: 1, 2 or 4
+template <typename F>
+void with_pairs(const pset& ps, F f) {
+  switch (ps.dev.ch / (2 * ps.tb)) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    default: f(std::integral_constant<int, 4>());
+  }
+}
+
+// column j of H and the rotations: classical Gram-Schmidt twice, then the Givens
+// step.  A set with fewer chunks than two per SM splits the inner products over
+// the basis vectors as well.
+template <typename T>
+void orthogonalise(cudaStream_t st, const pset& ps, const ws& W, int m, int j, size_t L, const T* V,
+                   T* w) {
+  const givens_dev G{W.H, W.cs, W.sn, W.gv, W.hn, W.res};
+  const int ny = std::max(1, std::min((j + AB) / AB, 304 / ps.Q));
+  const int JB = std::min(256, ((j + 1 + ny - 1) / ny + AB - 1) / AB * AB);
+  const dim3 grid(ps.Q, (j + JB) / JB);
+  const size_t red = sizeof(double2) * std::min(JB, j + 1) * (ps.tb / 32);
+  const size_t hs = sizeof(T) * (j + 1);
+  const size_t gs = (sizeof(double2) * 2 + sizeof(double)) * m + sizeof(double2);
+  with_pairs(ps, [&](auto pt) {
+    constexpr int PT = decltype(pt)::value;
+    for (int pass = 0; pass < 2; ++pass) {
+      k_dots<T, PT><<<grid, ps.tb, red, st>>>(j, JB, m, j, pass == 0, V, L, w, W.act, ps.dev,
+                                              W.part, W.cnt, W.hbuf, W.H);
+      CFIE_CHECK_LAUNCH();
+      if (pass == 0)
+        k_update<T, PT, false><<<ps.Q, ps.tb, hs, st>>>(j, m, V, L, W.hbuf, W.act, ps.dev, w,
+                                                        nullptr, W.cnt, G);
+      else
+        k_update<T, PT, true><<<ps.Q, ps.tb, std::max(hs, gs), st>>>(
+            j, m, V, L, W.hbuf, W.act, ps.dev, w, W.nrmp, W.cnt, G);
+      CFIE_CHECK_LAUNCH();
+    }
+  });
+}
+
+// x += V y
+template <typename T>
+void add_basis(cudaStream_t st, const pset& ps, const ws& W, int m, size_t L, const T* V,
+               double2* x) {
+  with_pairs(ps, [&](auto pt) {
+    k_xupdate<T, decltype(pt)::value><<<ps.Q, ps.tb, 0, st>>>(m, W.kd, ps.dev, V, L, W.y, x);
+  });
+  CFIE_CHECK_LAUNCH();
 }
 
 // Marks the problems of an Arnoldi step's matvec for the matvec callbacks.
@@ -587,9 +764,9 @@ void gmres_cycle(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps, c
   CFIE_CHECK_CUDA(
       cudaMemcpyAsync(W.norms, beta.data(), sizeof(double) * P, cudaMemcpyHostToDevice, st));
   if (W.f32)
-    k_start<float2><<<ps.Q, AT, 0, st>>>(W.act, ps.dev, W.norms, r, W.V32, W.vin);
+    k_start<float2><<<ps.Q, ps.tb, 0, st>>>(W.act, ps.dev, W.norms, r, W.V32, W.vin);
   else
-    k_start<double2><<<ps.Q, AT, 0, st>>>(W.act, ps.dev, W.norms, r, W.V, nullptr);
+    k_start<double2><<<ps.Q, ps.tb, 0, st>>>(W.act, ps.dev, W.norms, r, W.V, nullptr);
   CFIE_CHECK_LAUNCH();
   k_g_init<<<blocks_for((size_t)P * (m + 1)), 256, 0, st>>>(P, m, W.act, W.norms, W.gv);
   CFIE_CHECK_LAUNCH();
@@ -612,35 +789,18 @@ void gmres_cycle(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps, c
     }
     {
       prof_scope ps_(ctx, CFIE_K_ARNOLDI);
-      const size_t red_smem = sizeof(double2) * (j + 1) * (AT / 32);
       if (W.f32) {
-        k_to32<<<ps.Q, AT, 0, st>>>(W.act, ps.dev, W.w, W.w32);
+        k_to32<<<ps.Q, ps.tb, 0, st>>>(W.act, ps.dev, W.w, W.w32);
         CFIE_CHECK_LAUNCH();
+        orthogonalise<float2>(st, ps, W, m, j, L, W.V32, W.w32);
+      } else {
+        orthogonalise<double2>(st, ps, W, m, j, L, W.V, W.w);
       }
-      for (int pass = 0; pass < 2; ++pass) {
-        if (W.f32)
-          k_dots<float2><<<ps.Q, AT, red_smem, st>>>(j, W.V32, L, W.w32, W.act, ps.dev, W.part);
-        else
-          k_dots<double2><<<ps.Q, AT, red_smem, st>>>(j, W.V, L, W.w, W.act, ps.dev, W.part);
-        CFIE_CHECK_LAUNCH();
-        k_dots_reduce<<<P, 128, 0, st>>>(j, m, j, pass == 0, W.act, ps.dev, W.part, W.hbuf, W.H);
-        CFIE_CHECK_LAUNCH();
-        if (W.f32)
-          k_update<float2><<<ps.Q, AT, sizeof(double2) * (j + 1), st>>>(
-              j, W.V32, L, W.hbuf, W.act, ps.dev, W.w32, pass == 1 ? W.nrmp : nullptr);
-        else
-          k_update<double2><<<ps.Q, AT, sizeof(double2) * (j + 1), st>>>(
-              j, W.V, L, W.hbuf, W.act, ps.dev, W.w, pass == 1 ? W.nrmp : nullptr);
-        CFIE_CHECK_LAUNCH();
-      }
-      k_givens<<<P, 32, (sizeof(double2) * 2 + sizeof(double)) * m + sizeof(double2), st>>>(
-          m, j, W.act, ps.dev, W.nrmp, W.H, W.cs, W.sn, W.gv, W.hn, W.res);
-      CFIE_CHECK_LAUNCH();
       if (W.f32)
-        k_scale<float2><<<ps.Q, AT, 0, st>>>(W.act, ps.dev, W.hn, W.w32,
+        k_scale<float2><<<ps.Q, ps.tb, 0, st>>>(W.act, ps.dev, W.hn, W.w32,
                                              W.V32 + (size_t)(j + 1) * L, W.vin);
       else
-        k_scale<double2><<<ps.Q, AT, 0, st>>>(W.act, ps.dev, W.hn, W.w,
+        k_scale<double2><<<ps.Q, ps.tb, 0, st>>>(W.act, ps.dev, W.hn, W.w,
                                               W.V + (size_t)(j + 1) * L, nullptr);
       CFIE_CHECK_LAUNCH();
       stats.arnoldi_elems += arnoldi_elems(ps, act, j);
@@ -670,7 +830,7 @@ void gmres_cycle(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps, c
           cudaMemcpyAsync(W.act, act.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
   }
   CFIE_CHECK_CUDA(cudaMemcpyAsync(W.kd, kd.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
-  k_lsq<<<blocks_for(P, 64), 64, 0, st>>>(P, m, W.kd, W.H, W.gv, W.y);
+  k_lsq<<<P, 32, 2 * sizeof(double2) * m, st>>>(m, W.kd, W.H, W.gv, W.y);
   CFIE_CHECK_LAUNCH();
   // x += V y, or with right preconditioning x += P (V y)
   double2* xu = x;
@@ -680,10 +840,9 @@ void gmres_cycle(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps, c
     CFIE_CHECK_LAUNCH();
   }
   if (W.f32)
-    k_xupdate<float2><<<ps.Q, AT, 0, st>>>(m, W.kd, ps.dev, W.V32, L, W.y, xu);
+    add_basis<float2>(st, ps, W, m, L, W.V32, xu);
   else
-    k_xupdate<double2><<<ps.Q, AT, 0, st>>>(m, W.kd, ps.dev, W.V, L, W.y, xu);
-  CFIE_CHECK_LAUNCH();
+    add_basis<double2>(st, ps, W, m, L, W.V, xu);
   if (fns.prec) {
     fns.prec(xu, K.pz2.as<double2>());
     k_axpy<<<blocks_for(L), 256, 0, st>>>(L, K.pz2.as<double2>(), x);
@@ -700,9 +859,16 @@ void pset_build(pset& ps, const std::vector<size_t>& off, const std::vector<int>
   ps.P = (int)off.size();
   std::vector<int> nch(ps.P), chb(ps.P);
   std::vector<int2> items;
-  size_t L = 0;
+  size_t L = 0, total = 0;
+  // chunks of 2048 elements (256 threads, four pairs each), or shorter ones down
+  // to 128 (64 threads, one pair each) until there are about two per SM
+  for (int p = 0; p < ps.P; ++p) total += len[p];
+  int ch = 2048;
+  while (ch > 128 && total / ch < 304) ch /= 2;
+  ps.dev.ch = ch;
+  ps.tb = std::min(AT, ch / 2);
   for (int p = 0; p < ps.P; ++p) {
-    nch[p] = (len[p] + CH - 1) / CH;
+    nch[p] = (len[p] + ch - 1) / ch;
     chb[p] = (int)items.size();
     for (int c = 0; c < nch[p]; ++c) items.push_back(make_int2(p, c));
     L = std::max(L, off[p] + (size_t)len[p]);
@@ -746,7 +912,7 @@ void gmres_set(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps,
   m = std::max(1, std::min(m, std::min(maxit, MAXJ)));
   const bool f32 = refined && fns.basis32;
   stats.basis_fp32 = f32 ? 1 : 0;
-  ws W = workspace(K, ps, m, f32);
+  ws W = workspace(st, K, ps, m, f32);
   K.r.reserve(sizeof(double2) * L);
   if (fns.prec) {
     K.pz.reserve(sizeof(double2) * L);

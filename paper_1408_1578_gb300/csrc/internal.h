@@ -120,12 +120,14 @@ struct cfie_geom {
 struct pset_dev {
   const size_t* off;   // [P] segment offsets
   const int* len;      // [P] segment lengths
-  const int* nch;      // [P] 2048-element chunks per segment
+  const int* nch;      // [P] chunks per segment
   const int* chb;      // [P] first chunk slot of the segment
   const int2* items;   // [Q] (problem, chunk) work list
+  int ch;              // elements per chunk
 };
 struct pset {
   int P = 0, Q = 0;
+  int tb = 0;             // threads per CTA of the chunked kernels
   size_t L = 0;
   std::vector<int> len;   // host copy of the segment lengths
   pset_dev dev{};
