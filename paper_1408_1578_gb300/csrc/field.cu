@@ -15,8 +15,8 @@
 // staged in shared memory a tile at a time, the quarters added at the end.
 //
 // Bound: the FP64 pipe, about 60 instructions per kernel value and 4 per
-// density, so a kernel value is shared by up to 16 densities and padding
-// densities cost nothing; when the points alone do not fill the GPU the
+// density, so a kernel value is shared by up to 16 densities, with a kernel for
+// every few counts; when the points alone do not fill the GPU the
 // sources are split across CTAs and a second kernel adds the splits in a
 // fixed order.
 // Measured (GB300): 16 densities of n = 4096 nodes at 20000 points, sound hard,
@@ -89,13 +89,11 @@ k_field(int n, int npts, int nrhs, int tiles_per_split, double omega, double eta
                                 : make_double2(fma(A, v.y0, B * v.j1), fma(B, v.y1, -(A * v.j0)));
 #pragma unroll
       for (int k = 0; k < FRB; ++k) {
-        if (k < rn) {
-          const double2 qq = sq[jl][k];
-          acc[k].x = fma(c.x, qq.x, acc[k].x);
-          acc[k].x = fma(-c.y, qq.y, acc[k].x);
-          acc[k].y = fma(c.x, qq.y, acc[k].y);
-          acc[k].y = fma(c.y, qq.x, acc[k].y);
-        }
+        const double2 qq = sq[jl][k];
+        acc[k].x = fma(c.x, qq.x, acc[k].x);
+        acc[k].x = fma(-c.y, qq.y, acc[k].x);
+        acc[k].y = fma(c.x, qq.y, acc[k].y);
+        acc[k].y = fma(c.y, qq.x, acc[k].y);
       }
     }
   }
@@ -139,10 +137,11 @@ void launch_field(cfie_op* op, const double2* q, int nrhs, int npts, const doubl
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
   const int px = (npts + FPT - 1) / FPT, ry = (nrhs + FRB - 1) / FRB;
-  // about four CTAs per SM, as many splits of the sources as that takes (no
-  // more partial sums than 256 MB)
+  // about 16 CTAs per SM (two fit, so that the last of several waves is a small
+  // part), as many splits of the sources as that takes (no more partial sums
+  // than 256 MB)
   const size_t tot = (size_t)nrhs * npts;
-  long long splits = std::max<long long>(1, (4LL * sms + (long long)px * ry - 1) / ((long long)px * ry));
+  long long splits = std::max<long long>(1, (16LL * sms + (long long)px * ry - 1) / ((long long)px * ry));
   splits = std::min<long long>(splits, std::min<long long>(tiles, std::max<size_t>(1, ((size_t)1 << 24) / tot)));
   const int tps = (int)((tiles + splits - 1) / splits);
   const int ns = (tiles + tps - 1) / tps;
@@ -162,10 +161,18 @@ void launch_field(cfie_op* op, const double2* q, int nrhs, int npts, const doubl
 
 template <int BC>
 void field_bc(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts, double2* u) {
-  if (nrhs == 1)
+  // equal blocks of at most 16 densities
+  const int blocks = (nrhs + 15) / 16, per = (nrhs + blocks - 1) / blocks;
+  if (per == 1)
     launch_field<BC, 1>(op, q, nrhs, npts, pts, u);
-  else if (nrhs <= 4)
+  else if (per == 2)
+    launch_field<BC, 2>(op, q, nrhs, npts, pts, u);
+  else if (per <= 4)
     launch_field<BC, 4>(op, q, nrhs, npts, pts, u);
+  else if (per <= 8)
+    launch_field<BC, 8>(op, q, nrhs, npts, pts, u);
+  else if (per <= 12)
+    launch_field<BC, 12>(op, q, nrhs, npts, pts, u);
   else
     launch_field<BC, 16>(op, q, nrhs, npts, pts, u);
 }

@@ -125,7 +125,7 @@ __global__ void k_kress(int n, const double* __restrict__ cosk, const double* __
 // w_d for all d (R_d = R_{n-d}); spectral-derivative circulant c_d; diagonal entries.
 __global__ void k_finish(int n, double omega, double eta, int bc, const double* __restrict__ R,
                          double* __restrict__ w, double* __restrict__ ct, geom_dev g,
-                         double2* __restrict__ diag) {
+                         double2* __restrict__ diag) {   // w: w_d, then w_d / (pi h)
   int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= n) return;
   double h = 2.0 * CFIE_PI / n;
@@ -140,6 +140,7 @@ __global__ void k_finish(int n, double omega, double eta, int bc, const double* 
     w[d] = Rd - h * log(4.0 * sn * sn);
     ct[d] = 0.5 * ((d & 1) ? -1.0 : 1.0) * cs / sn;
   }
+  w[n + d] = w[d] / (CFIE_PI * h);
   // diagonal limits (node i = d)
   int i = d;
   double s = g.sp[i];
@@ -228,7 +229,7 @@ void kress_tables(cfie_op* op) {
   double* cosk = tmp.as<double>();
   double* invm = cosk + n;
   double* R = invm + n;
-  op->wtab.reserve(sizeof(double) * n);
+  op->wtab.reserve(sizeof(double) * 2 * (size_t)n);
   op->ctab.reserve(sizeof(double) * n);
   op->diag.reserve(sizeof(double2) * 2 * (size_t)n);
   k_tables<<<(n + 255) / 256, 256, 0, st>>>(n, cosk, invm);

@@ -216,7 +216,7 @@ struct cfie_op {
 
   dbuf geo;          // 6 n doubles and the Bessel tables (geom_dev)
   geom_dev g{};
-  dbuf wtab;         // n doubles: w_d = R_d - h ln(4 sin^2(pi d / n)), w_0 = R_0
+  dbuf wtab;         // n doubles: w_d = R_d - h ln(4 sin^2(pi d / n)), w_0 = R_0; n: w_d / (pi h)
   dbuf ctab;         // n doubles: spectral derivative circulant c_d = (-1)^d cot(pi d / n) / 2
   dbuf diag;         // complex diagonal entries: soft A_ii; hard (S_ii, D'_ii)
   double R0 = 0;

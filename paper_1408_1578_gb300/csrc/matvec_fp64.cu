@@ -30,10 +30,10 @@
 //
 // Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
 // scheduler): per pair about 70 instructions for the entry (hankel64.cuh) and
-// 4 (soft) or 8 (hard) per right-hand side for the sums, so the right-hand
-// sides of a block are counted out (no sums on padding columns; with one or
-// two the threads split the sources instead) and the entry is shared by up to
-// 64 (soft) or 32 (hard) of them.
+// 4 (soft) or 8 (hard) per right-hand side for the sums, so there is a kernel
+// for every few widths of a block (hardly any sums on padding columns; with one
+// or two the threads split the sources instead) and the entry is shared by up
+// to 64 (soft) or 32 (hard) of them.
 // Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 215 us; star n =
 // 4096, 16 right-hand sides, sound hard 15.8 -> 7.4 ms (of which 6.9 here).
 #include <algorithm>
@@ -181,10 +181,8 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
 #pragma unroll
       for (int q = 0; q < RQ; ++q) {
         const int r = rg + RG * q;
-        if (r < rbn) {
-          acc[0][q] = cmad(acc[0][q], a, S.X[0][jl][r]);
-          if constexpr (BC == 1) acc[NO - 1][q] = cmad(acc[NO - 1][q], b, S.X[NO - 1][jl][r]);
-        }
+        acc[0][q] = cmad(acc[0][q], a, S.X[0][jl][r]);
+        if constexpr (BC == 1) acc[NO - 1][q] = cmad(acc[NO - 1][q], b, S.X[NO - 1][jl][r]);
       }
     }
   }
@@ -218,6 +216,180 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
       }
     }
   }
+}
+
+// Up to four right-hand sides: each pair of nodes once for both of its entries.
+// (i, j) and (j, i) share the distance, the Hankel values and the Kress weight,
+// about 60 of the 75 FP64 instructions of an entry; what then remains per entry
+// is its normal and speed factors, the multiply-adds and two additions of the
+// reduction over the rows of the transposed product.
+//
+// A warp owns 32 rows (one per lane, sums in registers) and walks units of 8
+// sources: row blocks I and J = I + d (mod the number of blocks), d = 0 .. half
+// of it, cover every pair of blocks once; d = 0 takes its pairs in both orders.
+// The transposed sums of SB sources are reduced across the warp together (16
+// values: 16 additions instead of 80) and go out by (d, j), each written by one
+// warp; the direct sums by (split, i): the layout of the split partial sums
+// above with splits + nblk / 2 entries.
+// Measured (GB300), against one entry at a time: kite n = 1024 258 -> 144 us
+// (one right-hand side, sound soft), n = 4096 2.93 -> 1.50 ms, four 3.30 -> 1.95;
+// sound hard, n = 4096 3.26 -> 1.92 ms (one), 4.05 -> 2.82 (four).
+template <int BC, int R>
+__global__ void __launch_bounds__(32)
+k_pair_sym(int n, int nblk, double omega, double omega_inv, double eta_inv, double nf, double sf,
+           int units_per_warp, int splits, geom_dev g, const double* __restrict__ wks,
+           const double2* __restrict__ diag, const double2* __restrict__ xin,
+           const double2* __restrict__ uin, int nrhs, double2* __restrict__ part) {
+  constexpr int NO = BC ? 2 : 1;
+  constexpr int SB = 8 / (R * NO);     // sources whose transposed sums are reduced together
+  const int lane = threadIdx.x, I = blockIdx.x, i = 32 * I + lane;
+  const bool ok = i < n;
+  const int dmax = nblk / 2, units = 4 * (dmax + 1), nsp = splits + dmax;
+  // node data of a row or a source: coordinates, folded normal (soft nf nu;
+  // hard omega nu / |z'|), folded speed; densities of every output
+  auto normal = [&](int k, double& ax, double& ay) {
+    const double m = BC ? omega / g.sp[k] : nf;
+    ax = m * g.nx[k];
+    ay = m * g.ny[k];
+  };
+  // rows past n sit far away and contribute nothing
+  double tx = 1e3 * (lane + 2), ty = 1e3, tfx = 0.0, tfy = 0.0, te = 0.0;
+  double2 xi[R][NO], acc[R][NO];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int o = 0; o < NO; ++o) xi[r][o] = acc[r][o] = make_double2(0.0, 0.0);
+  if (ok) {
+    tx = g.x[i];
+    ty = g.y[i];
+    normal(i, tfx, tfy);
+    te = sf * g.sp[i];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (r < nrhs) {
+        xi[r][NO - 1] = xin[(size_t)r * n + i];
+        if (BC) xi[r][0] = uin[(size_t)r * n + i];
+      }
+  }
+  const int u1 = min(units, (int)(blockIdx.y + 1) * units_per_warp);
+  for (int u = blockIdx.y * units_per_warp; u < u1; ++u) {
+    const int d = u >> 2;
+    int J = I + d;
+    if (J >= nblk) J -= nblk;
+    const int jb = 32 * J + 8 * (u & 3);
+    // an even number of blocks meets its opposite pairs twice: the second time
+    // only writes the zeros that the reduction reads
+    const bool skip = d > 0 && 2 * d == nblk && I >= d;
+    // lanes 8 q .. 8 q + 7 hold the eight sources
+    const int jl = jb + (lane & 7);
+    double sx = 0.0, sy = 0.0, sfx = 0.0, sfy = 0.0, se = 0.0;
+    double2 xj[R][NO];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) xj[r][o] = make_double2(0.0, 0.0);
+    if (!skip && jl < n) {
+      sx = g.x[jl];
+      sy = g.y[jl];
+      normal(jl, sfx, sfy);
+      se = sf * g.sp[jl];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r < nrhs) {
+          xj[r][NO - 1] = xin[(size_t)r * n + jl];
+          if (BC) xj[r][0] = uin[(size_t)r * n + jl];
+        }
+    }
+#pragma unroll 1
+    for (int s0 = 0; s0 < 8; s0 += SB) {
+      double v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = 0.0;
+#pragma unroll
+      for (int b = 0; b < SB; ++b) {
+        const int s = s0 + b, j = jb + s;
+        if (skip || j >= n) continue;            // uniform
+        auto from = [&](double a) { return __shfl_sync(0xffffffffu, a, s); };
+        const double qx = from(sx), qy = from(sy), qfx = from(sfx), qfy = from(sfy), qe = from(se);
+        double2 q[R][NO];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int o = 0; o < NO; ++o) q[r][o] = make_double2(from(xj[r][o].x), from(xj[r][o].y));
+        int di = i - j;
+        if (di < 0) di += n;
+        const double wk = ok ? wks[di] : 0.0;
+        const double dx = tx - qx, dy = ty - qy;
+        double dist, rinv;
+        h64::distance(fma(dx, dx, dy * dy), dist, rinv);
+        const h64::values h = h64::bessel01(omega * dist, omega_inv * rinv, g.tab);
+        const double w0 = fma(wk, h.j0, h.y0), w1 = fma(wk, h.j1, h.y1);
+        const double ra = rinv * h.amp;
+        // entries from the receiving node's and the sending node's factors
+        double2 e[NO], et[NO];
+        if constexpr (BC == 0) {
+          const double A = qe * h.amp, B = fma(dx, qfx, dy * qfy) * ra;
+          e[0] = make_double2(fma(A, h.j0, -(B * w1)), fma(B, h.j1, A * w0));
+          const double At = te * h.amp, Bt = -(fma(dx, tfx, dy * tfy) * ra);
+          et[0] = make_double2(fma(At, h.j0, -(Bt * w1)), fma(Bt, h.j1, At * w0));
+        } else {
+          const double kn = fma(tfx, qfx, tfy * qfy) * eta_inv;
+          const double j0a = h.j0 * h.amp, w0a = w0 * h.amp, w1a = w1 * ra, j1a = h.j1 * ra;
+          const double D = fma(dx, tfx, dy * tfy) * qe;
+          e[0] = make_double2(-(qe * w0a), qe * j0a);
+          e[NO - 1] = make_double2(fma(kn, e[0].y, -(D * w1a)), fma(-kn, e[0].x, D * j1a));
+          const double Dt = -(fma(dx, qfx, dy * qfy) * te);
+          et[0] = make_double2(-(te * w0a), te * j0a);
+          et[NO - 1] = make_double2(fma(kn, et[0].y, -(Dt * w1a)), fma(-kn, et[0].x, Dt * j1a));
+        }
+        if (d == 0 && i == j) {
+          e[0] = BC ? diag[2 * i] : diag[i];
+          if constexpr (BC == 1) {
+            // C_ii = -D'_ii - i (omega^2 / eta) S_ii
+            const double k = omega * omega * eta_inv;
+            const double2 D = diag[2 * i + 1];
+            e[NO - 1] = make_double2(fma(k, e[0].y, -D.x), -fma(k, e[0].x, D.y));
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int o = 0; o < NO; ++o) {
+            acc[r][o] = cmad(acc[r][o], e[o], q[r][o]);
+            if (d > 0 && ok) {
+              const double2 t = cmad(make_double2(0.0, 0.0), et[o], xi[r][o]);
+              const int k = 2 * ((b * R + r) * NO + o);
+              v[k] = t.x;
+              v[k + 1] = t.y;
+            }
+          }
+      }
+      if (d == 0) continue;
+      // value k ends in the lanes whose bits 4 .. 1 are k, then bit 0 joins
+#pragma unroll
+      for (int w = 8, o = 16; w >= 1; w /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < w; ++k) {
+          const double mine = up ? v[k + w] : v[k], other = up ? v[k] : v[k + w];
+          v[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+      }
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+      const int k = lane >> 1, o = (k >> 1) % NO, r = (k >> 1) / NO % R, b = (k >> 1) / (NO * R);
+      const int j = jb + s0 + b;
+      if (!(lane & 1) && j < n && r < nrhs)
+        reinterpret_cast<double*>(
+            part + (((size_t)o * nsp + splits + d - 1) * nrhs + r) * n + j)[k & 1] = v[0];
+    }
+  }
+  if (!ok) return;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (r < nrhs)
+#pragma unroll
+      for (int o = 0; o < NO; ++o)
+        part[(((size_t)o * nsp + blockIdx.y) * nrhs + r) * n + i] = acc[r][o];
 }
 
 // Sum split partials in a fixed order: four threads per element take every
@@ -303,26 +475,52 @@ k_spectral_fp64(int n, const double* __restrict__ ct, const double* __restrict__
 }
 
 // How one product is cut: right-hand sides per CTA, targets per CTA, source
-// splits.  Four CTAs per SM keep the FP64 pipes busy; problems of fewer 64 x 32
-// tiles than eight per SM take 32-target tiles, whose last wave is fuller
-// (n = 1024: 512 tiles on 152 SMs are 3.4 each, 1024 are 6.7).
+// splits.  Two or three CTAs fit an SM; 16 per SM fill their waves (640 CTAs of
+// star n = 4096, 16 right-hand sides, sound hard, left the FP64 pipe idle 20 %
+// of the time).  Problems of fewer 64 x 32 tiles than eight per SM take
+// 32-target tiles.
+// Up to four right-hand sides take both entries of a pair of nodes at once
+// (k_pair_sym) while its partial sums, one per block distance, stay within 512
+// MB (or the caller's scratch): n = 46000 for one sound-soft right-hand side.
 struct pair_plan {
+  int sym;                  // 0, or the right-hand sides of k_pair_sym (1, 2, 4)
   int rbt, ti, rhsblocks, splits, tps;
+  int parts;                // partial sums per output and element
 };
 
-pair_plan plan_pair(int n, int nrhs, int hard, int device, int max_splits) {
-  pair_plan p;
+pair_plan plan_pair(int n, int nrhs, int hard, int device, size_t max_parts) {
+  pair_plan p{};
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  p.rbt = nrhs <= 2 ? nrhs : (nrhs <= 4 ? 4 : (nrhs <= 16 ? 16 : (hard ? 32 : 64)));
+  const size_t vec = sizeof(double2) * (hard ? 2 : 1) * (size_t)n * nrhs;
+  if (nrhs <= 4 && n >= 192) {   // below, a warp's chain over its 8 sources is the longer one
+    const int nblk = (n + 31) / 32, units = 4 * (nblk / 2 + 1);
+    const int want = (32 * sms + nblk - 1) / nblk;       // about 32 warps per SM
+    p.tps = (units + std::min(units, want) - 1) / std::min(units, want);
+    p.splits = (units + p.tps - 1) / p.tps;
+    p.parts = p.splits + nblk / 2;
+    if ((size_t)p.parts <= max_parts && p.parts * vec <= (size_t)512 << 20) {
+      p.sym = nrhs <= 2 ? nrhs : 4;
+      return p;
+    }
+  }
+  // equal blocks of at most 64 (soft) or 32 (hard) right-hand sides, each of the
+  // smallest size that has a kernel (a kernel's sums run over its whole block)
+  const int widest = hard ? 32 : 64;
+  p.rhsblocks = (nrhs + widest - 1) / widest;
+  const int per = (nrhs + p.rhsblocks - 1) / p.rhsblocks;
+  p.rbt = per <= 2 ? per : 4;
+  for (int r : {8, 12, 16, 24, 32, 48, 64})
+    if (p.rbt < per) p.rbt = r;
   p.rhsblocks = (nrhs + p.rbt - 1) / p.rbt;
   const int ntiles = (n + TJ - 1) / TJ;
   p.ti = (long long)((n + 63) / 64) * ntiles * p.rhsblocks < 8LL * sms && p.rbt <= 16 ? 32 : 64;
   const int rows = (n + p.ti - 1) / p.ti * p.rhsblocks;
-  const int target = (p.ti == 32 ? 8 : 4) * sms;
-  p.splits = std::max(1, std::min(std::min(ntiles, max_splits), (target + rows - 1) / rows));
+  const int target = 16 * sms;   // several waves of the two or three CTAs that fit an SM
+  p.splits = std::max<int>(1, std::min<size_t>(std::min<size_t>(ntiles, max_parts),
+                                               (target + rows - 1) / rows));
   p.tps = (ntiles + p.splits - 1) / p.splits;
-  p.splits = (ntiles + p.tps - 1) / p.tps;
+  p.splits = p.parts = (ntiles + p.tps - 1) / p.tps;
   return p;
 }
 
@@ -341,13 +539,31 @@ void launch_pair(cfie_op* op, const pair_plan& p, const double2* x, const double
   CFIE_CHECK_LAUNCH();
 }
 
+template <int BC, int R>
+void launch_sym(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
+                double2* part) {
+  const int n = op->n, nblk = (n + 31) / 32;
+  const double f = 0.25 * 0.7978845608028654 * op->h;   // hq c0
+  prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
+  k_pair_sym<BC, R><<<dim3(nblk, p.splits), 32, 0, op->ctx->stream>>>(
+      n, nblk, op->omega, 1.0 / op->omega, 1.0 / op->eta, op->omega * f, BC ? f : f * op->eta,
+      p.tps, p.splits, op->g, op->wtab.as<double>() + n, op->diag.as<double2>(), x, u, nrhs, part);
+  CFIE_CHECK_LAUNCH();
+}
+
 // partial sums of every output, then their reduction (soft: into y; hard: t = S
 // u and y = 1/2 x + C x)
 template <int BC>
 void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
               double2* part, double2* t, double2* y) {
   const bool small = p.ti == 32;
-  switch (p.rbt) {
+  if (p.sym == 1)
+    launch_sym<BC, 1>(op, p, x, u, nrhs, part);
+  else if (p.sym == 2)
+    launch_sym<BC, 2>(op, p, x, u, nrhs, part);
+  else if (p.sym == 4)
+    launch_sym<BC, 4>(op, p, x, u, nrhs, part);
+  else switch (p.rbt) {
     case 1:
       small ? launch_pair<BC, 32, 1>(op, p, x, u, nrhs, part)
             : launch_pair<BC, 64, 1>(op, p, x, u, nrhs, part);
@@ -360,14 +576,24 @@ void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* 
       small ? launch_pair<BC, 32, 4>(op, p, x, u, nrhs, part)
             : launch_pair<BC, 64, 4>(op, p, x, u, nrhs, part);
       break;
+    case 8:
+      small ? launch_pair<BC, 32, 8>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 8>(op, p, x, u, nrhs, part);
+      break;
+    case 12:
+      small ? launch_pair<BC, 32, 12>(op, p, x, u, nrhs, part)
+            : launch_pair<BC, 64, 12>(op, p, x, u, nrhs, part);
+      break;
     case 16:
       small ? launch_pair<BC, 32, 16>(op, p, x, u, nrhs, part)
             : launch_pair<BC, 64, 16>(op, p, x, u, nrhs, part);
       break;
-    default:
-      launch_pair<BC, 64, BC ? 32 : 64>(op, p, x, u, nrhs, part);
+    case 24: launch_pair<BC, 64, 24>(op, p, x, u, nrhs, part); break;
+    case 32: launch_pair<BC, 64, 32>(op, p, x, u, nrhs, part); break;
+    case 48: launch_pair<0, 64, 48>(op, p, x, u, nrhs, part); break;   // sound soft only
+    default: launch_pair<0, 64, 64>(op, p, x, u, nrhs, part);
   }
-  reduce_fp64(op, part, p.splits, x, t, y, nrhs);
+  reduce_fp64(op, part, p.parts, x, t, y, nrhs);
 }
 
 }  // namespace
@@ -394,7 +620,7 @@ void matvec_fp64(cfie_op* op, const double2* x, double2* y, int nrhs) {
   const bool hard = op->bc == CFIE_SOUND_HARD;
   const pair_plan p = plan_pair(op->n, nrhs, hard, op->ctx->device, 1 << 20);
   const size_t tot = (size_t)op->n * nrhs;
-  op->partial.reserve(sizeof(double2) * (hard ? 2 : 1) * (size_t)p.splits * tot);
+  op->partial.reserve(sizeof(double2) * (hard ? 2 : 1) * (size_t)p.parts * tot);
   double2* part = op->partial.as<double2>();
   if (!hard) {
     run_pair<0>(op, p, x, nullptr, nrhs, part, nullptr, y);
@@ -492,7 +718,7 @@ void matvec_fp64_static(cfie_op* op, const double2* x, double2* y, int nrhs) {
                      "(needs " + std::to_string(need) + " bytes)");
   // device address of the array on the context's (current) device
   unsigned char* base = static_cast<unsigned char*>(static_scratch_address(op->ctx->device));
-  const int fit = (int)std::min<size_t>((kStaticScratchBytes - fixed) / per_split, 1 << 20);
+  const size_t fit = (kStaticScratchBytes - fixed) / per_split;
   const pair_plan p = plan_pair(n, nrhs, hard, op->ctx->device, fit);
   double2* part = reinterpret_cast<double2*>(base + fixed);
   if (!hard) {
