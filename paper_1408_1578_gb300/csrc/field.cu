@@ -11,20 +11,21 @@
 //
 // discretised by the plain trapezoidal rule (spectrally accurate a few node
 // spacings away from the curve), FP64 throughout with the library's own
-// Hankel evaluation.  One thread per (point, quarter of the sources), sources
-// staged in shared memory a tile at a time, the quarters added at the end.
+// Hankel evaluation.  Up to four densities: one thread per (point, quarter of
+// the sources), sources staged in shared memory a tile at a time, the quarters
+// added at the end.  More: the block kernel of sums64.cuh.
 //
-// Bound: the FP64 pipe, about 60 instructions per kernel value and 4 per
-// density, so a kernel value is shared by up to 16 densities, with a kernel for
-// every few counts; when the points alone do not fill the GPU the
-// sources are split across CTAs and a second kernel adds the splits in a
-// fixed order.
+// Bound: the FP64 pipe, about 60 instructions per kernel value, which the
+// densities of a block share.  When the points alone do not fill the GPU the
+// sources are split across CTAs and a second kernel adds the splits in a fixed
+// order.
 // Measured (GB300): 16 densities of n = 4096 nodes at 20000 points, sound hard,
-// 70.2 -> 24.9 ms.
+// 70.2 -> 10.9 ms.
 #include <algorithm>
 
 #include "hankel64.cuh"
 #include "internal.h"
+#include "sums64.cuh"
 
 namespace {
 
@@ -47,8 +48,7 @@ k_field(int n, int npts, int nrhs, int tiles_per_split, double omega, double eta
   const int tid = threadIdx.x;
   const int pl = tid % FPT, quarter = tid / FPT;
   const int p = blockIdx.x * FPT + pl;
-  const int r0 = blockIdx.y * FRB;
-  const int rn = min(FRB, nrhs - r0);
+  const int rn = min(FRB, nrhs);
   const int j_begin = blockIdx.z * tiles_per_split * FTJ;
   const int j_end = min(n, j_begin + tiles_per_split * FTJ);
   const double f = 0.25 * 0.7978845608028654 * h;   // h c0 / 4
@@ -71,7 +71,7 @@ k_field(int n, int npts, int nrhs, int tiles_per_split, double omega, double eta
     }
     for (int e = tid; e < FTJ * FRB; e += FNT) {
       const int jl = e / FRB, k = e % FRB, j = j0 + jl;
-      sq[jl][k] = (j < n && k < rn) ? q[(size_t)(r0 + k) * n + j] : make_double2(0.0, 0.0);
+      sq[jl][k] = (j < n && k < rn) ? q[(size_t)k * n + j] : make_double2(0.0, 0.0);
     }
     __syncthreads();
     if (p >= npts) continue;
@@ -110,7 +110,7 @@ k_field(int n, int npts, int nrhs, int tiles_per_split, double omega, double eta
         s.x += buf[t * FPT + pl].x;
         s.y += buf[t * FPT + pl].y;
       }
-      dst[(size_t)(r0 + k) * npts + p] = s;
+      dst[(size_t)k * npts + p] = s;
     }
   }
 }
@@ -129,52 +129,80 @@ __global__ void k_field_sum(size_t tot, int splits, const double2* __restrict__ 
   u[e] = s;
 }
 
+// about 16 CTAs per SM (two fit, so that the last of several waves is a small
+// part): source splits of `tiles` tiles for `ctas` CTAs without, with no more
+// partial sums than 256 MB, and each one's tiles
+void split_sources(cfie_op* op, size_t tot, int tiles, long long ctas, int& splits, int& tps) {
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
+  long long s = std::max<long long>(1, (16LL * sms + ctas - 1) / ctas);
+  s = std::min<long long>(s, std::min<long long>(tiles, std::max<size_t>(1, ((size_t)1 << 24) / tot)));
+  tps = (int)((tiles + s - 1) / s);
+  splits = (tiles + tps - 1) / tps;
+}
+
+// where the partial sums of several splits go, and their sum
+double2* field_partials(cfie_op* op, size_t tot, int splits, double2* u) {
+  if (splits == 1) return u;
+  op->partial.reserve(sizeof(double2) * tot * splits);
+  return op->partial.as<double2>();
+}
+void sum_splits(cfie_op* op, size_t tot, int splits, const double2* part, double2* u) {
+  if (splits == 1) return;
+  k_field_sum<<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(tot, splits, part, u);
+  CFIE_CHECK_LAUNCH();
+}
+
 template <int BC, int FRB>
 void launch_field(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts,
                   double2* u) {
-  cudaStream_t st = op->ctx->stream;
-  const int n = op->n, tiles = (n + FTJ - 1) / FTJ;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op->ctx->device);
-  const int px = (npts + FPT - 1) / FPT, ry = (nrhs + FRB - 1) / FRB;
-  // about 16 CTAs per SM (two fit, so that the last of several waves is a small
-  // part), as many splits of the sources as that takes (no more partial sums
-  // than 256 MB)
+  const int n = op->n, px = (npts + FPT - 1) / FPT;
   const size_t tot = (size_t)nrhs * npts;
-  long long splits = std::max<long long>(1, (16LL * sms + (long long)px * ry - 1) / ((long long)px * ry));
-  splits = std::min<long long>(splits, std::min<long long>(tiles, std::max<size_t>(1, ((size_t)1 << 24) / tot)));
-  const int tps = (int)((tiles + splits - 1) / splits);
-  const int ns = (tiles + tps - 1) / tps;
-  double2* out = u;
-  if (ns > 1) {
-    op->partial.reserve(sizeof(double2) * tot * ns);
-    out = op->partial.as<double2>();
-  }
-  k_field<BC, FRB><<<dim3(px, ry, ns), FNT, 0, st>>>(n, npts, nrhs, tps, op->omega, op->eta, op->h,
-                                                     op->g, pts, q, out);
+  int splits, tps;
+  split_sources(op, tot, (n + FTJ - 1) / FTJ, px, splits, tps);
+  double2* out = field_partials(op, tot, splits, u);
+  k_field<BC, FRB><<<dim3(px, 1, splits), FNT, 0, op->ctx->stream>>>(
+      n, npts, nrhs, tps, op->omega, op->eta, op->h, op->g, pts, q, out);
   CFIE_CHECK_LAUNCH();
-  if (ns > 1) {
-    k_field_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, ns, out, u);
-    CFIE_CHECK_LAUNCH();
-  }
+  sum_splits(op, tot, splits, out, u);
+}
+
+// five and more densities: entries shared by up to 64, sums on the integer units
+void launch_block_field(cfie_op* op, bool hard, const double2* q, int nrhs, int npts,
+                        const double2* pts, double2* u) {
+  const double f = 0.25 * 0.7978845608028654 * op->h;   // h c0 / 4
+  const int width = sums64::block_width(nrhs, false), ti = sums64::block_rows(width, false);
+  const size_t tot = (size_t)nrhs * npts;
+  sums64::block_args a{};
+  split_sources(op, tot, (op->n + sums64::TJ - 1) / sums64::TJ,
+                (long long)((npts + ti - 1) / ti) * ((nrhs + width - 1) / width), a.splits,
+                a.tiles_per_split);
+  a.n = op->n;
+  a.rows = npts;
+  a.nrhs = nrhs;
+  a.rotate = hard;   // -S + D / (i eta) = -i (D / eta - i S)
+  a.omega = op->omega;
+  a.omega_inv = 1.0 / op->omega;
+  a.nf = hard ? op->omega * f / op->eta : op->omega * f;
+  a.sf = hard ? f : op->eta * f;
+  a.g = op->g;
+  a.pts = pts;
+  a.x = q;
+  a.out = field_partials(op, tot, a.splits, u);
+  sums64::run_block<sums64::FIELD>(a, ti, width, op->ctx->stream);
+  sum_splits(op, tot, a.splits, a.out, u);
 }
 
 template <int BC>
 void field_bc(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts, double2* u) {
-  // equal blocks of at most 16 densities
-  const int blocks = (nrhs + 15) / 16, per = (nrhs + blocks - 1) / blocks;
-  if (per == 1)
+  if (nrhs > 4)
+    launch_block_field(op, BC == 1, q, nrhs, npts, pts, u);
+  else if (nrhs == 1)
     launch_field<BC, 1>(op, q, nrhs, npts, pts, u);
-  else if (per == 2)
+  else if (nrhs == 2)
     launch_field<BC, 2>(op, q, nrhs, npts, pts, u);
-  else if (per <= 4)
-    launch_field<BC, 4>(op, q, nrhs, npts, pts, u);
-  else if (per <= 8)
-    launch_field<BC, 8>(op, q, nrhs, npts, pts, u);
-  else if (per <= 12)
-    launch_field<BC, 12>(op, q, nrhs, npts, pts, u);
   else
-    launch_field<BC, 16>(op, q, nrhs, npts, pts, u);
+    launch_field<BC, 4>(op, q, nrhs, npts, pts, u);
 }
 
 }  // namespace

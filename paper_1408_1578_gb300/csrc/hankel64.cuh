@@ -279,8 +279,9 @@ __device__ __forceinline__ void fill_tables(int j, double2* __restrict__ tab) {
 //   hard (eq. 2):  se = hq c0 |z'_j|, tx, ty = omega nu_i / |z'_i|;  A = se amp,
 //                  D = ((dx, dy) . (tx, ty)) A / r
 //                  S  = -A (y0 + wk j0) + i A j0,  D' = D (y1 + wk j1) - i D j1
-// omega_inv = 1 / omega, tab = the operator's tables.
-template <int BC>
+// omega_inv = 1 / omega, tab = the operator's tables.  KRESS false: no Kress term
+// (points off the curve).
+template <int BC, bool KRESS = true>
 __device__ __forceinline__ void pair_folded_fp64(double dx, double dy, double omega,
                                                  double omega_inv, double fx, double fy, double se,
                                                  double wk, const double2* __restrict__ tab,
@@ -289,7 +290,7 @@ __device__ __forceinline__ void pair_folded_fp64(double dx, double dy, double om
   h64::distance(fma(dx, dx, dy * dy), r, rinv);
   const h64::values v = h64::bessel01(omega * r, omega_inv * rinv, tab);
   const double A = se * v.amp;
-  const double w0 = fma(wk, v.j0, v.y0), w1 = fma(wk, v.j1, v.y1);
+  const double w0 = KRESS ? fma(wk, v.j0, v.y0) : v.y0, w1 = KRESS ? fma(wk, v.j1, v.y1) : v.y1;
   const double p = fma(dx, fx, dy * fy);
   if constexpr (BC == 0) {
     const double B = p * (rinv * v.amp);

@@ -19,23 +19,26 @@
 //          per right-hand side and pair fewer than S on three vectors and D')
 // Diagonal entries come precomputed (geometry.cu).
 //
-// Layout: a CTA of 4 TI threads owns TI = 64 (small problems: 32) targets and
-// walks a contiguous range of source tiles (TJ = 32 sources each).  For every
-// tile it evaluates the TI x TJ block of entries into shared memory (one warp
-// per target row, lanes over sources), then contracts it with the staged block
-// of right-hand sides.  Source ranges are split across CTAs when the row tiles
-// alone do not fill the GPU; the per-split partial sums go to a scratch buffer
-// and a second kernel adds them in a fixed order (deterministic results) and
-// applies the hard-path epilogue.
+// Kernels, by the number of right-hand sides:
+//   five and more: sums64.cuh (entries shared by a block of columns, its sums on
+//     the integer units)
+//   up to four: k_pair_sym (both entries of a pair of nodes at once)
+//   up to four of small problems, or where the transposed sums do not fit:
+//     k_pair_fp64.  A CTA of 4 TI threads owns TI = 64 (small problems: 32)
+//     targets and walks a contiguous range of source tiles (TJ = 32 sources
+//     each).  For every tile it evaluates the TI x TJ block of entries into
+//     shared memory (one warp per target row, lanes over sources), then
+//     contracts it with the staged block of right-hand sides; with one or two
+//     of those the threads split the sources instead.
+// In all of them source ranges are split across CTAs when the row tiles alone
+// do not fill the GPU; the per-split partial sums go to a scratch buffer and a
+// second kernel adds them in a fixed order (deterministic results) and applies
+// the hard-path epilogue.
 //
 // Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
-// scheduler): per pair about 70 instructions for the entry (hankel64.cuh) and
-// 4 (soft) or 8 (hard) per right-hand side for the sums, so there is a kernel
-// for every few widths of a block (hardly any sums on padding columns; with one
-// or two the threads split the sources instead) and the entry is shared by up
-// to 64 (soft) or 32 (hard) of them.
-// Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 215 us; star n =
-// 4096, 16 right-hand sides, sound hard 15.8 -> 7.4 ms (of which 6.9 here).
+// scheduler): per pair about 70 instructions for the entry (hankel64.cuh).
+// Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 138 us; star n =
+// 4096, 16 right-hand sides, sound hard 15.8 -> 3.2 ms.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -44,6 +47,7 @@
 
 #include "internal.h"
 #include "hankel64.cuh"
+#include "sums64.cuh"
 
 namespace {
 
@@ -504,17 +508,11 @@ pair_plan plan_pair(int n, int nrhs, int hard, int device, size_t max_parts) {
       return p;
     }
   }
-  // equal blocks of at most 64 (soft) or 32 (hard) right-hand sides, each of the
-  // smallest size that has a kernel (a kernel's sums run over its whole block)
-  const int widest = hard ? 32 : 64;
-  p.rhsblocks = (nrhs + widest - 1) / widest;
-  const int per = (nrhs + p.rhsblocks - 1) / p.rhsblocks;
-  p.rbt = per <= 2 ? per : 4;
-  for (int r : {8, 12, 16, 24, 32, 48, 64})
-    if (p.rbt < per) p.rbt = r;
+  p.rbt = nrhs <= 2 ? nrhs : nrhs <= 4 ? 4 : sums64::block_width(nrhs, hard);
   p.rhsblocks = (nrhs + p.rbt - 1) / p.rbt;
   const int ntiles = (n + TJ - 1) / TJ;
-  p.ti = (long long)((n + 63) / 64) * ntiles * p.rhsblocks < 8LL * sms && p.rbt <= 16 ? 32 : 64;
+  p.ti = (long long)((n + 63) / 64) * ntiles * p.rhsblocks < 8LL * sms ? 32 : 64;
+  if (p.rbt > 4) p.ti = std::min(p.ti, sums64::block_rows(p.rbt, hard));
   const int rows = (n + p.ti - 1) / p.ti * p.rhsblocks;
   const int target = 16 * sms;   // several waves of the two or three CTAs that fit an SM
   p.splits = std::max<int>(1, std::min<size_t>(std::min<size_t>(ntiles, max_parts),
@@ -563,35 +561,35 @@ void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* 
     launch_sym<BC, 2>(op, p, x, u, nrhs, part);
   else if (p.sym == 4)
     launch_sym<BC, 4>(op, p, x, u, nrhs, part);
-  else switch (p.rbt) {
-    case 1:
-      small ? launch_pair<BC, 32, 1>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 1>(op, p, x, u, nrhs, part);
-      break;
-    case 2:
-      small ? launch_pair<BC, 32, 2>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 2>(op, p, x, u, nrhs, part);
-      break;
-    case 4:
-      small ? launch_pair<BC, 32, 4>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 4>(op, p, x, u, nrhs, part);
-      break;
-    case 8:
-      small ? launch_pair<BC, 32, 8>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 8>(op, p, x, u, nrhs, part);
-      break;
-    case 12:
-      small ? launch_pair<BC, 32, 12>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 12>(op, p, x, u, nrhs, part);
-      break;
-    case 16:
-      small ? launch_pair<BC, 32, 16>(op, p, x, u, nrhs, part)
-            : launch_pair<BC, 64, 16>(op, p, x, u, nrhs, part);
-      break;
-    case 24: launch_pair<BC, 64, 24>(op, p, x, u, nrhs, part); break;
-    case 32: launch_pair<BC, 64, 32>(op, p, x, u, nrhs, part); break;
-    case 48: launch_pair<0, 64, 48>(op, p, x, u, nrhs, part); break;   // sound soft only
-    default: launch_pair<0, 64, 64>(op, p, x, u, nrhs, part);
+  else if (p.rbt == 1)
+    small ? launch_pair<BC, 32, 1>(op, p, x, u, nrhs, part)
+          : launch_pair<BC, 64, 1>(op, p, x, u, nrhs, part);
+  else if (p.rbt == 2)
+    small ? launch_pair<BC, 32, 2>(op, p, x, u, nrhs, part)
+          : launch_pair<BC, 64, 2>(op, p, x, u, nrhs, part);
+  else if (p.rbt == 4)
+    small ? launch_pair<BC, 32, 4>(op, p, x, u, nrhs, part)
+          : launch_pair<BC, 64, 4>(op, p, x, u, nrhs, part);
+  else {
+    const double f = 0.25 * 0.7978845608028654 * op->h;   // hq c0
+    prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
+    sums64::block_args a{};
+    a.n = a.rows = op->n;
+    a.nrhs = nrhs;
+    a.splits = p.splits;
+    a.tiles_per_split = p.tps;
+    a.omega = op->omega;
+    a.omega_inv = 1.0 / op->omega;
+    a.nf = op->omega * f;
+    a.sf = BC ? f : f * op->eta;
+    a.eta_inv = 1.0 / op->eta;
+    a.g = op->g;
+    a.wks = op->wtab.as<double>() + op->n;
+    a.diag = op->diag.as<double2>();
+    a.x = x;
+    a.u = u;
+    a.out = part;
+    sums64::run_block<BC>(a, p.ti, p.rbt, op->ctx->stream);
   }
   reduce_fp64(op, part, p.parts, x, t, y, nrhs);
 }

@@ -1,0 +1,312 @@
+// Sums of FP64 kernel entries over a block of right-hand sides, on the integer
+// units: y_r(i) = sum_j K_ij x_r(j) for five and more columns r.
+//
+// GB300 has 1.7 lanes of FP64 multiply-add per clock and SM, and 25 of 32 x 32
+// -> 64-bit integer multiply-add.  An entry takes about 60 FP64 instructions
+// (hankel64.cuh); its sums took 4 more per right-hand side, twice that for the
+// sound-hard operator's two.  Here a tile of 32 sources works in fixed point:
+// the 32 entries of a row share the exponent of the largest of them, the 32
+// densities of a column share theirs, each number is rounded to 57 bits and a
+// sign below it and kept as two 29-bit limbs.  Three integer multiply-adds
+// (high x high, the two mixed products) give a real product, the tile's sums
+// stay below 2^63, and at its end one conversion and one FP64 multiply-add take
+// each of them to the FP64 accumulator.  Within a tile an addend is off by
+// less than 2^-57 of the largest entry times the largest density, and
+// additions are exact, where FP64 rounds each to 2^-53 of the sum so far.
+// Measured (GB300): star n = 4096, 16 right-hand sides, sound hard, 6.2 -> 3.2 ms;
+// 16 densities at 20000 points 20.7 -> 10.9 ms.
+//
+// A tile with a value that this does not hold (infinities, NaN, exponents
+// beyond 2^+-420) takes FP64 multiply-adds instead.
+//
+// Layout: a CTA owns TI rows and walks its range of source tiles.  It evaluates
+// the TI x 32 block of entries into shared memory (one warp per row, lanes over
+// sources: the row's exponent is one reduction), then thread (row, group)
+// contracts its row with RBT / RG of the columns.
+#pragma once
+#include "hankel64.cuh"
+#include "internal.h"
+
+namespace sums64 {
+
+constexpr int TJ = 32;
+enum { SOFT = 0, HARD = 1, FIELD = 2 };
+
+// a number v < 2^(E - 1022), E a biased exponent, as v 2^(1079 - E) = hi 2^29 + lo
+// rounded to the nearest integer (|hi|, |lo| <= 2^28)
+__device__ __forceinline__ void to_limbs(double v, int E, int& hi, int& lo) {
+  const int h = __double2hiint(v), e = (h >> 20) & 0x7ff;
+  unsigned long long m =
+      ((unsigned long long)((h & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 5;
+  m = e ? m >> min(E - e, 63) : 0;   // subnormals round to zero
+  long long V = (long long)((m + 1) >> 1);
+  if (h < 0) V = -V;
+  hi = (int)((V + (1 << 28)) >> 29);
+  lo = (int)((unsigned)V - ((unsigned)hi << 29));
+}
+__device__ __forceinline__ double from_limbs(int hi, int lo, int E) {
+  if (E == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
+  return scalbn((double)(((long long)hi << 29) + lo), E - 1079);
+}
+__device__ __forceinline__ int4 to_limbs(double2 v, int E) {
+  int4 q;
+  to_limbs(v.x, E, q.x, q.y);
+  to_limbs(v.y, E, q.z, q.w);
+  return q;
+}
+// exponent of the largest of a warp's values; bad: one that the fixed-point sums
+// do not hold.  Zeros only: any exponent in range does.
+__device__ __forceinline__ int shared_exponent(double2 v, bool& bad) {
+  const unsigned a = __double2hiint(v.x) & 0x7fffffff, b = __double2hiint(v.y) & 0x7fffffff;
+  const int E = (int)(__reduce_max_sync(0xffffffffu, max(a, b)) >> 20);
+  if (E >= 600 && E <= 1500) return E;
+  bad |= __any_sync(0xffffffffu, (a | b | __double2loint(v.x) | __double2loint(v.y)) != 0);
+  return E ? E : 1023;
+}
+
+// sums of products of limbs: high x high, and the mixed ones 2^29 below
+struct fixed_acc {
+  long long h, m;
+  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
+    h += (long long)ah * bh;
+    m += (long long)ah * bl;
+    m += (long long)al * bh;
+  }
+  // scale: the high word of 2^(Ek + Ex - 2100)
+  __device__ __forceinline__ void flush(double& acc, int scale) const {
+    acc = fma((double)(h + ((m + (1 << 28)) >> 29)), __hiloint2double(scale, 0), acc);
+  }
+};
+
+struct block_args {
+  int n, rows, nrhs, splits, tiles_per_split;
+  bool rotate;                         // FIELD: times -i (sound hard)
+  double omega, omega_inv;
+  double nf, sf;                       // factors of the normal (HARD: of none) and the speed
+  double eta_inv;                      // HARD
+  geom_dev g;
+  const double* wks;                   // Kress weights / (pi h)
+  const double2 *diag, *pts, *x, *u;   // pts: FIELD; u: HARD
+  double2* out;                        // [output][split][column][row]
+};
+
+template <int MODE, int TI, int RBT>
+struct block_smem {
+  static constexpr int NO = MODE == HARD ? 2 : 1;
+  double tx[TI], ty[TI];
+  double tfx[NO == 2 ? TI : 1], tfy[NO == 2 ? TI : 1];   // HARD: omega nu / |z'|
+  double sx[TJ], sy[TJ], sfx[TJ], sfy[TJ], se[TJ];
+  double wk[TI + TJ];                    // Kress weights of the tile, by i - j
+  int4 K[NO][TI][TJ + 1];                // limbs (re, im): the entries; HARD: S, C
+  int4 X[NO][TJ][RBT];                   // densities; HARD: u, x
+  int ek[NO][TI], ex[NO][RBT];
+};
+
+template <int MODE, int TI, int RBT, int RG>
+__global__ void __launch_bounds__(TI* RG, 512 / (TI * RG))
+k_block64(block_args p) {
+  constexpr int NT = TI * RG, RQ = RBT / RG;
+  constexpr int NO = MODE == HARD ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  block_smem<MODE, TI, RBT>& S = *reinterpret_cast<block_smem<MODE, TI, RBT>*>(smem_raw);
+  const geom_dev& g = p.g;
+  const int tid = threadIdx.x, lane = tid & 31, n = p.n;
+  const int i0 = blockIdx.x * TI;
+  const int rb0 = blockIdx.z * RBT;
+  const int rbn = min(RBT, p.nrhs - rb0);
+  const int t_begin = blockIdx.y * p.tiles_per_split;
+  const int t_end = min((n + TJ - 1) / TJ, t_begin + p.tiles_per_split);
+
+  if (tid < TI) {
+    const int i = i0 + tid;
+    const bool ok = i < p.rows;
+    if constexpr (MODE == FIELD) {
+      const double2 z = ok ? p.pts[i] : make_double2(0.0, 0.0);
+      S.tx[tid] = z.x;
+      S.ty[tid] = z.y;
+    } else {
+      S.tx[tid] = ok ? g.x[i] : 0.0;
+      S.ty[tid] = ok ? g.y[i] : 0.0;
+    }
+    if constexpr (MODE == HARD) {
+      const double inv = ok ? p.omega / g.sp[i] : 0.0;
+      S.tfx[tid] = ok ? g.nx[i] * inv : 0.0;
+      S.tfy[tid] = ok ? g.ny[i] * inv : 0.0;
+    }
+  }
+
+  const int row = tid % TI, rg = tid / TI;
+  double2 acc[NO][RQ];
+#pragma unroll
+  for (int o = 0; o < NO; ++o)
+#pragma unroll
+    for (int q = 0; q < RQ; ++q) acc[o][q] = make_double2(0.0, 0.0);
+
+  for (int t = t_begin; t < t_end; ++t) {
+    const int j0 = t * TJ;
+    bool bad = false;
+    __syncthreads();
+    if (tid < TJ) {
+      const int j = j0 + tid;
+      const bool ok = j < n;
+      const double sp = ok ? g.sp[j] : 1.0;
+      const double m = MODE == HARD ? p.omega / sp : p.nf;
+      S.sx[tid] = ok ? g.x[j] : 0.0;
+      S.sy[tid] = ok ? g.y[j] : 0.0;
+      S.sfx[tid] = ok ? m * g.nx[j] : 0.0;
+      S.sfy[tid] = ok ? m * g.ny[j] : 0.0;
+      S.se[tid] = p.sf * sp;
+    }
+    if constexpr (MODE != FIELD)
+      for (int e = tid; e < TI + TJ - 1; e += NT) {
+        int d = (i0 - j0 + e - (TJ - 1)) % n;
+        if (d < 0) d += n;
+        S.wk[e] = p.wks[d];
+      }
+    for (int c = tid / 32; c < NO * RBT; c += NT / 32) {
+      const int o = c / RBT, r = c % RBT, j = j0 + lane;
+      const double2* src = o == NO - 1 ? p.x : p.u;
+      const double2 v = j < n && r < rbn ? src[(size_t)(rb0 + r) * n + j] : make_double2(0.0, 0.0);
+      const int E = shared_exponent(v, bad);
+      S.X[o][lane][r] = to_limbs(v, E);
+      if (lane == 0) S.ex[o][r] = E;
+    }
+    __syncthreads();
+
+    // ---- entries of the TI x TJ block
+    for (int il = tid / 32; il < TI; il += NT / 32) {
+      const int i = i0 + il, j = j0 + lane;
+      double2 a = make_double2(0.0, 0.0), b = a;
+      if (i < p.rows && j < n) {
+        if (MODE != FIELD && i == j) {
+          a = MODE == HARD ? p.diag[2 * i] : p.diag[i];
+          if (MODE == HARD) b = p.diag[2 * i + 1];
+        } else {
+          pair_folded_fp64<MODE == HARD, MODE != FIELD>(
+              S.tx[il] - S.sx[lane], S.ty[il] - S.sy[lane], p.omega, p.omega_inv,
+              MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
+              S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
+        }
+      }
+      if (MODE == FIELD && p.rotate) a = make_double2(a.y, -a.x);
+      int E = shared_exponent(a, bad);
+      S.K[0][il][lane] = to_limbs(a, E);
+      if (lane == 0) S.ek[0][il] = E;
+      if constexpr (MODE == HARD) {
+        // C = -D' - i (omega^2 / eta) (n_i . n_j) S
+        const double k = fma(S.tfx[il], S.sfx[lane], S.tfy[il] * S.sfy[lane]) * p.eta_inv;
+        const double2 c = make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y));
+        E = shared_exponent(c, bad);
+        S.K[NO - 1][il][lane] = to_limbs(c, E);
+        if (lane == 0) S.ek[NO - 1][il] = E;
+      }
+    }
+
+    // ---- contraction
+    if (__syncthreads_or(bad)) {
+      for (int jl = 0; jl < min(TJ, n - j0); ++jl)
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+          const int4 k = S.K[o][row][jl];
+          const double kr = from_limbs(k.x, k.y, S.ek[o][row]);
+          const double ki = from_limbs(k.z, k.w, S.ek[o][row]);
+          const double2* src = o == NO - 1 ? p.x : p.u;
+#pragma unroll
+          for (int q = 0; q < RQ; ++q) {
+            const int r = rg + RG * q;
+            if (r >= rbn) continue;
+            const double2 v = src[(size_t)(rb0 + r) * n + j0 + jl];
+            acc[o][q].x = fma(-ki, v.y, fma(kr, v.x, acc[o][q].x));
+            acc[o][q].y = fma(ki, v.x, fma(kr, v.y, acc[o][q].y));
+          }
+        }
+      continue;
+    }
+    fixed_acc re[NO][RQ], im[NO][RQ];
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+      for (int q = 0; q < RQ; ++q) re[o][q] = im[o][q] = fixed_acc{0, 0};
+#pragma unroll 2
+    for (int jl = 0; jl < TJ; ++jl)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const int4 k = S.K[o][row][jl];
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+          const int4 v = S.X[o][jl][rg + RG * q];
+          re[o][q].add(k.x, k.y, v.x, v.y);
+          re[o][q].add(-k.z, -k.w, v.z, v.w);
+          im[o][q].add(k.x, k.y, v.z, v.w);
+          im[o][q].add(k.z, k.w, v.x, v.y);
+        }
+      }
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+      for (int q = 0; q < RQ; ++q) {
+        const int scale = (S.ek[o][row] + S.ex[o][rg + RG * q] - 1077) << 20;
+        re[o][q].flush(acc[o][q].x, scale);
+        im[o][q].flush(acc[o][q].y, scale);
+      }
+  }
+
+  const int i = i0 + row;
+  if (i >= p.rows) return;
+#pragma unroll
+  for (int q = 0; q < RQ; ++q) {
+    const int r = rg + RG * q;
+    if (r < rbn)
+#pragma unroll
+      for (int o = 0; o < NO; ++o)
+        p.out[(((size_t)o * p.splits + blockIdx.y) * p.nrhs + rb0 + r) * p.rows + i] = acc[o][q];
+  }
+}
+
+template <int MODE, int TI, int RBT, int RG>
+void launch_block(const block_args& p, cudaStream_t stream) {
+  const size_t smem = sizeof(block_smem<MODE, TI, RBT>);
+  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_block64<MODE, TI, RBT, RG>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const dim3 grid((p.rows + TI - 1) / TI, p.splits, (p.nrhs + RBT - 1) / RBT);
+  k_block64<MODE, TI, RBT, RG><<<grid, TI * RG, smem, stream>>>(p);
+  CFIE_CHECK_LAUNCH();
+}
+
+// Columns per CTA: equal blocks of at most 64 (sound hard, where a column is two
+// sums: 32), each of the smallest width that has a kernel.
+inline int block_width(int nrhs, bool hard) {
+  const int widest = hard ? 32 : 64, blocks = (nrhs + widest - 1) / widest;
+  const int per = (nrhs + blocks - 1) / blocks;
+  for (int r : {8, 12, 16, 24, 32, 48})
+    if (per <= r) return r;
+  return 64;
+}
+// Rows per CTA: the sums of 64 rows and 32 columns (sound hard: 16) fill the
+// registers of the two CTAs that an SM holds; wider blocks have 32 rows.
+inline int block_rows(int width, bool hard) { return width > (hard ? 16 : 32) ? 32 : 64; }
+
+template <int MODE, int RBT>
+void run_width(const block_args& p, int ti, cudaStream_t stream) {
+  if constexpr (RBT > (MODE == HARD ? 16 : 32))
+    launch_block<MODE, 32, RBT, 8>(p, stream);
+  else if (ti == 32)
+    launch_block<MODE, 32, RBT, 4>(p, stream);
+  else
+    launch_block<MODE, 64, RBT, 4>(p, stream);
+}
+
+template <int MODE>
+void run_block(const block_args& p, int ti, int width, cudaStream_t stream) {
+  switch (width) {
+    case 8: run_width<MODE, 8>(p, ti, stream); break;
+    case 12: run_width<MODE, 12>(p, ti, stream); break;
+    case 16: run_width<MODE, 16>(p, ti, stream); break;
+    case 24: run_width<MODE, 24>(p, ti, stream); break;
+    case 32: run_width<MODE, 32>(p, ti, stream); break;
+    case 48: if constexpr (MODE != HARD) run_width<MODE, 48>(p, ti, stream); break;
+    default: if constexpr (MODE != HARD) run_width<MODE, 64>(p, ti, stream);
+  }
+}
+
+}  // namespace sums64

@@ -74,3 +74,55 @@ def test_field_splits(ctx, bc, npts, nrhs):
     want = np.stack([ofield.scattered_field(c, omega, omega, bc, q[k], xy) for k in range(nrhs)])
     assert np.max(np.abs(to_host(u) - want)) < TOL * np.max(np.abs(want))
     op.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+@pytest.mark.parametrize("n", [98, 1026])
+def test_fixed_point_sums_scales(ctx, bc, n):
+    """Sums in fixed point per tile of 32 sources: columns of any scale (those beyond 2^+-420
+    take FP64 sums), a tile of zeros, a range of 1e12 over the nodes, every block width.
+    Scaling by a power of two commutes with the product except for subnormal rounding."""
+    omega = n / 16.0
+    A = operators.cfie_matrix(geometry.kite(n), omega, omega, bc)
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp64")
+    for nrhs in (8, 12, 13, 24, 32, 48, 64):
+        X = inputs.random_density(n, nrhs, seed=nrhs)
+        X[1] *= 2.0 ** 900
+        X[2] *= 2.0 ** -900
+        X[3, 32:64] = 0.0
+        X[4] *= np.exp(-27.0 * np.linspace(0, 1, n))
+        x, y = to_dev(X), empty(nrhs, n)
+        op.apply_fp64(x, y)
+        got, want = to_host(y), (A @ X.T).T
+        s = np.ones(nrhs)
+        s[1], s[2] = 2.0 ** -900, 2.0 ** 900
+        assert np.max(col_rel(got * s[:, None], want * s[:, None])) < TOL, nrhs
+        # infinities and NaN stay in their columns
+        X[5, n // 3], X[6, 0] = np.inf, np.nan
+        op.apply_fp64(to_dev(X), y)
+        bad = to_host(y)
+        assert not np.isfinite(bad[5:7]).any()
+        keep = np.r_[0:5, 7:nrhs]
+        assert np.max(col_rel(bad[keep] * s[keep, None], want[keep] * s[keep, None])) < TOL, nrhs
+    op.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+@pytest.mark.parametrize("nrhs", [8, 12, 24, 40, 64])
+def test_field_block_widths(ctx, bc, nrhs):
+    n, omega, npts = 130, 9.0, 97
+    q = inputs.random_density(n, nrhs, seed=7)
+    q[2] *= 2.0 ** -900
+    rng = np.random.default_rng(nrhs)
+    pts = rng.uniform(2.0, 30.0, npts) * np.exp(2j * np.pi * rng.uniform(size=npts))
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp64")
+    u = empty(nrhs, npts)
+    op.field_eval(to_dev(q), to_dev(pts), u)
+    q[2] *= 2.0 ** 900
+    xy = np.stack([pts.real, pts.imag], 1)
+    want = np.stack([ofield.scattered_field(geometry.kite(n), omega, omega, bc, q[k], xy)
+                     for k in range(nrhs)])
+    got = to_host(u)
+    got[2] *= 2.0 ** 900
+    assert np.max(np.abs(got - want)) < TOL * np.max(np.abs(want))
+    op.close()
