@@ -15,12 +15,12 @@
 // the sources), sources staged in shared memory a tile at a time, the quarters
 // added at the end.  More: the block kernel of sums64.cuh.
 //
-// Bound: the FP64 pipe, about 60 instructions per kernel value, which the
+// Bound: the FP64 pipe, about 36 instructions per kernel value, which the
 // densities of a block share.  When the points alone do not fill the GPU the
 // sources are split across CTAs and a second kernel adds the splits in a fixed
 // order.
 // Measured (GB300): 16 densities of n = 4096 nodes at 20000 points, sound hard,
-// 70.2 -> 10.9 ms.
+// 70.2 -> 7.4 ms.
 #include <algorithm>
 
 #include "hankel64.cuh"

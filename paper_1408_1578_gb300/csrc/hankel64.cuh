@@ -2,13 +2,11 @@
 // of G(x, y) = (i/4) H0^(1)(omega |x - y|), paper Section 1), written from
 // published methods and tested against scipy / mpmath values:
 //
-//  x >= 20: Hankel's asymptotic expansion (Abramowitz & Stegun 9.2.5, 9.2.9,
-//           9.2.10):  H_nu^(1)(x) = sqrt(2/(pi x)) (P + i Q) exp(i chi),
-//           chi = x - (nu/2 + 1/4) pi,  P = sum_k (-1)^k a_2k x^-2k,
-//           Q = sum_k (-1)^k a_(2k+1) x^-(2k+1),
-//           a_k(nu) = prod_{m=1..k} (4 nu^2 - (2m-1)^2) / (8^k k!).
-//           Twenty-one terms reach double precision for x >= 20; fewer do
-//           further out (thirteen from 40, nine from 100, six from 400).
+//  x >= 20: Hankel's asymptotic expansion as modulus and phase (Abramowitz & Stegun
+//           9.2.28, 9.2.29): H_nu^(1)(x) = sqrt(2/(pi x)) m exp(i theta) with
+//           m = 1 + O(x^-2), theta = x - (nu/2 + 1/4) pi + O(1/x).  Eleven terms
+//           of each reach double precision for x >= 20; fewer do further out
+//           (eight from 32, five from 64).
 //  x <  20: J0 and g = Y0 - (2/pi) ln(x/2) J0, both entire, from their Taylor
 //           polynomials about the nearest multiple of 1/2 (degree 13: the next
 //           term is below 1e-18), with J1 = -J0' and Y1 = -Y0' from the same
@@ -19,43 +17,59 @@
 // lanes per clock and SM, latency 64 clocks), so a pair costs what its FP64
 // instructions cost and nothing else: shared square roots and reciprocals
 // (Newton's method from the special-function unit's estimate, which runs off
-// the FP64 pipe), one table look-up for sine and cosine, per-node factors.
-// About 70 FP64 instructions per far pair; 150 with the library's sqrt,
-// division and sincos and the full series everywhere.
+// the FP64 pipe), one table look-up for sine and cosine, per-node factors.  What
+// is small is kept off the FP64 pipe: everything that is added to the table's
+// sine and cosine is below 0.03, so that packed FP32 double-floats give it, and
+// FP64 numbers are taken apart and joined with integer instructions.
+// About 43 FP64 instructions per far pair of the sound-hard operator; 70 with the
+// series and the rotation in FP64, 150 with the library's sqrt, division and
+// sincos besides.  Measured (GB300), series in FP64 -> here: circle n = 1024, one
+// right-hand side 138 -> 96 us; star n = 4096, 16, sound hard 3.2 -> 2.35 ms; field of
+// 16 densities at 20000 points 10.9 -> 7.4 ms.  Values against quadruple
+// precision, rms over 20 < x < 50000: 3.8e-17 .. 6.3e-17 times amp (FP64
+// series 6.5e-17 .. 7.4e-17).
 #pragma once
 
 #include "internal.h"
+#include "packed32.cuh"
 
 namespace h64 {
 
-// a_k(nu) of the asymptotic expansion with the alternating sign folded in
-static __constant__ double kP0[11] = {1.0, -0.0703125, 0.112152099609375, -0.5725014209747314,
-                               6.074042001273483, -110.01714026924674, 3038.090510922384,
-                               -118838.42625678325, 6252951.493434797, -425939216.5047669,
-                               36468400807.06556};
-static __constant__ double kQ0[10] = {-0.125, 0.0732421875, -0.22710800170898438, 1.7277275025844574,
-                               -24.380529699556064, 551.3358961220206, -18257.755474293175,
-                               832859.3040162893, -50069589.531988926, 3836255180.2304335};
-static __constant__ double kP1[11] = {1.0, 0.1171875, -0.144195556640625, 0.6765925884246826,
-                               -6.883914268109947, 121.59789187653587, -3302.2722944808525,
-                               127641.2726461746, -6656367.718817688, 450278600.3050393,
-                               -38338575207.427895};
-static __constant__ double kQ1[10] = {0.375, -0.1025390625, 0.2775764465332031, -1.993531733751297,
-                               27.248827311268542, -603.8440767050702, 19718.37591223663,
-                               -890297.8767070678, 53104110.10968523, -4043620325.107754};
+// H_nu^(1)(x) = sqrt(2/(pi x)) m exp(i (x - (nu/2 + 1/4) pi + psi)), t = 1 / x:
+//   m = 1 + sum_k kMod[k-1] t^2k, psi = sum_k kPsi[k-1] t^(2k-1)
+// lane x: nu = 0, lane y: nu = 1.  From the series of m^2 (A&S 9.2.28), its
+// square root, and psi' = 1 / m^2 - 1 term by term.
+constexpr int kFarTerms = 11;
+static __constant__ float2 kMod[kFarTerms] = {
+    {-0.0625f, 0.1875f}, {0.103515625f, -0.193359375f}, {-0.5428466796875f, 0.8052978515625f},
+    {5.848699569702148f, -7.739953994750977f}, {-106.8867939710617f, 132.76182425022125f},
+    {2968.1429378427565f, -3543.303665366024f}, {-116538.47969683609f, 135394.22856918094f},
+    {6148451.462878801f, -7003141.574752433f}, {-419670939.1557855f, 470832610.30922693f},
+    {35988758012.12494f, -39896618143.18781f}, {-3787947157068.18f, 4158798688522.596f}};
+static __constant__ float2 kPsi[kFarTerms] = {
+    {-0.125f, 0.375f}, {0.06510416666666667f, -0.1640625f}, {-0.2095703125f, 0.3708984375f},
+    {1.6380658830915178f, -2.3693978445870534f}, {-23.475127749972874f, 30.624011993408203f},
+    {535.640519510616f, -659.185221823779f}, {-17837.279688947478f, 21156.314045527808f},
+    {816737.8421910767f, -944346.6095480548f}, {-49232732.339998595f, 55869739.657019265f},
+    {3779795380.667541f, -4228159535.534621f}, {-360101552365.56555f, 398251272117.5241f}};
+// what the FP32 numbers leave of the first four
+static __constant__ float2 kModL[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+static __constant__ float2 kPsiL[4] = {{0.0f, 0.0f}, {2.48352687e-09f, 0.0f}, {5.96046448e-09f, 1.1920929e-08f}, {-5.10896955e-08f, 3.4059797e-08f}};
 
-constexpr int kTrig = 1024;                     // table of sin, cos (2 pi j / kTrig - pi / 4)
+constexpr int kTrig = 1024;                     // table of sin, cos (2 pi j / kTrig - pi / 4),
+                                                // then both as double-floats (h, l, h, l)
 constexpr double kTrigInv = 162.97466172610083;  // kTrig / (2 pi)
-constexpr double kTrigC1 = 0.006135923151542565, kTrigC2 = 2.391888279584674e-19;  // 2 pi / kTrig
+constexpr double kTrigC1 = 0.006135923151542565;   // 2 pi / kTrig as a double ..
+constexpr float kTrigC2 = 3.898171832519376e-17f;  // .. and what is left, divided by it
 constexpr double kC0Inv = 1.2533141373155003;    // sqrt(pi / 2)
 constexpr double kTwoOverPi = 0.6366197723675814;
 constexpr double kGamma = 0.57721566490153286061;
 
 constexpr int kNear = 41;    // Taylor centres 0, 1/2, .. 20
 constexpr int kTaylor = 14;  // coefficients per centre
-// tables of one operator: kTrig (sin, cos) pairs, then kNear x kTaylor
+// tables of one operator: kTrig entries of sine and cosine, then kNear x kTaylor
 // coefficients (J0, g) of the Taylor polynomials
-constexpr int kTableDouble2 = kTrig + kNear * kTaylor;
+constexpr int kTableDouble2 = 2 * kTrig + kNear * kTaylor;
 
 // J0, J0', g, g' at x = 1/2, 1, .. 20 (50-digit mpmath values, rounded)
 static __constant__ double kCentre[kNear - 1][4] = {
@@ -132,64 +146,117 @@ struct values {
   double amp, j0, y0, j1, y1;
 };
 
-template <int NP, int NQ>
-__device__ __forceinline__ void series(double t2, double& P0, double& P1, double& Q0, double& Q1) {
-  P0 = kP0[NP];
-  P1 = kP1[NP];
-  Q0 = kQ0[NQ];
-  Q1 = kQ1[NQ];
-#pragma unroll
-  for (int k = NP - 1; k >= 0; --k) {
-    P0 = fma(P0, t2, kP0[k]);
-    P1 = fma(P1, t2, kP1[k]);
-  }
-#pragma unroll
-  for (int k = NQ - 1; k >= 0; --k) {
-    Q0 = fma(Q0, t2, kQ0[k]);
-    Q1 = fma(Q1, t2, kQ1[k]);
-  }
+// ---- FP64 numbers taken apart and put together on the integer units
+
+// FP32 number of the leading 24 bits of v (positive, in the FP32 range)
+__device__ __forceinline__ float leading(unsigned hi, unsigned lo) {
+  return __uint_as_float((hi - 0x38000000u) << 3 | lo >> 29);
+}
+// v = h + l, v positive and below 2^127; zero below 2^-126
+__device__ __forceinline__ void split(double v, float& h, float& l) {
+  const unsigned hi = __double2hiint(v), lo = __double2loint(v);
+  const bool in = hi >= 0x38100000u;
+  h = in ? leading(hi, lo) : 0.0f;
+  // 29 bits of weight 2^(e - 1075)
+  l = (float)(int)(lo & 0x1fffffff) * __int_as_float(max((int)(hi >> 20) - 948, 0) << 23);
+}
+// h + l in FP64, |l| <= 2^-24 |h| (2^-127 for h = 0)
+__device__ __forceinline__ double join(float h, float l) {
+  const unsigned b = __float_as_uint(h), m = b & 0x7fffffff;
+  // l in units of h's last place in FP64, its sign against h's
+  const unsigned s = (306u - max(m >> 23, 52u)) << 23 | (b & 0x80000000u);
+  int u = __float2int_rn(l * __uint_as_float(s));
+  if (u < 0 && (m & 0x7fffff) == 0) u *= 2;   // below a power of two places are half as large
+  const unsigned long long v =
+      ((unsigned long long)((m >> 3) + 0x38000000u) << 32 | m << 29) + (long long)u;
+  return __hiloint2double((int)((unsigned)(v >> 32) | (b & 0x80000000u)), (int)(unsigned)v);
 }
 
-// x >= 20, t = 1 / x
-__device__ __forceinline__ values asymptotic(double x, double t, const double2* __restrict__ tab) {
-  const double t2 = t * t;
-  double P0, P1, Q0, Q1;
-  // number of terms by the size of x (its high word, off the FP64 pipe), so
-  // that the first dropped one is below 2^-55 of the sum; the lanes of a
-  // warp hold neighbouring sources and mostly agree
+// c_1 + t2 (c_2 + .. + t2 c_N): terms 1 .. D in double-float, the others in FP32
+template <int N, int D>
+__device__ __forceinline__ d2 far_series(d2 t2, const float2* c, const float2* cl) {
+  float2 f = c[N - 1];
+#pragma unroll
+  for (int k = N - 2; k >= D; --k) f = fma2(f, t2.h, c[k]);
+  d2 v = {mul2(t2.h, f), f2(0.0f)};
+#pragma unroll
+  for (int k = D - 1; k >= 0; --k) {
+    if (k < D - 1) v = dd_mul(t2, v);
+    const d2 s = fast_sum(c[k], v.h);
+    v = {s.h, add2(s.l, add2(v.l, cl[k]))};
+  }
+  return v;
+}
+
+// x >= 20, t = 1 / x.  The angle x + psi = j 2 pi / kTrig + (d + psi), the table
+// holding sine and cosine S, C of the first part less pi / 4, and
+// |d + psi| < 0.023: with alpha = m cos(d + psi) - 1 and beta = m sin(d + psi)
+//   m cos = C + (C alpha - S beta),  m sin = S + (S alpha + C beta)
+// where the brackets are small: double-floats (2^-46) leave 2^-52 of the sum, far
+// below the x 2^-53 that the rounding of x itself moves it by.  Both orders
+// run in the lanes of packed FP32 pairs (about 130 instructions, the time of
+// three FP64 ones); FP64 are the reduction of x, the four last additions and amp.
+__device__ __forceinline__ values far(double x, double t, const double2* __restrict__ tab) {
+  float th, tl;
+  split(t, th, tl);
+  const d2 T = {f2(th), f2(tl)}, t2 = dd_mul(T, T);
+  // further out fewer terms matter, and fewer in double-float: the rounding and
+  // the dropped terms stay below 2^-53
+  d2 psi, mod;
   const int xh = __double2hiint(x);
-  if (xh >= 0x40790000)        // 400
-    series<3, 2>(t2, P0, P1, Q0, Q1);
-  else if (xh >= 0x40590000)   // 100
-    series<4, 4>(t2, P0, P1, Q0, Q1);
-  else if (xh >= 0x40440000)   // 40
-    series<6, 6>(t2, P0, P1, Q0, Q1);
-  else
-    series<10, 9>(t2, P0, P1, Q0, Q1);
-  Q0 *= t;
-  Q1 *= t;
-  // x = j 2 pi / kTrig + d; the table holds sine and cosine of the first part
-  // less pi / 4, and |d| <= pi / kTrig needs two terms of each series
-  // (remainders < 4e-22 and < 2e-18)
+  if (xh >= 0x40500000) {          // 64
+    psi = far_series<5, 2>(t2, kPsi, kPsiL);
+    mod = far_series<5, 2>(t2, kMod, kModL);
+  } else if (xh >= 0x40400000) {   // 32
+    psi = far_series<8, 3>(t2, kPsi, kPsiL);
+    mod = far_series<8, 3>(t2, kMod, kModL);
+  } else {
+    psi = far_series<kFarTerms, 4>(t2, kPsi, kPsiL);
+    mod = far_series<kFarTerms, 4>(t2, kMod, kModL);
+  }
+  psi = dd_mul(T, psi);
+  mod = dd_mul(t2, mod);
+  // x = j 2 pi / kTrig + d, |d| <= pi / kTrig < 2^-8, d in units of 2^-59
   constexpr double magic = 6755399441055744.0;   // 1.5 2^52
   const double u = fma(x, kTrigInv, magic);
   const int j = __double2loint(u) & (kTrig - 1);
-  const double jd = u - magic;
-  double d = fma(-jd, kTrigC1, x);
-  d = fma(-jd, kTrigC2, d);
-  const double2 sc = __ldg(tab + j);
-  const double d2 = d * d;
-  const double sd = fma(d * d2, fma(d2, 1.0 / 120.0, -1.0 / 6.0), d);
-  const double cm = d2 * fma(d2, 1.0 / 24.0, -0.5);            // cos d - 1
-  const double s = fma(sc.y, sd, fma(sc.x, cm, sc.x));
-  const double c = fma(-sc.x, sd, fma(sc.y, cm, sc.y));
+  const double w = fma(-(u - magic), kTrigC1, x) + 0x1.8p-7;
+  const unsigned wl = __double2loint(w);
+  const int wh = __double2hiint(w) - 0x3f880000;
+  const float dh = (float)(int)__funnelshift_l(wl, wh, 5) * 0x1p-32f;
+  const float dl = fmaf((float)(int)(wl & 0x7ffffff), 0x1p-59f,
+                        -(leading(__double2hiint(x), __double2loint(x)) * kTrigC2));
+  const double2 sc = __ldg(tab + 2 * j);
+  const float4 scf = __ldg(reinterpret_cast<const float4*>(tab) + 2 * j + 1);
+  // e = d + psi, q = e^2, y = sin(e) / e - 1, c = cos(e) - 1
+  d2 e = two_sum(f2(dh), psi.h);
+  e.l = add2(e.l, add2(f2(dl), psi.l));
+  e = dd_norm(e);
+  const d2 q = dd_norm(dd_mul(e, e));
+  d2 y = fast_sum(f2(-1.0f / 6.0f), mul2(q.h, fma2(q.h, f2(-1.0f / 5040.0f), f2(1.0f / 120.0f))));
+  y.l = add2(y.l, f2(4.967053731282552e-09f));     // 1 / 6 in FP32 less 1 / 6
+  y = dd_mul(q, y);
+  d2 c = fast_sum(f2(1.0f / 24.0f), mul2(q.h, f2(-1.0f / 720.0f)));
+  c.l = add2(c.l, f2(-1.241763432820638e-09f));    // 1 / 24 less that in FP32
+  c = dd_mul(q, c);
+  const d2 c2 = fast_sum(f2(-0.5f), c.h);
+  c = dd_mul(q, {c2.h, add2(c2.l, c.l)});
+  // times m = 1 + mod
+  d2 m = fast_sum(f2(1.0f), mod.h);
+  m.l = add2(m.l, mod.l);
+  const d2 alpha = dd_add(dd_mul(c, m), mod), em = dd_mul(e, m), ey = dd_mul(em, y);
+  d2 beta = fast_sum(em.h, ey.h);
+  beta.l = add2(beta.l, add2(em.l, ey.l));
+  const d2 S = {f2(scf.x), f2(scf.y)}, C = {f2(scf.z), f2(scf.w)};
+  const d2 re = dd_norm(dd_add(dd_mul(C, alpha), dd_neg(dd_mul(S, beta))));
+  const d2 im = dd_norm(dd_add(dd_mul(S, alpha), dd_mul(C, beta)));
   values v;
   v.amp = rsqrt_newton(x);
-  v.j0 = fma(P0, c, -(Q0 * s));
-  v.y0 = fma(P0, s, Q0 * c);
-  // chi_1 = chi - pi/2: cos chi_1 = s, sin chi_1 = -c
-  v.j1 = fma(P1, s, Q1 * c);
-  v.y1 = fma(Q1, s, -(P1 * c));
+  v.j0 = sc.y + join(re.h.x, re.l.x);
+  v.y0 = sc.x + join(im.h.x, im.l.x);
+  // chi_1 = chi - pi/2: cos chi_1 = sin, sin chi_1 = -cos
+  v.j1 = sc.x + join(im.h.y, im.l.y);
+  v.y1 = -(sc.y + join(re.h.y, re.l.y));
   return v;
 }
 
@@ -198,7 +265,7 @@ __device__ __forceinline__ values asymptotic(double x, double t, const double2* 
 __device__ __forceinline__ values taylor(double x, double t, const double2* __restrict__ tab) {
   const int k = __double2int_rn(2.0 * x);
   const double d = fma((double)k, -0.5, x);
-  const double2* a = tab + kTrig + k * kTaylor;
+  const double2* a = tab + 2 * kTrig + k * kTaylor;
   double2 q = __ldg(a + kTaylor - 1);
   double J = q.x, G = q.y, dJ = 0.0, dG = 0.0;
 #pragma unroll
@@ -221,7 +288,7 @@ __device__ __forceinline__ values taylor(double x, double t, const double2* __re
 
 // x > 0, t = 1 / x
 __device__ __forceinline__ values bessel01(double x, double t, const double2* __restrict__ tab) {
-  return __double2hiint(x) >= 0x40340000 ? asymptotic(x, t, tab) : taylor(x, t, tab);   // 20
+  return __double2hiint(x) >= 0x40340000 ? far(x, t, tab) : taylor(x, t, tab);   // 20
 }
 
 // tables of one operator (see kTableDouble2): thread j of the first kTrig
@@ -230,10 +297,13 @@ __device__ __forceinline__ void fill_tables(int j, double2* __restrict__ tab) {
   if (j < kTrig) {
     double s, c;
     sincospi(2.0 * j / kTrig - 0.25, &s, &c);
-    tab[j] = make_double2(s, c);
+    tab[2 * j] = make_double2(s, c);
+    const float sh = (float)s, ch = (float)c;
+    reinterpret_cast<float4*>(tab)[2 * j + 1] =
+        make_float4(sh, (float)(s - (double)sh), ch, (float)(c - (double)ch));
   } else if (j < kTrig + kNear) {
     const int k = j - kTrig;
-    double2* a = tab + kTrig + k * kTaylor;
+    double2* a = tab + 2 * kTrig + k * kTaylor;
     double J[kTaylor + 1], G[kTaylor + 1];
     if (k == 0) {
       // J0 = sum (-x^2/4)^m / (m!)^2,

@@ -787,7 +787,7 @@ __global__ void k_df_x(size_t len, const double2* __restrict__ x, float4* __rest
 }
 
 // set-up: per-node double-float data (df_nodes in pairdf.cuh); threads past the
-// nodes convert the sine / cosine table
+// nodes copy the sine / cosine table
 __global__ void k_df_geo(int n, geom_dev g, const double* __restrict__ w, double omega, double eta,
                          double h, int hard, const unsigned* __restrict__ bound,
                          float4* __restrict__ tgt, float4* __restrict__ tq, float4* __restrict__ src,
@@ -795,9 +795,7 @@ __global__ void k_df_geo(int n, geom_dev g, const double* __restrict__ w, double
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) {
     if (i - n < kDfTab) {
-      const double2 v = g.tab[i - n];
-      const df s = dmake(v.x), c = dmake(v.y);
-      tab[i - n] = make_float4(s.h, s.l, c.h, c.l);
+      tab[i - n] = reinterpret_cast<const float4*>(g.tab)[2 * (i - n) + 1];
     }
     return;
   }

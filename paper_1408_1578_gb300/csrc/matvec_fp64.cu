@@ -36,9 +36,9 @@
 // the hard-path epilogue.
 //
 // Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
-// scheduler): per pair about 70 instructions for the entry (hankel64.cuh).
-// Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 138 us; star n =
-// 4096, 16 right-hand sides, sound hard 15.8 -> 3.2 ms.
+// scheduler): per pair about 43 instructions for the entry (hankel64.cuh).
+// Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 96 us; star n =
+// 4096, 16 right-hand sides, sound hard 15.8 -> 2.35 ms.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -224,7 +224,7 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
 
 // Up to four right-hand sides: each pair of nodes once for both of its entries.
 // (i, j) and (j, i) share the distance, the Hankel values and the Kress weight,
-// about 60 of the 75 FP64 instructions of an entry; what then remains per entry
+// about 30 of the 43 FP64 instructions of an entry; what then remains per entry
 // is its normal and speed factors, the multiply-adds and two additions of the
 // reduction over the rows of the transposed product.
 //
@@ -235,7 +235,7 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
 // values: 16 additions instead of 80) and go out by (d, j), each written by one
 // warp; the direct sums by (split, i): the layout of the split partial sums
 // above with splits + nblk / 2 entries.
-// Measured (GB300), against one entry at a time: kite n = 1024 258 -> 144 us
+// Measured (GB300, entries of 75 instructions), against one entry at a time: kite n = 1024 258 -> 144 us
 // (one right-hand side, sound soft), n = 4096 2.93 -> 1.50 ms, four 3.30 -> 1.95;
 // sound hard, n = 4096 3.26 -> 1.92 ms (one), 4.05 -> 2.82 (four).
 template <int BC, int R>

@@ -3,6 +3,7 @@
 // comment of matvec_fp32.cu for the two-float phase and the asymptotic
 // Hankel expansion (A&S 9.2.5, 9.2.9, 9.2.10).
 #pragma once
+#include "packed32.cuh"
 
 // FP32 geometry of an operator: coordinates times omega as hi/lo pairs,
 // unnormalised normal, speed.
@@ -261,13 +262,6 @@ __device__ __forceinline__ float2 entry_folded32(float4 tg, float4 tq, float4 sc
 // issue slots.  Signs sit in the per-node data and in the constants
 // where they can.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
 // as pair_phase, for the two sources
 struct pair_phase2 {

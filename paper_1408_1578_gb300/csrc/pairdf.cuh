@@ -66,34 +66,7 @@ __host__ __device__ __forceinline__ df dmake(double v) {
   return {h, (float)(v - (double)h)};
 }
 
-// ---------------------------------------------------------------------------
-// packed double-float
-// ---------------------------------------------------------------------------
-struct d2 {
-  float2 h, l;
-};
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return add2(a, neg2(b)); }
-__device__ __forceinline__ d2 dd_neg(d2 a) { return {neg2(a.h), neg2(a.l)}; }
-// a + b exactly, |a| >= |b| or a == 0
-__device__ __forceinline__ d2 fast_sum(float2 a, float2 b) {
-  const float2 s = add2(a, b);
-  return {s, sub2(b, sub2(s, a))};
-}
-__device__ __forceinline__ d2 two_sum(float2 a, float2 b) {
-  const float2 s = add2(a, b), v = sub2(s, a);
-  return {s, add2(sub2(a, sub2(s, v)), sub2(b, v))};
-}
-__device__ __forceinline__ d2 dd_add(d2 a, d2 b) {
-  const d2 s = two_sum(a.h, b.h);
-  return {s.h, add2(s.l, add2(a.l, b.l))};
-}
-__device__ __forceinline__ d2 dd_norm(d2 a) { return fast_sum(a.h, a.l); }
-__device__ __forceinline__ d2 dd_mul(d2 a, d2 b) {
-  const float2 p = mul2(a.h, b.h);
-  float2 e = fma2(a.h, b.h, neg2(p));
-  e = fma2(a.h, b.l, e);
-  return {p, fma2(a.l, b.h, e)};
-}
+// packed double-float, one of its two lanes
 __device__ __forceinline__ df lane0(d2 a) { return {a.h.x, a.l.x}; }
 __device__ __forceinline__ df lane1(d2 a) { return {a.h.y, a.l.y}; }
 

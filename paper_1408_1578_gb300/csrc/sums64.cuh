@@ -2,7 +2,7 @@
 // units: y_r(i) = sum_j K_ij x_r(j) for five and more columns r.
 //
 // GB300 has 1.7 lanes of FP64 multiply-add per clock and SM, and 25 of 32 x 32
-// -> 64-bit integer multiply-add.  An entry takes about 60 FP64 instructions
+// -> 64-bit integer multiply-add.  An entry takes about 40 FP64 instructions
 // (hankel64.cuh); its sums took 4 more per right-hand side, twice that for the
 // sound-hard operator's two.  Here a tile of 32 sources works in fixed point:
 // the 32 entries of a row share the exponent of the largest of them, the 32

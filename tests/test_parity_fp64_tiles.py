@@ -1,6 +1,6 @@
 """FP64 matvec and field at the edges of their tilings: right-hand-side blocks of 1, 2, 4, 16,
 32 / 64 and their remainders, 32- and 64-target tiles with ragged ends, source splits, pairs on
-both sides of every change of the Hankel evaluation (omega r = 20, 40, 100, 400).
+both sides of every change of the Hankel evaluation (omega r = 20, 32, 64).
 
 Bounds: 1e-12 per right-hand side (the FP64 resolution of the Hankel argument, 4e-16 omega
 diam, is below it at every size here), as for the other FP64 parity tests."""
