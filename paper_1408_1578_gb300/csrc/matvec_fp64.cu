@@ -19,19 +19,11 @@
 //          per right-hand side and pair fewer than S on three vectors and D')
 // Diagonal entries come precomputed (geometry.cu).
 //
-// Kernels, by the number of right-hand sides:
-//   five and more: sums64.cuh (entries shared by a block of columns, its sums on
-//     the integer units)
-//   up to four: k_pair_sym (both entries of a pair of nodes at once)
-//   up to four of small problems, or where the transposed sums do not fit:
-//     k_pair_fp64.  A CTA of 4 TI threads owns TI = 64 (small problems: 32)
-//     targets and walks a contiguous range of source tiles (TJ = 32 sources
-//     each).  For every tile it evaluates the TI x TJ block of entries into
-//     shared memory (one warp per target row, lanes over sources), then
-//     contracts it with the staged block of right-hand sides; with one or two
-//     of those the threads split the sources instead.
-// In all of them source ranges are split across CTAs when the row tiles alone
-// do not fill the GPU; the per-split partial sums go to a scratch buffer and a
+// Kernels: k_pair_sym (both entries of a pair of nodes at once) for a few
+// right-hand sides, else sums64.cuh (entries shared by a block of columns, sums on
+// the integer units).
+// In both of them source ranges are split across CTAs when the rows alone do
+// not fill the GPU; the per-split partial sums go to a scratch buffer and a
 // second kernel adds them in a fixed order (deterministic results) and applies
 // the hard-path epilogue.
 //
@@ -51,8 +43,6 @@
 
 namespace {
 
-constexpr int TJ = 32;
-
 __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
   acc.x = fma(a.x, b.x, acc.x);
   acc.x = fma(-a.y, b.y, acc.x);
@@ -61,168 +51,7 @@ __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
   return acc;
 }
 
-template <int BC, int TI, int RBT>
-struct pair_smem {
-  // targets: coordinates; hard: omega nu / |z'| and (omega^2 / eta) nu / |z'|
-  double tx[TI], ty[TI], tfx[BC ? TI : 1], tfy[BC ? TI : 1], tux[BC ? TI : 1], tuy[BC ? TI : 1];
-  // sources: coordinates, folded factors (soft: nu, hard: unit normal), speed factor
-  double sx[TJ], sy[TJ], sfx[TJ], sfy[TJ], se[TJ];
-  double wk[TI + TJ];                    // Kress weights / (pi h) of the tile, by i - j
-  double2 A[TI][TJ + 1];                 // soft: A; hard: S
-  double2 B[BC ? TI : 1][TJ + 1];        // hard: C
-  double2 X[BC ? 2 : 1][TJ][RBT];        // soft: x ; hard: u, x
-};
-
-template <int BC, int TI, int RBT>
-__global__ void __launch_bounds__(4 * TI)
-k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restrict__ wtab,
-            const double2* __restrict__ diag, const double2* __restrict__ xin,
-            const double2* __restrict__ uin, int nrhs, int splits, int tiles_per_split,
-            double2* __restrict__ part) {
-  constexpr int NT = 4 * TI;
-  constexpr int RG = RBT < 4 ? RBT : 4;   // groups of threads over the right-hand sides ..
-  constexpr int JG = 4 / RG;              // .. and, with fewer than four of those, the sources
-  constexpr int RQ = RBT / RG;            // right-hand sides per thread
-  constexpr int NO = BC ? 2 : 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  pair_smem<BC, TI, RBT>& S = *reinterpret_cast<pair_smem<BC, TI, RBT>*>(smem_raw);
-  const int tid = threadIdx.x;
-  const int i0 = blockIdx.x * TI;
-  const int split = blockIdx.y;
-  const int rb0 = blockIdx.z * RBT;
-  const int rbn = min(RBT, nrhs - rb0);
-  const int ntiles = (n + TJ - 1) / TJ;
-  const int t_begin = split * tiles_per_split;
-  const int t_end = min(ntiles, t_begin + tiles_per_split);
-  const double h = 2.0 * CFIE_PI / n;
-  const double f = 0.25 * 0.7978845608028654 * h;   // hq c0
-  const double wscale = 1.0 / (CFIE_PI * h), omega_inv = 1.0 / omega;
-
-  if (tid < TI) {
-    const int i = i0 + tid;
-    const bool ok = i < n;
-    S.tx[tid] = ok ? g.x[i] : 0.0;
-    S.ty[tid] = ok ? g.y[i] : 0.0;
-    if constexpr (BC == 1) {
-      const double inv = ok ? omega / g.sp[i] : 0.0, k = omega / eta;
-      S.tfx[tid] = ok ? g.nx[i] * inv : 0.0;
-      S.tfy[tid] = ok ? g.ny[i] * inv : 0.0;
-      S.tux[tid] = S.tfx[tid] * k;
-      S.tuy[tid] = S.tfy[tid] * k;
-    }
-  }
-
-  const int il2 = tid % TI;                // contraction: target row
-  const int rg = (tid / TI) % RG;          // right-hand-side group
-  const int jg = (tid / TI) / RG;          // source group
-  double2 acc[NO][RQ];
-#pragma unroll
-  for (int o = 0; o < NO; ++o)
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) acc[o][q] = make_double2(0.0, 0.0);
-
-  for (int t = t_begin; t < t_end; ++t) {
-    const int j0 = t * TJ;
-    __syncthreads();
-    if (tid < TJ) {
-      const int j = j0 + tid;
-      const bool ok = j < n;
-      const double sp = ok ? g.sp[j] : 1.0;
-      const double m = BC ? 1.0 / sp : omega * f;
-      S.sx[tid] = ok ? g.x[j] : 0.0;
-      S.sy[tid] = ok ? g.y[j] : 0.0;
-      S.sfx[tid] = ok ? m * g.nx[j] : 0.0;
-      S.sfy[tid] = ok ? m * g.ny[j] : 0.0;
-      S.se[tid] = BC ? f * sp : f * eta * sp;
-    }
-    for (int e = tid; e < TI + TJ - 1; e += NT) {
-      int d = (i0 - j0 + e - (TJ - 1)) % n;
-      if (d < 0) d += n;
-      S.wk[e] = wtab[d] * wscale;
-    }
-    for (int e = tid; e < TJ * RBT; e += NT) {
-      const int jl = e / RBT, r = e % RBT;
-      const int j = j0 + jl;
-      double2 xv = make_double2(0.0, 0.0), uv = xv;
-      if (j < n && r < rbn) {
-        xv = xin[(size_t)(rb0 + r) * n + j];
-        if (BC) uv = uin[(size_t)(rb0 + r) * n + j];
-      }
-      S.X[NO - 1][jl][r] = xv;
-      if constexpr (BC == 1) S.X[0][jl][r] = uv;
-    }
-    __syncthreads();
-
-    // ---- entries of the TI x TJ block: one warp per row, lane = source
-    for (int e = tid; e < TI * TJ; e += NT) {
-      const int il = e / TJ, jl = e % TJ;
-      const int i = i0 + il, j = j0 + jl;
-      double2 a = make_double2(0.0, 0.0), b = a;
-      if (i < n && j < n) {
-        if (i == j) {
-          a = BC ? diag[2 * i] : diag[i];
-          if (BC) b = diag[2 * i + 1];
-        } else {
-          pair_folded_fp64<BC>(S.tx[il] - S.sx[jl], S.ty[il] - S.sy[jl], omega, omega_inv,
-                               BC ? S.tfx[il] : S.sfx[jl], BC ? S.tfy[il] : S.sfy[jl], S.se[jl],
-                               S.wk[il - jl + TJ - 1], g.tab, a, b);
-        }
-      }
-      S.A[il][jl] = a;
-      if constexpr (BC == 1) {
-        // C = -D' - i (omega^2 / eta) (n_i . n_j) S
-        const double k = fma(S.tux[il], S.sfx[jl], S.tuy[il] * S.sfy[jl]);
-        S.B[il][jl] = make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y));
-      }
-    }
-    __syncthreads();
-
-    // ---- contraction
-    const int jn = min(TJ, n - j0);
-    for (int jl = jg; jl < jn; jl += JG) {
-      const double2 a = S.A[il2][jl];
-      const double2 b = BC ? S.B[il2][jl] : a;
-#pragma unroll
-      for (int q = 0; q < RQ; ++q) {
-        const int r = rg + RG * q;
-        acc[0][q] = cmad(acc[0][q], a, S.X[0][jl][r]);
-        if constexpr (BC == 1) acc[NO - 1][q] = cmad(acc[NO - 1][q], b, S.X[NO - 1][jl][r]);
-      }
-    }
-  }
-
-  if constexpr (JG > 1) {   // join the source groups (RQ = 1) in the entries' place
-    double2* red = &S.A[0][0];
-    static_assert(NO * JG * RG * TI <= TI * (TJ + 1), "group sums exceed the entry block");
-    __syncthreads();
-#pragma unroll
-    for (int o = 0; o < NO; ++o) red[((o * JG + jg) * RG + rg) * TI + il2] = acc[o][0];
-    __syncthreads();
-    if (jg > 0) return;
-#pragma unroll
-    for (int o = 0; o < NO; ++o)
-#pragma unroll
-      for (int k = 1; k < JG; ++k) {
-        const double2 v = red[((o * JG + k) * RG + rg) * TI + il2];
-        acc[o][0].x += v.x;
-        acc[o][0].y += v.y;
-      }
-  }
-  const int i = i0 + il2;
-  if (i < n) {
-#pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-      const int r = rg + RG * q;
-      if (r < rbn) {
-#pragma unroll
-        for (int o = 0; o < NO; ++o)
-          part[(((size_t)o * splits + split) * nrhs + rb0 + r) * n + i] = acc[o][q];
-      }
-    }
-  }
-}
-
-// Up to four right-hand sides: each pair of nodes once for both of its entries.
+// A few right-hand sides: each pair of nodes once for both of its entries.
 // (i, j) and (j, i) share the distance, the Hankel values and the Kress weight,
 // about 30 of the 43 FP64 instructions of an entry; what then remains per entry
 // is its normal and speed factors, the multiply-adds and two additions of the
@@ -233,11 +62,11 @@ k_pair_fp64(int n, double omega, double eta, geom_dev g, const double* __restric
 // of it, cover every pair of blocks once; d = 0 takes its pairs in both orders.
 // The transposed sums of SB sources are reduced across the warp together (16
 // values: 16 additions instead of 80) and go out by (d, j), each written by one
-// warp; the direct sums by (split, i): the layout of the split partial sums
-// above with splits + nblk / 2 entries.
-// Measured (GB300, entries of 75 instructions), against one entry at a time: kite n = 1024 258 -> 144 us
-// (one right-hand side, sound soft), n = 4096 2.93 -> 1.50 ms, four 3.30 -> 1.95;
-// sound hard, n = 4096 3.26 -> 1.92 ms (one), 4.05 -> 2.82 (four).
+// warp; the direct sums by (split, i): the layout of the block kernel's split
+// partial sums with splits + nblk / 2 entries.
+// Measured (GB300, kite), against the block kernel: sound soft, one right-hand
+// side n = 512 83 -> 60 us, n = 4096 1.51 -> 1.10 ms; four n = 1024 155 -> 131 us,
+// n = 8192 5.46 -> 5.64 ms; sound hard, one n = 4096 1.86 -> 1.46 ms, two 1.87 -> 1.80.
 template <int BC, int R>
 __global__ void __launch_bounds__(32)
 k_pair_sym(int n, int nblk, double omega, double omega_inv, double eta_inv, double nf, double sf,
@@ -483,12 +312,15 @@ k_spectral_fp64(int n, const double* __restrict__ ct, const double* __restrict__
 // star n = 4096, 16 right-hand sides, sound hard, left the FP64 pipe idle 20 %
 // of the time).  Problems of fewer 64 x 32 tiles than eight per SM take
 // 32-target tiles.
-// Up to four right-hand sides take both entries of a pair of nodes at once
-// (k_pair_sym) while its partial sums, one per block distance, stay within 512
-// MB (or the caller's scratch): n = 46000 for one sound-soft right-hand side.
+// k_pair_sym takes up to four sums (sound soft: four right-hand sides, sound
+// hard: two; with three, sound hard n = 4096, 2.39 ms against the block
+// kernel's 1.87) from n = 400 on: below, the block kernel has at most one tile per
+// SM (kite n = 384, one right-hand side 57 against 52 us), and while its partial
+// sums, one per block distance, stay within 512 MB (or the caller's scratch):
+// n = 46000 for one sound-soft right-hand side.
 struct pair_plan {
   int sym;                  // 0, or the right-hand sides of k_pair_sym (1, 2, 4)
-  int rbt, ti, rhsblocks, splits, tps;
+  int rbt, ti, splits, tps;
   int parts;                // partial sums per output and element
 };
 
@@ -497,7 +329,7 @@ pair_plan plan_pair(int n, int nrhs, int hard, int device, size_t max_parts) {
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   const size_t vec = sizeof(double2) * (hard ? 2 : 1) * (size_t)n * nrhs;
-  if (nrhs <= 4 && n >= 192) {   // below, a warp's chain over its 8 sources is the longer one
+  if (nrhs <= (hard ? 2 : 4) && n >= 400) {
     const int nblk = (n + 31) / 32, units = 4 * (nblk / 2 + 1);
     const int want = (32 * sms + nblk - 1) / nblk;       // about 32 warps per SM
     p.tps = (units + std::min(units, want) - 1) / std::min(units, want);
@@ -508,33 +340,17 @@ pair_plan plan_pair(int n, int nrhs, int hard, int device, size_t max_parts) {
       return p;
     }
   }
-  p.rbt = nrhs <= 2 ? nrhs : nrhs <= 4 ? 4 : sums64::block_width(nrhs, hard);
-  p.rhsblocks = (nrhs + p.rbt - 1) / p.rbt;
-  const int ntiles = (n + TJ - 1) / TJ;
-  p.ti = (long long)((n + 63) / 64) * ntiles * p.rhsblocks < 8LL * sms ? 32 : 64;
-  if (p.rbt > 4) p.ti = std::min(p.ti, sums64::block_rows(p.rbt, hard));
-  const int rows = (n + p.ti - 1) / p.ti * p.rhsblocks;
+  p.rbt = sums64::block_width(nrhs, hard);
+  const int rhsblocks = (nrhs + p.rbt - 1) / p.rbt, ntiles = (n + sums64::TJ - 1) / sums64::TJ;
+  p.ti = sums64::block_rows(p.rbt, hard);
+  if ((long long)((n + 63) / 64) * ntiles * rhsblocks < 8LL * sms) p.ti = 32;
+  const int rows = (n + p.ti - 1) / p.ti * rhsblocks;
   const int target = 16 * sms;   // several waves of the two or three CTAs that fit an SM
   p.splits = std::max<int>(1, std::min<size_t>(std::min<size_t>(ntiles, max_parts),
                                                (target + rows - 1) / rows));
   p.tps = (ntiles + p.splits - 1) / p.splits;
   p.splits = p.parts = (ntiles + p.tps - 1) / p.tps;
   return p;
-}
-
-template <int BC, int TI, int RBT>
-void launch_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
-                 double2* part) {
-  const int n = op->n;
-  const size_t smem = sizeof(pair_smem<BC, TI, RBT>);
-  CFIE_CHECK_CUDA(cudaFuncSetAttribute(k_pair_fp64<BC, TI, RBT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((n + TI - 1) / TI, p.splits, p.rhsblocks);
-  prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
-  k_pair_fp64<BC, TI, RBT><<<grid, 4 * TI, smem, op->ctx->stream>>>(
-      n, op->omega, op->eta, op->g, op->wtab.as<double>(), op->diag.as<double2>(), x, u, nrhs,
-      p.splits, p.tps, part);
-  CFIE_CHECK_LAUNCH();
 }
 
 template <int BC, int R>
@@ -554,22 +370,12 @@ void launch_sym(cfie_op* op, const pair_plan& p, const double2* x, const double2
 template <int BC>
 void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
               double2* part, double2* t, double2* y) {
-  const bool small = p.ti == 32;
   if (p.sym == 1)
     launch_sym<BC, 1>(op, p, x, u, nrhs, part);
   else if (p.sym == 2)
     launch_sym<BC, 2>(op, p, x, u, nrhs, part);
-  else if (p.sym == 4)
-    launch_sym<BC, 4>(op, p, x, u, nrhs, part);
-  else if (p.rbt == 1)
-    small ? launch_pair<BC, 32, 1>(op, p, x, u, nrhs, part)
-          : launch_pair<BC, 64, 1>(op, p, x, u, nrhs, part);
-  else if (p.rbt == 2)
-    small ? launch_pair<BC, 32, 2>(op, p, x, u, nrhs, part)
-          : launch_pair<BC, 64, 2>(op, p, x, u, nrhs, part);
-  else if (p.rbt == 4)
-    small ? launch_pair<BC, 32, 4>(op, p, x, u, nrhs, part)
-          : launch_pair<BC, 64, 4>(op, p, x, u, nrhs, part);
+  else if (BC == 0 && p.sym == 4)
+    launch_sym<0, 4>(op, p, x, u, nrhs, part);
   else {
     const double f = 0.25 * 0.7978845608028654 * op->h;   // hq c0
     prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);

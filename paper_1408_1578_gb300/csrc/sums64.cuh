@@ -1,5 +1,5 @@
 // Sums of FP64 kernel entries over a block of right-hand sides, on the integer
-// units: y_r(i) = sum_j K_ij x_r(j) for five and more columns r.
+// units: y_r(i) = sum_j K_ij x_r(j).
 //
 // GB300 has 1.7 lanes of FP64 multiply-add per clock and SM, and 25 of 32 x 32
 // -> 64-bit integer multiply-add.  An entry takes about 40 FP64 instructions
@@ -278,7 +278,7 @@ void launch_block(const block_args& p, cudaStream_t stream) {
 inline int block_width(int nrhs, bool hard) {
   const int widest = hard ? 32 : 64, blocks = (nrhs + widest - 1) / widest;
   const int per = (nrhs + blocks - 1) / blocks;
-  for (int r : {8, 12, 16, 24, 32, 48})
+  for (int r : {4, 8, 12, 16, 24, 32, 48})
     if (per <= r) return r;
   return 64;
 }
@@ -299,6 +299,7 @@ void run_width(const block_args& p, int ti, cudaStream_t stream) {
 template <int MODE>
 void run_block(const block_args& p, int ti, int width, cudaStream_t stream) {
   switch (width) {
+    case 4: run_width<MODE, 4>(p, ti, stream); break;
     case 8: run_width<MODE, 8>(p, ti, stream); break;
     case 12: run_width<MODE, 12>(p, ti, stream); break;
     case 16: run_width<MODE, 16>(p, ti, stream); break;
