@@ -29,10 +29,10 @@
 // pairs (pair32.cuh), which issue half as often as scalar instructions, four
 // independent chains at a time; the sources are warp-uniform loads from a ring
 // filled three tiles ahead.  Measured (GB300), kernel alone: kite n = 32768, 64
-// right-hand sides 2.95 -> 2.53 ms (packed pairs in the former layout, a row
+// right-hand sides 2.95 -> 2.44 ms (packed pairs in the former layout, a row
 // per half warp: 2.97, bound by shared-memory cycles and by waits for the
 // source loads); ellipse n = 32768, 1 right-hand side, sound hard, 4.90 (S and
-// D' in two passes) -> 2.98 ms; two pairs at a time instead of four: 2.60 ms.
+// D' in two passes) -> 2.97 ms; two pairs at a time instead of four: 0.07 ms more.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -83,6 +83,14 @@ struct tc_params {
   const float2* band;    // near entries: soft A, or S, then C
 };
 
+// v << 16 as a byte permutation: the compiler turns the shift into a multiply-add,
+// on the pipe that bounds the producers (kite n = 32768 2.53 -> 2.51 ms)
+__device__ __forceinline__ uint32_t shl16(uint32_t v) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, 0x1044;" : "=r"(r) : "r"(v));
+  return r;
+}
+
 // bf16 hi / lo split of eight entries of one row (adjacent sources): the packed
 // words of the four planes (hi re, hi im, lo re, lo im) of each operator
 template <int NO>
@@ -91,7 +99,7 @@ struct split_words {
   __device__ __forceinline__ static void split(float2 e, uint32_t& hi, uint32_t& lo) {
     const __nv_bfloat162 b = __floats2bfloat162_rn(e.x, e.y);
     hi = *reinterpret_cast<const uint32_t*>(&b);
-    const float2 h = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+    const float2 h = make_float2(__uint_as_float(shl16(hi)), __uint_as_float(hi & 0xffff0000u));
     const float2 d = add2(e, neg2(h));
     const __nv_bfloat162 c = __floats2bfloat162_rn(d.x, d.y);
     lo = *reinterpret_cast<const uint32_t*>(&c);

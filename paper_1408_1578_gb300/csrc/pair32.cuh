@@ -117,8 +117,8 @@ __device__ __forceinline__ pair_phase pair_phase32(float txh, float txl, float t
   return f;
 }
 
-// The same distance and phase to the accuracy of the fused tensor-core
-// kernel, whose entries reach the tensor cores as bf16 hi + lo pairs (2^-17
+// The same distance and phase to the accuracy of the stored and the fused
+// tensor-core kernels, whose entries reach the tensor cores as bf16 hi + lo pairs (2^-17
 // relative): the lo part of x comes from H - xh^2 (one fma, of the size of C)
 // plus C instead of from the exact sum H + C, the Cody-Waite constant has two
 // parts (the third, k C3, is 1.6e-12 omega r rad) and the lo part of pi/4 is
@@ -164,7 +164,7 @@ __device__ __forceinline__ void hankel_asym32(float ti, float s, float c, float&
   y1 = fmaf(Q1, s, -P1 * c);
 }
 
-// Two terms of each of P and Q (the fused tensor-core kernel): the remainder
+// Two terms of each of P and Q (the stored operators): the remainder
 // is below the first omitted term, < 2.2e-6 relative for x >= 16 and
 // < 1.4e-8 for x >= 64, near the bf16 hi + lo split's 2^-17.
 __device__ __forceinline__ void hankel_asym32_tc(float ti, float s, float c, float& j0, float& y0,
@@ -211,47 +211,19 @@ __device__ __forceinline__ void pair_entries_fp32(const omega32& P, float txh, f
   }
 }
 
-// Entry kinds: the sound-soft combination of eq. 1, or one of the two layer
-// operators S, D' of the sound-hard operator of eq. 2
-enum { KIND_SOFT = 0, KIND_S = 1, KIND_DP = 2 };
-
-// The same entries with the per-node factors folded in, to the fused
-// tensor-core kernel's accuracy (phase and series above): tg, sc = target and
-// source coordinates, tq = target factors (D'
-// only), sq = source factors, wk = Kress weight / (pi h); see the packed
-// layout above.  With A = sq ra and B = omega hq c0 (nu_j . (z_i - z_j)) ra / r,
-//   soft:  re = A j0 - B (y1 + wk j1),      im = B j1 + A (y0 + wk j0)
-//   S:     re = -A' (y0 + wk j0),            im = A' j0        (A' = hq c0 |z'_j| ra)
-//   D':    re = D (y1 + wk j1),              im = -D j1
-// with D = omega (nu_i . (z_i - z_j)) / |z'_i| hq c0 |z'_j| ra / r.
-template <int KIND>
-__device__ __forceinline__ float2 entry_finish32(const pair_phase& f, float4 tq, float4 sq,
-                                                 float wk) {
+// The sound-soft entry with the per-node factors folded in, to the accuracy of
+// the operators' bf16 hi + lo planes (phase and series above): tg, sc = target
+// and source coordinates, sq = source factors, wk = Kress weight / (pi h); see
+// the packed layout above.  With A = hq c0 eta |z'_j| ra and B = omega hq c0
+// (nu_j . (z_i - z_j)) ra / r,
+//   re = A j0 - B (y1 + wk j1),      im = B j1 + A (y0 + wk j0)
+__device__ __forceinline__ float2 entry_folded32(float4 tg, float4 sc, float4 sq, float wk) {
+  const pair_phase f = pair_phase32_tc(tg.x, tg.y, tg.z, tg.w, sc.x, sc.y, sc.z, sc.w);
   float j0, y0, j1, y1;
   hankel_asym32_tc(f.xinv, f.s, f.c, j0, y0, j1, y1);
-  float2 a;
-  if constexpr (KIND == KIND_SOFT) {
-    const float A = sq.z * f.ra;
-    const float B = fmaf(f.dx, sq.x, f.dy * sq.y) * (f.xinv * f.ra);
-    a.x = fmaf(A, j0, -B * fmaf(wk, j1, y1));
-    a.y = fmaf(B, j1, A * fmaf(wk, j0, y0));
-  } else if constexpr (KIND == KIND_S) {
-    const float A = sq.w * f.ra;
-    a.x = -A * fmaf(wk, j0, y0);
-    a.y = A * j0;
-  } else {
-    const float D = fmaf(f.dx, tq.x, f.dy * tq.y) * (f.xinv * f.ra) * sq.w;
-    a.x = D * fmaf(wk, j1, y1);
-    a.y = -D * j1;
-  }
-  return a;
-}
-
-template <int KIND>
-__device__ __forceinline__ float2 entry_folded32(float4 tg, float4 tq, float4 sc, float4 sq,
-                                                 float wk) {
-  return entry_finish32<KIND>(pair_phase32_tc(tg.x, tg.y, tg.z, tg.w, sc.x, sc.y, sc.z, sc.w), tq,
-                              sq, wk);
+  const float A = sq.z * f.ra;
+  const float B = fmaf(f.dx, sq.x, f.dy * sq.y) * (f.xinv * f.ra);
+  return make_float2(fmaf(A, j0, -B * fmaf(wk, j1, y1)), fmaf(B, j1, A * fmaf(wk, j0, y0)));
 }
 
 // ---------------------------------------------------------------------------
@@ -265,7 +237,7 @@ __device__ __forceinline__ float2 entry_folded32(float4 tg, float4 tq, float4 sc
 
 // as pair_phase, for the two sources
 struct pair_phase2 {
-  float2 dx, dy, xinv, ra, s, c;
+  float2 dx, dy, xinv, ra, chi;   // chi = x - pi/4 less a multiple of 2 pi
 };
 
 // pair_phase32_tc for both sources: t0, t1 the target's (xh, xh, xl, xl), (yh,
@@ -287,28 +259,33 @@ __device__ __forceinline__ pair_phase2 phase32_pair(float4 t0, float4 t1, float4
   const float2 xl = fma2(e, mul2(f.xinv, f2(0.5f)), f2(-kPi4H));             // x lo - pi/4
   const float2 kr = add2(fma2(xh, f2(kInv2Pi), f2(-0.125f)), f2(12582912.0f));
   const float2 k = add2(kr, f2(-12582912.0f));
-  const float2 chi = add2(fma2(k, f2(-kC2), fma2(k, f2(-kC1), xh)), xl);     // first fma exact
-  sincos_sfu(chi.x, &f.s.x, &f.c.x);
-  sincos_sfu(chi.y, &f.s.y, &f.c.y);
+  f.chi = add2(fma2(k, f2(-kC2), fma2(k, f2(-kC1), xh)), xl);                // first fma exact
   return f;
 }
 
-// j0, w0 = y0 + wk j0, j1, w1 = y1 + wk j1 of both sources (hankel_asym32_tc)
+// H_nu(x) = c0 ra m_nu exp(i (chi + psi_nu - nu pi / 2)) of both sources, as
+// modulus and phase (A&S 9.2.28, 9.2.29: two terms each): j0 = m0 c0, w0 = y0 + wk
+// j0 = m0 u0, j1 = m1 s1, w1 = y1 + wk j1 = m1 u1.  Two more sines and cosines on the
+// special-function unit than with P and Q, but six packed instructions of 52
+// fewer on the FMA pipe, which bounds the fused kernel: kite n = 32768, 64 right-hand
+// sides 2.51 -> 2.44 ms.
 struct hankel_pair {
-  float2 j0, w0, j1, w1;
+  float2 m0, m1, c0, u0, s1, u1;
 };
 __device__ __forceinline__ hankel_pair hankel32_pair(const pair_phase2& f, float2 wk) {
   const float2 ti = f.xinv, t2 = mul2(ti, ti);
-  const float2 ns = neg2(f.s);
-  const float2 P0 = fma2(t2, f2(-0.0703125f), f2(1.0f));
-  const float2 Q0 = mul2(ti, fma2(t2, f2(0.0732421875f), f2(-0.125f)));
-  const float2 P1n = fma2(t2, f2(-0.1171875f), f2(-1.0f));
-  const float2 Q1 = mul2(ti, fma2(t2, f2(-0.1025390625f), f2(0.375f)));
+  const float2 a0 = fma2(ti, fma2(t2, f2(25.0f / 384.0f), f2(-0.125f)), f.chi);
+  const float2 a1 = fma2(ti, fma2(t2, f2(-21.0f / 128.0f), f2(0.375f)), f.chi);
   hankel_pair h;
-  h.j0 = fma2(P0, f.c, mul2(Q0, ns));
-  h.w0 = fma2(wk, h.j0, fma2(P0, f.s, mul2(Q0, f.c)));
-  h.j1 = fma2(P1n, ns, mul2(Q1, f.c));
-  h.w1 = fma2(wk, h.j1, fma2(P1n, f.c, mul2(Q1, f.s)));
+  float2 s0, c1;
+  sincos_sfu(a0.x, &s0.x, &h.c0.x);
+  sincos_sfu(a0.y, &s0.y, &h.c0.y);
+  sincos_sfu(a1.x, &h.s1.x, &c1.x);
+  sincos_sfu(a1.y, &h.s1.y, &c1.y);
+  h.m0 = fma2(t2, f2(-0.0625f), f2(1.0f));
+  h.m1 = fma2(t2, f2(0.1875f), f2(1.0f));
+  h.u0 = fma2(wk, h.c0, s0);
+  h.u1 = fma2(wk, h.s1, neg2(c1));
   return h;
 }
 
@@ -333,23 +310,25 @@ template <int OP>
 __device__ __forceinline__ entry_pair finish32_pair(const pair_phase2& f, float4 tq, float4 s2,
                                                     float2 sc, float2 wk) {
   const hankel_pair h = hankel32_pair(f, wk);
-  const float2 A = mul2(sc, f.ra);
+  const float2 A = mul2(sc, f.ra), A0 = mul2(A, h.m0);
   entry_pair e;
   if constexpr (OP == OP_SOFT) {
-    const float2 B = mul2(fma2(f.dx, lo2(s2), mul2(f.dy, hi2(s2))), mul2(f.xinv, f.ra));
-    e.re = fma2(A, h.j0, mul2(neg2(B), h.w1));
-    e.im = fma2(A, h.w0, mul2(B, h.j1));
+    const float2 B = mul2(fma2(f.dx, lo2(s2), mul2(f.dy, hi2(s2))),
+                          mul2(h.m1, mul2(f.xinv, f.ra)));
+    e.re = fma2(A0, h.c0, mul2(neg2(B), h.u1));
+    e.im = fma2(A0, h.u0, mul2(B, h.s1));
   } else {
-    const float2 sr = mul2(A, h.j0), si = mul2(A, h.w0);
+    const float2 sr = mul2(A0, h.c0), si = mul2(A0, h.u0);
     if constexpr (OP == OP_S || OP == OP_SC) {
       e.re = sr;
       e.im = si;
     }
     if constexpr (OP == OP_C || OP == OP_SC) {
-      const float2 D = mul2(fma2(f.dx, lo2(tq), mul2(f.dy, hi2(tq))), mul2(f.xinv, A));
+      const float2 D = mul2(fma2(f.dx, lo2(tq), mul2(f.dy, hi2(tq))),
+                            mul2(h.m1, mul2(f.xinv, A)));
       const float2 kn = fma2(lo2(tq), lo2(s2), mul2(hi2(tq), hi2(s2)));
-      const float2 cr = fma2(kn, sr, mul2(neg2(D), h.w1));
-      const float2 ci = fma2(kn, si, mul2(D, h.j1));
+      const float2 cr = fma2(kn, sr, mul2(neg2(D), h.u1));
+      const float2 ci = fma2(kn, si, mul2(D, h.s1));
       if constexpr (OP == OP_C) {
         e.re = cr;
         e.im = ci;

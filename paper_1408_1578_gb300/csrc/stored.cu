@@ -94,8 +94,7 @@ k_assemble(int n, int pitch, int b, int bd, const float4* __restrict__ pk,
       // the folded entry of the fused matvec, to the accuracy the bf16 hi + lo
       // planes keep (packed coordinates and factors, Kress table / (pi h) at
       // i - j + n)
-      a = entry_folded32<KIND_SOFT>(pk[i], make_float4(0.f, 0.f, 0.f, 0.f), pk[j], pk[n + j],
-                                    wkt[i - j + n].x);
+      a = entry_folded32(pk[i], pk[j], pk[n + j], wkt[i - j + n].x);
     }
     // largest far entry of the row (outside the double-float band of width bd):
     // the row exponent of the tensor-core residual
