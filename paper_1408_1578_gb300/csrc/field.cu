@@ -13,12 +13,12 @@
 // spacings away from the curve), FP64 throughout with the library's own
 // Hankel evaluation: the block kernel of sums64.cuh.
 //
-// Bound: the FP64 pipe, about 36 instructions per kernel value, which the
+// Bound: the FP64 pipe, about 31 instructions per kernel value, which the
 // densities of a block share.  When the points alone do not fill the GPU the
 // sources are split across CTAs and a second kernel adds the splits in a fixed
 // order.
 // Measured (GB300): 16 densities of n = 4096 nodes at 20000 points, sound hard,
-// 70.2 -> 7.4 ms.
+// 70.2 -> 6.8 ms.
 #include <algorithm>
 
 #include "hankel64.cuh"
@@ -46,7 +46,7 @@ __global__ void k_field_sum(size_t tot, int splits, const double2* __restrict__ 
 void field_eval(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts,
                 double2* u) {
   const bool hard = op->bc == CFIE_SOUND_HARD;
-  const double f = 0.25 * 0.7978845608028654 * op->h;   // h c0 / 4
+  const double f = h64::pair_factor(op->omega, op->h);   // h c0 / 4
   const int width = sums64::block_width(nrhs, false), ti = sums64::block_rows(width, false);
   const int tiles = (op->n + sums64::TJ - 1) / sums64::TJ;
   const size_t tot = (size_t)nrhs * npts;
@@ -67,6 +67,7 @@ void field_eval(cfie_op* op, const double2* q, int nrhs, int npts, const double2
   a.rotate = hard;   // -S + D / (i eta) = -i (D / eta - i S)
   a.omega = op->omega;
   a.omega_inv = 1.0 / op->omega;
+  a.near = h64::near_amp(op->omega);
   a.nf = hard ? op->omega * f / op->eta : op->omega * f;
   a.sf = hard ? f : op->eta * f;
   a.g = op->g;

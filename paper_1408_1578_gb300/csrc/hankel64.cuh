@@ -21,11 +21,11 @@
 // is small is kept off the FP64 pipe: everything that is added to the table's
 // sine and cosine is below 0.03, so that packed FP32 double-floats give it, and
 // FP64 numbers are taken apart and joined with integer instructions.
-// About 43 FP64 instructions per far pair of the sound-hard operator; 70 with the
+// About 38 FP64 instructions per far pair of the sound-hard operator; 70 with the
 // series and the rotation in FP64, 150 with the library's sqrt, division and
 // sincos besides.  Measured (GB300), series in FP64 -> here: circle n = 1024, one
-// right-hand side 138 -> 96 us; star n = 4096, 16, sound hard 3.2 -> 2.35 ms; field of
-// 16 densities at 20000 points 10.9 -> 7.4 ms.  Values against quadruple
+// right-hand side 138 -> 96 us; star n = 4096, 16, sound hard 3.2 -> 2.22 ms; field of
+// 16 densities at 20000 points 10.9 -> 6.8 ms.  Values against quadruple
 // precision, rms over 20 < x < 50000: 3.8e-17 .. 6.3e-17 times amp (FP64
 // series 6.5e-17 .. 7.4e-17).
 #pragma once
@@ -125,23 +125,8 @@ __device__ __forceinline__ double rsqrt_newton(double a) {
   return fma(e * y, fma(e, 0.375, 0.5), y);
 }
 
-// distance r = sqrt(r2) and 1 / r.  The plain functions take the arguments
-// near the ends of the exponent range, where the estimate flushes to zero.
-__device__ __forceinline__ void distance(double r2, double& r, double& rinv) {
-  const unsigned hi = (unsigned)__double2hiint(r2);
-  if (hi - 0x02000000u < 0x7c000000u) {   // 2^-991 < r2 < 2^993
-    rinv = rsqrt_newton(r2);
-    const double r0 = r2 * rinv;
-    const double half = __hiloint2double(__double2hiint(rinv) - 0x00100000, __double2loint(rinv));
-    r = fma(fma(-r0, r0, r2), half, r0);
-  } else {
-    r = sqrt(r2);
-    rinv = 1.0 / r;
-  }
-}
-
-// J0 = amp j0, Y0 = amp y0, J1 = amp j1, Y1 = amp y1, with c0 = sqrt(2/pi)
-// left out of amp: J = c0 amp j
+// J0 = c0 amp j0, Y0 = c0 amp y0, J1 = c0 amp j1, Y1 = c0 amp y1 with c0 =
+// sqrt(2 / (pi omega)), which the callers' per-node factors take
 struct values {
   double amp, j0, y0, j1, y1;
 };
@@ -172,6 +157,44 @@ __device__ __forceinline__ double join(float h, float l) {
   return __hiloint2double((int)((unsigned)(v >> 32) | (b & 0x80000000u)), (int)(unsigned)v);
 }
 
+// distance r, 1 / r and q = r^(-1/2) from r^2
+struct polar {
+  double r, rinv, q;
+};
+// One Newton step of third order for r2^(-1/4) gives all three: y from the
+// special-function unit (|e| < 2^-18 for e = 1 - r2 y^4), q = y (1 + e / 4 + 5
+// e^2 / 32), whose second factor, less 1, takes a double-float; 8 FP64
+// instructions where separate steps for 1 / r and x^(-1/2) take 13.  The plain
+// functions take what is outside FP32's range.
+__device__ __forceinline__ polar distance(double r2) {
+  polar p;
+  const unsigned hi = __double2hiint(r2);
+  if (hi - 0x38700000u < 0x0f000000u) {   // 2^-120 <= r2 < 2^120
+    float y = leading(hi, __double2loint(r2));
+    asm("sqrt.approx.ftz.f32 %0, %0;" : "+f"(y));
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(y));
+    const float s0 = y * y;
+    const double s = join(s0, fmaf(y, y, -s0));            // y^2, exact
+    const double w = fma(-(r2 * s), s, 1.0) + 0x1.8p-17;   // e in units of 2^-69
+    const unsigned wl = __double2loint(w);
+    const int wh = __double2hiint(w) - 0x3ee80000;
+    const float eh = (float)(int)__funnelshift_l(wl, wh, 5) * 0x1p-42f;
+    const float el = (float)(int)(wl & 0x7ffffff) * 0x1p-69f;
+    const float gh = 0.25f * eh, gl = fmaf(0.15625f * eh, eh, 0.25f * el);
+    const float yg = y * gh, c = fmaf(y, gl, fmaf(y, gh, -yg)), h = yg + c;
+    p.q = join(y, 0.0f) + join(h, c - (h - yg));
+    p.rinv = p.q * p.q;
+    const double r0 = r2 * p.rinv;
+    const double half = __hiloint2double(__double2hiint(p.rinv) - 0x00100000, __double2loint(p.rinv));
+    p.r = fma(fma(-r0, r0, r2), half, r0);
+  } else {
+    p.r = sqrt(r2);
+    p.rinv = 1.0 / p.r;
+    p.q = sqrt(p.rinv);
+  }
+  return p;
+}
+
 // c_1 + t2 (c_2 + .. + t2 c_N): terms 1 .. D in double-float, the others in FP32
 template <int N, int D>
 __device__ __forceinline__ d2 far_series(d2 t2, const float2* c, const float2* cl) {
@@ -195,8 +218,8 @@ __device__ __forceinline__ d2 far_series(d2 t2, const float2* c, const float2* c
 // where the brackets are small: double-floats (2^-46) leave 2^-52 of the sum, far
 // below the x 2^-53 that the rounding of x itself moves it by.  Both orders
 // run in the lanes of packed FP32 pairs (about 130 instructions, the time of
-// three FP64 ones); FP64 are the reduction of x, the four last additions and amp.
-__device__ __forceinline__ values far(double x, double t, const double2* __restrict__ tab) {
+// three FP64 ones); FP64 are the reduction of x and the four last additions.
+__device__ __forceinline__ values far(double x, double t, double amp, const double2* __restrict__ tab) {
   float th, tl;
   split(t, th, tl);
   const d2 T = {f2(th), f2(tl)}, t2 = dd_mul(T, T);
@@ -251,7 +274,7 @@ __device__ __forceinline__ values far(double x, double t, const double2* __restr
   const d2 re = dd_norm(dd_add(dd_mul(C, alpha), dd_neg(dd_mul(S, beta))));
   const d2 im = dd_norm(dd_add(dd_mul(S, alpha), dd_mul(C, beta)));
   values v;
-  v.amp = rsqrt_newton(x);
+  v.amp = amp;
   v.j0 = sc.y + join(re.h.x, re.l.x);
   v.y0 = sc.x + join(im.h.x, im.l.x);
   // chi_1 = chi - pi/2: cos chi_1 = sin, sin chi_1 = -cos
@@ -262,7 +285,7 @@ __device__ __forceinline__ values far(double x, double t, const double2* __restr
 
 // 0 < x < 20, t = 1 / x: Taylor polynomials about c = k / 2, k nearest 2 x,
 // Horner's scheme for each value and derivative
-__device__ __forceinline__ values taylor(double x, double t, const double2* __restrict__ tab) {
+__device__ __forceinline__ values taylor(double x, double t, double amp, const double2* __restrict__ tab) {
   const int k = __double2int_rn(2.0 * x);
   const double d = fma((double)k, -0.5, x);
   const double2* a = tab + 2 * kTrig + k * kTaylor;
@@ -278,7 +301,7 @@ __device__ __forceinline__ values taylor(double x, double t, const double2* __re
   }
   const double lg = log(0.5 * x);
   values v;
-  v.amp = kC0Inv;
+  v.amp = amp;
   v.j0 = J;
   v.j1 = -dJ;
   v.y0 = fma(kTwoOverPi * lg, J, G);
@@ -286,9 +309,10 @@ __device__ __forceinline__ values taylor(double x, double t, const double2* __re
   return v;
 }
 
-// x > 0, t = 1 / x
-__device__ __forceinline__ values bessel01(double x, double t, const double2* __restrict__ tab) {
-  return __double2hiint(x) >= 0x40340000 ? far(x, t, tab) : taylor(x, t, tab);   // 20
+// x = omega r > 0, t = 1 / x, q = r^(-1/2), near = sqrt(pi omega / 2)
+__device__ __forceinline__ values bessel01(double x, double t, double q, double near,
+                                           const double2* __restrict__ tab) {
+  return __double2hiint(x) >= 0x40340000 ? far(x, t, q, tab) : taylor(x, t, near, tab);   // 20
 }
 
 // tables of one operator (see kTableDouble2): thread j of the first kTrig
@@ -337,37 +361,42 @@ __device__ __forceinline__ void fill_tables(int j, double2* __restrict__ tab) {
   }
 }
 
+// hq c0 and sqrt(pi omega / 2) of the folded entries below
+__host__ __device__ __forceinline__ double pair_factor(double omega, double h) {
+  return 0.25 * 0.7978845608028654 * h / sqrt(omega);
+}
+__host__ __device__ __forceinline__ double near_amp(double omega) { return kC0Inv * sqrt(omega); }
+
 }  // namespace h64
 
 // Nystrom entries of one off-diagonal pair (i != j) in FP64, (dx, dy) =
 // z_i - z_j, with the per-node factors folded in (hq = h / 4, c0 =
-// sqrt(2/pi), nu the unnormalised normal, |z'| the speed, wk = Kress weight
-// / (pi h); h64::values' amp is x^(-1/2)):
+// sqrt(2 / (pi omega)), nu the unnormalised normal, |z'| the speed, wk = Kress weight
+// / (pi h); h64::values' amp is r^(-1/2)):
 //   soft (eq. 1):  sx, sy = omega hq c0 nu_j,  se = hq c0 eta |z'_j|;  A = se amp,
 //                  B = ((dx, dy) . (sx, sy)) amp / r
 //                  re = A j0 - B (y1 + wk j1),  im = B j1 + A (y0 + wk j0)
 //   hard (eq. 2):  se = hq c0 |z'_j|, tx, ty = omega nu_i / |z'_i|;  A = se amp,
 //                  D = ((dx, dy) . (tx, ty)) A / r
 //                  S  = -A (y0 + wk j0) + i A j0,  D' = D (y1 + wk j1) - i D j1
-// omega_inv = 1 / omega, tab = the operator's tables.  KRESS false: no Kress term
+// omega_inv = 1 / omega, near = sqrt(pi omega / 2), tab = the operator's tables.  KRESS false: no Kress term
 // (points off the curve).
 template <int BC, bool KRESS = true>
 __device__ __forceinline__ void pair_folded_fp64(double dx, double dy, double omega,
-                                                 double omega_inv, double fx, double fy, double se,
-                                                 double wk, const double2* __restrict__ tab,
+                                                 double omega_inv, double near, double fx, double fy,
+                                                 double se, double wk, const double2* __restrict__ tab,
                                                  double2& a, double2& b) {
-  double r, rinv;
-  h64::distance(fma(dx, dx, dy * dy), r, rinv);
-  const h64::values v = h64::bessel01(omega * r, omega_inv * rinv, tab);
+  const h64::polar d = h64::distance(fma(dx, dx, dy * dy));
+  const h64::values v = h64::bessel01(omega * d.r, omega_inv * d.rinv, d.q, near, tab);
   const double A = se * v.amp;
   const double w0 = KRESS ? fma(wk, v.j0, v.y0) : v.y0, w1 = KRESS ? fma(wk, v.j1, v.y1) : v.y1;
   const double p = fma(dx, fx, dy * fy);
   if constexpr (BC == 0) {
-    const double B = p * (rinv * v.amp);
+    const double B = p * (d.rinv * v.amp);
     a = make_double2(fma(A, v.j0, -(B * w1)), fma(B, v.j1, A * w0));
     b = make_double2(0.0, 0.0);
   } else {
-    const double D = p * (rinv * A);
+    const double D = p * (d.rinv * A);
     a = make_double2(-(A * w0), A * v.j0);
     b = make_double2(D * w1, -(D * v.j1));
   }
@@ -383,13 +412,12 @@ __device__ __forceinline__ void pair_entries_fp64(double dx, double dy, double o
                                                   double sj, double nxi, double nyi, double si,
                                                   const double2* __restrict__ tab, double2& a,
                                                   double2& b) {
-  constexpr double c0q = 0.25 * 0.7978845608028654;   // c0 / 4
-  const double f = c0q * h, wk = w / (CFIE_PI * h);
+  const double f = h64::pair_factor(omega, h), near = h64::near_amp(omega), wk = w / (CFIE_PI * h);
   if constexpr (BC == 0)
-    pair_folded_fp64<0>(dx, dy, omega, 1.0 / omega, omega * f * nxj, omega * f * nyj, f * eta * sj,
+    pair_folded_fp64<0>(dx, dy, omega, 1.0 / omega, near, omega * f * nxj, omega * f * nyj, f * eta * sj,
                         wk, tab, a, b);
   else
-    pair_folded_fp64<1>(dx, dy, omega, 1.0 / omega, omega * nxi / si, omega * nyi / si, f * sj, wk,
+    pair_folded_fp64<1>(dx, dy, omega, 1.0 / omega, near, omega * nxi / si, omega * nyi / si, f * sj, wk,
                         tab, a, b);
 }
 

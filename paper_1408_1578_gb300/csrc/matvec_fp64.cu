@@ -28,9 +28,9 @@
 // the hard-path epilogue.
 //
 // Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
-// scheduler): per pair about 43 instructions for the entry (hankel64.cuh).
+// scheduler): per pair about 38 instructions for the entry (hankel64.cuh).
 // Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 96 us; star n =
-// 4096, 16 right-hand sides, sound hard 15.8 -> 2.35 ms.
+// 4096, 16 right-hand sides, sound hard 15.8 -> 2.22 ms.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -53,7 +53,7 @@ __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
 
 // A few right-hand sides: each pair of nodes once for both of its entries.
 // (i, j) and (j, i) share the distance, the Hankel values and the Kress weight,
-// about 30 of the 43 FP64 instructions of an entry; what then remains per entry
+// about 27 of the 38 FP64 instructions of an entry; what then remains per entry
 // is its normal and speed factors, the multiply-adds and two additions of the
 // reduction over the rows of the transposed product.
 //
@@ -69,8 +69,8 @@ __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
 // n = 8192 5.46 -> 5.64 ms; sound hard, one n = 4096 1.86 -> 1.46 ms, two 1.87 -> 1.80.
 template <int BC, int R>
 __global__ void __launch_bounds__(32)
-k_pair_sym(int n, int nblk, double omega, double omega_inv, double eta_inv, double nf, double sf,
-           int units_per_warp, int splits, geom_dev g, const double* __restrict__ wks,
+k_pair_sym(int n, int nblk, double omega, double omega_inv, double near, double eta_inv, double nf,
+           double sf, int units_per_warp, int splits, geom_dev g, const double* __restrict__ wks,
            const double2* __restrict__ diag, const double2* __restrict__ xin,
            const double2* __restrict__ uin, int nrhs, double2* __restrict__ part) {
   constexpr int NO = BC ? 2 : 1;
@@ -153,11 +153,10 @@ k_pair_sym(int n, int nblk, double omega, double omega_inv, double eta_inv, doub
         if (di < 0) di += n;
         const double wk = ok ? wks[di] : 0.0;
         const double dx = tx - qx, dy = ty - qy;
-        double dist, rinv;
-        h64::distance(fma(dx, dx, dy * dy), dist, rinv);
-        const h64::values h = h64::bessel01(omega * dist, omega_inv * rinv, g.tab);
+        const h64::polar p = h64::distance(fma(dx, dx, dy * dy));
+        const h64::values h = h64::bessel01(omega * p.r, omega_inv * p.rinv, p.q, near, g.tab);
         const double w0 = fma(wk, h.j0, h.y0), w1 = fma(wk, h.j1, h.y1);
-        const double ra = rinv * h.amp;
+        const double ra = p.rinv * h.amp;
         // entries from the receiving node's and the sending node's factors
         double2 e[NO], et[NO];
         if constexpr (BC == 0) {
@@ -357,10 +356,10 @@ template <int BC, int R>
 void launch_sym(cfie_op* op, const pair_plan& p, const double2* x, const double2* u, int nrhs,
                 double2* part) {
   const int n = op->n, nblk = (n + 31) / 32;
-  const double f = 0.25 * 0.7978845608028654 * op->h;   // hq c0
+  const double f = h64::pair_factor(op->omega, op->h);   // hq c0
   prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
   k_pair_sym<BC, R><<<dim3(nblk, p.splits), 32, 0, op->ctx->stream>>>(
-      n, nblk, op->omega, 1.0 / op->omega, 1.0 / op->eta, op->omega * f, BC ? f : f * op->eta,
+      n, nblk, op->omega, 1.0 / op->omega, h64::near_amp(op->omega), 1.0 / op->eta, op->omega * f, BC ? f : f * op->eta,
       p.tps, p.splits, op->g, op->wtab.as<double>() + n, op->diag.as<double2>(), x, u, nrhs, part);
   CFIE_CHECK_LAUNCH();
 }
@@ -377,7 +376,7 @@ void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* 
   else if (BC == 0 && p.sym == 4)
     launch_sym<0, 4>(op, p, x, u, nrhs, part);
   else {
-    const double f = 0.25 * 0.7978845608028654 * op->h;   // hq c0
+    const double f = h64::pair_factor(op->omega, op->h);   // hq c0
     prof_scope ps(op->ctx, CFIE_K_MATVEC_FP64);
     sums64::block_args a{};
     a.n = a.rows = op->n;
@@ -386,6 +385,7 @@ void run_pair(cfie_op* op, const pair_plan& p, const double2* x, const double2* 
     a.tiles_per_split = p.tps;
     a.omega = op->omega;
     a.omega_inv = 1.0 / op->omega;
+    a.near = h64::near_amp(op->omega);
     a.nf = op->omega * f;
     a.sf = BC ? f : f * op->eta;
     a.eta_inv = 1.0 / op->eta;

@@ -81,7 +81,7 @@ struct fixed_acc {
 struct block_args {
   int n, rows, nrhs, splits, tiles_per_split;
   bool rotate;                         // FIELD: times -i (sound hard)
-  double omega, omega_inv;
+  double omega, omega_inv, near;       // near = sqrt(pi omega / 2)
   double nf, sf;                       // factors of the normal (HARD: of none) and the speed
   double eta_inv;                      // HARD
   geom_dev g;
@@ -94,7 +94,8 @@ template <int MODE, int TI, int RBT>
 struct block_smem {
   static constexpr int NO = MODE == HARD ? 2 : 1;
   double tx[TI], ty[TI];
-  double tfx[NO == 2 ? TI : 1], tfy[NO == 2 ? TI : 1];   // HARD: omega nu / |z'|
+  // HARD: omega nu / |z'| and (omega / eta) nu / |z'|
+  double tfx[NO == 2 ? TI : 1], tfy[NO == 2 ? TI : 1], tux[NO == 2 ? TI : 1], tuy[NO == 2 ? TI : 1];
   double sx[TJ], sy[TJ], sfx[TJ], sfy[TJ], se[TJ];
   double wk[TI + TJ];                    // Kress weights of the tile, by i - j
   int4 K[NO][TI][TJ + 1];                // limbs (re, im): the entries; HARD: S, C
@@ -132,6 +133,8 @@ k_block64(block_args p) {
       const double inv = ok ? p.omega / g.sp[i] : 0.0;
       S.tfx[tid] = ok ? g.nx[i] * inv : 0.0;
       S.tfy[tid] = ok ? g.ny[i] * inv : 0.0;
+      S.tux[tid] = S.tfx[tid] * p.eta_inv;
+      S.tuy[tid] = S.tfy[tid] * p.eta_inv;
     }
   }
 
@@ -184,7 +187,7 @@ k_block64(block_args p) {
         } else {
           pair_folded_fp64<MODE == HARD, MODE != FIELD>(
               S.tx[il] - S.sx[lane], S.ty[il] - S.sy[lane], p.omega, p.omega_inv,
-              MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
+              p.near, MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
               S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
         }
       }
@@ -194,7 +197,7 @@ k_block64(block_args p) {
       if (lane == 0) S.ek[0][il] = E;
       if constexpr (MODE == HARD) {
         // C = -D' - i (omega^2 / eta) (n_i . n_j) S
-        const double k = fma(S.tfx[il], S.sfx[lane], S.tfy[il] * S.sfy[lane]) * p.eta_inv;
+        const double k = fma(S.tux[il], S.sfx[lane], S.tuy[il] * S.sfy[lane]);
         const double2 c = make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y));
         E = shared_exponent(c, bad);
         S.K[NO - 1][il][lane] = to_limbs(c, E);
