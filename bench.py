@@ -176,9 +176,10 @@ def measured_peaks():
 SMS, FP32_LANES = 152, 128
 # FP32 pair entries (two-float phase, asymptotics) by summation variant: the
 # CUDA-core kernel evaluates both hard entries from one phase; the tensor-core
-# kernel folds the per-node factors in, keeps the accuracy of its bf16 hi + lo
-# operands (two-term series, no exact sum in the phase) and evaluates S (36)
-# and D' (42) in two passes
+# kernel folds the per-node factors in and keeps the accuracy of its bf16 hi + lo
+# operands (two-term series, no exact sum in the phase), S (36) and D' (42).  A
+# fixed unit of work: the kernels now spend fewer (modulus and phase instead of
+# P and Q, S and C from one phase), which raises the fraction reported
 ENTRY_OPS = {("soft", 1): 74, ("hard", 1): 87, ("soft", 2): 54, ("hard", 2): 36 + 42}
 SUM_OPS = {"soft": 4, "hard": 8}         # FP32 FMAs per pair and right-hand side (CUDA-core sums)
 DF_ENTRY_OPS = 563                       # double-float pair entry of the residual kernel

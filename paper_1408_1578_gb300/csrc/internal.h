@@ -236,13 +236,14 @@ struct cfie_op {
   dbuf df_geo, df_band, df_part, df_x;
   int df_b = -1;
   dbuf df_rowexp;    // sound soft: row exponents of the far entries (tensor-core residual)
-  rtc_plan rtc[3];   // tensor-core residual plans for 16, 32, 64 right-hand sides per pass
+  rtc_plan rtc[4];   // tensor-core residual plans for 16, 32, 48, 64 right-hand sides per pass
   int res_variant = 0;   // residual: 0 automatic, 1 CUDA-core Dot2, 2 tensor cores
 
   // FP32 matvec variant: 0 = autotuned, 1 = FP32-pipe contraction, 2 = tensor cores
   int variant = 0, tuned_nrhs = -1, tuned_choice = 1;
   int basis32 = 1;   // inner Krylov basis in FP32 for the refined precisions
-  tc_plan tc[3];   // plans: up to 32, up to 64 right-hand sides; S and C together, up to 32
+  // plans: up to 32, up to 64 right-hand sides; S and C together, up to 32, up to 40
+  tc_plan tc[4];
 
   // stored path (CFIE_STORED): bf16 hi/lo planes of A and the contraction plan
   dbuf stored;

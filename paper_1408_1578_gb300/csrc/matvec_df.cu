@@ -200,13 +200,13 @@ __global__ void __launch_bounds__(DNT) k_pair_df(df_params P, size_t xstride) {
 // integer multiple of the same power of two and stays below 2^14 of it, so a
 // chunk of 128 sources (256 terms with the split complex product for L = 2,
 // 512 for L = 3, 768 for L = 4, 1024 for L = 5) sums exactly in FP32 whatever
-// the tensor core's rounding.  With up to 32 right-hand sides per pass the
+// the tensor core's rounding.  With up to 48 right-hand sides per pass the
 // tensor memory holds five accumulators: L = 2, 3, 4, 5 exact and L = 6, 7
 // together (below 2^-32 of the leading level).  With 64 right-hand sides only
 // four fit (4 x 128 columns) and L = 5 shares the accumulator of L = 6, 7,
 // whose additions the tensor core does not round to nearest (measured: 1e-12
 // relative for the sound-soft residual; the sound-hard passes, whose
-// hypersingular part magnifies it tenfold, take at most 32 right-hand sides).
+// hypersingular part magnifies it tenfold, take at most 48 right-hand sides).
 // Every 128 sources the producer warps
 // join the levels in double-float: L = 2 + 3 and L >= 4 each as an exact
 // TwoSum pair, then one double-float addition (adding the lower levels to the
@@ -233,7 +233,7 @@ constexpr int RST = 2;        // pipeline stages
 constexpr int RCK = 8;        // tiles per TMEM chunk (128 sources)
 // level accumulators: L = 2, 3, 4, 5 and L >= 6 when they fit, else L >= 5 shared
 template <int NB>
-__host__ __device__ constexpr int rlevels() { return NB <= 32 ? 5 : 4; }
+__host__ __device__ constexpr int rlevels() { return NB <= 48 ? 5 : 4; }
 constexpr int RPROD = 16;     // producer warps
 constexpr int RWTMA = RPROD, RWMMA = RPROD + 1;
 // 18 warps (the producers also drain the accumulators): at most 5 per
@@ -925,7 +925,7 @@ int launch_df(cfie_op* op, df_params P, int nrhs) {
 template <int NB, int OP>
 void run_rtc(cfie_op* op, df_params P, const double2* x, double2* y, int r0, int nr) {
   constexpr int NC = 2 * NB;
-  rtc_plan& T = op->rtc[NB == 16 ? 0 : (NB == 32 ? 1 : 2)];
+  rtc_plan& T = op->rtc[NB == 16 ? 0 : (NB == 32 ? 1 : (NB == 48 ? 2 : 3))];
   const int n = op->n;
   cudaStream_t st = op->ctx->stream;
   if (!T.built) {
@@ -996,12 +996,14 @@ template <int OP>
 void run_rtc_block(cfie_op* op, const df_params& P, const double2* x, double2* y, int r0,
                    int nr) {
   if constexpr (OP == OP_SOFT) {
-    if (nr > 32) {
+    if (nr > 48) {
       run_rtc<64, OP>(op, P, x, y, r0, nr);
       return;
     }
   }
-  if (nr > 16)
+  if (nr > 32)
+    run_rtc<48, OP>(op, P, x, y, r0, nr);
+  else if (nr > 16)
     run_rtc<32, OP>(op, P, x, y, r0, nr);
   else
     run_rtc<16, OP>(op, P, x, y, r0, nr);
@@ -1162,13 +1164,14 @@ void matvec_df(cfie_op* op, const double2* x, double2* y, int nrhs) {
     df_params PC = P;
     PC.x = xv + tot;
     PC.band = P.band + (size_t)n * (2 * (size_t)P.b + 1);
-    // passes of at most 32 right-hand sides, whose tensor memory holds an
+    // passes of at most 48 right-hand sides, whose tensor memory holds an
     // exact accumulator for every level up to L = 5: the hypersingular part
     // magnifies the rounding of the shared L >= 5 accumulator of 64-wide
     // passes to ~1e-11 relative (sound soft: ~1e-12)
-    for (int r0 = 0; r0 < nrhs; r0 += 32) {
-      run_rtc_block<OP_S>(op, P, u, t, r0, std::min(32, nrhs - r0));
-      run_rtc_block<OP_C>(op, PC, x, y, r0, std::min(32, nrhs - r0));
+    const int passes = (nrhs + 47) / 48, per = (nrhs + passes - 1) / passes;
+    for (int r0 = 0; r0 < nrhs; r0 += per) {
+      run_rtc_block<OP_S>(op, P, u, t, r0, std::min(per, nrhs - r0));
+      run_rtc_block<OP_C>(op, PC, x, y, r0, std::min(per, nrhs - r0));
     }
   } else {
     int splits;

@@ -12,6 +12,7 @@
 // Kress tables, plane-wave data, refined GMRES; the Krylov basis stays on the
 // device for the life of the solve.  Finished requests keep their solution and
 // timing on the host until released.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <condition_variable>
@@ -55,7 +56,9 @@ size_t footprint_bytes(const cfie_request& r) {
   f += n * 129 * 8 * 2;               // near-field band (b <= 64), both operators
   f += vec / 2 * (16 * ops + 3);      // FP32 split partials and staging
   f += vec * 4 * ops;                 // FP64 residual partials (a few splits)
-  f += n * 200 + ((size_t)64 << 20);  // tables, small buffers, slack
+  if (r.precision == CFIE_FP64)       // FP64 matvec partials: one per block distance, or of
+    f += k <= 4 ? std::min((size_t)512 << 20, vec * (n / 64 + 32) * 2) : (size_t)96 << 20;   // splits
+  f += n * 360 + ((size_t)64 << 20);  // tables, small buffers, slack
   if (r.precision == CFIE_TENSOR_REFINED) {
     const size_t pitch = (n + 63) / 64 * 64, rows = (n + 127) / 128 * 128;
     f += 8 * rows * pitch;              // stored bf16 hi/lo planes (re, im), whole row blocks

@@ -41,3 +41,18 @@ def test_variants_at_tile_edges(ctx, bc, n):
             assert np.max(col_rel(got[-1], want)) < 1e-4, (nrhs, variant)
         assert np.max(col_rel(got[1], got[0])) < 5e-5, nrhs
     op.close()
+
+
+@pytest.mark.parametrize("nrhs", [33, 40, 41, 66, 80, 81])
+def test_sound_hard_pass_widths(ctx, nrhs):
+    """S and C together in passes of 32 or 40, or one after the other in passes of 64: both sides
+    of every change."""
+    n, omega = 386, 32.0
+    A = operators.cfie_matrix(geometry.kite(n), omega, omega, "hard")
+    op = ctx.kite().discretise(n, omega, bc="hard", precision="fp32")
+    op.set_variant(2)
+    X = inputs.random_density(n, nrhs, seed=nrhs)
+    y = empty(nrhs, n)
+    op.apply(to_dev(X), y)
+    assert np.max(col_rel(to_host(y), (A @ X.T).T)) < 1e-4
+    op.close()

@@ -35,3 +35,18 @@ def test_residual_at_tile_edges(ctx, bc, n, omega):
             op.apply_residual(to_dev(X), y)
             assert np.max(col_rel(to_host(y), want)) < 1e-11, (nrhs, variant)
     op.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+@pytest.mark.parametrize("nrhs", [32, 40, 48, 49, 64, 72, 96, 97])
+def test_residual_pass_widths(ctx, bc, nrhs):
+    """Passes of 16, 32, 48 and 64 right-hand sides, both sides of every change."""
+    n, omega = 386, 32.0
+    A = operators.cfie_matrix(geometry.kite(n), omega, omega, bc)
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp32")
+    op.set_residual_variant(2)
+    X = inputs.random_density(n, nrhs, seed=nrhs)
+    y = empty(nrhs, n)
+    op.apply_residual(to_dev(X), y)
+    assert np.max(col_rel(to_host(y), (A @ X.T).T)) < 1e-11
+    op.close()
