@@ -298,8 +298,11 @@ cfie_status cfie_apply(cfie_op* op, const void* x_dev, void* y_dev, int nrhs);
  * times both variants once on the context stream and the process keeps the
  * faster), 1 = register-blocked FP32 sums on the CUDA cores (any operator),
  * 2 = tensor cores (entries split bf16 hi + lo, tcgen05 contraction; for the
- * sound-hard operator S is applied to the three vectors of Maue's identity and
- * D' to the density, each a pass of the same kernel).  Variant 1 evaluates the
+ * sound-hard operator S is applied to d/ds x and C = -D' - i (omega^2 / eta)
+ * (n_i . n_j) S to x, together up to 40 right-hand sides).  Autotune gives
+ * products that are launches and latency in either variant (one right-hand side,
+ * n <= 2304; sound hard, n <= 1152 to 2304 by the number of right-hand sides)
+ * variant 1, the more accurate, without timing.  Variant 1 evaluates the
  * FP32 entries to full FP32 accuracy, variant 2 to the accuracy its bf16
  * hi + lo operands keep (two-term Hankel series, a few 1e-6 relative next to
  * the near band); both stay far inside the 1e-4 of a raw FP32 matvec. */
@@ -333,10 +336,10 @@ cfie_status cfie_apply_fp64_static(cfie_op* op, const void* x_dev, void* y_dev, 
  * true residuals: for CFIE_FP32_REFINED / CFIE_TENSOR_REFINED operators of
  * either boundary condition the same entries as cfie_apply_fp64 evaluated in
  * double-float arithmetic on the FP32 pipe (hi + lo pairs, error-free products
- * and sums; for the sound-hard operator S and D' so, the spectral derivatives
- * in FP64; a few 1e-12 relative), otherwise the FP64 matvec (also when the
- * near band of the double-float form would exceed 4 GB).  Arguments as
- * cfie_apply. */
+ * and sums; for the sound-hard operator S and C (see cfie_op_set_variant) so,
+ * the spectral derivatives in FP64; a few 1e-12 relative), otherwise the FP64
+ * matvec (also when the near band of the double-float form would exceed 4 GB).
+ * Arguments as cfie_apply. */
 cfie_status cfie_apply_residual(cfie_op* op, const void* x_dev, void* y_dev, int nrhs);
 
 /* Solve A x = f for nrhs independent right-hand sides by restarted GMRES
@@ -360,7 +363,7 @@ cfie_status cfie_gmres_solve(cfie_op* op, const void* f_dev, void* x_dev, int nr
  * inside cfie_gmres_solve), all to a few 1e-12 relative: variant 1 evaluates the
  * entries in double-float (FP32 pairs) and sums with compensated Dot2 on the
  * CUDA cores; variant 2 evaluates the far entries in double-float (for the
- * sound-hard operator S and D' in separate passes), splits entries and
+ * sound-hard operator S and C in separate passes), splits entries and
  * densities into six 8-bit slices on per-row / per-column power-of-two grids
  * and sums the slice products on the tensor cores, exactly in FP32 for the
  * three leading levels, with the near band on the CUDA cores; 0 (default)

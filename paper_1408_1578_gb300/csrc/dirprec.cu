@@ -103,6 +103,7 @@ k_dirprec_e(int n, int m, double omega, double eta, double ds, geom_dev g,
   const double h = 2.0 * CFIE_PI / n;
   double ar = 0.0, ai = 0.0;
   float sr32 = 0.f, si32 = 0.f;
+  const pair_consts pc = make_pair_consts(omega, eta, h);
   const long long tot = (long long)ci * cj;
   for (long long idx = threadIdx.x; idx < tot; idx += blockDim.x) {
     const int x = (int)(idx / cj), y = (int)(idx % cj);
@@ -125,7 +126,7 @@ k_dirprec_e(int n, int m, double omega, double eta, double ds, geom_dev g,
       si32 = fmaf(a.x, p2, fmaf(a.y, p1, si32));
     } else {
       double2 a, unused;
-      pair_entries_fp64<0>(g.x[gi] - g.x[gj], g.y[gi] - g.y[gj], omega, eta, h, wtab[d], g.nx[gj],
+      pair_entries_fp64<0>(g.x[gi] - g.x[gj], g.y[gi] - g.y[gj], pc, wtab[n + d], g.nx[gj],
                            g.ny[gj], g.sp[gj], g.nx[gi], g.ny[gi], g.sp[gi], g.tab, a, unused);
       ar += a.x * pr - a.y * pim;
       ai += a.x * pim + a.y * pr;

@@ -402,23 +402,28 @@ __device__ __forceinline__ void pair_folded_fp64(double dx, double dy, double om
   }
 }
 
-// The same entries from plain node data (set-up kernels): w = Kress table
-// entry w_{(i-j) mod n}, h = 2 pi / n.
+// The same entries from plain node data (set-up kernels): wk = Kress weight
+// w_{(i-j) mod n} / (pi h).
 //   soft:  a = h K + w K1 for K = L - i eta M (eq. 1)
 //   hard:  a = S_ij = h M + w M1, b = D'_ij = h L' + w L'1 (eq. 2)
+// The operator's constants come ready: per entry their root and quotients cost as
+// much as the entry.
+struct pair_consts {
+  double omega, omega_inv, near, f, eta;
+};
+__host__ __device__ __forceinline__ pair_consts make_pair_consts(double omega, double eta,
+                                                                 double h) {
+  return {omega, 1.0 / omega, h64::near_amp(omega), h64::pair_factor(omega, h), eta};
+}
 template <int BC>
-__device__ __forceinline__ void pair_entries_fp64(double dx, double dy, double omega, double eta,
-                                                  double h, double w, double nxj, double nyj,
-                                                  double sj, double nxi, double nyi, double si,
+__device__ __forceinline__ void pair_entries_fp64(double dx, double dy, const pair_consts& c,
+                                                  double wk, double nxj, double nyj, double sj,
+                                                  double nxi, double nyi, double si,
                                                   const double2* __restrict__ tab, double2& a,
                                                   double2& b) {
-  const double f = h64::pair_factor(omega, h), near = h64::near_amp(omega), wk = w / (CFIE_PI * h);
-  if constexpr (BC == 0)
-    pair_folded_fp64<0>(dx, dy, omega, 1.0 / omega, near, omega * f * nxj, omega * f * nyj, f * eta * sj,
-                        wk, tab, a, b);
-  else
-    pair_folded_fp64<1>(dx, dy, omega, 1.0 / omega, near, omega * nxi / si, omega * nyi / si, f * sj, wk,
-                        tab, a, b);
+  const double m = BC == 0 ? c.omega * c.f : c.omega / si;
+  pair_folded_fp64<BC>(dx, dy, c.omega, c.omega_inv, c.near, m * (BC == 0 ? nxj : nxi),
+                       m * (BC == 0 ? nyj : nyi), c.f * sj * (BC == 0 ? c.eta : 1.0), wk, tab, a, b);
 }
 
 // C_ij = -D'_ij - i (omega^2 / eta) (n_i . n_j) S_ij, the operator that the

@@ -860,7 +860,7 @@ k_df_scan(int n, double omega, geom_dev g, int* __restrict__ bmax) {
   if ((threadIdx.x & 31) == 0) atomicMax(bmax, best);
 }
 
-__global__ void k_df_band(int n, int b, int hard, double omega, double eta, geom_dev g,
+__global__ void k_df_band(int n, int b, int hard, pair_consts pc, geom_dev g,
                           const double* __restrict__ wtab, const double2* __restrict__ diag,
                           float4* __restrict__ band) {
   const int bw = 2 * b + 1;
@@ -878,16 +878,16 @@ __global__ void k_df_band(int n, int b, int hard, double omega, double eta, geom
     int d = i - j;
     if (d < 0) d += n;
     if (hard)
-      pair_entries_fp64<1>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, 2.0 * CFIE_PI / n,
-                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
+      pair_entries_fp64<1>(g.x[i] - g.x[j], g.y[i] - g.y[j], pc, wtab[n + d],
+                           g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
     else
-      pair_entries_fp64<0>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, 2.0 * CFIE_PI / n,
-                           wtab[d], g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
+      pair_entries_fp64<0>(g.x[i] - g.x[j], g.y[i] - g.y[j], pc, wtab[n + d],
+                           g.nx[j], g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, b2);
   }
   const df re = dmake(a.x), im = dmake(a.y);
   band[e] = make_float4(re.h, re.l, im.h, im.l);
   if (hard) {
-    const double2 c = hard_combined(g, omega, eta, i, j, a, b2);
+    const double2 c = hard_combined(g, pc.omega, pc.eta, i, j, a, b2);
     const df br = dmake(c.x), bi = dmake(c.y);
     band[(size_t)n * bw + e] = make_float4(br.h, br.l, bi.h, bi.l);
   }
@@ -1078,9 +1078,9 @@ void df_prepare(cfie_op* op) {
       n, op->g, op->wtab.as<double>(), op->omega, op->eta, op->h, hard, bound, g4, g4 + 2 * (size_t)n,
       g4 + 3 * (size_t)n, g4 + 6 * (size_t)n, g4 + 8 * (size_t)n);
   CFIE_CHECK_LAUNCH();
-  k_df_band<<<nbk((size_t)n * bw), 256, 0, st>>>(n, b, hard, op->omega, op->eta, op->g,
-                                                  op->wtab.as<double>(), op->diag.as<double2>(),
-                                                  op->df_band.as<float4>());
+  k_df_band<<<nbk((size_t)n * bw), 256, 0, st>>>(
+      n, b, hard, make_pair_consts(op->omega, op->eta, op->h), op->g, op->wtab.as<double>(),
+      op->diag.as<double2>(), op->df_band.as<float4>());
   CFIE_CHECK_LAUNCH();
   if (op->layout != CFIE_STORED) {   // stored operators get them from the assembly
     op->df_rowexp.reserve(sizeof(int) * (size_t)n * (hard ? 2 : 1));

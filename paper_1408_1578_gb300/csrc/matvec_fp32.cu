@@ -424,7 +424,7 @@ __global__ void k_band_from_df(int n, int b, int bd, int ops, const float4* __re
 }
 
 template <int BC>
-__global__ void k_band_fill(int n, int b, double omega, double eta, geom_dev g,
+__global__ void k_band_fill(int n, int b, pair_consts pc, geom_dev g,
                             const double* __restrict__ wtab, const double2* __restrict__ diag,
                             float2* __restrict__ band, float2* __restrict__ band2) {
   const int bw = 2 * b + 1;
@@ -446,13 +446,12 @@ __global__ void k_band_fill(int n, int b, double omega, double eta, geom_dev g,
   } else {
     int d = i - j;
     if (d < 0) d += n;
-    const double h = 2.0 * CFIE_PI / n;
-    pair_entries_fp64<BC>(g.x[i] - g.x[j], g.y[i] - g.y[j], omega, eta, h, wtab[d], g.nx[j],
+    pair_entries_fp64<BC>(g.x[i] - g.x[j], g.y[i] - g.y[j], pc, wtab[n + d], g.nx[j],
                           g.ny[j], g.sp[j], g.nx[i], g.ny[i], g.sp[i], g.tab, a, bb);
   }
   band[e] = make_float2((float)a.x, (float)a.y);
   if (BC) {
-    const double2 c = hard_combined(g, omega, eta, i, j, a, bb);
+    const double2 c = hard_combined(g, pc.omega, pc.eta, i, j, a, bb);
     band2[e] = make_float2((float)c.x, (float)c.y);
   }
 }
@@ -553,16 +552,17 @@ void fp32_band(cfie_op* op) {
   cudaStream_t st = op->ctx->stream;
   float2* band = op->band.as<float2>();
   const bool hard = op->bc == CFIE_SOUND_HARD;
+  const pair_consts pc = make_pair_consts(op->omega, op->eta, op->h);
   if (op->df_b >= b) {
     k_band_from_df<<<nblk((size_t)n * bw), 256, 0, st>>>(n, b, op->df_b, hard ? 2 : 1,
                                                           op->df_band.as<float4>(), band);
   } else if (!hard) {
-    k_band_fill<0><<<nblk((size_t)n * bw), 256, 0, st>>>(n, b, op->omega, op->eta, op->g,
+    k_band_fill<0><<<nblk((size_t)n * bw), 256, 0, st>>>(n, b, pc, op->g,
                                                           op->wtab.as<double>(),
                                                           op->diag.as<double2>(), band, nullptr);
   } else {
     k_band_fill<1><<<nblk((size_t)n * bw), 256, 0, st>>>(
-        n, b, op->omega, op->eta, op->g, op->wtab.as<double>(), op->diag.as<double2>(), band,
+        n, b, pc, op->g, op->wtab.as<double>(), op->diag.as<double2>(), band,
         band + (size_t)n * bw);
   }
   CFIE_CHECK_LAUNCH();
