@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(DNT) k_pair_df(df_params P, size_t xstride) {
 //
 // Bound: the producers' FP32 arithmetic, about 340 operations per pair (290 for
 // the entry, 52 for the slices), issued in packed pairs.  Measured (GB300): kite
-// n = 32768, 64 right-hand sides 27.4 -> 16.8 ms (710 -> 340 instructions per
-// pair); star n = 4096, 16, sound hard: 1.88 -> 0.76 ms (two passes instead of
+// n = 32768, 64 right-hand sides 27.4 -> 16.7 ms (710 -> 340 operations per
+// pair); star n = 4096, 16, sound hard: 1.88 -> 0.77 ms (two passes instead of
 // three, the band sums 0.77 -> 0.1 ms).  The drain (one pass over the accumulators
 // per 128 sources, 40 operations per element) in packed pairs of columns: 18.1 ->
 // 16.8 ms.

@@ -18,8 +18,8 @@
 //    A table in shared memory holds sine and cosine of J 2 pi / 1024 - pi / 4; with
 //    |d| <= pi / 1024, sin d - d needs FP32 only (2e-6 d) and cos d - 1 two terms.
 //  * Hankel's asymptotic expansion (A&S 9.2.5, 9.2.9, 9.2.10) carries its leading
-//    terms in double-float and the small corrections in FP32: for omega r >= 48
-//    four terms of P and Q; pairs with 20 <= omega r < 48 (next to the band) are
+//    terms in double-float and the small corrections in FP32: for omega r >= 64
+//    four terms of P and Q; pairs with 20 <= omega r < 64 (next to the band) are
 //    redone one by one with seven and their first corrections in double-float.
 //    The dropped terms are below 1e-13.
 #pragma once
@@ -27,11 +27,14 @@
 #include "pair32.cuh"
 
 constexpr float kXD = 20.0f;   // asymptotic expansion for omega r >= 20
-constexpr float kXS = 48.0f;   // short series (small terms in FP32) for omega r >= 48
+// Short series (small terms in FP32) from here on: at 48 the products were off by up
+// to 1.3 times as much as with full series (2.5e-13 against 2.1e-13, ellipse n = 592),
+// at 64 by less than those (1.2e-13) for 0.6 to 1.6 % more time.
+constexpr float kXS = 64.0f;
 constexpr int kDfTab = 1024;   // (sin h, l, cos h, l) of 2 pi j / 1024 - pi / 4
 
 // ---------------------------------------------------------------------------
-// scalar double-float (drains, running sums, the 20 <= omega r < 48 series)
+// scalar double-float (drains, running sums, the 20 <= omega r < 64 series)
 // ---------------------------------------------------------------------------
 struct df {
   float h, l;
@@ -76,7 +79,7 @@ struct df_hankel2 {
   d2 dx, dy, t, ra, j0, y0, j1, y1;
 };
 
-// one source with 20 <= omega r < 48 (t = 1/x, sine and cosine of the phase):
+// one source with 20 <= omega r < 64 (t = 1/x, sine and cosine of the phase):
 // terms up to t^14 (P) and t^15 (Q), the first omitted one below 1e-14 at x =
 // 20; the t^2 term of P and the t^3 term of Q (up to 2e-4 and 1e-5 there) in
 // double-float
@@ -199,7 +202,7 @@ __device__ __forceinline__ df_hankel2 hankel_df2(float3 tx, float3 ty, float4 s0
     sn = turn(Sh, Sl, Ch, Cl);
     cs = turn(Ch, Cl, neg2(Sh), neg2(Sl));
   }
-  // x >= 48: terms up to t^8 (P) and t^7 (Q), the corrections in FP32 (t^2 with
+  // x >= 64: terms up to t^8 (P) and t^7 (Q), the corrections in FP32 (t^2 with
   // the lo part of t: its FP32 error, times the 0.07 t^2 term, stays below 3e-12
   // of P)
   const float2 th = H.t.h;

@@ -1,6 +1,6 @@
 """Residual matvecs at the edges of their tilings, both summation variants: 128-row tiles with
 ragged ends, tiles inside, across and outside the double-float band, pairs on both sides of
-omega r = 20 (band) and 48 (short series), right-hand-side passes of 4, 16, 32 and 64.
+omega r = 20 (band) and 64 (short series), right-hand-side passes of 4, 16, 32, 48 and 64.
 
 Bound 1e-11 per right-hand side, as for the other residual tests."""
 import numpy as np
