@@ -193,12 +193,18 @@ SLICE_OPS = 48                           # six 8-bit slices of the re / im parts
 FP64_NOMINAL_TFLOPS = 1.25               # GB300 FP64 (nominal; FMA = 2 flops)
 
 
+# FP32 operations per pair that the sound-soft tensor-core kernels now spend on
+# entries (packed FP32 and special-function operations; residual: with slicing):
+# "frac_spent" beside the fraction in the units of work above, which stay fixed so
+# that rates compare across versions and can exceed the peak
+SPENT_OPS = {"matvec_fp32": 52, "matvec_fp64": 342}
+
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one
 # ncu capture of the current kernel at the same launch configuration, keyed by
 # (kernel class, curve, n, nrhs, matvec variant); absent = not captured.
 NCU_TRAFFIC = {
-    ("matvec_fp32", "kite", 32768, 64, 2): 79.033088e6 + 11.152128e6,
-    ("matvec_fp64", "kite", 32768, 64, 2): 3.288266e9 + 157.754112e6,
+    ("matvec_fp32", "kite", 32768, 64, 2): 80.063232e6 + 12.190208e6,
+    ("matvec_fp64", "kite", 32768, 64, 2): 3.398163e9 + 206.532864e6,
 }
 
 
@@ -228,6 +234,8 @@ def kernel_rooflines(kt, spec, stats, peaks, src, n, solves_timed):
                                 + ("source sums on the tensor cores, not counted" if v == 2
                                    else f"{SUM_OPS[bc]} FMA per pair per right-hand side") + ")",
                         "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz"}
+            if v == 2 and bc == "soft":
+                out[cls]["frac_spent"] = a / fp32_peak * SPENT_OPS[cls] / ops
         elif cls == "matvec_fp64" and prec != "fp64" and stats.get("residual_variant") == 2:
             ent, sl = (DF_ENTRY_OPS, SLICE_OPS) if bc == "soft" else (DF_HARD_PASS_OPS, 2 * SLICE_OPS)
             ops = ent + sl
@@ -238,6 +246,8 @@ def kernel_rooflines(kt, spec, stats, peaks, src, n, solves_timed):
                                 "(double-float entries, slicing; slice products on the tensor "
                                 "cores, not counted)",
                         "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz"}
+            if bc == "soft":
+                out[cls]["frac_spent"] = a / fp32_peak * SPENT_OPS[cls] / ops
         elif cls == "matvec_fp64" and prec != "fp64":
             # S applied to the 3 vectors of Maue's identity and D' to x: 4 sums per RHS
             ent, terms = (DF_ENTRY_OPS, 1) if bc == "soft" else (DF_HARD_OPS, 4)
