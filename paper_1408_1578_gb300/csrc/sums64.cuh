@@ -11,7 +11,7 @@
 // (high x high, the two mixed products) give a real product, the tile's sums
 // stay below 2^63, and at its end one conversion and one FP64 multiply-add take
 // each of them to the FP64 accumulator.  Within a tile an addend is off by
-// less than 2^-57 of the largest entry times the largest density, and
+// at most 2^-56 of the largest entry times the largest density, and
 // additions are exact, where FP64 rounds each to 2^-53 of the sum so far.
 // Measured (GB300): star n = 4096, 16 right-hand sides, sound hard, 6.2 -> 3.2 ms;
 // 16 densities at 20000 points 20.7 -> 10.9 ms.
@@ -180,17 +180,11 @@ k_block64(block_args p) {
     for (int il = tid / 32; il < TI; il += NT / 32) {
       const int i = i0 + il, j = j0 + lane;
       double2 a = make_double2(0.0, 0.0), b = a;
-      if (i < p.rows && j < n) {
-        if (MODE != FIELD && i == j) {
-          a = MODE == HARD ? p.diag[2 * i] : p.diag[i];
-          if (MODE == HARD) b = p.diag[2 * i + 1];
-        } else {
-          pair_folded_fp64<MODE == HARD, MODE != FIELD>(
-              S.tx[il] - S.sx[lane], S.ty[il] - S.sy[lane], p.omega, p.omega_inv,
-              p.near, MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
-              S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
-        }
-      }
+      if (i < p.rows && j < n && (MODE == FIELD || i != j))
+        pair_folded_fp64<MODE == HARD, MODE != FIELD>(
+            S.tx[il] - S.sx[lane], S.ty[il] - S.sy[lane], p.omega, p.omega_inv, p.near,
+            MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
+            S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
       if (MODE == FIELD && p.rotate) a = make_double2(a.y, -a.x);
       int E = shared_exponent(a, bad);
       S.K[0][il][lane] = to_limbs(a, E);
@@ -206,8 +200,36 @@ k_block64(block_args p) {
     }
 
     // ---- contraction
-    if (__syncthreads_or(bad)) {
-      for (int jl = 0; jl < min(TJ, n - j0); ++jl)
+    const bool slow = __syncthreads_or(bad);
+    const int self = MODE == FIELD ? -1 : i0 + row - j0;   // the diagonal entry's source
+    if (MODE != FIELD && self >= 0 && self < TJ && i0 + row < n) {
+      // in FP64: sound soft it holds the 1/2 of the identity, whose exponent would
+      // take twelve bits from the other entries of the tile
+      const int i = i0 + row;
+      double2 d[NO];
+      d[0] = MODE == HARD ? p.diag[2 * i] : p.diag[i];
+      if constexpr (MODE == HARD) {
+        // C_ii = -D'_ii - i (omega^2 / eta) S_ii
+        const double k = p.omega * p.omega * p.eta_inv;
+        const double2 D = p.diag[2 * i + 1];
+        d[NO - 1] = make_double2(fma(k, d[0].y, -D.x), -fma(k, d[0].x, D.y));
+      }
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const double2* src = o == NO - 1 ? p.x : p.u;
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+          const int r = rg + RG * q;
+          if (r >= rbn) continue;
+          const double2 v = src[(size_t)(rb0 + r) * n + i];
+          acc[o][q].x = fma(-d[o].y, v.y, fma(d[o].x, v.x, acc[o][q].x));
+          acc[o][q].y = fma(d[o].y, v.x, fma(d[o].x, v.y, acc[o][q].y));
+        }
+      }
+    }
+    if (slow) {
+      for (int jl = 0; jl < min(TJ, n - j0); ++jl) {
+        if (jl == self) continue;
 #pragma unroll
         for (int o = 0; o < NO; ++o) {
           const int4 k = S.K[o][row][jl];
@@ -223,6 +245,7 @@ k_block64(block_args p) {
             acc[o][q].y = fma(ki, v.x, fma(kr, v.y, acc[o][q].y));
           }
         }
+      }
       continue;
     }
     fixed_acc re[NO][RQ], im[NO][RQ];

@@ -126,3 +126,25 @@ def test_field_block_widths(ctx, bc, nrhs):
     got[2] *= 2.0 ** 900
     assert np.max(np.abs(got - want)) < TOL * np.max(np.abs(want))
     op.close()
+
+
+@pytest.mark.parametrize("bc", ["soft", "hard"])
+def test_unit_columns(ctx, bc):
+    """Unit densities give the matrix entry by entry, next to the diagonal too: the entries of a
+    column to 1e-12 of the column's largest off-diagonal one (sound soft the diagonal, 1/2, is a
+    thousand times that)."""
+    n, omega, j = 1026, 60.0, 517
+    A = operators.cfie_matrix(geometry.kite(n), omega, omega, bc)
+    op = ctx.kite().discretise(n, omega, bc=bc, precision="fp64")
+    X = np.zeros((8, n), complex)
+    X[np.arange(8), j + 40 * np.arange(8)] = 1.0
+    y = empty(8, n)
+    op.apply_fp64(to_dev(X), y)
+    got = to_host(y)
+    for k in range(8):
+        c = A[:, j + 40 * k].copy()
+        off = np.arange(n) != j + 40 * k
+        scale = np.max(np.abs(c[off])) if bc == "soft" else np.max(np.abs(c))
+        assert np.max(np.abs(got[k] - c)[off]) < TOL * scale, k
+        assert abs(got[k] - c)[~off].max() < TOL * np.max(np.abs(c)), k
+    op.close()
