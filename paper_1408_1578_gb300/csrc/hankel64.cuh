@@ -284,9 +284,11 @@ __device__ __forceinline__ values far(double x, double t, double amp, const doub
 }
 
 // 0 < x < 20, t = 1 / x: Taylor polynomials about c = k / 2, k nearest 2 x,
-// Horner's scheme for each value and derivative
+// Horner's scheme for each value and derivative.  A NaN with its sign set (a field
+// point that is not a number) also comes here; as an integer it is -2^31, which
+// must not address the table.
 __device__ __forceinline__ values taylor(double x, double t, double amp, const double2* __restrict__ tab) {
-  const int k = __double2int_rn(2.0 * x);
+  const int k = min(max(__double2int_rn(2.0 * x), 0), kNear - 1);
   const double d = fma((double)k, -0.5, x);
   const double2* a = tab + 2 * kTrig + k * kTaylor;
   double2 q = __ldg(a + kTaylor - 1);
