@@ -16,8 +16,12 @@
 // Measured (GB300): star n = 4096, 16 right-hand sides, sound hard, 6.2 -> 3.2 ms;
 // 16 densities at 20000 points 20.7 -> 10.9 ms.
 //
-// A tile with a value that this does not hold (infinities, NaN, exponents
-// beyond 2^+-420) takes FP64 multiply-adds instead.
+// So an addend loses what lies between the largest entry times the largest
+// density and itself, which is at most the smaller of the two ranges: where a row's
+// entries in a tile range over more than 2^kSpread and so does a column of
+// densities, the row's sums of that tile are FP64 multiply-adds with the entries as
+// they were evaluated.  So they are in a tile with a value that fixed point does not
+// hold (infinities, NaN, exponents beyond 2^+-420).
 //
 // Layout: a CTA owns TI rows and walks its range of source tiles.  It evaluates
 // the TI x 32 block of entries into shared memory (one warp per row, lanes over
@@ -44,24 +48,34 @@ __device__ __forceinline__ void to_limbs(double v, int E, int& hi, int& lo) {
   hi = (int)((V + (1 << 28)) >> 29);
   lo = (int)((unsigned)V - ((unsigned)hi << 29));
 }
-__device__ __forceinline__ double from_limbs(int hi, int lo, int E) {
-  if (E == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
-  return scalbn((double)(((long long)hi << 29) + lo), E - 1079);
-}
 __device__ __forceinline__ int4 to_limbs(double2 v, int E) {
   int4 q;
   to_limbs(v.x, E, q.x, q.y);
   to_limbs(v.y, E, q.z, q.w);
   return q;
 }
-// exponent of the largest of a warp's values; bad: one that the fixed-point sums
-// do not hold.  Zeros only: any exponent in range does.
-__device__ __forceinline__ int shared_exponent(double2 v, bool& bad) {
+// Range of a row's or a column's 32 values, from which the sums' form follows.  An
+// addend is off by 2^-56 of the largest entry times the largest density, so with
+// one of the ranges up to 2^kSpread a tile's sum is off by about 2^(kSpread - 53) of
+// sum |K x| at the very worst (one small product alone), where even values leave
+// 2^-56.  Random densities range wider than 2^7 in 5 of 1000 columns of a tile
+// (normal) or 1 of 2000 (uniform), entries where sound hard C, or the 1 +- cos of the
+// others, goes through zero.  Measured (GB300), against no limit at all: 2^7 star n
+// = 4096, 16, sound hard 2.25 -> 2.25 ms, field 6.85 -> 6.85 ms; 2^6 2.28, 6.99 ms.
+constexpr int kSpread = 7;
+constexpr int kRaw = 1 << 16;   // with a row's exponent: entries kept in FP64
+struct tile_range {
+  int e;           // exponent of the largest (zeros only: any)
+  bool out, wide;  // not held in fixed point; smallest of the valid ones 2^-kSpread below
+};
+__device__ __forceinline__ tile_range range_of(double2 v, bool valid) {
   const unsigned a = __double2hiint(v.x) & 0x7fffffff, b = __double2hiint(v.y) & 0x7fffffff;
-  const int E = (int)(__reduce_max_sync(0xffffffffu, max(a, b)) >> 20);
-  if (E >= 600 && E <= 1500) return E;
-  bad |= __any_sync(0xffffffffu, (a | b | __double2loint(v.x) | __double2loint(v.y)) != 0);
-  return E ? E : 1023;
+  const unsigned m = max(a, b);
+  const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+  const int least = (int)(__reduce_min_sync(0xffffffffu, valid ? m : 0xffffffffu) >> 20);
+  if (E >= 600 && E <= 1500) return {E, false, E - least > kSpread};
+  const bool any = __any_sync(0xffffffffu, (a | b | __double2loint(v.x) | __double2loint(v.y)) != 0);
+  return {E ? E : 1023, any, false};
 }
 
 // sums of products of limbs: high x high, and the mixed ones 2^29 below
@@ -98,9 +112,10 @@ struct block_smem {
   double tfx[NO == 2 ? TI : 1], tfy[NO == 2 ? TI : 1], tux[NO == 2 ? TI : 1], tuy[NO == 2 ? TI : 1];
   double sx[TJ], sy[TJ], sfx[TJ], sfy[TJ], se[TJ];
   double wk[TI + TJ];                    // Kress weights of the tile, by i - j
-  int4 K[NO][TI][TJ + 1];                // limbs (re, im): the entries; HARD: S, C
+  int4 K[NO][TI][TJ + 1];                // limbs (re, im): the entries; HARD: S, C; raw rows: double2
   int4 X[NO][TJ][RBT];                   // densities; HARD: u, x
   int ek[NO][TI], ex[NO][RBT];
+  int cols[NO];                          // 1: a wide column of densities, 2: one out of range
 };
 
 template <int MODE, int TI, int RBT, int RG>
@@ -138,6 +153,8 @@ k_block64(block_args p) {
     }
   }
 
+  if (tid < NO) S.cols[tid] = 0;
+
   const int row = tid % TI, rg = tid / TI;
   double2 acc[NO][RQ];
 #pragma unroll
@@ -147,7 +164,6 @@ k_block64(block_args p) {
 
   for (int t = t_begin; t < t_end; ++t) {
     const int j0 = t * TJ;
-    bool bad = false;
     __syncthreads();
     if (tid < TJ) {
       const int j = j0 + tid;
@@ -170,37 +186,50 @@ k_block64(block_args p) {
       const int o = c / RBT, r = c % RBT, j = j0 + lane;
       const double2* src = o == NO - 1 ? p.x : p.u;
       const double2 v = j < n && r < rbn ? src[(size_t)(rb0 + r) * n + j] : make_double2(0.0, 0.0);
-      const int E = shared_exponent(v, bad);
-      S.X[o][lane][r] = to_limbs(v, E);
-      if (lane == 0) S.ex[o][r] = E;
+      const tile_range span = range_of(v, j < n);
+      S.X[o][lane][r] = to_limbs(v, span.e);
+      if (lane == 0) {
+        S.ex[o][r] = span.e;
+        if (span.out || span.wide) atomicOr(&S.cols[o], span.out ? 2 : 1);
+      }
     }
     __syncthreads();
 
     // ---- entries of the TI x TJ block
     for (int il = tid / 32; il < TI; il += NT / 32) {
       const int i = i0 + il, j = j0 + lane;
+      const bool in = i < p.rows && j < n && (MODE == FIELD || i != j);
       double2 a = make_double2(0.0, 0.0), b = a;
-      if (i < p.rows && j < n && (MODE == FIELD || i != j))
+      if (in)
         pair_folded_fp64<MODE == HARD, MODE != FIELD>(
             S.tx[il] - S.sx[lane], S.ty[il] - S.sy[lane], p.omega, p.omega_inv, p.near,
             MODE == HARD ? S.tfx[il] : S.sfx[lane], MODE == HARD ? S.tfy[il] : S.sfy[lane],
             S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
       if (MODE == FIELD && p.rotate) a = make_double2(a.y, -a.x);
-      int E = shared_exponent(a, bad);
-      S.K[0][il][lane] = to_limbs(a, E);
-      if (lane == 0) S.ek[0][il] = E;
+      auto keep = [&](int o, double2 v) {
+        const tile_range span = range_of(v, in);
+        const int c = S.cols[o];
+        const bool raw = span.out || (c & 2) || (c && span.wide);
+        int4 q;
+        if (raw)
+          q = make_int4(__double2loint(v.x), __double2hiint(v.x), __double2loint(v.y),
+                        __double2hiint(v.y));
+        else
+          q = to_limbs(v, span.e);
+        S.K[o][il][lane] = q;
+        if (lane == 0) S.ek[o][il] = raw ? span.e | kRaw : span.e;
+      };
+      keep(0, a);
       if constexpr (MODE == HARD) {
         // C = -D' - i (omega^2 / eta) (n_i . n_j) S
         const double k = fma(S.tux[il], S.sfx[lane], S.tuy[il] * S.sfy[lane]);
-        const double2 c = make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y));
-        E = shared_exponent(c, bad);
-        S.K[NO - 1][il][lane] = to_limbs(c, E);
-        if (lane == 0) S.ek[NO - 1][il] = E;
+        keep(NO - 1, make_double2(fma(k, a.y, -b.x), -fma(k, a.x, b.y)));
       }
     }
 
     // ---- contraction
-    const bool slow = __syncthreads_or(bad);
+    __syncthreads();
+    if (tid < NO) S.cols[tid] = 0;
     const int self = MODE == FIELD ? -1 : i0 + row - j0;   // the diagonal entry's source
     if (MODE != FIELD && self >= 0 && self < TJ && i0 + row < n) {
       // in FP64: sound soft it holds the 1/2 of the identity, whose exponent would
@@ -227,27 +256,6 @@ k_block64(block_args p) {
         }
       }
     }
-    if (slow) {
-      for (int jl = 0; jl < min(TJ, n - j0); ++jl) {
-        if (jl == self) continue;
-#pragma unroll
-        for (int o = 0; o < NO; ++o) {
-          const int4 k = S.K[o][row][jl];
-          const double kr = from_limbs(k.x, k.y, S.ek[o][row]);
-          const double ki = from_limbs(k.z, k.w, S.ek[o][row]);
-          const double2* src = o == NO - 1 ? p.x : p.u;
-#pragma unroll
-          for (int q = 0; q < RQ; ++q) {
-            const int r = rg + RG * q;
-            if (r >= rbn) continue;
-            const double2 v = src[(size_t)(rb0 + r) * n + j0 + jl];
-            acc[o][q].x = fma(-ki, v.y, fma(kr, v.x, acc[o][q].x));
-            acc[o][q].y = fma(ki, v.x, fma(kr, v.y, acc[o][q].y));
-          }
-        }
-      }
-      continue;
-    }
     fixed_acc re[NO][RQ], im[NO][RQ];
 #pragma unroll
     for (int o = 0; o < NO; ++o)
@@ -268,13 +276,34 @@ k_block64(block_args p) {
         }
       }
 #pragma unroll
-    for (int o = 0; o < NO; ++o)
+    for (int o = 0; o < NO; ++o) {
+      const int ek = S.ek[o][row];
+      if (!(ek & kRaw)) {
 #pragma unroll
-      for (int q = 0; q < RQ; ++q) {
-        const int scale = (S.ek[o][row] + S.ex[o][rg + RG * q] - 1077) << 20;
-        re[o][q].flush(acc[o][q].x, scale);
-        im[o][q].flush(acc[o][q].y, scale);
+        for (int q = 0; q < RQ; ++q) {
+          const int scale = (ek + S.ex[o][rg + RG * q] - 1077) << 20;
+          re[o][q].flush(acc[o][q].x, scale);
+          im[o][q].flush(acc[o][q].y, scale);
+        }
+        continue;
       }
+      // the row's entries are in FP64, the sums above meaningless
+      const double2* src = o == NO - 1 ? p.x : p.u;
+#pragma unroll 1
+      for (int jl = 0; jl < min(TJ, n - j0); ++jl) {
+        if (jl == self) continue;
+        const int4 k = S.K[o][row][jl];
+        const double kr = __hiloint2double(k.y, k.x), ki = __hiloint2double(k.w, k.z);
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+          const int r = rg + RG * q;
+          if (r >= rbn) continue;
+          const double2 v = src[(size_t)(rb0 + r) * n + j0 + jl];
+          acc[o][q].x = fma(-ki, v.y, fma(kr, v.x, acc[o][q].x));
+          acc[o][q].y = fma(ki, v.x, fma(kr, v.y, acc[o][q].y));
+        }
+      }
+    }
   }
 
   const int i = i0 + row;
