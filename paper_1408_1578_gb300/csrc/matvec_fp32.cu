@@ -351,7 +351,8 @@ __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w
   pk[i] = make_float4(xh, xl, yh, yl);
   pk[n + i] = make_float4((float)(omega * f * nx), (float)(omega * f * ny),
                           (float)(f * eta * sp), (float)(f * sp));
-  pk[2 * n + i] = make_float4((float)(omega * nx / sp), (float)(omega * ny / sp), 0.f, 0.f);
+  pk[2 * n + i] =
+      make_float4((float)(2.0 * omega * nx / sp), (float)(2.0 * omega * ny / sp), 0.f, 0.f);
   // source data by pairs: value v of node i at 4 (i / 2 * 2 + v / 2) + 2 (v % 2) + i % 2
   float* sq = sp4 + (size_t)(i / 2) * 8 + (i & 1);
   sq[0] = -xh;
@@ -359,8 +360,8 @@ __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w
   sq[4] = -yh;
   sq[6] = -yl;
   sq += (size_t)4 * n;
-  sq[0] = (float)(hard ? omega / eta * nx / sp : omega * f * nx);
-  sq[2] = (float)(hard ? omega / eta * ny / sp : omega * f * ny);
+  sq[0] = (float)(hard ? 0.5 * omega / eta * nx / sp : 2.0 * omega * f * nx);
+  sq[2] = (float)(hard ? 0.5 * omega / eta * ny / sp : 2.0 * omega * f * ny);
   sq[4] = (float)(hard ? f * sp : f * eta * sp);
   sq[6] = 0.f;
 }

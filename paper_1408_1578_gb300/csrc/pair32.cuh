@@ -12,15 +12,16 @@
 // tensor-core kernel, starting on 16-byte boundaries:
 //   n float4 coordinates      (omega x hi, lo, omega y hi, lo)
 //   n float4 source factors   (omega hq c0 nu1, omega hq c0 nu2, hq c0 eta |z'|, hq c0 |z'|)
-//   n float4 target factors   (omega nu1 / |z'|, omega nu2 / |z'|, 0, 0)
+//   n float4 target factors   2 omega (nu1, nu2) / |z'|, 0, 0
 //   2 n + 8 float2: the Kress table twice over divided by pi h, entry
 //   k = i - j + n holding the weights of sources j and j + 1,
 //   (w_{k mod n}, w_{(k - 1) mod n}) / (pi h), then zeros
 //   n float4 source coordinates by pairs j, j + 1 (n is even), negated:
 //   (-xh_j, -xh_j+1, -xl_j, -xl_j+1), (-yh_j, ..)
 //   n float4 source factors by pairs, (a_j, a_j+1, b_j, b_j+1), (c_j, c_j+1, 0, 0):
-//   soft a, b = omega hq c0 nu, c = hq c0 eta |z'|; hard a, b = (omega / eta)
+//   soft a, b = 2 omega hq c0 nu, c = hq c0 eta |z'|; hard a, b = (omega / (2 eta))
 //   nu / |z'|, c = hq c0 |z'|
+// (the entries of pairs carry 1 / (2 x) in the place of 1 / x)
 // with hq = h / 4 and c0 = sqrt(2 / pi) (nu = unnormalised normal, |z'| = speed).
 struct geo32 {
   float *xh, *xl, *yh, *yl, *nx, *ny, *sp;
@@ -237,7 +238,7 @@ __device__ __forceinline__ float2 entry_folded32(float4 tg, float4 sc, float4 sq
 
 // as pair_phase, for the two sources
 struct pair_phase2 {
-  float2 dx, dy, xinv, ra, chi;   // chi = x - pi/4 less a multiple of 2 pi
+  float2 dx, dy, half, ra, chi;   // half = 1 / (2 x), chi = x - pi/4 less a multiple of 2 pi
 };
 
 // pair_phase32_tc for both sources: t0, t1 the target's (xh, xh, xl, xl), (yh,
@@ -252,11 +253,12 @@ __device__ __forceinline__ pair_phase2 phase32_pair(float4 t0, float4 t1, float4
   f.dy = add2(dyh, dyl);
   const float2 C = fma2(dxl, add2(dxh, f.dx), mul2(dyl, add2(dyh, f.dy)));
   const float2 x2 = add2(H, C);
-  f.xinv = make_float2(rsqrt_sfu(x2.x), rsqrt_sfu(x2.y));
-  const float2 xh = mul2(x2, f.xinv);
+  const float2 xinv = make_float2(rsqrt_sfu(x2.x), rsqrt_sfu(x2.y));
+  const float2 xh = mul2(x2, xinv);
   f.ra = make_float2(rsqrt_sfu(xh.x), rsqrt_sfu(xh.y));
   const float2 e = add2(fma2(neg2(xh), xh, H), C);                // x^2 - xh^2
-  const float2 xl = fma2(e, mul2(f.xinv, f2(0.5f)), f2(-kPi4H));             // x lo - pi/4
+  f.half = mul2(xinv, f2(0.5f));
+  const float2 xl = fma2(e, f.half, f2(-kPi4H));                             // x lo - pi/4
   const float2 kr = add2(fma2(xh, f2(kInv2Pi), f2(-0.125f)), f2(12582912.0f));
   const float2 k = add2(kr, f2(-12582912.0f));
   f.chi = add2(fma2(k, f2(-kC2), fma2(k, f2(-kC1), xh)), xl);                // first fma exact
@@ -265,25 +267,31 @@ __device__ __forceinline__ pair_phase2 phase32_pair(float4 t0, float4 t1, float4
 
 // H_nu(x) = c0 ra m_nu exp(i (chi + psi_nu - nu pi / 2)) of both sources, as
 // modulus and phase (A&S 9.2.28, 9.2.29: two terms each): j0 = m0 c0, w0 = y0 + wk
-// j0 = m0 u0, j1 = m1 s1, w1 = y1 + wk j1 = m1 u1.  Two more sines and cosines on the
-// special-function unit than with P and Q, but six packed instructions of 52
-// fewer on the FMA pipe, which bounds the fused kernel: kite n = 32768, 64 right-hand
-// sides 2.51 -> 2.44 ms.
+// j0 = m0 u0, j1 = m1 s1, w1 = y1 + wk j1 = m1 u1.  m1 = 1 + 3 t^2 / 16 - 0.193 t^4 ..
+// takes psi_1 / t = 3/8 - 0.164 t^2 times t^2 / 2, which costs nothing and holds -0.082
+// of the third term: at omega r = 16 the entries are off by 1.6e-6 of H0 and 1.7e-6 of
+// H1 (two terms of P and Q: 1.7e-6 and 2.2e-6; m1 with two terms 2.9e-6, with three
+// 3.5e-7 and 4 % more time for the kite).  Everything is in u = t^2 / 4 and h = t / 2,
+// which the phase needs anyway; the factors of two sit in the node data.  Two more
+// sines and cosines on the special-function unit than with P and Q, but six packed
+// instructions of 52 fewer on the FMA pipe, which bounds the fused kernel: kite n =
+// 32768, 64 right-hand sides 2.51 -> 2.45 ms.
 struct hankel_pair {
   float2 m0, m1, c0, u0, s1, u1;
 };
 __device__ __forceinline__ hankel_pair hankel32_pair(const pair_phase2& f, float2 wk) {
-  const float2 ti = f.xinv, t2 = mul2(ti, ti);
-  const float2 a0 = fma2(ti, fma2(t2, f2(25.0f / 384.0f), f2(-0.125f)), f.chi);
-  const float2 a1 = fma2(ti, fma2(t2, f2(-21.0f / 128.0f), f2(0.375f)), f.chi);
+  const float2 u = mul2(f.half, f.half);   // t^2 / 4
+  const float2 q1 = fma2(u, f2(-21.0f / 16.0f), f2(0.75f));
+  const float2 a0 = fma2(f.half, fma2(u, f2(25.0f / 48.0f), f2(-0.25f)), f.chi);
+  const float2 a1 = fma2(f.half, q1, f.chi);
   hankel_pair h;
   float2 s0, c1;
   sincos_sfu(a0.x, &s0.x, &h.c0.x);
   sincos_sfu(a0.y, &s0.y, &h.c0.y);
   sincos_sfu(a1.x, &h.s1.x, &c1.x);
   sincos_sfu(a1.y, &h.s1.y, &c1.y);
-  h.m0 = fma2(t2, f2(-0.0625f), f2(1.0f));
-  h.m1 = fma2(t2, f2(0.1875f), f2(1.0f));
+  h.m0 = fma2(u, f2(-0.25f), f2(1.0f));
+  h.m1 = fma2(u, q1, f2(1.0f));
   h.u0 = fma2(wk, h.c0, s0);
   h.u1 = fma2(wk, h.s1, neg2(c1));
   return h;
@@ -292,8 +300,8 @@ __device__ __forceinline__ hankel_pair hankel32_pair(const pair_phase2& f, float
 // Operators of the fused kernel: the sound-soft one (eq. 1); of the sound-hard
 // one (eq. 2, Maue's identity summed over the pairs) S' = -i S, applied to u =
 // d/ds x, and C = -D' - i (omega^2 / eta) (n_i . n_j) S, applied to x; or both
-// from one phase.  With A = c ra, B (soft) = (a, b).(dx, dy) ra / x, D =
-// (tq).(dx, dy) A / x, kn = tq.(a, b) = (omega^2 / eta) n_i . n_j:
+// from one phase.  With A = c ra, B (soft) = (a, b).(dx, dy) ra / (2 x), D =
+// (tq).(dx, dy) A / (2 x), kn = tq.(a, b) = (omega^2 / eta) n_i . n_j:
 //   soft: re = A j0 - B w1,           im = A w0 + B j1
 //   S':   re = A j0,                  im = A w0
 //   C:    re = kn A j0 - D w1,        im = kn A w0 + D j1
@@ -304,7 +312,7 @@ struct entry_pair {
   float2 re2, im2;   // OP_SC: C (the first is S')
 };
 
-// tq = (tx, tx, ty, ty) target factors omega nu / |z'| (hard), s2, s3 the source
+// tq = (tx, tx, ty, ty) target factors 2 omega nu / |z'| (hard), s2, s3 the source
 // factors by pairs
 template <int OP>
 __device__ __forceinline__ entry_pair finish32_pair(const pair_phase2& f, float4 tq, float4 s2,
@@ -314,7 +322,7 @@ __device__ __forceinline__ entry_pair finish32_pair(const pair_phase2& f, float4
   entry_pair e;
   if constexpr (OP == OP_SOFT) {
     const float2 B = mul2(fma2(f.dx, lo2(s2), mul2(f.dy, hi2(s2))),
-                          mul2(h.m1, mul2(f.xinv, f.ra)));
+                          mul2(h.m1, mul2(f.half, f.ra)));
     e.re = fma2(A0, h.c0, mul2(neg2(B), h.u1));
     e.im = fma2(A0, h.u0, mul2(B, h.s1));
   } else {
@@ -325,7 +333,7 @@ __device__ __forceinline__ entry_pair finish32_pair(const pair_phase2& f, float4
     }
     if constexpr (OP == OP_C || OP == OP_SC) {
       const float2 D = mul2(fma2(f.dx, lo2(tq), mul2(f.dy, hi2(tq))),
-                            mul2(h.m1, mul2(f.xinv, A)));
+                            mul2(h.m1, mul2(f.half, A)));
       const float2 kn = fma2(lo2(tq), lo2(s2), mul2(hi2(tq), hi2(s2)));
       const float2 cr = fma2(kn, sr, mul2(neg2(D), h.u1));
       const float2 ci = fma2(kn, si, mul2(D, h.s1));

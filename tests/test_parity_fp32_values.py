@@ -1,0 +1,46 @@
+"""FP32 entries of the tensor-core sums on their own."""
+import numpy as np
+import pytest
+
+from oracle import geometry, operators
+from paper_1408_1578_gb300 import inputs
+from tests.gpu_util import empty, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1408_1578_gb300 import cfie
+    c = cfie.Context(0)
+    yield c
+    c.close()
+
+
+def test_amplitude_next_to_the_band(ctx):
+    """Unit columns give single entries; with eta small against omega they are H1 times plain
+    factors.  Their mean amplitude over the pairs with 16.4 < omega r < 17.4, the largest arguments
+    of the short series, is no further off than with two terms of P and Q (the leading dropped one
+    is 0.144 / x^4), and 3e-7 for the arithmetic: two special-function values of 1.2e-7, one and a
+    half of them in the amplitude, FP32 per-node factors (6e-8), and the bf16 hi + lo splits (up to
+    3e-6, but of either sign) averaged over a thousand distances."""
+    n, omega, m = 4096, 64.0, 64
+    eta = omega * 1e-6
+    c = geometry.ellipse(n, 1.0, 0.8)
+    op = ctx.ellipse(1.0, 0.8).discretise(n, omega, eta=eta, bc="soft", precision="fp32")
+    op.set_variant(2)
+    cols = (3 * np.arange(m) - 96) % n          # about the slowest node, where the band is widest
+    rows = np.arange(-450, 450) % n
+    X = np.zeros((m, n), complex)
+    X[np.arange(m), cols] = 1.0
+    y = empty(m, n)
+    op.apply(to_dev(X), y)
+    got = to_host(y)[:, rows]
+    D, S = (operators.layer_rows(c, omega, rows, k)[:, cols].T for k in "DS")
+    A = D - 1j * eta * S
+    x = omega * np.hypot(*(c.z[rows][None, :, :] - c.z[cols][:, None, :]).transpose(2, 0, 1))
+    pick = (x > 16.4) & (x < 17.4)
+    assert pick.sum() > 1000
+    bias = np.mean(np.abs(got[pick]) / np.abs(A[pick])) - 1.0
+    assert abs(bias) < np.mean(0.144195556640625 / x[pick] ** 4) + 3e-7, bias
+    op.close()
