@@ -210,8 +210,9 @@ __global__ void __launch_bounds__(NT, 2) k_pair_fp32(pair_params P) {
 }
 
 // y = sum of split partials, as FP32 pairs (TwoSum, errors gathered: 48 bits,
-// without the FP64 pipe); hard: t = S u (complex64 for the derivative) and
-// y = 1/2 x + C x
+// without the FP64 pipe), in FP64 where those are not finite (TwoSum makes NaN of
+// an infinity, and the sum may pass the range of FP32); hard: t = S u (complex64
+// for the derivative) and y = 1/2 x + C x
 template <int BC>
 __global__ void k_reduce32(size_t tot, int splits, const float2* __restrict__ part,
                            const double2* __restrict__ x, float2* __restrict__ t_out,
@@ -234,6 +235,14 @@ __global__ void k_reduce32(size_t tot, int splits, const float2* __restrict__ pa
       two_sum(v.y, err.y, p.y);
     }
     s[o] = make_double2((double)v.x + (double)err.x, (double)v.y + (double)err.y);
+    if (!isfinite(err.x) || !isfinite(err.y)) {
+      s[o] = make_double2(0.0, 0.0);
+      for (int sp = 0; sp < splits; ++sp) {
+        const float2 p = part[((size_t)o * splits + sp) * tot + e];
+        s[o].x += p.x;
+        s[o].y += p.y;
+      }
+    }
   }
   if (BC == 0) {
     y[e] = s[0];

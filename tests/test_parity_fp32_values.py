@@ -1,8 +1,9 @@
-"""FP32 entries of the tensor-core sums on their own."""
+"""FP32 entries of the tensor-core sums on their own, and densities that are not finite."""
 import numpy as np
 import pytest
 
 from oracle import geometry, operators
+from paper_1408_1578_gb300 import inputs
 from paper_1408_1578_gb300 import inputs
 from tests.gpu_util import empty, to_dev, to_host
 
@@ -43,4 +44,22 @@ def test_amplitude_next_to_the_band(ctx):
     assert pick.sum() > 1000
     bias = np.mean(np.abs(got[pick]) / np.abs(A[pick])) - 1.0
     assert abs(bias) < np.mean(0.144195556640625 / x[pick] ** 4) + 3e-7, bias
+    op.close()
+
+
+def test_infinite_density_gives_infinities(ctx):
+    """A density with one infinite real part: every product of its column is infinite, as FP64
+    sums of the splits' partial sums have it; the other columns stay as they are."""
+    n, omega, nrhs = 512, 30.0, 9
+    op = ctx.kite().discretise(n, omega, bc="soft", precision="fp32")
+    op.set_variant(1)
+    X = inputs.random_density(n, nrhs, seed=2)
+    y0, y1 = empty(nrhs, n), empty(nrhs, n)
+    op.apply(to_dev(X), y0)
+    X[3, 100] = complex(np.inf, 0.0)
+    op.apply(to_dev(X), y1)
+    a, b = to_host(y0), to_host(y1)
+    assert np.isinf(b[3].real).all() and np.isinf(b[3].imag).all()
+    keep = np.arange(nrhs) != 3
+    assert np.array_equal(a[keep], b[keep])
     op.close()
