@@ -23,9 +23,10 @@
 // partial sums in a fixed order by the problem's last CTA to finish.
 //
 // Bound: HBM (or L2, when the basis fits) for large sets, latency for small
-// ones.  The chunk length (128 to 2048 elements) is chosen so that the set has
-// about two CTAs per SM, the inner products of a small set are also split over
-// the basis vectors, loads of four basis vectors are in flight at once, the four
+// ones.  The chunk length (128 to 2048 elements) is chosen so that the columns of
+// one operator have about two CTAs per SM (a set with several lengths takes a launch
+// for each), the inner products of a small set are also split over the basis
+// vectors, loads of four basis vectors are in flight at once, the four
 // pairs of sums are reduced across a warp together (9 shuffles instead of 40;
 // on GB300 the FP64 additions of a plain reduction cost more than the products),
 // and an Arnoldi step is 5 launches instead of 9.  Measured (GB300): unrestarted
@@ -72,12 +73,12 @@ struct chunk_ref {
 };
 
 __device__ __forceinline__ chunk_ref chunk_of(const pset_dev& ps, int item) {
-  const int2 it = ps.items[item];
+  const int4 it = __ldg(reinterpret_cast<const int4*>(ps.items) + ps.first + item);
   chunk_ref r;
-  r.p = it.x;
-  r.base = ps.off[it.x] + (size_t)it.y * ps.ch;
-  r.cnt = min(ps.ch, ps.len[it.x] - it.y * ps.ch);
-  r.slot = ps.chb[it.x] + it.y;
+  r.base = (size_t)(unsigned)it.x | (size_t)(unsigned)it.y << 32;
+  r.cnt = it.z;
+  r.p = it.w;
+  r.slot = ps.first + item;
   return r;
 }
 
@@ -127,6 +128,7 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
   if (!act[c.p]) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int j0 = blockIdx.y * JB, j1 = min(J + 1, j0 + JB);
+  const int nch = ps.nch[c.p], chb = ps.chb[c.p];   // early, for the last CTA
   two<T> wr[PT];
 #pragma unroll
   for (int e = 0; e < PT; ++e) {
@@ -134,7 +136,10 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
     wr[e].a = wr[e].b = basis_t<T>::make(0.0, 0.0);
     if (q < c.cnt) wr[e] = load2(w + c.base + q);
   }
-  for (int jj = j0; jj < j1; jj += AB) {
+  // (an advancing pointer: with the index of the vector in each address the compiler
+  // kept half of the loads in flight, kite n = 8192, 64 directions, 30.5 ms against 29.9)
+  const T* vp = V + (size_t)j0 * L + c.base;
+  for (int jj = j0; jj < j1; jj += AB, vp += AB * L) {
     two<T> v[AB][PT];
 #pragma unroll
     for (int b = 0; b < AB; ++b)
@@ -142,7 +147,7 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
       for (int e = 0; e < PT; ++e) {
         const int q = 2 * (e * blockDim.x + threadIdx.x);
         v[b][e].a = v[b][e].b = basis_t<T>::make(0.0, 0.0);
-        if (q < c.cnt && jj + b < j1) v[b][e] = load2(V + (size_t)(jj + b) * L + c.base + q);
+        if (q < c.cnt && jj + b < j1) v[b][e] = load2(vp + b * L + q);
       }
     S s[2 * AB];
 #pragma unroll
@@ -189,7 +194,6 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
     }
     partial[(size_t)c.slot * (J + 1) + jj] = t;
   }
-  const int nch = ps.nch[c.p], chb = ps.chb[c.p];
   if (!last_cta(counter + c.p, nch * gridDim.y)) return;
   for (int jj = threadIdx.x; jj <= J; jj += blockDim.x) {
     double2 t = make_double2(0.0, 0.0);
@@ -333,6 +337,7 @@ k_update(int J, int m, const T* __restrict__ V, size_t L, const double2* __restr
       }
     }
   }
+  const int nch = GIVENS ? ps.nch[c.p] : 0, chb = GIVENS ? ps.chb[c.p] : 0;
   S ss = 0;
 #pragma unroll
   for (int e = 0; e < PT; ++e) {
@@ -353,7 +358,6 @@ k_update(int J, int m, const T* __restrict__ V, size_t L, const double2* __restr
       for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q];
       nrm_partial[c.slot] = t;
     }
-    const int nch = ps.nch[c.p], chb = ps.chb[c.p];
     if (!last_cta(counter + c.p, nch)) return;
     if (threadIdx.x < 32) {
       double s2 = 0.0;
@@ -521,10 +525,13 @@ k_residual(pset_dev ps, const double2* __restrict__ f, const double2* __restrict
            double2* __restrict__ r, double* __restrict__ rr, double* __restrict__ ff) {
   const chunk_ref c = chunk_of(ps, blockIdx.x);
   double sr = 0.0, sf = 0.0;
+  // pairs of elements as in the other kernels: the order of the sums is the
+  // chunk's, not the CTA's
 #pragma unroll 4
-  for (int q = threadIdx.x; q < c.cnt; q += blockDim.x) {
-    {
-      const size_t idx = c.base + q;
+  for (int q = 2 * threadIdx.x; q < c.cnt; q += 2 * blockDim.x) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const size_t idx = c.base + q + u;
       const double2 fv = f[idx];
       double2 v = fv;
       if (ax) {
@@ -688,13 +695,18 @@ void residual_norms(cudaStream_t st, krylov_ws& K, const pset& ps, const ws& W,
   fn.assign(K.host + P, K.host + 2 * P);
 }
 
-// pairs of elements per thread of the chunked kernels: 1, 2 or 4
+// f(items, group, pairs per thread) for the items of each chunk length
 template <typename F>
-void with_pairs(const pset& ps, F f) {
-  switch (ps.dev.ch / (2 * ps.tb)) {
-    case 1: f(std::integral_constant<int, 1>()); break;
-    case 2: f(std::integral_constant<int, 2>()); break;
-    default: f(std::integral_constant<int, 4>());
+void each_group(const pset& ps, F f) {
+  for (const pset_group& g : ps.groups) {
+    pset_dev d = ps.dev;
+    d.first = g.first;
+    switch (g.pairs) {
+      case 1: f(d, g, std::integral_constant<int, 1>()); break;
+      case 2: f(d, g, std::integral_constant<int, 2>()); break;
+      default: f(d, g, std::integral_constant<int, 4>());
+    }
+    CFIE_CHECK_LAUNCH();
   }
 }
 
@@ -707,35 +719,33 @@ void orthogonalise(cudaStream_t st, const pset& ps, const ws& W, int m, int j, s
   const givens_dev G{W.H, W.cs, W.sn, W.gv, W.hn, W.res};
   const int ny = std::max(1, std::min((j + AB) / AB, 304 / ps.Q));
   const int JB = std::min(256, ((j + 1 + ny - 1) / ny + AB - 1) / AB * AB);
-  const dim3 grid(ps.Q, (j + JB) / JB);
-  const size_t red = sizeof(double2) * std::min(JB, j + 1) * (ps.tb / 32);
   const size_t hs = sizeof(T) * (j + 1);
   const size_t gs = (sizeof(double2) * 2 + sizeof(double)) * m + sizeof(double2);
-  with_pairs(ps, [&](auto pt) {
-    constexpr int PT = decltype(pt)::value;
-    for (int pass = 0; pass < 2; ++pass) {
-      k_dots<T, PT><<<grid, ps.tb, red, st>>>(j, JB, m, j, pass == 0, V, L, w, W.act, ps.dev,
-                                              W.part, W.cnt, W.hbuf, W.H);
-      CFIE_CHECK_LAUNCH();
+  for (int pass = 0; pass < 2; ++pass) {
+    each_group(ps, [&](const pset_dev& d, const pset_group& g, auto pt) {
+      const size_t red = sizeof(double2) * std::min(JB, j + 1) * (g.tb / 32);
+      k_dots<T, decltype(pt)::value><<<dim3(g.count, (j + JB) / JB), g.tb, red, st>>>(
+          j, JB, m, j, pass == 0, V, L, w, W.act, d, W.part, W.cnt, W.hbuf, W.H);
+    });
+    each_group(ps, [&](const pset_dev& d, const pset_group& g, auto pt) {
+      constexpr int PT = decltype(pt)::value;
       if (pass == 0)
-        k_update<T, PT, false><<<ps.Q, ps.tb, hs, st>>>(j, m, V, L, W.hbuf, W.act, ps.dev, w,
-                                                        nullptr, W.cnt, G);
+        k_update<T, PT, false>
+            <<<g.count, g.tb, hs, st>>>(j, m, V, L, W.hbuf, W.act, d, w, nullptr, W.cnt, G);
       else
-        k_update<T, PT, true><<<ps.Q, ps.tb, std::max(hs, gs), st>>>(
-            j, m, V, L, W.hbuf, W.act, ps.dev, w, W.nrmp, W.cnt, G);
-      CFIE_CHECK_LAUNCH();
-    }
-  });
+        k_update<T, PT, true><<<g.count, g.tb, std::max(hs, gs), st>>>(
+            j, m, V, L, W.hbuf, W.act, d, w, W.nrmp, W.cnt, G);
+    });
+  }
 }
 
 // x += V y
 template <typename T>
 void add_basis(cudaStream_t st, const pset& ps, const ws& W, int m, size_t L, const T* V,
                double2* x) {
-  with_pairs(ps, [&](auto pt) {
-    k_xupdate<T, decltype(pt)::value><<<ps.Q, ps.tb, 0, st>>>(m, W.kd, ps.dev, V, L, W.y, x);
+  each_group(ps, [&](const pset_dev& d, const pset_group& g, auto pt) {
+    k_xupdate<T, decltype(pt)::value><<<g.count, g.tb, 0, st>>>(m, W.kd, d, V, L, W.y, x);
   });
-  CFIE_CHECK_LAUNCH();
 }
 
 // Marks the problems of an Arnoldi step's matvec for the matvec callbacks.
@@ -855,29 +865,41 @@ void gmres_cycle(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps, c
 }  // namespace
 
 void pset_build(pset& ps, const std::vector<size_t>& off, const std::vector<int>& len,
-                cudaStream_t st) {
+                const std::vector<size_t>& own, cudaStream_t st) {
   ps.P = (int)off.size();
-  std::vector<int> nch(ps.P), chb(ps.P);
-  std::vector<int2> items;
-  size_t L = 0, total = 0;
-  // chunks of 2048 elements (256 threads, four pairs each), or shorter ones down
-  // to 128 (64 threads, one pair each) until there are about two per SM
-  for (int p = 0; p < ps.P; ++p) total += len[p];
-  int ch = 2048;
-  while (ch > 128 && total / ch < 304) ch /= 2;
-  ps.dev.ch = ch;
-  ps.tb = std::min(AT, ch / 2);
+  ps.L = 0;
+  ps.len = len;
+  ps.groups.clear();
+  std::vector<int> nch(ps.P), chb(ps.P), ch(ps.P);
+  std::vector<chunk_item> items;
+  // Chunks of 2048 elements (256 threads, four pairs each), or shorter ones down to
+  // 128 (64 threads, one pair) until the problem's own operator has about two per
+  // SM.  What else is in the set does not change the order of a problem's sums, so
+  // that a solve gives the same bits alone and in a batch.  (With the length from the
+  // whole set's size a batch of 32 stars, n up to 16384, 32 directions each, takes 31 ms
+  // instead of 40 for these kernels, of 174 in all; a balanced tree over units of a warp,
+  // the same for every length, 30 ms, but 5 to 10 % more in small sets.)
   for (int p = 0; p < ps.P; ++p) {
-    nch[p] = (len[p] + ch - 1) / ch;
-    chb[p] = (int)items.size();
-    for (int c = 0; c < nch[p]; ++c) items.push_back(make_int2(p, c));
-    L = std::max(L, off[p] + (size_t)len[p]);
+    ch[p] = 2048;
+    while (ch[p] > 128 && own[p] / ch[p] < 304) ch[p] /= 2;
+    ps.L = std::max(ps.L, off[p] + (size_t)len[p]);
+  }
+  for (int c = 128; c <= 2048; c *= 2) {
+    pset_group g{(int)items.size(), 0, std::min(AT, c / 2), std::max(1, c / (2 * AT))};
+    for (int p = 0; p < ps.P; ++p) {
+      if (ch[p] != c) continue;
+      chb[p] = (int)items.size();
+      for (int at = 0; at < len[p]; at += c)
+        items.push_back({off[p] + (size_t)at, std::min(c, len[p] - at), p});
+      nch[p] = (int)items.size() - chb[p];
+    }
+    g.count = (int)items.size() - g.first;
+    if (!g.count) continue;
+    ps.groups.push_back(g);
+    ps.tb = g.tb;
   }
   ps.Q = (int)items.size();
-  ps.L = L;
-  ps.len = len;
-  const size_t bytes = sizeof(size_t) * ps.P + sizeof(int) * 3 * ps.P + sizeof(int2) * ps.Q + 128;
-  ps.buf.reserve(bytes);
+  ps.buf.reserve(sizeof(chunk_item) * ps.Q + sizeof(int) * 2 * ps.P + 64);
   char* b = ps.buf.as<char>();
   size_t o = 0;
   auto put = [&](const void* src, size_t n) {
@@ -886,11 +908,10 @@ void pset_build(pset& ps, const std::vector<size_t>& off, const std::vector<int>
     o += (n + 15) & ~size_t(15);
     return at;
   };
-  ps.dev.off = (const size_t*)put(off.data(), sizeof(size_t) * ps.P);
-  ps.dev.len = (const int*)put(len.data(), sizeof(int) * ps.P);
+  ps.dev.items = (const chunk_item*)put(items.data(), sizeof(chunk_item) * ps.Q);
   ps.dev.nch = (const int*)put(nch.data(), sizeof(int) * ps.P);
   ps.dev.chb = (const int*)put(chb.data(), sizeof(int) * ps.P);
-  ps.dev.items = (const int2*)put(items.data(), sizeof(int2) * ps.Q);
+  ps.dev.first = 0;
   CFIE_CHECK_CUDA(cudaStreamSynchronize(st));  // the host vectors die on return
 }
 
@@ -898,7 +919,7 @@ void pset_uniform(pset& ps, int n, int nrhs, cudaStream_t st) {
   std::vector<size_t> off(nrhs);
   std::vector<int> len(nrhs, n);
   for (int k = 0; k < nrhs; ++k) off[k] = (size_t)k * n;
-  pset_build(ps, off, len, st);
+  pset_build(ps, off, len, std::vector<size_t>(nrhs, (size_t)n * nrhs), st);
 }
 
 void gmres_set(cudaStream_t st, cfie_ctx* ctx, krylov_ws& K, const pset& ps,

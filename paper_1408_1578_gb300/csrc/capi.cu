@@ -736,7 +736,7 @@ cfie_status cfie_batch_create(cfie_ctx* ctx, int count, cfie_op* const* ops, con
     b = new cfie_batch();
     b->ctx = ctx;
     b->all_stored = true;
-    std::vector<size_t> poff;
+    std::vector<size_t> poff, pown;
     std::vector<int> plen;
     long long at = 0;
     for (int k = 0; k < count; ++k) {
@@ -750,13 +750,14 @@ cfie_status cfie_batch_create(cfie_ctx* ctx, int count, cfie_op* const* ops, con
       for (int r = 0; r < nrhs[k]; ++r) {
         poff.push_back((size_t)(at + (long long)r * ops[k]->n));
         plen.push_back(ops[k]->n);
+        pown.push_back((size_t)ops[k]->n * nrhs[k]);
       }
       at += (long long)ops[k]->n * nrhs[k];
       b->all_stored = b->all_stored && ops[k]->layout == CFIE_STORED;
     }
     b->L = (size_t)at;
     b->prec = ops[0]->prec;
-    pset_build(b->ps, poff, plen, ctx->stream);
+    pset_build(b->ps, poff, plen, pown, ctx->stream);
     if (b->all_stored && ctx->tune_batches)
       gemm_plan_tune(b->plan, ctx, b->ops, b->nrhs, b->off, b->L, b->tune_ms);
     else if (b->all_stored)

@@ -117,19 +117,26 @@ struct cfie_geom {
 };
 
 // A set of independent GMRES problems laid out as segments of one vector.
+struct chunk_item {    // elements base .. base + cnt - 1, of problem p
+  size_t base;
+  int cnt, p;
+};
 struct pset_dev {
-  const size_t* off;   // [P] segment offsets
-  const int* len;      // [P] segment lengths
-  const int* nch;      // [P] chunks per segment
-  const int* chb;      // [P] first chunk slot of the segment
-  const int2* items;   // [Q] (problem, chunk) work list
-  int ch;              // elements per chunk
+  const int* nch;            // [P] chunks per segment
+  const int* chb;            // [P] first item of the segment
+  const chunk_item* items;   // [Q] work list, a segment's items in order
+  int first;                 // item of CTA 0
+};
+// Items of one chunk length: CTAs of tb threads, `pairs` pairs of elements each
+struct pset_group {
+  int first, count, tb, pairs;
 };
 struct pset {
   int P = 0, Q = 0;
-  int tb = 0;             // threads per CTA of the chunked kernels
+  int tb = 0;             // threads per CTA of the kernels that take every item
   size_t L = 0;
   std::vector<int> len;   // host copy of the segment lengths
+  std::vector<pset_group> groups;
   pset_dev dev{};
   dbuf buf;
 };
@@ -373,8 +380,9 @@ void matvec_fp32_tc(cfie_op* op, const double2* x, double2* y, int nrhs);
 int tc_take_error(cfie_op* op);
 int df_take_error(cfie_op* op);
 // arnoldi.cu
+// own[p]: elements of all right-hand sides of problem p's operator
 void pset_build(pset& ps, const std::vector<size_t>& off, const std::vector<int>& len,
-                cudaStream_t st);
+                const std::vector<size_t>& own, cudaStream_t st);
 void pset_uniform(pset& ps, int n, int nrhs, cudaStream_t st);
 void measure_peaks(cfie_ctx* ctx, cfie_peaks* out);
 void field_eval(cfie_op* op, const double2* q, int nrhs, int npts, const double2* pts,
