@@ -64,9 +64,10 @@ __device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {
 // values: 16 additions instead of 80) and go out by (d, j), each written by one
 // warp; the direct sums by (split, i): the layout of the block kernel's split
 // partial sums with splits + nblk / 2 entries.
-// Measured (GB300, kite), against the block kernel: sound soft, one right-hand
-// side n = 512 83 -> 60 us, n = 4096 1.51 -> 1.10 ms; four n = 1024 155 -> 131 us,
-// n = 8192 5.46 -> 5.64 ms; sound hard, one n = 4096 1.86 -> 1.46 ms, two 1.87 -> 1.80.
+// Measured (GB300, kite), against the block kernel, which takes up to four columns
+// in the same time: sound soft, one right-hand side n = 512 86 -> 69 us, n = 4096 1.39
+// -> 0.97 ms, n = 16384 18.8 -> 14.3 ms, two 18.8 -> 16.5 ms; sound hard, one n = 4096
+// 1.71 -> 1.38 ms.
 template <int BC, int R>
 __global__ void __launch_bounds__(32)
 k_pair_sym(int n, int nblk, double omega, double omega_inv, double near, double eta_inv, double nf,
@@ -311,12 +312,15 @@ k_spectral_fp64(int n, const double* __restrict__ ct, const double* __restrict__
 // star n = 4096, 16 right-hand sides, sound hard, left the FP64 pipe idle 20 %
 // of the time).  Problems of fewer 64 x 32 tiles than eight per SM take
 // 32-target tiles.
-// k_pair_sym takes up to four sums (sound soft: four right-hand sides, sound
-// hard: two; with three, sound hard n = 4096, 2.39 ms against the block
-// kernel's 1.87) from n = 400 on: below, the block kernel has at most one tile per
-// SM (kite n = 384, one right-hand side 57 against 52 us), and while its partial
-// sums, one per block distance, stay within 512 MB (or the caller's scratch):
-// n = 46000 for one sound-soft right-hand side.
+// k_pair_sym takes one or two sums per entry (sound soft: right-hand sides, sound
+// hard: two each), and three or four up to n = 2048, where its smaller units fill the
+// GPU better (four right-hand sides, n = 1024 159 -> 131 us, 2048 386 -> 414 kite and
+// 394 -> 375 circle; further up the reduction of each sum over the rows costs more
+// than the shared evaluation saves: n = 3072 807 -> 826 us, 8192 4.96 -> 5.37 ms, sound
+// hard, two, 3072 1078 -> 1088 us, 8192 6.02 -> 6.37 ms).  From n = 400 on: below, the
+// block kernel has at most one tile per SM (kite n = 384, one right-hand side 57
+// against 52 us).  And while its partial sums, one per block distance, stay within
+// 512 MB (or the caller's scratch): n = 46000 for one sound-soft right-hand side.
 struct pair_plan {
   int sym;                  // 0, or the right-hand sides of k_pair_sym (1, 2, 4)
   int rbt, ti, splits, tps;
@@ -328,7 +332,8 @@ pair_plan plan_pair(int n, int nrhs, int hard, int device, size_t max_parts) {
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   const size_t vec = sizeof(double2) * (hard ? 2 : 1) * (size_t)n * nrhs;
-  if (nrhs <= (hard ? 2 : 4) && n >= 400) {
+  const int sums = nrhs * (hard ? 2 : 1);
+  if (n >= 400 && (sums <= 2 || (sums <= 4 && n <= 2048))) {
     const int nblk = (n + 31) / 32, units = 4 * (nblk / 2 + 1);
     const int want = (32 * sms + nblk - 1) / nblk;       // about 32 warps per SM
     p.tps = (units + std::min(units, want) - 1) / std::min(units, want);
