@@ -309,7 +309,9 @@ cfie_status cfie_apply(cfie_op* op, const void* x_dev, void* y_dev, int nrhs);
 cfie_status cfie_op_set_variant(cfie_op* op, int variant);
 
 /* y = A x in FP64 whatever the operator's precision (the matvec used for true
- * residuals). */
+ * residuals).  Takes partial sums from the device's pool for the call, up to 512
+ * MB or (sound hard: twice) the size of y, and the operator keeps at most 64 MB
+ * of them. */
 cfie_status cfie_apply_fp64(cfie_op* op, const void* x_dev, void* y_dev, int nrhs);
 
 /* y = A x in FP64, like cfie_apply_fp64, but without allocating any device
@@ -410,7 +412,9 @@ cfie_status cfie_op_set_block_gmres(cfie_op* op, int on);
  * column-major.  Points must lie off the curve; the rule is spectrally
  * accurate a few node spacings (2 pi / n in the parameter) away from it and
  * loses accuracy closer in.  Pointers 16-byte aligned; u must not overlap q or
- * pts.  Asynchronous on the context stream. */
+ * pts.  Takes up to 256 MB of partial sums from the device's pool for the call,
+ * of which the operator keeps at most 64 MB.  Asynchronous on the context
+ * stream. */
 cfie_status cfie_field_eval(cfie_op* op, const void* q_dev, int nrhs, int npts,
                             const void* pts_dev, void* u_dev);
 

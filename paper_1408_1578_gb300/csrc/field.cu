@@ -82,5 +82,6 @@ void field_eval(cfie_op* op, const double2* q, int nrhs, int npts, const double2
   if (a.splits > 1) {
     k_field_sum<<<(unsigned)((tot + 255) / 256), 256, 0, op->ctx->stream>>>(tot, a.splits, a.out, u);
     CFIE_CHECK_LAUNCH();
+    op->partial.trim();
   }
 }

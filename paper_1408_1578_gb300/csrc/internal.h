@@ -64,6 +64,10 @@ struct stream_scope {
   stream_scope& operator=(const stream_scope&) = delete;
 };
 
+// scratch that an operator keeps between calls at most (the pool hands a larger one
+// out again in a microsecond, next to products of a millisecond and more)
+constexpr size_t kKeepScratch = (size_t)64 << 20;
+
 struct dbuf {
   void* p = nullptr;
   size_t bytes = 0;
@@ -82,6 +86,10 @@ struct dbuf {
     release();
     CFIE_CHECK_CUDA(cudaMallocAsync(&p, need, alloc_stream()));
     bytes = need;
+  }
+  // give a large buffer back to the pool once the work that uses it is queued
+  void trim() {
+    if (bytes > kKeepScratch) release();
   }
   template <class T>
   T* as() const { return static_cast<T*>(p); }

@@ -433,6 +433,7 @@ void matvec_fp64(cfie_op* op, const double2* x, double2* y, int nrhs) {
   double2* part = op->partial.as<double2>();
   if (!hard) {
     run_pair<0>(op, p, x, nullptr, nrhs, part, nullptr, y);
+    op->partial.trim();
     return;
   }
   op->tmp1.reserve(sizeof(double2) * tot);
@@ -442,6 +443,7 @@ void matvec_fp64(cfie_op* op, const double2* x, double2* y, int nrhs) {
   // u = (1/s) Dt x
   spectral_apply(op, x, u, nullptr, make_double2(1.0, 0.0), nrhs);
   run_pair<1>(op, p, x, u, nrhs, part, t, y);
+  op->partial.trim();
   // y += (1/(i eta)) (1/s) Dt t
   spectral_apply(op, t, y, y, make_double2(0.0, -1.0 / op->eta), nrhs);
 }
