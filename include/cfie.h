@@ -301,8 +301,8 @@ cfie_status cfie_apply(cfie_op* op, const void* x_dev, void* y_dev, int nrhs);
  * sound-hard operator S is applied to d/ds x and C = -D' - i (omega^2 / eta)
  * (n_i . n_j) S to x, together up to 40 right-hand sides).  Autotune gives
  * products that are launches and latency in either variant (one right-hand side,
- * n <= 2304; sound hard, n <= 1152 to 2304 by the number of right-hand sides)
- * variant 1, the more accurate, without timing.  Variant 1 evaluates the
+ * n <= 2304; sound hard, n <= 1152 to 2304 by the number of right-hand sides, up
+ * to 64) variant 1, the more accurate, without timing.  Variant 1 evaluates the
  * FP32 entries to full FP32 accuracy, variant 2 to the accuracy its bf16
  * hi + lo operands keep (two-term Hankel series, a few 1e-6 relative next to
  * the near band); both stay far inside the 1e-4 of a raw FP32 matvec. */

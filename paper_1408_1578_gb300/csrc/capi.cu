@@ -101,23 +101,23 @@ void prof_harvest(cfie_ctx* c, bool wait) {
 
 namespace {
 
-// Process-wide choice between the two FP32 matvec variants, keyed by
-// (boundary condition, n, nrhs): each is timed once with CUDA events on the
-// operator's stream and the faster one is kept.
+// Process-wide choice between the two FP32 matvec variants, keyed by boundary
+// condition, n, nrhs and the tensor-core form's passes: each is timed once with
+// CUDA events on the operator's stream and the faster one is kept.
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int>, int> g_tuned;
+std::map<std::tuple<int, int, int, int>, int> g_tuned;
 
 // Sizes at which a product is launches and latency in either variant (tens of
 // microseconds; timed on a GB300, both within a third of each other) take the
 // CUDA-core sums without timing: they are the more accurate, 1e-6 against 2e-6
 // (sound soft) and 6e-6 (sound hard) relative.  Sound soft, one right-hand
-// side: 27 against 37 us at n = 1024, 51 against 50 at 2050; sound hard:
-// 85 against 104 us at n = 512, 64 right-hand sides, 114 against 110 at n =
-// 2048, 8 (CUDA cores against tensor cores).
+// side: 27 against 37 us at n = 1024, 51 against 50 at 2050; sound hard, measured
+// up to 64 right-hand sides: 85 against 104 us at n = 512, 64, 114 against 110 at n
+// = 2048, 8 (CUDA cores against tensor cores).
 bool prefers_fp32_sums(const cfie_op* op, int nrhs) {
   const int n = op->n;
   if (nrhs == 1 && n <= 2304) return true;
-  return op->bc == CFIE_SOUND_HARD &&
+  return op->bc == CFIE_SOUND_HARD && nrhs <= 64 &&
          (n <= 1152 || (n <= 1600 && nrhs < 32) || (n <= 2304 && nrhs < 16));
 }
 
@@ -125,12 +125,13 @@ int tuned_variant(cfie_op* op, const double2* x, double2* y, int nrhs) {
   if (op->variant) return op->variant;
   if (prefers_fp32_sums(op, nrhs)) return 1;
   // decisions are shared by operators of similar shape (n up to the next power
-  // of two, right-hand sides in octaves), so that a server seeing a new n and
-  // nrhs with every request does not time both variants every time
+  // of two, right-hand sides in octaves with the same number of passes, which
+  // steps inside an octave), so that a server seeing a new n and nrhs with every
+  // request does not time both variants every time
   int nb = 1, rb = 1;
   while (nb < op->n) nb *= 2;
-  while (rb * 2 <= std::min(nrhs, 64)) rb *= 2;
-  const auto key = std::make_tuple((int)op->bc, nb, rb);
+  while (rb * 2 <= nrhs) rb *= 2;
+  const auto key = std::make_tuple((int)op->bc, nb, rb, tc_passes(op, nrhs));
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tuned.find(key);

@@ -385,6 +385,7 @@ void matvec_df(cfie_op* op, const double2* x, double2* y, int nrhs);
 void matvec_residual(cfie_op* op, const double2* x, double2* y, int nrhs);
 // matvec_tc.cu
 void matvec_fp32_tc(cfie_op* op, const double2* x, double2* y, int nrhs);
+int tc_passes(const cfie_op* op, int nrhs);   // its passes over the pairs
 int tc_take_error(cfie_op* op);
 int df_take_error(cfie_op* op);
 // arnoldi.cu

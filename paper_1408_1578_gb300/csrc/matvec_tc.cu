@@ -625,7 +625,23 @@ void run_blocks(cfie_op* op, const double2* x, const float2* u, float2* t, doubl
   }
 }
 
+// Sound hard: passes of S and C together, 0 where each on its own is the less.  S and C
+// from one phase take 1.25 to 1.3 passes of one operator, but the tensor memory and
+// the stages hold 40 right-hand sides of both against 64 of one (n = 6002, 33
+// right-hand sides: 405 -> 325 us with the derivatives; n = 16384, 72: 2.50 -> 1.80 ms).
+int joint_passes(int nrhs) {
+  const int both = (nrhs + 39) / 40, each = 2 * ((nrhs + 63) / 64);
+  return 4 * both < 3 * each ? both : 0;
+}
+
 }  // namespace
+
+int tc_passes(const cfie_op* op, int nrhs) {
+  const int blocks = (nrhs + 63) / 64;
+  if (op->bc == CFIE_SOUND_SOFT) return blocks;
+  const int both = joint_passes(nrhs);
+  return both ? both : 2 * blocks;
+}
 
 void matvec_fp32_tc(cfie_op* op, const double2* x, double2* y, int nrhs) {
   if (op->bc == CFIE_SOUND_SOFT) {
@@ -639,12 +655,7 @@ void matvec_fp32_tc(cfie_op* op, const double2* x, double2* y, int nrhs) {
   float2* u32 = op->xin32.as<float2>();
   float2* t32 = u32 + tot;
   spectral32_apply(op, x, u32, nrhs);
-  // S and C from one phase take 1.25 to 1.3 passes of one operator, but the tensor
-  // memory and the stages hold 40 right-hand sides of both against 64 of one:
-  // together while that is the less (n = 6002, 33 right-hand sides: 405 ->
-  // 325 us with the derivatives; n = 16384, 72: 2.50 -> 1.80 ms)
-  const int both = (nrhs + 39) / 40, each = 2 * ((nrhs + 63) / 64);
-  if (4 * both < 3 * each) {
+  if (const int both = joint_passes(nrhs)) {
     const int per = (nrhs + both - 1) / both;
     for (int r0 = 0; r0 < nrhs; r0 += per) {
       const int nr = std::min(per, nrhs - r0);
