@@ -369,8 +369,9 @@ fft_args<T> args_of(const fft_plan& F, int n, T* work) {
 
 // Transforms per CTA (2^lc of length 2^lM, out of 2^lOther): about 2048
 // elements, at least 64 contiguous bytes per row of the columns, fewer when
-// the launch would leave SMs idle.  Shared memory: two buffers, at most
-// 2 (2^11 elements x 2) or 2 (2^10 x (4 + 1)) of 16 bytes, 164 KB.
+// the launch would leave SMs idle.  Shared memory: two buffers, for n <= 2^20 (N <=
+// 2^21) at most 2 (2^11 elements x 2) or 2 (2^10 x (4 + 1)) of 16 bytes, 160 KB;
+// spectral_fft refuses what does not fit.
 template <typename T>
 int per_cta(int lM, int lOther, int cols, int lmin) {
   int lc = std::max(lmin, 11 - lM);
@@ -409,6 +410,7 @@ void spectral_fft(cfie_op* op, const X* in, O* out, const O* base, double2 scale
   R.lc = per_cta<T>(R.l2, R.l1, cols, 0);
   const dim3 gc(1u << (C.l2 - C.lc), cols), gr(1u << (R.l1 - R.lc), cols);
   const size_t sc = smem_of<T>(C.l1, C.lc), sr = smem_of<T>(R.l2, R.lc);
+  CFIE_REQUIRE(std::max(sc, sr) <= kSmemMax, "spectral derivative: transform too long");
   const double* osc = F.osc.as<double>();
   prof_scope ps(op->ctx, CFIE_K_SPECTRAL);
   FFT_LAUNCH((k_fft_cols<T, COL_IN, X, O>), gc, sc, st, C, in, osc, scale, base, out);
