@@ -170,34 +170,64 @@ def measured_peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
-# Algorithmic work per (target, source) pair of each kernel class, counted from
-# the kernels' per-pair formulas (FP32 add / mul / fma / min / max / rint and
-# each special-function unit op = 1 operation, IEEE division or square root = 8).
+# Two counts per (target, source) pair of each kernel class.
+#
+# A fixed unit of work, so that rates ("achieved") compare across versions: the
+# operations of the kernels' first per-pair formulas (FP32 add / mul / fma / min / max /
+# rint and each special-function unit op = 1 operation, IEEE division or square root =
+# 8).  SMS x FP32_LANES x clock bounds operations, not these units.
 SMS, FP32_LANES = 152, 128
-# FP32 pair entries (two-float phase, asymptotics) by summation variant: the
-# CUDA-core kernel evaluates both hard entries from one phase; the tensor-core
-# kernel folds the per-node factors in and keeps the accuracy of its bf16 hi + lo
-# operands (two-term series, no exact sum in the phase), S (36) and D' (42).  A
-# fixed unit of work: the kernels now spend fewer (modulus and phase instead of
-# P and Q, S and C from one phase), which raises the fraction reported
 ENTRY_OPS = {("soft", 1): 74, ("hard", 1): 87, ("soft", 2): 54, ("hard", 2): 36 + 42}
 SUM_OPS = {"soft": 4, "hard": 8}         # FP32 FMAs per pair and right-hand side (CUDA-core sums)
 DF_ENTRY_OPS = 563                       # double-float pair entry of the residual kernel
 # sound hard: the phase and Hankel part (431) with the S assembly (39) and the D'
-# assembly (78); the CUDA-core kernel takes both from one phase, the sliced
-# tensor-core kernel evaluates them in separate passes
+# assembly (78)
 DF_HARD_OPS = 431 + 39 + 78
 DF_HARD_PASS_OPS = (431 + 39) + (431 + 78)
 DF_TERM_OPS = 48                         # Dot2 complex product-sum per pair and right-hand side
 SLICE_OPS = 48                           # six 8-bit slices of the re / im parts of one entry
+#
+# What the kernels now execute on the pipe that bounds them, counted from their
+# sources: lanes of FP32 add / mul / fma (two of a packed instruction; special
+# functions and conversions run on other pipes), or FP64 instructions.  Fractions of a
+# roofline are in these ("frac_spent", and "frac" wherever the unit of work holds
+# operations that are no longer executed).
+SPENT_FP32 = {"soft": 24 + 9 + 11 + 2,   # phase, modulus and phase, entry, bf16 hi + lo split
+              "joint": 24 + 9 + 15 + 4,  # S and C from one phase
+              "apart": (24 + 5 + 4 + 2) + (24 + 9 + 15 + 2)}
+SPENT_DF_HANKEL = 204                    # of these 42 for the orders S does not use
+SPENT_DF = {"soft": SPENT_DF_HANKEL + 96, "hard": SPENT_DF_HANKEL + 126}   # CUDA-core sums
+SPENT_SLICES = 52
+SPENT_RTC = {"soft": SPENT_DF_HANKEL + 96 + SPENT_SLICES,
+             "hard": (SPENT_DF_HANKEL - 42 + 33 + SPENT_SLICES) +
+                     (SPENT_DF_HANKEL + 120 + SPENT_SLICES)}
+# FP64 multiply-adds and additions per clock and SM (measured; nominal 1.25 TFLOP/s is 2)
+FP64_LANES = 1.7
 FP64_NOMINAL_TFLOPS = 1.25               # GB300 FP64 (nominal; FMA = 2 flops)
 
 
-# FP32 operations per pair that the sound-soft tensor-core kernels now spend on
-# entries (packed FP32 and special-function operations; residual: with slicing):
-# "frac_spent" beside the fraction in the units of work above, which stay fixed so
-# that rates compare across versions and can exceed the peak
-SPENT_OPS = {"matvec_fp32": 52, "matvec_fp64": 342}
+def spent_fp64(n, nrhs, bc):
+    """FP64 instructions per pair of the FP64 product: few columns, the kernel that evaluates a
+    pair of nodes once for both entries (25 shared, 8 or 12.5 per entry, 10 per sum of an entry
+    and its transpose); else the block kernel (33 or 38 per entry, and per right-hand side and
+    operator two conversions and two multiply-adds for each 32 sources)."""
+    ops = 2 if bc == "hard" else 1
+    sums = ops * nrhs
+    if n >= 400 and (sums <= 2 or (sums <= 4 and n <= 2048)):
+        return (25 + 2 * (12.5 if bc == "hard" else 8) + 10 * sums) / 2
+    return (38 if bc == "hard" else 33) + 4 * sums / 32
+
+
+def spent_fp32(nrhs, bc):
+    """FP32 lane operations per pair of the tensor-core product."""
+    blocks = -(-nrhs // 64)
+    if bc == "soft":
+        return SPENT_FP32["soft"] * blocks
+    both = -(-nrhs // 40)
+    if 4 * both < 6 * blocks:
+        return SPENT_FP32["joint"] * both
+    return SPENT_FP32["apart"] * blocks
+
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one
 # ncu capture of the current kernel at the same launch configuration, keyed by
@@ -206,6 +236,18 @@ NCU_TRAFFIC = {
     ("matvec_fp32", "kite", 32768, 64, 2): 80.063232e6 + 12.190208e6,
     ("matvec_fp64", "kite", 32768, 64, 2): 3.398163e9 + 206.532864e6,
 }
+
+
+def alu_entry(ops, spent, n, per, pipe_peak, work, clock_hz):
+    """Roofline entry of a pair kernel: `ops` per pair in the unit of work, `spent` executed,
+    `per` seconds a product, `pipe_peak` in executed operations.  frac is in executed operations;
+    peak is the rate of the unit of work at which it would be 1."""
+    a = ops * n * n / per / 1e12
+    frac = spent * n * n / per / 1e12 / pipe_peak
+    return {"bound": "alu", "achieved": a, "peak": a / frac, "unit": "Top/s", "frac": frac,
+            "frac_spent": frac, "traffic": None, "spent_per_pair": spent,
+            "work": f"{work}; {spent:g} executed on the pipe that bounds it",
+            "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz, in executed ops"}
 
 
 def kernel_rooflines(kt, spec, stats, peaks, src, n, solves_timed):
@@ -227,45 +269,44 @@ def kernel_rooflines(kt, spec, stats, peaks, src, n, solves_timed):
             # per matvec (the sound-hard tensor-core form, and passes of more
             # than 64 right-hand sides, take several launches per matvec)
             mv = stats.get("inner_matvecs", 0) * solves_timed
-            a = ops * n * n / (sec / mv if mv else avg) / 1e12
-            out[cls] = {"bound": "alu", "achieved": a, "peak": fp32_peak, "unit": "Top/s",
-                        "frac": a / fp32_peak, "traffic": None,
-                        "work": f"{ops} FP32 ops per pair (variant {v}: "
-                                + ("source sums on the tensor cores, not counted" if v == 2
-                                   else f"{SUM_OPS[bc]} FMA per pair per right-hand side") + ")",
-                        "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz"}
-            if v == 2 and bc == "soft":
-                out[cls]["frac_spent"] = a / fp32_peak * SPENT_OPS[cls] / ops
+            per = sec / mv if mv else avg
+            spent = spent_fp32(nrhs, bc) if v == 2 else ops
+            out[cls] = alu_entry(ops, spent, n, per, fp32_peak,
+                                 f"{ops} FP32 ops per pair (variant {v}: "
+                                 + ("source sums on the tensor cores, not counted" if v == 2
+                                    else f"{SUM_OPS[bc]} FMA per pair per right-hand side") + ")",
+                                 clock_hz)
+            if v == 2 and bc == "soft":     # the unit of work stays below the pipe's peak
+                out[cls].update(peak=fp32_peak, frac=out[cls]["achieved"] / fp32_peak)
         elif cls == "matvec_fp64" and prec != "fp64" and stats.get("residual_variant") == 2:
             ent, sl = (DF_ENTRY_OPS, SLICE_OPS) if bc == "soft" else (DF_HARD_PASS_OPS, 2 * SLICE_OPS)
-            ops = ent + sl
-            a = ops * n * n / avg / 1e12
-            out[cls] = {"bound": "alu", "achieved": a, "peak": fp32_peak, "unit": "Top/s",
-                        "frac": a / fp32_peak, "traffic": None,
-                        "work": f"tensor-core residual: {ent} + {sl} FP32 ops per pair "
-                                "(double-float entries, slicing; slice products on the tensor "
-                                "cores, not counted)",
-                        "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz"}
-            if bc == "soft":
-                out[cls]["frac_spent"] = a / fp32_peak * SPENT_OPS[cls] / ops
+            passes = -(-nrhs // (64 if bc == "soft" else 48))
+            # passes of 48 and a remainder each evaluate the entries; sound hard: launches
+            # of S and of C, of which avg is the mean
+            per = avg * passes * (1 if bc == "soft" else 2)
+            out[cls] = alu_entry(ent + sl, SPENT_RTC[bc] * passes, n, per, fp32_peak,
+                                 f"tensor-core residual: {ent} + {sl} FP32 ops per pair "
+                                 "(double-float entries, slicing; slice products on the tensor "
+                                 "cores, not counted)", clock_hz)
+            out[cls]["achieved"] = (ent + sl) * n * n / avg / 1e12
+            out[cls]["peak"] = out[cls]["achieved"] / out[cls]["frac"]
         elif cls == "matvec_fp64" and prec != "fp64":
-            # S applied to the 3 vectors of Maue's identity and D' to x: 4 sums per RHS
+            # unit of work: S on the 3 vectors of Maue's identity and D' on x (4 sums per
+            # right-hand side); executed: S and C (2)
             ent, terms = (DF_ENTRY_OPS, 1) if bc == "soft" else (DF_HARD_OPS, 4)
-            ops = ent + DF_TERM_OPS * terms * nrhs
-            a = ops * n * n / avg / 1e12
-            out[cls] = {"bound": "alu", "achieved": a, "peak": fp32_peak, "unit": "Top/s",
-                        "frac": a / fp32_peak, "traffic": None,
-                        "work": f"double-float residual: {ent} + {DF_TERM_OPS * terms} x nrhs "
-                                "FP32 ops per pair",
-                        "peak_source": f"152 SMs x 128 FP32 lanes x {clock_hz / 1e6:.0f} MHz"}
+            spent = SPENT_DF[bc] + DF_TERM_OPS * (1 if bc == "soft" else 2) * nrhs
+            out[cls] = alu_entry(ent + DF_TERM_OPS * terms * nrhs, spent, n, avg, fp32_peak,
+                                 f"double-float residual: {ent} + {DF_TERM_OPS * terms} x nrhs "
+                                 "FP32 ops per pair", clock_hz)
         elif cls == "matvec_fp64":
             dfma = (4 if bc == "soft" else 8) * nrhs
-            a = dfma * n * n / avg / 1e12
-            pk = FP64_NOMINAL_TFLOPS / 2
-            out[cls] = {"bound": "alu", "achieved": a, "peak": pk, "unit": "T DFMA/s",
-                        "frac": a / pk, "traffic": None,
-                        "work": f"{dfma} DFMA per pair (source sums only: a lower bound)",
-                        "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (not measured)"}
+            spent = spent_fp64(n, nrhs, bc)
+            pk = SMS * FP64_LANES * clock_hz / 1e12
+            out[cls] = alu_entry(dfma, spent, n, avg, pk,
+                                 f"{dfma} DFMA per pair (source sums alone, which now run on the "
+                                 "integer units from five sums per entry on)", clock_hz)
+            out[cls].update(unit="T DFMA/s", peak_source=f"{SMS} SMs x {FP64_LANES} FP64 lanes "
+                            f"(measured) x {clock_hz / 1e6:.0f} MHz")
         elif cls == "matvec_tensor":
             pitch = (n + 63) // 64 * 64
             b = n * pitch * 8
@@ -830,8 +871,8 @@ def _brief(r):
     out["workload"] = r["config"]["workload"]
     if r.get("roofline"):
         rf = r["roofline"]
-        out["roofline"] = {k: rf[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac")
-                           if k in rf}
+        out["roofline"] = {k: rf[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac",
+                                              "frac_spent") if k in rf}
     if "one_at_a_time_summary" in r:
         out["one_at_a_time_summary"] = r["one_at_a_time_summary"]
     return out
