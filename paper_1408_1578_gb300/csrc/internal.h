@@ -244,7 +244,7 @@ struct cfie_op {
   dbuf geo32;        // hi/lo coordinates + FP32 normals / speeds
   dbuf band;         // near-field band entries (complex64), n x (2 b + 1) per operator
   int band_b = -1;
-  dbuf xin32, xin32b; // FP32 staging of the input (and hard-path helpers)
+  dbuf xin32;        // FP32 staging of the input (and hard-path helpers)
   fft_plan fft;       // sound hard: FFT spectral derivative
 
   // FP64-accurate residual matvec in double-float arithmetic (sound-soft)
@@ -255,7 +255,7 @@ struct cfie_op {
   int res_variant = 0;   // residual: 0 automatic, 1 CUDA-core Dot2, 2 tensor cores
 
   // FP32 matvec variant: 0 = autotuned, 1 = FP32-pipe contraction, 2 = tensor cores
-  int variant = 0, tuned_nrhs = -1, tuned_choice = 1;
+  int variant = 0;
   int basis32 = 1;   // inner Krylov basis in FP32 for the refined precisions
   // plans: up to 32, up to 64 right-hand sides; S and C together, up to 32, up to 40
   tc_plan tc[4];

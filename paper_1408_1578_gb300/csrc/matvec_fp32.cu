@@ -28,8 +28,8 @@
 // into shared memory, source-major; then the tile is contracted with the staged
 // right-hand sides, each thread accumulating 4 targets x R/8 right-hand sides in
 // registers (complex multiply-add on the FP32 pipe).  Source ranges are split
-// across CTAs to fill the GPU; partial sums (complex64) are added in FP64 in a
-// fixed order by the reduction kernel.
+// across CTAs to fill the GPU; partial sums (complex64) are added in pairs of FP32
+// in a fixed order by the reduction kernel.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -258,52 +258,6 @@ __global__ void k_to32(size_t len, const double2* __restrict__ in, float2* __res
   if (e < len) out[e] = make_float2((float)in[e].x, (float)in[e].y);
 }
 
-// out[k][i] (+)= (scale / s_i) sum_j c_{(i-j) mod n} in[k][j] in FP32 with
-// blocked accumulation (256-source partial sums); out complex64 or complex128
-constexpr int SPT = 256;
-template <bool OUT64>
-__global__ void __launch_bounds__(SPT)
-k_spectral32(int n, const float* __restrict__ ct, const double* __restrict__ sp,
-             const float2* __restrict__ in, double2 scale, float2* __restrict__ out32,
-             double2* __restrict__ out64) {
-  __shared__ float2 xs[SPT];
-  const int i = blockIdx.x * SPT + threadIdx.x;
-  const int k = blockIdx.y;
-  const float2* ink = in + (size_t)k * n;
-  float2 outer = make_float2(0.f, 0.f);
-  for (int j0 = 0; j0 < n; j0 += SPT) {
-    __syncthreads();
-    const int jj = j0 + threadIdx.x;
-    xs[threadIdx.x] = jj < n ? ink[jj] : make_float2(0.f, 0.f);
-    __syncthreads();
-    if (i < n) {
-      const int jn = min(SPT, n - j0);
-      int idx = i - j0;
-      if (idx < 0) idx += n;
-      float2 acc = make_float2(0.f, 0.f);
-      for (int q = 0; q < jn; ++q) {
-        const float c = ct[idx];
-        acc.x = fmaf(c, xs[q].x, acc.x);
-        acc.y = fmaf(c, xs[q].y, acc.y);
-        idx = idx == 0 ? n - 1 : idx - 1;
-      }
-      outer.x += acc.x;
-      outer.y += acc.y;
-    }
-  }
-  if (i < n) {
-    const double inv = 1.0 / sp[i];
-    const double sx = scale.x * inv, sy = scale.y * inv;
-    const double2 v = make_double2(sx * outer.x - sy * outer.y, sx * outer.y + sy * outer.x);
-    const size_t e = (size_t)k * n + i;
-    if (OUT64) {
-      out64[e] = make_double2(out64[e].x + v.x, out64[e].y + v.y);
-    } else {
-      out32[e] = make_float2((float)v.x, (float)v.y);
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // set-up kernels
 // ---------------------------------------------------------------------------
@@ -324,9 +278,8 @@ __global__ void k_coord_bound(int n, geom_dev g, unsigned* __restrict__ bound) {
 // 2^23.1 of them, exact as well; the lo parts (|lo| <= 2^(e-11)) keep the rest
 // to ~2^(e-35).
 __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w,
-                        const double* __restrict__ ct, const unsigned* __restrict__ bound,
-                        double omega, double eta, double h, float* __restrict__ w32,
-                        float* __restrict__ c32, float4* __restrict__ pk,
+                        const unsigned* __restrict__ bound, double omega, double eta, double h,
+                        float* __restrict__ w32, float4* __restrict__ pk,
                         float2* __restrict__ wkt, int hard, float* __restrict__ sp4) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < 8) wkt[2 * n + i] = make_float2(0.f, 0.f);
@@ -347,7 +300,6 @@ __global__ void k_geo32(int n, geom_dev g, geo32 o, const double* __restrict__ w
   o.ny[i] = (float)g.ny[i];
   o.sp[i] = (float)g.sp[i];
   w32[i] = (float)w[i];
-  c32[i] = (float)ct[i];
   // the Kress table twice over, divided by pi h, indexed by i - j + n (no
   // cyclic wrap), paired with the weight of the next source; the zero tail is
   // written above
@@ -540,13 +492,12 @@ void fp32_prepare(cfie_op* op) {
   float* base = op->geo32.as<float>();
   geo32 o{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n, base + 6 * n};
   float* w32 = base + 7 * n;
-  float* c32 = base + 8 * n;
   unsigned* bound = reinterpret_cast<unsigned*>(base + geo32_bound_offset(n));
   CFIE_CHECK_CUDA(cudaMemsetAsync(bound, 0, sizeof(unsigned), st));
   k_coord_bound<<<nblk(n), 256, 0, st>>>(n, op->g, bound);
   CFIE_CHECK_LAUNCH();
-  k_geo32<<<nblk(n), 256, 0, st>>>(n, op->g, o, op->wtab.as<double>(), op->ctab.as<double>(),
-                                    bound, op->omega, op->eta, op->h, w32, c32,
+  k_geo32<<<nblk(n), 256, 0, st>>>(n, op->g, o, op->wtab.as<double>(), bound, op->omega, op->eta,
+                                    op->h, w32,
                                     reinterpret_cast<float4*>(base + geo32_pack_offset(n)),
                                     reinterpret_cast<float2*>(base + geo32_wk_offset(n)),
                                     op->bc == CFIE_SOUND_HARD, base + geo32_pair_offset(n));

@@ -7,9 +7,8 @@
 
 // FP32 geometry of an operator: coordinates times omega as hi/lo pairs,
 // unnormalised normal, speed.
-// Stored in one buffer: 9 n floats xh, xl, yh, yl, nx, ny, sp, w32 (Kress
-// table), c32 (spectral-derivative circulant); then, for the fused
-// tensor-core kernel, starting on 16-byte boundaries:
+// Stored in one buffer: 8 n floats xh, xl, yh, yl, nx, ny, sp, w32 (Kress
+// table); then, for the fused tensor-core kernel, starting on 16-byte boundaries:
 //   n float4 coordinates      (omega x hi, lo, omega y hi, lo)
 //   n float4 source factors   (omega hq c0 nu1, omega hq c0 nu2, hq c0 eta |z'|, hq c0 |z'|)
 //   n float4 target factors   2 omega (nu1, nu2) / |z'|, 0, 0
@@ -27,7 +26,7 @@ struct geo32 {
   float *xh, *xl, *yh, *yl, *nx, *ny, *sp;
 };
 
-inline size_t geo32_pack_offset(int n) { return ((size_t)9 * n + 3) & ~size_t(3); }
+inline size_t geo32_pack_offset(int n) { return ((size_t)8 * n + 3) & ~size_t(3); }
 inline size_t geo32_wk_offset(int n) { return geo32_pack_offset(n) + (size_t)12 * n; }
 inline size_t geo32_pair_offset(int n) {
   return (geo32_wk_offset(n) + (size_t)4 * n + 16 + 3) & ~size_t(3);
@@ -231,9 +230,9 @@ __device__ __forceinline__ float2 entry_folded32(float4 tg, float4 sc, float4 sq
 // Two entries of one target at once (the adjacent sources j, j + 1), in packed
 // FP32 pairs: add, mul and fma on float2 issue once for two lanes of
 // arithmetic (measured: the same 121 lane-ops per clock and SM as scalar FMAs
-// at half the issue slots), and the producers of the fused kernel are bound by
-// issue slots.  Signs sit in the per-node data and in the constants
-// where they can.
+// at half the issue slots); the producers of the fused kernel were bound by issue
+// slots with scalar ones and are by the FMA pipe now.  Signs sit in the per-node
+// data and in the constants where they can.
 // ---------------------------------------------------------------------------
 
 // as pair_phase, for the two sources
