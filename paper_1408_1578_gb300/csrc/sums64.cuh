@@ -61,19 +61,24 @@ __device__ __forceinline__ int4 to_limbs(double2 v, int E) {
 // 2^-56.  Random densities range wider than 2^7 in 5 of 1000 columns of a tile
 // (normal) or 1 of 2000 (uniform), entries where sound hard C, or the 1 +- cos of the
 // others, goes through zero.  Measured (GB300), against no limit at all: 2^7 star n
-// = 4096, 16, sound hard 2.25 -> 2.25 ms, field 6.85 -> 6.85 ms; 2^6 2.28, 6.99 ms.
+// = 4096, 16, sound hard 2.25 -> 2.25 ms, field 6.85 -> 6.85 ms; 2^6 2.28, 6.99 ms; with
+// a row's smallest entry looked for only where a column ranges that wide 2.24, 6.81 ms.
 constexpr int kSpread = 7;
 constexpr int kRaw = 1 << 16;   // with a row's exponent: entries kept in FP64
 struct tile_range {
   int e;           // exponent of the largest (zeros only: any)
   bool out, wide;  // not held in fixed point; smallest of the valid ones 2^-kSpread below
 };
-__device__ __forceinline__ tile_range range_of(double2 v, bool valid) {
+// (wide: whether that matters)
+__device__ __forceinline__ tile_range range_of(double2 v, bool valid, bool wide) {
   const unsigned a = __double2hiint(v.x) & 0x7fffffff, b = __double2hiint(v.y) & 0x7fffffff;
   const unsigned m = max(a, b);
   const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-  const int least = (int)(__reduce_min_sync(0xffffffffu, valid ? m : 0xffffffffu) >> 20);
-  if (E >= 600 && E <= 1500) return {E, false, E - least > kSpread};
+  if (E >= 600 && E <= 1500) {
+    if (wide)
+      wide = E - (int)(__reduce_min_sync(0xffffffffu, valid ? m : 0xffffffffu) >> 20) > kSpread;
+    return {E, false, wide};
+  }
   const bool any = __any_sync(0xffffffffu, (a | b | __double2loint(v.x) | __double2loint(v.y)) != 0);
   return {E ? E : 1023, any, false};
 }
@@ -186,7 +191,7 @@ k_block64(block_args p) {
       const int o = c / RBT, r = c % RBT, j = j0 + lane;
       const double2* src = o == NO - 1 ? p.x : p.u;
       const double2 v = j < n && r < rbn ? src[(size_t)(rb0 + r) * n + j] : make_double2(0.0, 0.0);
-      const tile_range span = range_of(v, j < n);
+      const tile_range span = range_of(v, j < n, true);
       S.X[o][lane][r] = to_limbs(v, span.e);
       if (lane == 0) {
         S.ex[o][r] = span.e;
@@ -207,9 +212,9 @@ k_block64(block_args p) {
             S.se[lane], MODE == FIELD ? 0.0 : S.wk[il - lane + TJ - 1], g.tab, a, b);
       if (MODE == FIELD && p.rotate) a = make_double2(a.y, -a.x);
       auto keep = [&](int o, double2 v) {
-        const tile_range span = range_of(v, in);
         const int c = S.cols[o];
-        const bool raw = span.out || (c & 2) || (c && span.wide);
+        const tile_range span = range_of(v, in, c == 1);
+        const bool raw = span.out || (c & 2) || span.wide;
         int4 q;
         if (raw)
           q = make_int4(__double2loint(v.x), __double2hiint(v.x), __double2loint(v.y),
