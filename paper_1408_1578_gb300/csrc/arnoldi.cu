@@ -136,8 +136,10 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
     wr[e].a = wr[e].b = basis_t<T>::make(0.0, 0.0);
     if (q < c.cnt) wr[e] = load2(w + c.base + q);
   }
-  // (an advancing pointer: with the index of the vector in each address the compiler
-  // kept half of the loads in flight, kite n = 8192, 64 directions, 30.5 ms against 29.9)
+  // Two pairs per thread: an advancing pointer.  With the index of the vector in each
+  // address the compiler kept half of the loads in flight there (32 registers, kite n =
+  // 8192, 64 directions, 30.5 ms against 29.9), and with the pointer fewer at four pairs
+  // (n = 32768: these kernels 35.9 ms a solve against 33.0).
   const T* vp = V + (size_t)j0 * L + c.base;
   for (int jj = j0; jj < j1; jj += AB, vp += AB * L) {
     two<T> v[AB][PT];
@@ -147,7 +149,8 @@ k_dots(int J, int JB, int m, int col, int first, const T* __restrict__ V, size_t
       for (int e = 0; e < PT; ++e) {
         const int q = 2 * (e * blockDim.x + threadIdx.x);
         v[b][e].a = v[b][e].b = basis_t<T>::make(0.0, 0.0);
-        if (q < c.cnt && jj + b < j1) v[b][e] = load2(vp + b * L + q);
+        if (q < c.cnt && jj + b < j1)
+          v[b][e] = load2(PT == 2 ? vp + b * L + q : V + (size_t)(jj + b) * L + c.base + q);
       }
     S s[2 * AB];
 #pragma unroll
