@@ -315,7 +315,8 @@ def kernel_rooflines(kt, spec, stats, peaks, src, n, solves_timed):
                         "frac": a / peaks["hbm_gbs"], "traffic": None,
                         "work": "stored bf16 hi/lo matrix (8 bytes per entry) read once per matvec",
                         "peak_source": src}
-        elif cls == "arnoldi":
+        elif cls == "arnoldi" and not spec.get("solver", "").startswith("block"):
+            # (block GMRES orthogonalises by GEMMs over blocks, not by passes per vector)
             elems = stats.get("arnoldi_elems", 0) * solves_timed
             esize = 8 if stats.get("basis_fp32") else 16
             b = 4 * elems * esize
