@@ -31,7 +31,7 @@
 // on GB300 the FP64 additions of a plain reduction cost more than the products),
 // and an Arnoldi step is 5 launches instead of 9.  Measured (GB300): unrestarted
 // FP64 solve of n = 1024, 30 steps, 15.2 -> 9.1 ms (490 -> 290 us a step, 227 of
-// them the matvec); kite n = 8192, 64 directions, 88 steps, 34.2 -> 30.4 ms.
+// them the matvec); kite n = 8192, 64 directions, 88 steps, 34.2 -> 29.8 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

@@ -30,7 +30,7 @@
 // Bound: the FP64 pipe (one instruction of a warp per 64 clocks and
 // scheduler): per pair about 38 instructions for the entry (hankel64.cuh).
 // Measured (GB300): circle n = 1024, 1 right-hand side 1120 -> 96 us; star n =
-// 4096, 16 right-hand sides, sound hard 15.8 -> 2.22 ms.
+// 4096, 16 right-hand sides, sound hard 15.8 -> 2.25 ms.
 #include <algorithm>
 #include <mutex>
 #include <string>

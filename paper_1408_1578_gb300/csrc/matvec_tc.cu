@@ -12,24 +12,26 @@
 // FP32 accumulation in tensor memory.  The sound-hard operator (eq. 2 with
 // Maue's identity) is two operators over the same pairs, S on u = d/ds x and
 // C = -D' - i (omega^2 / eta) (n_i . n_j) S on x (n1 S n1 + n2 S n2 has the
-// entries (n_i . n_j) S_ij); up to 32 right-hand sides one pass evaluates both
-// from one phase, above that each has a pass of its own (both sets of operand
-// planes of 64 right-hand sides do not fit two stages of shared memory).
+// entries (n_i . n_j) S_ij); a pass of up to 40 right-hand sides evaluates both from
+// one phase, and where that takes more work than a pass of up to 64 for each, they
+// have passes of their own (joint_passes; the operand planes of both for 64
+// right-hand sides do not fit two stages of shared memory).
 // Work is split stream-K: the (128-row tile, 32-source tile) pairs form one
 // list and each CTA (one per SM) takes a contiguous range, cut into segments
-// that end at row-tile boundaries.  Warp roles (22 warps): 0-15 evaluate pair
-// entries into the stage ring, 16 issues the TMA loads of the right-hand sides,
-// of each tile's source geometry and of its Kress window, 17 issues the MMAs
-// (double-buffered accumulators), 18-21 drain finished accumulators into
-// per-segment partial sums, which a second kernel adds in a fixed order.  All
-// mbarrier waits are bounded (error flag, drain, TMEM freed on every path).
+// that end at row-tile boundaries.  Warp roles (24 warps, two of them only to fill
+// the last warpgroup): 0-15 evaluate pair entries into the stage ring, 16 issues the
+// TMA loads of the right-hand sides, of each tile's source geometry and of its
+// Kress window, 17 issues the MMAs (double-buffered accumulators), 18-21 drain
+// finished accumulators into per-segment partial sums, which a second kernel adds
+// in a fixed order.  All mbarrier waits are bounded (error flag, drain, TMEM freed
+// on every path).
 //
-// Bound: the producers' FP32 arithmetic (FMA pipe 75 % busy, ncu).  A lane keeps
-// one target and evaluates the entries of eight adjacent sources in packed FP32
+// Bound: the producers' FP32 arithmetic (FMA pipe 64 % busy, its heavy half 70 %,
+// ncu).  A lane keeps one target and evaluates the entries of eight adjacent sources in packed FP32
 // pairs (pair32.cuh), which issue half as often as scalar instructions, four
 // independent chains at a time; the sources are warp-uniform loads from a ring
 // filled three tiles ahead.  Measured (GB300), kernel alone: kite n = 32768, 64
-// right-hand sides 2.95 -> 2.44 ms (packed pairs in the former layout, a row
+// right-hand sides 2.95 -> 2.45 ms (packed pairs in the former layout, a row
 // per half warp: 2.97, bound by shared-memory cycles and by waits for the
 // source loads); ellipse n = 32768, 1 right-hand side, sound hard, 4.90 (S and
 // D' in two passes) -> 2.97 ms; two pairs at a time instead of four: 0.07 ms more.
@@ -54,8 +56,8 @@ constexpr int TBK = 32;      // sources per tile (32 bf16 = one 64-byte swizzle 
 // warps add it into their running sums.  The tensor core's FP32 accumulation
 // does not round to nearest: its error grows with the number of MMAs summed
 // into one accumulator (~2e-8 relative per MMA), so chunks of 256 sources keep
-// that bias near 2e-6 whatever n is, while the running sums (FP32 adds, rounded
-// to nearest) and the FP64 segment reduction add only unbiased rounding.
+// that bias near 2e-6 whatever n is, while the running sums and the segment
+// reduction (FP32 adds, rounded to nearest) add only unbiased rounding.
 constexpr int CK = 8;
 constexpr int WKW = TBM + TBK + 2;   // Kress window of a tile (+ alignment slack)
 // Source data (geometry, Kress window) are fetched this many tiles ahead, into
