@@ -18,15 +18,11 @@ def ctx():
     c.close()
 
 
-def test_amplitude_next_to_the_band(ctx):
-    """Unit columns give single entries; with eta small against omega they are H1 times plain
-    factors.  Their mean amplitude over the pairs with 16.4 < omega r < 17.4, the largest arguments
-    of the short series, is no further off than with two terms of P and Q (the leading dropped one
-    is 0.144 / x^4), and 3e-7 for the arithmetic: two special-function values of 1.2e-7, one and a
-    half of them in the amplitude, FP32 per-node factors (6e-8), and the bf16 hi + lo splits (up to
-    3e-6, but of either sign) averaged over a thousand distances."""
+def _entries_next_to_the_band(ctx, ratio):
+    """Products of unit columns over the exact entries, and omega r, of the pairs with
+    16.4 < omega r < 17.4 (the largest arguments of the short series) at eta = ratio omega."""
     n, omega, m = 4096, 64.0, 64
-    eta = omega * 1e-6
+    eta = omega * ratio
     c = geometry.ellipse(n, 1.0, 0.8)
     op = ctx.ellipse(1.0, 0.8).discretise(n, omega, eta=eta, bc="soft", precision="fp32")
     op.set_variant(2)
@@ -37,14 +33,33 @@ def test_amplitude_next_to_the_band(ctx):
     y = empty(m, n)
     op.apply(to_dev(X), y)
     got = to_host(y)[:, rows]
+    op.close()
     D, S = (operators.layer_rows(c, omega, rows, k)[:, cols].T for k in "DS")
     A = D - 1j * eta * S
     x = omega * np.hypot(*(c.z[rows][None, :, :] - c.z[cols][:, None, :]).transpose(2, 0, 1))
     pick = (x > 16.4) & (x < 17.4)
     assert pick.sum() > 1000
-    bias = np.mean(np.abs(got[pick]) / np.abs(A[pick])) - 1.0
-    assert abs(bias) < np.mean(0.144195556640625 / x[pick] ** 4) + 3e-7, bias
-    op.close()
+    return got[pick] / A[pick], x[pick]
+
+
+def test_amplitude_next_to_the_band(ctx):
+    """Unit columns give single entries; with eta small against omega they are H1 times plain
+    factors.  Their mean amplitude is no further off than with two terms of P and Q (the leading
+    dropped one is 0.144 / x^4), and 3e-7 for the arithmetic: two special-function values of
+    1.2e-7, one and a half of them in the amplitude, FP32 per-node factors (6e-8), and the bf16
+    hi + lo splits (up to 3e-6, but of either sign) averaged over a thousand distances."""
+    q, x = _entries_next_to_the_band(ctx, 1e-6)
+    bias = np.mean(np.abs(q)) - 1.0
+    assert abs(bias) < np.mean(0.144195556640625 / x ** 4) + 3e-7, bias
+
+
+@pytest.mark.parametrize("ratio", [1e6, 1e-6])
+def test_phase_next_to_the_band(ctx, ratio):
+    """The mean phase of H0 (eta large) and H1 (small): the argument 4e-7, sine and cosine 3.6e-7,
+    the third term of the phase 3e-7, and 4e-7 for the splits.  (Its second term is 1.5e-5 and
+    3.7e-5 there.)"""
+    q, _ = _entries_next_to_the_band(ctx, ratio)
+    assert abs(np.mean(np.angle(q))) < 1.5e-6, np.mean(np.angle(q))
 
 
 def test_infinite_density_gives_infinities(ctx):
